@@ -422,15 +422,30 @@ __device__ __noinline__ bool meets_aabb(const RayState& r, const int32_t Oloc[3]
     return true;
 }
 
+__device__ __forceinline__ float ray_norm(const RayState& r) {
+    return sqrtf(__fadd_rn(__fadd_rn(__fmul_rn(r.d[0], r.d[0]), __fmul_rn(r.d[1], r.d[1])), __fmul_rn(r.d[2], r.d[2])));
+}
+
 // With a view distance, a hit farther than it is a miss (FP64, fixed order).
+static __device__ __noinline__ bool within_view_f64(int32_t Ne, float de, float x, float y, float z, float view_dist) {
+    const double d0 = x, d1 = y, d2 = z;
+    const double dd = (double)Ne / (4096.0 * fabs((double)de)) * sqrt(d0 * d0 + d1 * d1 + d2 * d2);
+    return dd <= (double)view_dist;
+}
+
+// FP64 runs at about 2 operations per clock and SM here; the FP32 distance
+// (eight roundings, within 2^-20 of the FP64 one while |d| is in its normal
+// range) settles every hit that is not that close to the limit (the margin is
+// 2^-17).  Open world, 2560x1440: 814 -> 801 us a frame.
 __device__ __forceinline__ bool within_view(const SceneDev& S, const RayState& r, const HitRec& hit) {
-    if (S.view_dist <= 0.0f) return true;
-    double dd = 0.0;
-    if (hit.e < 3) {
-        const double d0 = r.d[0], d1 = r.d[1], d2 = r.d[2];
-        dd = (double)hit.Ne / (4096.0 * fabs((double)r.d[hit.e])) * sqrt(d0 * d0 + d1 * d1 + d2 * d2);
+    if (S.view_dist <= 0.0f || hit.e == 3) return true;
+    const float de = r.d[hit.e], dn = ray_norm(r);
+    const float est = (float)hit.Ne * (1.0f / 4096.0f) / fabsf(de) * dn;
+    if (dn > 0x1p-40f && dn < 0x1p40f) {
+        if (est < S.view_dist * (1.0f - 0x1p-17f)) return true;
+        if (est > S.view_dist * (1.0f + 0x1p-17f)) return false;
     }
-    return dd <= (double)S.view_dist;
+    return within_view_f64(hit.Ne, de, r.d[0], r.d[1], r.d[2], S.view_dist);
 }
 
 // Write the output record of a hit that trace_chunk found in the chunk region
@@ -463,10 +478,6 @@ __device__ __forceinline__ bool emit_hit(const SceneDev& S, const RayState& r, c
 __device__ __forceinline__ void emit_miss(uint4* __restrict__ out_hit, float* __restrict__ out_t, size_t pix) {
     out_hit[pix] = make_uint4(0u, 0u, 0u, 0xFFu | (7u << 16));
     out_t[pix] = __int_as_float(0x7F800000);
-}
-
-__device__ __forceinline__ float ray_norm(const RayState& r) {
-    return sqrtf(__fadd_rn(__fadd_rn(__fmul_rn(r.d[0], r.d[0]), __fmul_rn(r.d[1], r.d[1])), __fmul_rn(r.d[2], r.d[2])));
 }
 
 // The beam-pass bound of pixel (px, py) of a W x H view: the minimum over

@@ -17,6 +17,10 @@ constexpr uint32_t kNone = 0xFFFFFFFFu;
 constexpr uint32_t kResidentBit = 0x80000000u;
 constexpr int kFix = 12;            // camera origin fixed point: multiples of 2^-12
 constexpr int kMaxLevels = 10;      // log2(512) + 1
+// A device node's prefix words hold 24 bits of prefix and the child's mask
+// above them, except in a node of this side (2^kWideLevel voxels of its LOD).
+constexpr int kWideLevel = 9, kWideSide = 1 << kWideLevel;
+constexpr uint32_t kPrefixBits = 0xFFFFFFu;
 constexpr int kMaxImageHeight = 65535 * 8;  // 8-row casting blocks, at most 65535 in grid y
 
 // One (chunk, LOD) as resident on the device, and (per frame) the selected

@@ -14,6 +14,7 @@
 #include "aok_internal.h"
 #include "aok_select.cuh"
 #include "aok_trace.cuh"
+#include "aok_walk.cuh"
 
 using namespace aok;
 
@@ -50,15 +51,20 @@ __device__ __forceinline__ int32_t beam_bound_lut(const BeamLookup& b, int px, i
 // space in front of the nearest voxel they can meet.  At most 72 registers:
 // 7 blocks per SM (the loop needs no more; no spills).
 template <bool COUNT, bool BEAM = false>
-__global__ void __launch_bounds__(128, 7) cast_kernel(SceneDev S, CamDev C, const ChunkRef* __restrict__ frame,
+__global__ void __launch_bounds__(128, 7) cast_kernel(const __grid_constant__ SceneDev S,
+                                                   const __grid_constant__ CamDev C,
+                                                   const ChunkRef* __restrict__ frame,
                                                    uint4* __restrict__ out_hit, float* __restrict__ out_t,
                                                    uint32_t* __restrict__ counts, const BeamLookup beam) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int px = blockIdx.x * 16 + (warp & 1) * 8 + (lane & 7);
     const int py = blockIdx.y * 8 + (warp >> 1) * 4 + (lane >> 3);
+    const uint32_t lanes = __ballot_sync(0xFFFFFFFFu, px < C.W && py < C.H);
     if (px >= C.W || py >= C.H) return;
     const int32_t Dn = BEAM ? beam_bound_lut(beam, px, py) : 0;
-    trace_pixel<COUNT, false, BEAM>(S, C, frame, px, py, out_hit, out_t, counts, (size_t)py * C.W + px, nullptr, Dn);
+    const size_t pix = (size_t)py * C.W + px;
+    if (COUNT) trace_pixel<true, false, BEAM>(S, C, frame, px, py, out_hit, out_t, counts, pix, nullptr, Dn);
+    else cast_pixel<BEAM>(S, C, frame, px, py, out_hit, out_t, pix, Dn, lanes);
 }
 
 // The same casting with every pool index checked (CheckDev); BEAM: with the
@@ -109,8 +115,9 @@ __global__ void __launch_bounds__(256) cast_persistent(const __grid_constant__ B
             const int32_t local = (int32_t)(tile - vbeg);
             const int px = (local % tiles_x) * tw + (lane & (tw - 1));
             const int py = (local / tiles_x) * th + (lane >> P.tile_w_log);
+            const uint32_t lanes = __ballot_sync(0xFFFFFFFFu, px < v.cam.W && py < v.cam.H);
             if (px < v.cam.W && py < v.cam.H)
-                trace_pixel<false>(v.scene, v.cam, v.frame, px, py, v.hit, v.t, nullptr, (size_t)py * v.cam.W + px);
+                cast_pixel<false>(v.scene, v.cam, v.frame, px, py, v.hit, v.t, (size_t)py * v.cam.W + px, 0, lanes);
         }
     }
     // the last CTA to finish re-arms the counters for the next launch
@@ -145,11 +152,11 @@ __global__ void __launch_bounds__(128, 7) cast_grid(const __grid_constant__ Batc
     const int32_t local = (int32_t)(blk - v.tile_begin);
     const int px = (local % bw) * 2 * tw + (warp & 1) * tw + (lane & (tw - 1));
     const int py = (local / bw) * 2 * th + (warp >> 1) * th + (lane >> twl);
+    const uint32_t lanes = __ballot_sync(0xFFFFFFFFu, px < v.cam.W && py < v.cam.H);
     if (px < v.cam.W && py < v.cam.H) {
         // with a bound of 0 (no beam pass for this view) the march is the plain one
         const int32_t Dn = beam_bound(v.beam, P.beam_tag, v.cam.W, v.cam.H, px, py);
-        trace_pixel<false, false, true>(v.scene, v.cam, v.frame, px, py, v.hit, v.t, nullptr,
-                                        (size_t)py * v.cam.W + px, nullptr, Dn);
+        cast_pixel<true>(v.scene, v.cam, v.frame, px, py, v.hit, v.t, (size_t)py * v.cam.W + px, Dn, lanes);
     }
 }
 

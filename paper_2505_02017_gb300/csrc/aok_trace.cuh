@@ -347,7 +347,7 @@ __device__ __forceinline__ bool trace_chunk(const SceneDev& S, const ChunkRef& r
         const int rk = __popc(sj.y & ((1u << oct) - 1u));
         const uint64_t at = (uint64_t)sj.x + 3 + 2 * rk;
         if (out_of<CHECK>(at, ck ? ck->n_nodes : 0, ck, 1u)) return false;
-        idx += nodes[at];
+        idx += nodes[at] & (j - n == kWideLevel ? ~0u : kPrefixBits);
         if (COUNT) cnt.rbytes += rk * ((j - 1 == n + 2) ? 8u : 4u);  // the paper-format resolve
     }
     const int bit = (u0 & 3) + 4 * (u1 & 3) + 16 * (u2 & 3);

@@ -1,0 +1,587 @@
+// The casting kernels' voxel walk: the march of aok_trace.cuh (chunk grid,
+// then each chunk's sparse voxel DAG, Aokana Sec. 3.5) with every ordering
+// decision made in FP32 together with a bound on its error.  A decision closer
+// than its bound ends the fast walk, and the ray goes on in a second instance
+// of the same walk that settles such decisions by exact comparisons, so that
+// results stay those of the exact real ray.
+//
+// Why: the exact march spends two 32 x 32 -> 64-bit products (half-rate
+// multiplies) and a 64-bit compare on every comparison of plane crossings, and
+// compares again at every level it descends.  Here a crossing is one FMA, the
+// nearest of three and its distance from the second one are a minimum and
+// three compares, and a cell's coordinates at all levels are found at once
+// when an occupied cell is entered, so that descending costs no comparison.
+// Bound: instruction issue (about 70% of it) and the divergence of neighbour
+// rays (19 of 32 lanes).  Frames, exact march -> this walk: city 1920x1080
+// 484 -> 334 us, overview 3840x2160 743 -> 530, open world 2560x1440
+// 801 -> 557, 24 views 6404 -> 4278, 320x180 147 -> 83, 256x256 74 -> 54 us.
+//
+// Numbers.  The ray is taken in the frame mirrored so that d >= 0.  Its
+// parameter t counts from a base point on the ray, known to 2^-24 of a voxel:
+// an integer voxel B and a fraction x in [0, 1) per axis.  Plane j (in voxels
+// of the chunk's LOD, from the base's voxel) is crossed at
+// T = j g - x g, g = 1 / d.  With u = 2^-24: the approximate reciprocal is
+// within 2u of 1 / d, x and the product x g within u each, the FMA within u
+// of T, so |error of T| <= 3u T + 2u g; up to three steps T += g inside a
+// leaf block add u T each.  Two crossings are told apart when they differ by
+// more than eps (T + g_max), eps = 14 u (both errors, and the rounding of
+// that sum).  A coordinate x + T d at the entry of a cell, used for its
+// integer part, is then within eps (T + g_max) d_max as well (3u T d + 2u g d
+// from T, u each from the FMA, x and x - 1/2; g_max d_max >= 1) and is used
+// when it lies farther than that from every integer.
+#pragma once
+#include "aok_trace.cuh"
+
+namespace aok {
+
+constexpr float kWalkEps = 0x1.Cp-21f;
+constexpr float kZeroInv = 1e35f;       // 1 / d of a zero component: its planes lie past every other crossing
+constexpr uint32_t kMagicBits = 0x4B000000u;  // 2^23: kMagicBits | i is the float 2^23 + i for 0 <= i < 2^23
+constexpr float kRound = 12582912.0f;   // 1.5 * 2^23: adding it rounds to an integer
+// A base point farther back than this (voxels of the ray's largest component)
+// is replaced when an occupied cell is entered, which keeps the bounds small.
+constexpr float kRebase = 96.0f;
+
+template <class T>
+__device__ __forceinline__ T sel3(int e, T a, T b, T c) {
+    return e == 0 ? a : (e == 1 ? b : c);
+}
+
+__device__ __forceinline__ float rcp_approx(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// 2^n, |n| < 127
+__device__ __forceinline__ float pow2(int n) { return __int_as_float((127 + n) << 23); }
+
+struct WalkRay {
+    float ad[3], inv[3];  // |d|, 1 / |d|
+    float gmax, dmax;     // largest 1 / |d| of a moving axis, largest |d|
+};
+
+// Where a walk goes on: the chunk cell and the plane (e, Ne) it is entered or
+// continued at (e = 3: the origin; e < 0: the walk has not started).
+struct WalkAt {
+    int32_t cc[3], e, Ne;
+};
+
+// The decisions that FP32 leaves open, exactly (trace_chunk's comparisons and
+// its rules for ties): Na / |da| < Nb / |db| ...
+static __device__ __noinline__ bool exact_less(int32_t Na, float da, int32_t Nb, float db) {
+    int32_t ma, Ea, mb, Eb;
+    decompose(da, ma, Ea);
+    decompose(db, mb, Eb);
+    return tlt(Na, ma, Nb, mb, Eb - Ea);
+}
+// ... and the axis of the nearest of three exit planes, at a tie the higher one.
+static __device__ __noinline__ int exact_nearest(int32_t N0, int32_t N1, int32_t N2, float d0, float d1, float d2) {
+    const bool xy = exact_less(N0, d0, N1, d1);
+    return exact_less(xy ? N0 : N1, xy ? d0 : d1, N2, d2) ? (xy ? 0 : 1) : 2;
+}
+
+// Base point of the ray where it crosses plane (e, Ne) (e = 3: the origin):
+// voxel B and fraction x per axis of the mirrored world.  The quotient
+// Ne / |d_e| is carried as a sum of two floats (residual by FMA), so that the
+// point's error is below 2^-12 numerator units at any distance.  False if a
+// coordinate lies within 2^-10 units (2^-22 voxels) of a voxel plane; EXACT
+// then places it by comparison: a plane crossed no later than the base point
+// is passed.
+template <bool EXACT>
+__device__ __forceinline__ bool walk_base(const WalkRay& w, const int32_t Ow[3], int e, int32_t Ne, int32_t B[3],
+                                          float x[3]) {
+    float q1 = 0.0f, q2 = 0.0f;
+    const float ade = sel3(e, w.ad[0], w.ad[1], w.ad[2]);
+    if (e < 3) {
+        const float inv = sel3(e, w.inv[0], w.inv[1], w.inv[2]);
+        const float Nf = (float)Ne, Nl = (float)(Ne - (int32_t)Nf);
+        q1 = Nf * inv;
+        q2 = (__fmaf_rn(-q1, ade, Nf) + Nl) * inv;
+    }
+    bool clear = true;
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        const float p1 = q1 * w.ad[a];
+        const float p2 = __fmaf_rn(q2, w.ad[a], __fmaf_rn(q1, w.ad[a], -p1));
+        const int32_t i1 = __float2int_rd(p1);
+        float f = (p1 - (float)i1) + p2;
+        const int32_t i2 = __float2int_rd(f);
+        const bool plane = a == e;
+        const int32_t I = (int32_t)((uint32_t)Ow[a] + (uint32_t)(plane ? Ne : i1 + i2));
+        f = plane ? 0.0f : f - (float)i2;
+        float lo = (float)(I & 4095) + f;
+        B[a] = I >> kFix;
+        // exact where nothing moved the coordinate off the origin's (e = 3, a zero component) or it is the plane itself
+        if (!plane && e < 3 && w.ad[a] > 0.0f && !(fabsf(lo - 2048.0f) < 2048.0f - 0x1p-10f)) {
+            clear = false;
+            if (EXACT) {
+                const int32_t P = lo < 2048.0f ? B[a] : B[a] + 1;
+                const int32_t Np = (int32_t)(((uint32_t)P << kFix) - (uint32_t)Ow[a]);
+                const int32_t Bn = exact_less(Ne, ade, Np, w.ad[a]) ? P - 1 : P;
+                lo += 4096.0f * (float)(B[a] - Bn);
+                B[a] = Bn;
+            }
+        }
+        x[a] = lo * (1.0f / 4096.0f);
+    }
+    return clear;
+}
+
+// Cast the pixel's ray and write its record.  BEAM: restart past the beam
+// pass's bound Dn (0: none).  lanes: the warp's lanes that call it.  False
+// (never with EXACT; nothing written): undecided at `at`, where an EXACT walk
+// takes over.  The loops have one way out each, and the outer one is left by
+// all lanes together: a return from inside them cost the warp its convergence
+// (7 active lanes instead of 19, 2.5 times the time).
+template <bool EXACT, bool BEAM>
+__device__ __forceinline__ bool walk_pixel(const SceneDev& S, const CamDev& C, const ChunkRef* __restrict__ frame,
+                                           int px, int py, uint4* __restrict__ out_hit, float* __restrict__ out_t,
+                                           size_t pix, int32_t Dn, uint32_t lanes, WalkAt& at) {
+    RayState r;  // d and mir only
+    ray_dir(C, px, py, r.d);
+    r.mir = (r.d[0] < 0.0f ? 1u : 0u) | (r.d[1] < 0.0f ? 2u : 0u) | (r.d[2] < 0.0f ? 4u : 0u);
+    WalkRay w;
+    w.dmax = fmaxf(fmaxf(fabsf(r.d[0]), fabsf(r.d[1])), fabsf(r.d[2]));
+    // only ratios of the components matter: bring an unusual scale to a normal one
+    float scale = 1.0f;
+    if (!(w.dmax > 0x1p-40f)) scale = 0x1p100f;
+    if (w.dmax > 0x1p40f) scale = 0x1p-88f;
+    w.dmax *= scale;
+    w.gmax = 0.0f;
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        w.ad[a] = fabsf(r.d[a]) * scale;
+        w.inv[a] = w.ad[a] > 0.0f ? rcp_approx(w.ad[a]) : kZeroInv;
+        if (w.ad[a] > 0.0f) w.gmax = fmaxf(w.gmax, w.inv[a]);
+    }
+    const int cs = S.mlog + kFix;
+    int32_t Ow[3], Wfix[3];
+    bool inside = true;
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        Wfix[a] = S.grid[a] << cs;
+        Ow[a] = ((r.mir >> a) & 1u) ? Wfix[a] - C.O[a] : C.O[a];
+        inside = inside && Ow[a] >= 0 && Ow[a] < Wfix[a];
+    }
+    bool tie = EXACT;        // (a tie is possible: the hit's entry face is checked for it)
+    bool miss = false, undecided = false;
+    int e = 3;
+    int32_t Ne = 0;
+    const bool resumed = EXACT && at.e >= 0;
+    if (resumed) {
+        e = at.e;
+        Ne = at.Ne;
+    } else if (!inside) {
+        // enter the world box: latest entry plane against the earliest exit plane
+        float tin = -1.0f, tin2 = -1.0f, tout = 3.0e38f;
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            if (Ow[a] >= Wfix[a] || (w.ad[a] == 0.0f && Ow[a] < 0)) miss = true;
+            const float ti = Ow[a] < 0 ? (float)(-Ow[a]) * w.inv[a] : -1.0f;
+            tout = fminf(tout, (float)(Wfix[a] - Ow[a]) * w.inv[a]);
+            if (ti > tin) { tin2 = tin; tin = ti; e = a; }
+            else tin2 = fmaxf(tin2, ti);
+        }
+        if (tin > tout * (1.0f + kWalkEps)) {
+            miss = true;
+        } else if (!miss && !(tin < tout * (1.0f - kWalkEps) && tin2 < tin * (1.0f - kWalkEps))) {
+            undecided = true;
+            if (EXACT) {
+                e = -1;
+                int ex = 0;
+                for (int a = 0; a < 3; a++) {
+                    const int32_t O = sel3(a, Ow[0], Ow[1], Ow[2]);
+                    const float da = sel3(a, w.ad[0], w.ad[1], w.ad[2]);
+                    if (O < 0 && (e < 0 || exact_less(-sel3(e, Ow[0], Ow[1], Ow[2]), sel3(e, w.ad[0], w.ad[1], w.ad[2]), -O, da)))
+                        e = a;
+                    if (a > 0 && exact_less(sel3(a, Wfix[0], Wfix[1], Wfix[2]) - O, da,
+                                            sel3(ex, Wfix[0], Wfix[1], Wfix[2]) - sel3(ex, Ow[0], Ow[1], Ow[2]),
+                                            sel3(ex, w.ad[0], w.ad[1], w.ad[2])))
+                        ex = a;
+                }
+                miss = !exact_less(-sel3(e, Ow[0], Ow[1], Ow[2]), sel3(e, w.ad[0], w.ad[1], w.ad[2]),
+                                   sel3(ex, Wfix[0], Wfix[1], Wfix[2]) - sel3(ex, Ow[0], Ow[1], Ow[2]),
+                                   sel3(ex, w.ad[0], w.ad[1], w.ad[2]));
+            }
+        }
+        Ne = -sel3(e, Ow[0], Ow[1], Ow[2]);
+    }
+    if (BEAM && Dn > 0 && !miss && !resumed) {
+        // the beam restart of trace_pixel_t; where its order against the world
+        // box is undecided the march simply starts at the box
+        int as = 0;
+        if (w.ad[1] > w.ad[0]) as = 1;
+        if (w.ad[2] > fmaxf(w.ad[0], w.ad[1])) as = 2;
+        const int32_t O = sel3(as, Ow[0], Ow[1], Ow[2]);
+        const int32_t Nl = (int32_t)(((uint32_t)(Dn - 1) + (uint32_t)O) & ~4095u) - O;
+        if (Dn == INT_MAX || Nl >= sel3(as, Wfix[0], Wfix[1], Wfix[2]) - O) {
+            miss = true;  // nothing solid for this ray
+        } else if (Nl > 0) {
+            const float ts = (float)Nl * sel3(as, w.inv[0], w.inv[1], w.inv[2]);
+            const float te = e < 3 ? (float)Ne * sel3(e, w.inv[0], w.inv[1], w.inv[2]) : 0.0f;
+            float tout = 3.0e38f;
+#pragma unroll
+            for (int a = 0; a < 3; a++)
+                if (a != as) tout = fminf(tout, (float)(Wfix[a] - Ow[a]) * w.inv[a]);
+            if (ts > tout * (1.0f + kWalkEps)) {
+                miss = true;  // left the world box before the restart point
+            } else if (ts < tout * (1.0f - kWalkEps) && ts > te * (1.0f + kWalkEps)) {
+                e = as;
+                Ne = Nl;
+            }
+        }
+    }
+    at.e = -1;
+    int32_t B[3], cc[3];
+    float x[3];
+    undecided = !walk_base<EXACT>(w, Ow, e, Ne, B, x) || undecided;
+#pragma unroll
+    for (int a = 0; a < 3; a++) cc[a] = resumed ? at.cc[a] : max(0, min(B[a] >> S.mlog, S.grid[a] - 1));
+    undecided = !EXACT && undecided && !miss;
+    bool alive = !miss && !undecided, found = false;
+    int32_t u[3];
+    HitRec hit;
+    uint4 ra, rb;  // the current chunk's frame entry
+    const float dn = sqrtf(w.ad[0] * w.ad[0] + w.ad[1] * w.ad[1] + w.ad[2] * w.ad[2]);  // for the view distance
+    const uint32_t* __restrict__ nodes = S.nodes;
+    bool based = true;  // the base point lies on the entry of the current chunk
+    while (EXACT ? alive : __any_sync(lanes, alive)) {
+        bool traced = false;
+        if (alive) {
+#pragma unroll
+            for (int a = 0; a < 3; a++) u[a] = ((r.mir >> a) & 1u) ? S.grid[a] - 1 - cc[a] : cc[a];
+            const uint4* fr = reinterpret_cast<const uint4*>(
+                frame + ((size_t)u[0] + (size_t)S.grid[0] * ((size_t)u[1] + (size_t)S.grid[1] * u[2])));
+            ra = __ldg(fr);
+            rb = __ldg(fr + 1);
+            if (S.view_dist > 0.0f && e < 3) {
+                const float tent = (float)Ne * (1.0f / 4096.0f) * sel3(e, w.inv[0], w.inv[1], w.inv[2]);
+                if (tent * dn > S.view_dist * 1.00001f + 1.0f) alive = false;
+            }
+            if (alive && ra.x != kNone) {
+                // skip chunks whose solid-voxel AABB (grown by 1/16 voxel) the ray misses
+                const int32_t M = 1 << S.mlog;
+                const int32_t lo[3] = {(int32_t)(rb.x & 0xFFFFu), (int32_t)(rb.x >> 16), (int32_t)(rb.y & 0xFFFFu)};
+                const int32_t hi[3] = {(int32_t)(rb.y >> 16), (int32_t)(rb.z & 0xFFFFu), (int32_t)(rb.z >> 16)};
+                float tn = 0.0f, tf = 3.0e38f;
+#pragma unroll
+                for (int a = 0; a < 3; a++) {
+                    const bool m = (r.mir >> a) & 1u;
+                    const int32_t off = (cc[a] << S.mlog) - B[a];
+                    tn = fmaxf(tn, ((float)(off + (m ? M - hi[a] : lo[a])) - (x[a] + 0.0625f)) * w.inv[a]);
+                    tf = fminf(tf, ((float)(off + (m ? M - lo[a] : hi[a])) - (x[a] - 0.0625f)) * w.inv[a]);
+                }
+                traced = tn <= tf;
+            }
+        }
+        if (EXACT ? traced : __any_sync(lanes, traced)) {
+            // Voxel coordinates of the current cell at every level, in voxels
+            // of the LOD, axis a shifted left by a: the octant of level k is
+            // then bits k, k + 1, k + 2 of the three merged words.
+            bool go = traced, occ = false;
+            int n = 0, R = 3, k = 2;
+            float gtol = 0.0f, dmaxn = 0.0f;
+            uint32_t V0 = 0, V1 = 0, V2 = 0;
+            float Kp[3], gs[3], hp[3], xm[3], dv[3];
+            // {node, child mask} of the path's interior levels R .. 3; an
+            // EXACT walk keeps to the octree inside leaf blocks too (at a tie
+            // the cells visited depend on it) and holds level 2 as well
+            constexpr int kLow = EXACT ? 2 : 3;
+            uint2 st[kMaxLevels - kLow];
+            uint32_t pidx = 0, pm8 = 0, o = 0;
+            uint64_t lmu = 0;
+            // numerator of the plane at scaled coordinate P of axis a
+            auto plane = [&](int a, uint32_t P) -> int32_t {
+                return (((sel3(a, cc[0], cc[1], cc[2]) << S.mlog) + (int32_t)((P >> a) << n)) << kFix) -
+                       sel3(a, Ow[0], Ow[1], Ow[2]);
+            };
+            // crossing parameters and coordinates from the base point, the
+            // latter kept within the cell of coordinates V with bits `low` free
+            auto rebase = [&](uint32_t low) {
+                const float up = pow2(n), down = pow2(-n);
+                uint32_t J[3] = {V0, V1 >> 1, V2 >> 2};
+#pragma unroll
+                for (int a = 0; a < 3; a++) {
+                    const int32_t l = B[a] - (cc[a] << S.mlog);
+                    J[a] = (uint32_t)max((int32_t)(J[a] & ~low), min(l >> n, (int32_t)(J[a] | low)));
+                    const float xn = ((float)(l - (int32_t)(J[a] << n)) + x[a]) * down;
+                    const float g = w.inv[a] * up;
+                    gs[a] = g * (1.0f / (float)(1 << a));
+                    hp[a] = __fmaf_rn(-xn, g, gs[a]);
+                    xm[a] = xn - 0.5f;
+                    dv[a] = w.ad[a] * down;
+                    Kp[a] = __uint_as_float(kMagicBits | (J[a] << a));
+                }
+                V0 = J[0];
+                V1 = J[1] << 1;
+                V2 = J[2] << 2;
+            };
+            // octant of the level-k cell in its parent, stored order: bits k,
+            // k + 1, k + 2 of the three words merged (m = ~0 << k)
+            uint32_t m = ~0u;
+            auto octant = [&]() -> uint32_t {
+                const uint32_t hi = (V2 & (m << 2)) | (V1 & ~(m << 2));
+                return ((((hi & (m << 1)) | (V0 & ~(m << 1))) >> k) & 7u) ^ r.mir;
+            };
+            if (traced) {
+                n = (int)ra.y;
+                R = S.mlog - n;
+                gtol = kWalkEps * w.gmax * pow2(n);
+                dmaxn = w.dmax * pow2(-n);
+                pidx = ra.x;
+                pm8 = nodes[pidx] & 0xFFu;
+                if (!based) undecided = !walk_base<EXACT>(w, Ow, e, Ne, B, x) && !EXACT;
+                if (!EXACT) { at.e = e; at.Ne = Ne; }
+                rebase((1u << R) - 1u);
+                st[R - kLow] = make_uint2(pidx, pm8);
+                k = R - 1;
+                m = ~0u << k;
+                o = octant();
+                occ = (pm8 >> o) & 1u;
+            }
+            while (go) {
+                while (occ && k > (EXACT ? 0 : 2)) {
+                    // into the occupied cell: its node and child mask
+                    if (EXACT && k == 1) {
+                        // the voxel bits of a leaf block's 2x2x2 group
+                        const uint64_t v = lmu >> ((o & 1u) * 2 + (o & 2u) * 4 + (o & 4u) * 8);
+                        pm8 = (uint32_t)((v & 3) | ((v >> 2) & 0xC) | ((v >> 12) & 0x30) | ((v >> 14) & 0xC0));
+                    } else {
+                        const uint2 ch = __ldg(reinterpret_cast<const uint2*>(
+                            nodes + pidx + 2 + 2 * __popc(pm8 & ~(~0u << o))));
+                        pidx = ch.x;
+                        pm8 = ch.y >> 24;
+                        if (k == kWideLevel - 1) pm8 = nodes[pidx] & 0xFFu;
+                        if (EXACT && k == 2) {
+                            lmu = __ldg(S.leaves + pidx);
+                            uint64_t q = lmu | (lmu >> 1);
+                            q |= q >> 4;
+                            q |= q >> 16;  // the occupied groups
+                            pm8 = (uint32_t)((q & 1) | ((q >> 1) & 2) | ((q >> 6) & 4) | ((q >> 7) & 8) |
+                                             ((q >> 28) & 16) | ((q >> 29) & 32) | ((q >> 34) & 64) | ((q >> 35) & 128));
+                        }
+                        st[k - kLow] = make_uint2(pidx, pm8);
+                    }
+                    k--;
+                    m = ~0u << k;
+                    o = octant();
+                    occ = (pm8 >> o) & 1u;
+                }
+                float tm = 0.0f;
+                if (EXACT) {
+                    go = !occ;  // occupied at level 0: the hit
+                } else if (occ) {
+                    // a 4^3 leaf block: voxel by voxel, to a set bit or out of
+                    // it; i: bit of the voxel in the mirrored frame
+                    lmu = __ldg(S.leaves + __ldg(nodes + pidx + 2 + 2 * __popc(pm8 & ~(~0u << o))));
+                    float T0 = __fmaf_rn(__uint_as_float(V0 | kMagicBits) - Kp[0], gs[0], hp[0]);
+                    float T1 = __fmaf_rn(__uint_as_float(V1 | 1u | kMagicBits) - Kp[1], gs[1], hp[1]);
+                    float T2 = __fmaf_rn(__uint_as_float(V2 | 3u | kMagicBits) - Kp[2], gs[2], hp[2]);
+                    uint32_t i = (V0 & 3u) | ((V1 & 6u) << 1) | ((V2 & 12u) << 2), inc = 0;
+                    const uint32_t mi = ((r.mir & 1u) | ((r.mir & 2u) << 1) | ((r.mir & 4u) << 2)) * 3u;
+                    for (;;) {
+                        const uint32_t j = i ^ mi;
+                        occ = (((j & 32u) ? (uint32_t)(lmu >> 32) : (uint32_t)lmu) >> (j & 31u)) & 1u;
+                        if (occ) break;
+                        tm = fminf(fminf(T0, T1), T2);
+                        const float thr = __fmaf_rn(tm, 1.0f + kWalkEps, gtol);
+                        const bool p0 = T0 <= thr, p1 = T1 <= thr, p2 = T2 <= thr;
+                        undecided = undecided || (p0 ? p1 || p2 : p1 == p2);
+                        if (p0) { T0 = T0 + gs[0]; inc = 1u; }
+                        else if (p1) { T1 = __fmaf_rn(gs[1], 2.0f, T1); inc = 4u; }
+                        else { T2 = __fmaf_rn(gs[2], 4.0f, T2); inc = 16u; }
+                        i += inc;
+                        if (!(i & (3u * inc))) break;  // left the block
+                    }
+                    if (occ) {
+                        if (inc) e = inc == 1u ? 0 : (inc == 4u ? 1 : 2);
+                        V0 = (V0 & ~3u) | (i & 3u);
+                        V1 = (V1 & ~6u) | ((i >> 1) & 6u);
+                        V2 = (V2 & ~12u) | ((i >> 2) & 12u);
+                        go = false;  // the hit
+                    }
+                }
+                // leave empty cells through their nearest exit face until an
+                // occupied one or the chunk's end
+                uint32_t m0 = m;
+                while (!occ) {
+                    const uint32_t E0 = V0 | ~m | kMagicBits, E1 = V1 | ~(m << 1) | kMagicBits,
+                                   E2 = V2 | ~(m << 2) | kMagicBits;
+                    const float T0 = __fmaf_rn(__uint_as_float(E0) - Kp[0], gs[0], hp[0]);
+                    const float T1 = __fmaf_rn(__uint_as_float(E1) - Kp[1], gs[1], hp[1]);
+                    const float T2 = __fmaf_rn(__uint_as_float(E2) - Kp[2], gs[2], hp[2]);
+                    tm = fminf(fminf(T0, T1), T2);
+                    const float thr = __fmaf_rn(tm, 1.0f + kWalkEps, gtol);
+                    bool p0 = T0 <= thr, p1 = T1 <= thr;
+                    const bool p2 = T2 <= thr;
+                    const bool amb = p0 ? p1 || p2 : p1 == p2;
+                    if (EXACT) {
+                        if (amb) {
+                            const int a = exact_nearest(plane(0, E0 + (1u - kMagicBits)), plane(1, E1 + (1u - kMagicBits)),
+                                                        plane(2, E2 + (1u - kMagicBits)), w.ad[0], w.ad[1], w.ad[2]);
+                            p0 = a == 0;
+                            p1 = a == 1;
+                            tm = sel3(a, T0, T1, T2);
+                        }
+                    } else {
+                        undecided = undecided || amb;
+                    }
+                    uint32_t nv;
+                    if (p0) { nv = V0 = E0 + (1u - kMagicBits); e = 0; }
+                    else if (p1) { nv = V1 = E1 + (1u - kMagicBits); e = 1; }
+                    else { nv = V2 = E2 + (1u - kMagicBits); e = 2; }
+                    m0 = m;
+                    // the level of the cell entered: k for a sibling, else
+                    // that of the lowest set bit (the parent was left)
+                    const int K = __ffs((int)nv) - 1 - e;
+                    if (K >= R) { go = false; break; }  // left the chunk
+                    if (K != k) {
+                        const uint2 par = st[K + 1 - kLow];
+                        pidx = par.x;
+                        pm8 = par.y;
+                    }
+                    k = K;
+                    m = ~0u << k;
+                    o = octant();
+                    occ = (pm8 >> o) & 1u;
+                }
+                if (go) {
+                    // the entered cell's coordinates below the level it was
+                    // left at (the crossed axis' are zero: it is on a face);
+                    // at a tie, below the level it was entered at
+                    if (EXACT) m0 = m;
+                    const float lim = 0.5f - __fmaf_rn(tm, kWalkEps, gtol) * dmaxn;
+                    const float x0 = __fmaf_rn(tm, dv[0], xm[0]), x1 = __fmaf_rn(tm, dv[1], xm[1]),
+                                x2 = __fmaf_rn(tm, dv[2], xm[2]);
+                    const float r0 = (x0 + kRound) - kRound, r1 = (x1 + kRound) - kRound, r2 = (x2 + kRound) - kRound;
+                    const bool clear = fabsf(x0 - r0) < (e == 0 ? 1.0f : lim) && fabsf(x1 - r1) < (e == 1 ? 1.0f : lim) &&
+                                       fabsf(x2 - r2) < (e == 2 ? 1.0f : lim);
+                    if (tm * w.dmax > kRebase || !clear) {
+                        // far from the base point, or next to a voxel plane: a new base here
+                        const int32_t Nt = plane(e, sel3(e, V0, V1, V2));
+                        if (!EXACT && !undecided) { at.e = e; at.Ne = Nt; }
+                        undecided = (!walk_base<EXACT>(w, Ow, e, Nt, B, x) && !EXACT) || undecided;
+                        rebase(~m0);
+                    } else {
+                        const uint32_t k0 = e == 0 ? ~0u : m0, k1 = e == 1 ? ~0u : m0 << 1, k2 = e == 2 ? ~0u : m0 << 2;
+                        V0 = (V0 & k0) | (__float_as_uint(r0 + Kp[0]) & ~k0);
+                        V1 = (V1 & k1) | (__float_as_uint(__fmaf_rn(r1, 2.0f, Kp[1])) & ~k1);
+                        V2 = (V2 & k2) | (__float_as_uint(__fmaf_rn(r2, 4.0f, Kp[2])) & ~k2);
+                    }
+                }
+            }
+            if (undecided) {
+                if (!EXACT && alive) {
+#pragma unroll
+                    for (int a = 0; a < 3; a++) at.cc[a] = cc[a];
+                    alive = false;
+                }
+            } else if (traced && occ) {
+                hit.c[0] = (int32_t)V0;
+                hit.c[1] = (int32_t)(V1 >> 1);
+                hit.c[2] = (int32_t)(V2 >> 2);
+                hit.e = e;
+                // depth-first index (Sec. 3.3), as in trace_chunk
+                const uint32_t side = (1u << R) - 1u;
+                const uint32_t u0 = (r.mir & 1u) ? side - V0 : V0;
+                const uint32_t u1 = (r.mir & 2u) ? side - (V1 >> 1) : V1 >> 1;
+                const uint32_t u2 = (r.mir & 4u) ? side - (V2 >> 2) : V2 >> 2;
+                uint32_t idx = 0;
+                for (int j = R; j >= 3; j--) {
+                    const int sh = j - 1;
+                    const uint32_t oct = ((u0 >> sh) & 1u) | (((u1 >> sh) & 1u) << 1) | (((u2 >> sh) & 1u) << 2);
+                    const uint2 sj = st[j - kLow];
+                    idx += nodes[sj.x + 3 + 2 * __popc(sj.y & ((1u << oct) - 1u))] & (j == kWideLevel ? ~0u : kPrefixBits);
+                }
+                const int bit = (int)((u0 & 3u) + 4 * (u1 & 3u) + 16 * (u2 & 3u));
+                hit.idx = idx + (uint32_t)__popcll(lmu & ((1ull << bit) - 1ull));
+                found = true;
+                alive = false;
+            }
+        }
+        if (alive && !traced) {
+            // over this chunk cell: its nearest exit face
+            float T[3];
+#pragma unroll
+            for (int a = 0; a < 3; a++)
+                T[a] = __fmaf_rn((float)(((cc[a] + 1) << S.mlog) - B[a]), w.inv[a], -x[a] * w.inv[a]);
+            const float thr = __fmaf_rn(fminf(fminf(T[0], T[1]), T[2]), 1.0f + kWalkEps, kWalkEps * w.gmax);
+            const bool p0 = T[0] <= thr, p1 = T[1] <= thr, p2 = T[2] <= thr;
+            const int en = p0 ? 0 : (p1 ? 1 : 2);
+            if (p0 ? p1 || p2 : p1 == p2) {
+                if (EXACT) {
+                    e = exact_nearest(((cc[0] + 1) << cs) - Ow[0], ((cc[1] + 1) << cs) - Ow[1],
+                                      ((cc[2] + 1) << cs) - Ow[2], w.ad[0], w.ad[1], w.ad[2]);
+                } else {
+#pragma unroll
+                    for (int a = 0; a < 3; a++) at.cc[a] = cc[a];
+                    at.e = e;
+                    at.Ne = Ne;
+                    undecided = true;
+                    alive = false;
+                }
+            } else {
+                e = en;
+            }
+        }
+        if (alive) {
+            based = false;
+            cc[0] += e == 0;
+            cc[1] += e == 1;
+            cc[2] += e == 2;
+            const int32_t ce = sel3(e, cc[0], cc[1], cc[2]);
+            if (ce >= sel3(e, S.grid[0], S.grid[1], S.grid[2])) alive = false;
+            Ne = (ce << cs) - sel3(e, Ow[0], Ow[1], Ow[2]);
+        }
+    }
+    if (!EXACT && undecided) return false;
+    if (found) {
+        const int n = (int)ra.y;
+        hit.Ne = 0;
+        if (e < 3)  // the voxel's face that the ray enters through
+            hit.Ne = (((sel3(e, cc[0], cc[1], cc[2]) << S.mlog) + (sel3(e, hit.c[0], hit.c[1], hit.c[2]) << n)) << kFix) -
+                     sel3(e, Ow[0], Ow[1], Ow[2]);
+        if (EXACT && tie && (e == 1 || e == 2)) {
+            // entered through an edge or a corner: the lowest of its axes (lowest_entry_face)
+            const int32_t Nh = hit.Ne;
+            const float de = sel3(e, w.ad[0], w.ad[1], w.ad[2]);
+            for (int b = e - 1; b >= 0; b--) {
+                const float db = b ? w.ad[1] : w.ad[0];
+                const int32_t Nb = ((((b ? cc[1] : cc[0]) << S.mlog) + ((b ? hit.c[1] : hit.c[0]) << n)) << kFix) -
+                                   (b ? Ow[1] : Ow[0]);
+                if (db > 0.0f && !exact_less(Nh, de, Nb, db) && !exact_less(Nb, db, Nh, de)) {
+                    hit.e = b;
+                    hit.Ne = Nb;
+                }
+            }
+        }
+        ChunkRef ref;
+        ref.lod = ra.y;
+        ref.mat_base = (uint64_t)ra.z | (uint64_t)ra.w << 32;
+        ref.nblocks = rb.w;
+        found = emit_hit(S, r, ref, u, hit, ray_norm(r), out_hit, out_t, pix);
+    }
+    if (!found) emit_miss(out_hit, out_t, pix);
+    return true;
+}
+
+// The rest of an undecided ray.  Out of line: about one ray in three thousand
+// needs it, and inside the walk its comparisons cost every ray registers.
+template <bool BEAM>
+__device__ __noinline__ void walk_rest(const SceneDev& S, const CamDev& C, const ChunkRef* __restrict__ frame, int px,
+                                       int py, uint4* __restrict__ out_hit, float* __restrict__ out_t, size_t pix,
+                                       int32_t Dn, WalkAt at) {
+    walk_pixel<true, BEAM>(S, C, frame, px, py, out_hit, out_t, pix, Dn, 0u, at);
+}
+
+template <bool BEAM>
+__device__ __forceinline__ void cast_pixel(const SceneDev& S, const CamDev& C, const ChunkRef* __restrict__ frame,
+                                           int px, int py, uint4* __restrict__ out_hit, float* __restrict__ out_t,
+                                           size_t pix, int32_t Dn, uint32_t lanes) {
+    WalkAt at;
+    if (!walk_pixel<false, BEAM>(S, C, frame, px, py, out_hit, out_t, pix, Dn, lanes, at))
+        walk_rest<BEAM>(S, C, frame, px, py, out_hit, out_t, pix, Dn, at);
+}
+
+}  // namespace aok

@@ -5,10 +5,8 @@ from dataclasses import replace
 import numpy as np
 import pytest
 
-import oracle as orc
 import scenegen as sg
-from gpu_util import compare, decode
-from worlds import HAND32
+from worlds import HAND32, MED64, MULTI32
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -43,4 +41,57 @@ def test_view_distance_at_the_limit(ctx, rel):
     found = bool((int(hit[0, 0, 3]) >> 19) & 1)
     assert found == (20.5 <= vd)
     assert float(t[0, 0]) == (20.5 if found else np.inf)
+    sc.destroy()
+
+
+# The FP32 walk against the exact march (aok_render_counted runs it), every
+# pixel of every record: generic views, and directions and origins on voxel
+# and chunk planes, where crossings tie.
+WALK_WORLDS = [replace(HAND32, name="chunk8", seed=5, wx=64, wy=64, wz=64, chunk=8, n_lods=1, octaves=3, period0=32,
+                       h_min=8, h_max=40, crust=2, n_boxes=12, box_min=2, box_max=9),
+               MULTI32, MED64, replace(MULTI32, name="multi32far", view_dist=60.0), sg.city(2, 1024)]
+WALK_DIRS = [(1.0, 1.0, -1.0), (-1.0, 2.0, -2.0), (1.0, -1.0, -0.5), (1.0, 0.0, -1.0), (0.0, 0.0, -1.0), (1.0, 1e-6, -0.2)]
+
+
+def _equal_to_march(ctx, sc, cam, tau):
+    hit, t = _render(ctx, sc, cam, tau)
+    hit2, t2 = aok.alloc_frame(cam.W, cam.H)
+    counts = torch.zeros((cam.H, cam.W, 3), dtype=torch.int32, device="cuda")
+    aok.render_counted(ctx, sc, cam, tau, hit2, t2, counts)
+    torch.cuda.synchronize()
+    assert torch.equal(hit, hit2) and torch.equal(t.view(torch.int32), t2.view(torch.int32))
+    return float(((hit[..., 3] >> 19) & 1).float().mean())
+
+
+@pytest.mark.parametrize("beam", [0, 1])
+@pytest.mark.parametrize("spec", WALK_WORLDS, ids=lambda s: s.name)
+def test_walk_equals_exact_march(ctx, spec, beam):
+    w = sg.World(spec)
+    sc = aok.Scene.from_world(ctx, w)
+    cams = [sg.orbit_camera(spec, 3 + s, 211 + s, 97 + s, radius=1.3 * spec.wx) for s in range(2)]
+    cams += [sg.ground_camera(w, s, 203, 117, z_lo=3, z_hi=max(6, spec.wz // 16)) for s in range(2)]
+    for d in WALK_DIRS:
+        cams.append(sg.make_camera((spec.wx / 2, spec.wy / 2, spec.wz * 0.75), d, 63, 41))
+        cams.append(sg.make_camera((-5.0, spec.wy / 4, spec.wz * 0.75 + 0.25), d, 33, 64))
+        cams.append(sg.make_camera((spec.wx * 0.75, spec.wy / 2, spec.wz + 8.0), d, 71, 44))
+    aok.beam_tune(ctx, 8, 2, 0 if beam else 1 << 40, 0)
+    hits = sum(_equal_to_march(ctx, sc, c, tau) for c in cams for tau in (1.0, 3.0))
+    aok.beam_tune(ctx)
+    assert hits > 1.0
+    sc.destroy()
+
+
+@pytest.mark.parametrize("scale", [2.0 ** -80, 2.0 ** -41, 2.0 ** 41, 2.0 ** 60])
+def test_walk_of_scaled_directions(ctx, scale):
+    # only the ratios of a direction's components matter to the walk
+    w = sg.World(MED64)
+    sc = aok.Scene.from_world(ctx, w)
+    cam = sg.ground_camera(w, 4, 160, 90, z_lo=4, z_hi=40)
+    want, _ = _render(ctx, sc, cam, 1.5)
+    cam.R = (cam.R.astype(np.float64) * np.array([1.0, 1.0, scale])).astype(np.float32)
+    cam.tan_half_fovy = np.float32(float(cam.tan_half_fovy) * scale)
+    # u and v scale with tan_half_fovy, the view axis with its column: the same rays, longer or shorter
+    got, _ = _render(ctx, sc, cam, 1.5 / scale)
+    assert torch.equal(want, got)
+    _equal_to_march(ctx, sc, cam, 1.5 / scale)
     sc.destroy()

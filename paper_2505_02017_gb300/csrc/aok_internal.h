@@ -63,10 +63,10 @@ struct CamDev {
     int32_t W, H;
     int32_t O[3];           // origin * 2^kFix (exact)
     float of[3];            // origin as float
-    float planes[4][4];     // view-pyramid side planes: n . (p - o) <= 0 inside (n, unused)
+    float planes[4][3];     // view-pyramid side planes: n . (p - o) <= 0 inside
     double sf;              // StreamingFactor for Eq. 1
     float aspect;           // (float)W / (float)H, one IEEE rounding
-    float pad;
+    float rW, rH;           // 1 / (float)W, 1 / (float)H, one IEEE rounding each
 };
 
 // Device buffers of the tile-chunk pipeline (Sec. 3.5) for one resolution.

@@ -130,6 +130,8 @@ int make_cam(aok_ctx* ctx, const Scene* sc, const aok_camera* cam, double tau, C
     out->W = cam->width;
     out->H = cam->height;
     out->aspect = (float)cam->width / (float)cam->height;  // the ray's W / H: one IEEE binary32 division
+    out->rW = 1.0f / (float)cam->width;
+    out->rH = 1.0f / (float)cam->height;
     for (int a = 0; a < 3; a++) {
         const double o = cam->origin[a];
         if (!std::isfinite(o) || std::fabs(o) >= 131072.0) return AOK_E_INVALID;
@@ -162,7 +164,6 @@ int make_cam(aok_ctx* ctx, const Scene* sc, const aok_camera* cam, double tau, C
         if (s * dot < 0) for (int i = 0; i < 3; i++) n[i] = -n[i];
         double len = std::sqrt(n[0] * n[0] + n[1] * n[1] + n[2] * n[2]);
         for (int i = 0; i < 3; i++) out->planes[p][i] = len > 0 ? (float)(n[i] / len) : 0.0f;
-        out->planes[p][3] = 0.0f;
     }
     // StreamingFactor from the pixel threshold (fixed FP64 operation order)
     const double fpx = (double)cam->height / (2.0 * (double)cam->tan_half_fovy);

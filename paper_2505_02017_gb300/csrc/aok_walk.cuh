@@ -138,20 +138,26 @@ template <bool EXACT, bool BEAM>
 __device__ __forceinline__ bool walk_pixel(const SceneDev& S, const CamDev& C, const ChunkRef* __restrict__ frame,
                                            int px, int py, uint4* __restrict__ out_hit, float* __restrict__ out_t,
                                            size_t pix, int32_t Dn, uint32_t lanes, WalkAt& at) {
-    RayState r;  // d and mir only
-    ray_dir(C, px, py, r.d);
-    r.mir = (r.d[0] < 0.0f ? 1u : 0u) | (r.d[1] < 0.0f ? 2u : 0u) | (r.d[2] < 0.0f ? 4u : 0u);
+    float d[3];
+    ray_dir(C, px, py, d);
+    const uint32_t mir = (d[0] < 0.0f ? 1u : 0u) | (d[1] < 0.0f ? 2u : 0u) | (d[2] < 0.0f ? 4u : 0u);
+    bool undecided = false, miss = false, odd = false;
+    // Only ratios of the components matter to the walk: EXACT brings an
+    // unusual scale to a normal one, the fast walk leaves such a ray to it.
     WalkRay w;
-    w.dmax = fmaxf(fmaxf(fabsf(r.d[0]), fabsf(r.d[1])), fabsf(r.d[2]));
-    // only ratios of the components matter: bring an unusual scale to a normal one
+    w.dmax = fmaxf(fmaxf(fabsf(d[0]), fabsf(d[1])), fabsf(d[2]));
     float scale = 1.0f;
-    if (!(w.dmax > 0x1p-40f)) scale = 0x1p100f;
-    if (w.dmax > 0x1p40f) scale = 0x1p-88f;
-    w.dmax *= scale;
+    if (EXACT) {
+        if (!(w.dmax > 0x1p-40f)) scale = 0x1p100f;
+        if (w.dmax > 0x1p40f) scale = 0x1p-88f;
+        w.dmax *= scale;
+    } else {
+        odd = !(w.dmax > 0x1p-40f && w.dmax < 0x1p40f);
+    }
     w.gmax = 0.0f;
 #pragma unroll
     for (int a = 0; a < 3; a++) {
-        w.ad[a] = fabsf(r.d[a]) * scale;
+        w.ad[a] = EXACT ? fabsf(d[a]) * scale : fabsf(d[a]);
         w.inv[a] = w.ad[a] > 0.0f ? rcp_approx(w.ad[a]) : kZeroInv;
         if (w.ad[a] > 0.0f) w.gmax = fmaxf(w.gmax, w.inv[a]);
     }
@@ -161,11 +167,9 @@ __device__ __forceinline__ bool walk_pixel(const SceneDev& S, const CamDev& C, c
 #pragma unroll
     for (int a = 0; a < 3; a++) {
         Wfix[a] = S.grid[a] << cs;
-        Ow[a] = ((r.mir >> a) & 1u) ? Wfix[a] - C.O[a] : C.O[a];
+        Ow[a] = ((mir >> a) & 1u) ? Wfix[a] - C.O[a] : C.O[a];
         inside = inside && Ow[a] >= 0 && Ow[a] < Wfix[a];
     }
-    bool tie = EXACT;        // (a tie is possible: the hit's entry face is checked for it)
-    bool miss = false, undecided = false;
     int e = 3;
     int32_t Ne = 0;
     const bool resumed = EXACT && at.e >= 0;
@@ -207,59 +211,64 @@ __device__ __forceinline__ bool walk_pixel(const SceneDev& S, const CamDev& C, c
         }
         Ne = -sel3(e, Ow[0], Ow[1], Ow[2]);
     }
+    bool restarted = false;
     if (BEAM && Dn > 0 && !miss && !resumed) {
-        // the beam restart of trace_pixel_t; where its order against the world
-        // box is undecided the march simply starts at the box
+        // the beam restart of trace_pixel_t (from the box, if that order is undecided)
         int as = 0;
         if (w.ad[1] > w.ad[0]) as = 1;
         if (w.ad[2] > fmaxf(w.ad[0], w.ad[1])) as = 2;
         const int32_t O = sel3(as, Ow[0], Ow[1], Ow[2]);
         const int32_t Nl = (int32_t)(((uint32_t)(Dn - 1) + (uint32_t)O) & ~4095u) - O;
-        if (Dn == INT_MAX || Nl >= sel3(as, Wfix[0], Wfix[1], Wfix[2]) - O) {
+        if (Dn == INT_MAX || Nl >= (sel3(as, S.grid[0], S.grid[1], S.grid[2]) << cs) - O) {
             miss = true;  // nothing solid for this ray
-        } else if (Nl > 0) {
-            const float ts = (float)Nl * sel3(as, w.inv[0], w.inv[1], w.inv[2]);
-            const float te = e < 3 ? (float)Ne * sel3(e, w.inv[0], w.inv[1], w.inv[2]) : 0.0f;
-            float tout = 3.0e38f;
-#pragma unroll
-            for (int a = 0; a < 3; a++)
-                if (a != as) tout = fminf(tout, (float)(Wfix[a] - Ow[a]) * w.inv[a]);
-            if (ts > tout * (1.0f + kWalkEps)) {
-                miss = true;  // left the world box before the restart point
-            } else if (ts < tout * (1.0f - kWalkEps) && ts > te * (1.0f + kWalkEps)) {
-                e = as;
-                Ne = Nl;
-            }
+        } else if (Nl > 0 && (e == 3 || (float)Nl * sel3(as, w.inv[0], w.inv[1], w.inv[2]) >
+                                            (float)Ne * sel3(e, w.inv[0], w.inv[1], w.inv[2]) * (1.0f + kWalkEps))) {
+            e = as;
+            Ne = Nl;
+            restarted = true;
         }
     }
-    at.e = -1;
+    int eb = -1;  // base point's plane is (eb, Ne); < 0: the walk has not started
     int32_t B[3], cc[3];
     float x[3];
-    undecided = !walk_base<EXACT>(w, Ow, e, Ne, B, x) || undecided;
+    const bool clear = walk_base<EXACT>(w, Ow, e, Ne, B, x);
+    bool outside = false;
 #pragma unroll
-    for (int a = 0; a < 3; a++) cc[a] = resumed ? at.cc[a] : max(0, min(B[a] >> S.mlog, S.grid[a] - 1));
-    undecided = !EXACT && undecided && !miss;
+    for (int a = 0; a < 3; a++) {
+        cc[a] = resumed ? at.cc[a] : B[a] >> S.mlog;
+        outside = outside || (uint32_t)cc[a] >= (uint32_t)S.grid[a];
+        if (EXACT) cc[a] = max(0, min(cc[a], S.grid[a] - 1));  // (entered through an edge of the box)
+    }
+    if (restarted && outside && (EXACT || clear)) miss = true;  // left the world box before the restart point
+    undecided = !EXACT && (odd || (!miss && (undecided || outside || !clear)));
     bool alive = !miss && !undecided, found = false;
-    int32_t u[3];
     HitRec hit;
-    uint4 ra, rb;  // the current chunk's frame entry
-    const float dn = sqrtf(w.ad[0] * w.ad[0] + w.ad[1] * w.ad[1] + w.ad[2] * w.ad[2]);  // for the view distance
+    // the current chunk cell's entry of the frame table
+    auto chunk_entry = [&](int32_t u[3]) -> const uint4* {
+#pragma unroll
+        for (int a = 0; a < 3; a++) u[a] = ((mir >> a) & 1u) ? S.grid[a] - 1 - cc[a] : cc[a];
+        return reinterpret_cast<const uint4*>(
+            frame + ((uint32_t)u[0] + (uint32_t)S.grid[0] * ((uint32_t)u[1] + (uint32_t)S.grid[1] * (uint32_t)u[2])));
+    };
     const uint32_t* __restrict__ nodes = S.nodes;
     bool based = true;  // the base point lies on the entry of the current chunk
     while (EXACT ? alive : __any_sync(lanes, alive)) {
         bool traced = false;
+        uint32_t root = kNone, lod = 0;
         if (alive) {
-#pragma unroll
-            for (int a = 0; a < 3; a++) u[a] = ((r.mir >> a) & 1u) ? S.grid[a] - 1 - cc[a] : cc[a];
-            const uint4* fr = reinterpret_cast<const uint4*>(
-                frame + ((size_t)u[0] + (size_t)S.grid[0] * ((size_t)u[1] + (size_t)S.grid[1] * u[2])));
-            ra = __ldg(fr);
-            rb = __ldg(fr + 1);
+            int32_t u[3];
+            const uint4* fr = chunk_entry(u);
+            const uint4 ra = __ldg(fr), rb = __ldg(fr + 1);
+            root = ra.x;
+            lod = ra.y;
             if (S.view_dist > 0.0f && e < 3) {
+                const float dn = sqrtf(w.ad[0] * w.ad[0] + w.ad[1] * w.ad[1] + w.ad[2] * w.ad[2]);
                 const float tent = (float)Ne * (1.0f / 4096.0f) * sel3(e, w.inv[0], w.inv[1], w.inv[2]);
                 if (tent * dn > S.view_dist * 1.00001f + 1.0f) alive = false;
             }
-            if (alive && ra.x != kNone) {
+            if (BEAM && restarted) {
+                traced = alive && root != kNone;  // restarted in this chunk, next to solid voxels: no use asking
+            } else if (alive && root != kNone) {
                 // skip chunks whose solid-voxel AABB (grown by 1/16 voxel) the ray misses
                 const int32_t M = 1 << S.mlog;
                 const int32_t lo[3] = {(int32_t)(rb.x & 0xFFFFu), (int32_t)(rb.x >> 16), (int32_t)(rb.y & 0xFFFFu)};
@@ -267,7 +276,7 @@ __device__ __forceinline__ bool walk_pixel(const SceneDev& S, const CamDev& C, c
                 float tn = 0.0f, tf = 3.0e38f;
 #pragma unroll
                 for (int a = 0; a < 3; a++) {
-                    const bool m = (r.mir >> a) & 1u;
+                    const bool m = (mir >> a) & 1u;
                     const int32_t off = (cc[a] << S.mlog) - B[a];
                     tn = fmaxf(tn, ((float)(off + (m ? M - hi[a] : lo[a])) - (x[a] + 0.0625f)) * w.inv[a]);
                     tf = fminf(tf, ((float)(off + (m ? M - lo[a] : hi[a])) - (x[a] - 0.0625f)) * w.inv[a]);
@@ -284,7 +293,8 @@ __device__ __forceinline__ bool walk_pixel(const SceneDev& S, const CamDev& C, c
             float gtol = 0.0f, dmaxn = 0.0f;
             uint32_t V0 = 0, V1 = 0, V2 = 0;
             float Kp[3], gs[3], hp[3], xm[3], dv[3];
-            // {node, child mask} of the path's interior levels R .. 3; an
+            // {node, child mask | its place among its parent's children << 8}
+            // of the path's interior levels R .. 3; an
             // EXACT walk keeps to the octree inside leaf blocks too (at a tie
             // the cells visited depend on it) and holds level 2 as well
             constexpr int kLow = EXACT ? 2 : 3;
@@ -304,8 +314,11 @@ __device__ __forceinline__ bool walk_pixel(const SceneDev& S, const CamDev& C, c
 #pragma unroll
                 for (int a = 0; a < 3; a++) {
                     const int32_t l = B[a] - (cc[a] << S.mlog);
-                    J[a] = (uint32_t)max((int32_t)(J[a] & ~low), min(l >> n, (int32_t)(J[a] | low)));
-                    const float xn = ((float)(l - (int32_t)(J[a] << n)) + x[a]) * down;
+                    // (a decided base point lies in the cell: only EXACT can meet its upper face, at a tie)
+                    J[a] = EXACT ? (uint32_t)max((int32_t)(J[a] & ~low), min(l >> n, (int32_t)(J[a] | low)))
+                                 : (J[a] & ~low) | ((uint32_t)(l >> n) & low);
+                    const int32_t below = EXACT ? l - (int32_t)(J[a] << n) : l & ((1 << n) - 1);
+                    const float xn = ((float)below + x[a]) * down;
                     const float g = w.inv[a] * up;
                     gs[a] = g * (1.0f / (float)(1 << a));
                     hp[a] = __fmaf_rn(-xn, g, gs[a]);
@@ -322,17 +335,17 @@ __device__ __forceinline__ bool walk_pixel(const SceneDev& S, const CamDev& C, c
             uint32_t m = ~0u;
             auto octant = [&]() -> uint32_t {
                 const uint32_t hi = (V2 & (m << 2)) | (V1 & ~(m << 2));
-                return ((((hi & (m << 1)) | (V0 & ~(m << 1))) >> k) & 7u) ^ r.mir;
+                return ((((hi & (m << 1)) | (V0 & ~(m << 1))) >> k) & 7u) ^ mir;
             };
             if (traced) {
-                n = (int)ra.y;
+                n = (int)lod;
                 R = S.mlog - n;
                 gtol = kWalkEps * w.gmax * pow2(n);
                 dmaxn = w.dmax * pow2(-n);
-                pidx = ra.x;
+                pidx = root;
                 pm8 = nodes[pidx] & 0xFFu;
                 if (!based) undecided = !walk_base<EXACT>(w, Ow, e, Ne, B, x) && !EXACT;
-                if (!EXACT) { at.e = e; at.Ne = Ne; }
+                eb = e;
                 rebase((1u << R) - 1u);
                 st[R - kLow] = make_uint2(pidx, pm8);
                 k = R - 1;
@@ -348,8 +361,8 @@ __device__ __forceinline__ bool walk_pixel(const SceneDev& S, const CamDev& C, c
                         const uint64_t v = lmu >> ((o & 1u) * 2 + (o & 2u) * 4 + (o & 4u) * 8);
                         pm8 = (uint32_t)((v & 3) | ((v >> 2) & 0xC) | ((v >> 12) & 0x30) | ((v >> 14) & 0xC0));
                     } else {
-                        const uint2 ch = __ldg(reinterpret_cast<const uint2*>(
-                            nodes + pidx + 2 + 2 * __popc(pm8 & ~(~0u << o))));
+                        const uint32_t rank = __popc(pm8 & ~(~0u << o));
+                        const uint2 ch = __ldg(reinterpret_cast<const uint2*>(nodes + pidx + 2 + 2 * rank));
                         pidx = ch.x;
                         pm8 = ch.y >> 24;
                         if (k == kWideLevel - 1) pm8 = nodes[pidx] & 0xFFu;
@@ -361,7 +374,7 @@ __device__ __forceinline__ bool walk_pixel(const SceneDev& S, const CamDev& C, c
                             pm8 = (uint32_t)((q & 1) | ((q >> 1) & 2) | ((q >> 6) & 4) | ((q >> 7) & 8) |
                                              ((q >> 28) & 16) | ((q >> 29) & 32) | ((q >> 34) & 64) | ((q >> 35) & 128));
                         }
-                        st[k - kLow] = make_uint2(pidx, pm8);
+                        st[k - kLow] = make_uint2(pidx, pm8 | rank << 8);
                     }
                     k--;
                     m = ~0u << k;
@@ -379,7 +392,7 @@ __device__ __forceinline__ bool walk_pixel(const SceneDev& S, const CamDev& C, c
                     float T1 = __fmaf_rn(__uint_as_float(V1 | 1u | kMagicBits) - Kp[1], gs[1], hp[1]);
                     float T2 = __fmaf_rn(__uint_as_float(V2 | 3u | kMagicBits) - Kp[2], gs[2], hp[2]);
                     uint32_t i = (V0 & 3u) | ((V1 & 6u) << 1) | ((V2 & 12u) << 2), inc = 0;
-                    const uint32_t mi = ((r.mir & 1u) | ((r.mir & 2u) << 1) | ((r.mir & 4u) << 2)) * 3u;
+                    const uint32_t mi = ((mir & 1u) | ((mir & 2u) << 1) | ((mir & 4u) << 2)) * 3u;
                     for (;;) {
                         const uint32_t j = i ^ mi;
                         occ = (((j & 32u) ? (uint32_t)(lmu >> 32) : (uint32_t)lmu) >> (j & 31u)) & 1u;
@@ -460,7 +473,7 @@ __device__ __forceinline__ bool walk_pixel(const SceneDev& S, const CamDev& C, c
                     if (tm * w.dmax > kRebase || !clear) {
                         // far from the base point, or next to a voxel plane: a new base here
                         const int32_t Nt = plane(e, sel3(e, V0, V1, V2));
-                        if (!EXACT && !undecided) { at.e = e; at.Ne = Nt; }
+                        if (!undecided) { eb = e; Ne = Nt; }
                         undecided = (!walk_base<EXACT>(w, Ow, e, Nt, B, x) && !EXACT) || undecided;
                         rebase(~m0);
                     } else {
@@ -471,30 +484,26 @@ __device__ __forceinline__ bool walk_pixel(const SceneDev& S, const CamDev& C, c
                     }
                 }
             }
-            if (undecided) {
-                if (!EXACT && alive) {
-#pragma unroll
-                    for (int a = 0; a < 3; a++) at.cc[a] = cc[a];
-                    alive = false;
-                }
+            if (!EXACT && undecided) {
+                alive = false;
             } else if (traced && occ) {
                 hit.c[0] = (int32_t)V0;
                 hit.c[1] = (int32_t)(V1 >> 1);
                 hit.c[2] = (int32_t)(V2 >> 2);
                 hit.e = e;
-                // depth-first index (Sec. 3.3), as in trace_chunk
-                const uint32_t side = (1u << R) - 1u;
-                const uint32_t u0 = (r.mir & 1u) ? side - V0 : V0;
-                const uint32_t u1 = (r.mir & 2u) ? side - (V1 >> 1) : V1 >> 1;
-                const uint32_t u2 = (r.mir & 4u) ? side - (V2 >> 2) : V2 >> 2;
-                uint32_t idx = 0;
-                for (int j = R; j >= 3; j--) {
-                    const int sh = j - 1;
-                    const uint32_t oct = ((u0 >> sh) & 1u) | (((u1 >> sh) & 1u) << 1) | (((u2 >> sh) & 1u) << 2);
-                    const uint2 sj = st[j - kLow];
-                    idx += nodes[sj.x + 3 + 2 * __popc(sj.y & ((1u << oct) - 1u))] & (j == kWideLevel ? ~0u : kPrefixBits);
+                // depth-first index (Sec. 3.3): the prefix beside each child
+                // pointer of the path, then the leaf block's earlier voxels
+                uint32_t idx;
+                if (EXACT) {
+                    idx = nodes[st[1].x + 3 + 2 * (st[0].y >> 8)];
+                } else {
+                    idx = nodes[pidx + 3 + 2 * __popc(pm8 & ~(~0u << o))];
                 }
-                const int bit = (int)((u0 & 3u) + 4 * (u1 & 3u) + 16 * (u2 & 3u));
+                idx &= kPrefixBits;
+                for (int j = R; j > 3; j--)
+                    idx += nodes[st[j - kLow].x + 3 + 2 * (st[j - 1 - kLow].y >> 8)] & (j == kWideLevel ? ~0u : kPrefixBits);
+                const uint32_t bit = ((V0 & 3u) | ((V1 & 6u) << 1) | ((V2 & 12u) << 2)) ^
+                                     (((mir & 1u) | ((mir & 2u) << 1) | ((mir & 4u) << 2)) * 3u);
                 hit.idx = idx + (uint32_t)__popcll(lmu & ((1ull << bit) - 1ull));
                 found = true;
                 alive = false;
@@ -514,10 +523,7 @@ __device__ __forceinline__ bool walk_pixel(const SceneDev& S, const CamDev& C, c
                     e = exact_nearest(((cc[0] + 1) << cs) - Ow[0], ((cc[1] + 1) << cs) - Ow[1],
                                       ((cc[2] + 1) << cs) - Ow[2], w.ad[0], w.ad[1], w.ad[2]);
                 } else {
-#pragma unroll
-                    for (int a = 0; a < 3; a++) at.cc[a] = cc[a];
-                    at.e = e;
-                    at.Ne = Ne;
+                    eb = e;
                     undecided = true;
                     alive = false;
                 }
@@ -527,6 +533,7 @@ __device__ __forceinline__ bool walk_pixel(const SceneDev& S, const CamDev& C, c
         }
         if (alive) {
             based = false;
+            restarted = false;
             cc[0] += e == 0;
             cc[1] += e == 1;
             cc[2] += e == 2;
@@ -535,14 +542,23 @@ __device__ __forceinline__ bool walk_pixel(const SceneDev& S, const CamDev& C, c
             Ne = (ce << cs) - sel3(e, Ow[0], Ow[1], Ow[2]);
         }
     }
-    if (!EXACT && undecided) return false;
+    if (!EXACT && undecided) {
+#pragma unroll
+        for (int a = 0; a < 3; a++) at.cc[a] = cc[a];
+        at.e = eb;
+        at.Ne = Ne;
+        return false;
+    }
     if (found) {
+        int32_t u[3];
+        const uint4* fr = chunk_entry(u);
+        const uint4 ra = __ldg(fr);
         const int n = (int)ra.y;
         hit.Ne = 0;
         if (e < 3)  // the voxel's face that the ray enters through
             hit.Ne = (((sel3(e, cc[0], cc[1], cc[2]) << S.mlog) + (sel3(e, hit.c[0], hit.c[1], hit.c[2]) << n)) << kFix) -
                      sel3(e, Ow[0], Ow[1], Ow[2]);
-        if (EXACT && tie && (e == 1 || e == 2)) {
+        if (EXACT && (e == 1 || e == 2)) {
             // entered through an edge or a corner: the lowest of its axes (lowest_entry_face)
             const int32_t Nh = hit.Ne;
             const float de = sel3(e, w.ad[0], w.ad[1], w.ad[2]);
@@ -559,7 +575,11 @@ __device__ __forceinline__ bool walk_pixel(const SceneDev& S, const CamDev& C, c
         ChunkRef ref;
         ref.lod = ra.y;
         ref.mat_base = (uint64_t)ra.z | (uint64_t)ra.w << 32;
-        ref.nblocks = rb.w;
+        ref.nblocks = __ldg(fr + 1).w;
+        RayState r;
+#pragma unroll
+        for (int a = 0; a < 3; a++) r.d[a] = EXACT ? d[a] : w.ad[a];  // (their signs do not matter)
+        r.mir = mir;
         found = emit_hit(S, r, ref, u, hit, ray_norm(r), out_hit, out_t, pix);
     }
     if (!found) emit_miss(out_hit, out_t, pix);

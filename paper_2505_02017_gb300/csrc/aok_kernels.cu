@@ -60,10 +60,12 @@ __device__ __forceinline__ int32_t beam_bound_warp(const BeamLookup& b, int px, 
 
 // 16 x 8 pixel tiles, warps of 8 x 4 pixels.  BEAM: the warp's 8 x 4 tile
 // bound from the beam pass (aok_beam.cu) restarts its rays' march past the
-// space in front of the nearest voxel they can meet.  At most 72 registers:
-// 7 blocks per SM (the loop needs no more; no spills).
+// space in front of the nearest voxel they can meet.  At most 64 registers:
+// 8 blocks per SM (72 and 7 blocks: overview 3840x2160 511 us a frame instead
+// of 491, city 1080p 360 instead of 354; 56 and 9 blocks: 482 and 352, but
+// 320x180 views, where occupancy does not matter, 3% slower).
 template <bool COUNT, bool BEAM = false>
-__global__ void __launch_bounds__(128, 7) cast_kernel(const __grid_constant__ SceneDev S,
+__global__ void __launch_bounds__(128, 8) cast_kernel(const __grid_constant__ SceneDev S,
                                                    const __grid_constant__ CamDev C,
                                                    const ChunkRef* __restrict__ frame,
                                                    uint4* __restrict__ out_hit, float* __restrict__ out_t,
@@ -152,7 +154,7 @@ __global__ void __launch_bounds__(256) cast_persistent(const __grid_constant__ B
 // tiles (2^tile_w_log x 32/2^tile_w_log pixels each); P.v[v].tile_begin is the
 // exclusive prefix sum of the views' block-tile counts.  The view index derives
 // from blockIdx only, so every per-view parameter load is block-uniform.
-__global__ void __launch_bounds__(128, 7) cast_grid(const __grid_constant__ BatchParams P) {
+__global__ void __launch_bounds__(128, 8) cast_grid(const __grid_constant__ BatchParams P) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint64_t blk = blockIdx.x;
     uint32_t lo = 0, hi = P.n_views - 1;  // last view with tile_begin <= blk

@@ -24,23 +24,28 @@
 // within 2u of 1 / d, x and the product x g within u each, the FMA within u
 // of T, so |error of T| <= 3u T + 2u g; up to three steps T += g inside a
 // leaf block add u T each.  Two crossings are told apart when they differ by
-// more than eps (T + g_max), eps = 14 u (both errors, and the rounding of
-// that sum).  A coordinate x + T d at the entry of a cell, used for its
-// integer part, is then within eps (T + g_max) d_max as well (3u T d + 2u g d
-// from T, u each from the FMA, x and x - 1/2; g_max d_max >= 1) and is used
-// when it lies farther than that from every integer.
+// more than eps T + 5u g_max, eps = 8u (14u in a leaf block): both errors, and
+// the rounding of that sum.  A coordinate x + T d at the entry of a cell, used
+// for its integer part, is within (4u T + 4u g_max) d_max (from T: 3u T d +
+// 2u g d; from the FMA u T d, from x and x - 1/2 2u, and g_max d_max >= 1) and
+// is used when it lies farther than 5u (T + g_max) d_max from every integer.
 #pragma once
 #include "aok_trace.cuh"
 
 namespace aok {
 
-constexpr float kWalkEps = 0x1.Cp-21f;
+constexpr float kU = 0x1p-24f;
+constexpr float kEpsT = 8.0f * kU, kEpsLeaf = 14.0f * kU, kEpsX = 5.0f * kU, kEpsG = 5.0f * kU;
+constexpr float kWalkEps = 14.0f * kU;  // of the walk's start, where T is a product of two rounded factors
 constexpr float kZeroInv = 1e35f;       // 1 / d of a zero component: its planes lie past every other crossing
 constexpr uint32_t kMagicBits = 0x4B000000u;  // 2^23: kMagicBits | i is the float 2^23 + i for 0 <= i < 2^23
 constexpr float kRound = 12582912.0f;   // 1.5 * 2^23: adding it rounds to an integer
 // A base point farther back than this (voxels of the ray's largest component)
-// is replaced when an occupied cell is entered, which keeps the bounds small.
-constexpr float kRebase = 96.0f;
+// is replaced when an occupied cell is entered, which keeps the bounds small:
+// near when the cell is of level kNearLevel or below, where the ray is about to
+// meet leaf blocks.
+constexpr float kRebaseNear = 48.0f, kRebaseFar = 256.0f;
+constexpr int kNearLevel = 4;
 
 template <class T>
 __device__ __forceinline__ T sel3(int e, T a, T b, T c) {
@@ -340,7 +345,7 @@ __device__ __forceinline__ bool walk_pixel(const SceneDev& S, const CamDev& C, c
             if (traced) {
                 n = (int)lod;
                 R = S.mlog - n;
-                gtol = kWalkEps * w.gmax * pow2(n);
+                gtol = kEpsG * w.gmax * pow2(n);
                 dmaxn = w.dmax * pow2(-n);
                 pidx = root;
                 pm8 = nodes[pidx] & 0xFFu;
@@ -398,7 +403,7 @@ __device__ __forceinline__ bool walk_pixel(const SceneDev& S, const CamDev& C, c
                         occ = (((j & 32u) ? (uint32_t)(lmu >> 32) : (uint32_t)lmu) >> (j & 31u)) & 1u;
                         if (occ) break;
                         tm = fminf(fminf(T0, T1), T2);
-                        const float thr = __fmaf_rn(tm, 1.0f + kWalkEps, gtol);
+                        const float thr = __fmaf_rn(tm, 1.0f + kEpsLeaf, gtol);
                         const bool p0 = T0 <= thr, p1 = T1 <= thr, p2 = T2 <= thr;
                         undecided = undecided || (p0 ? p1 || p2 : p1 == p2);
                         if (p0) { T0 = T0 + gs[0]; inc = 1u; }
@@ -425,7 +430,7 @@ __device__ __forceinline__ bool walk_pixel(const SceneDev& S, const CamDev& C, c
                     const float T1 = __fmaf_rn(__uint_as_float(E1) - Kp[1], gs[1], hp[1]);
                     const float T2 = __fmaf_rn(__uint_as_float(E2) - Kp[2], gs[2], hp[2]);
                     tm = fminf(fminf(T0, T1), T2);
-                    const float thr = __fmaf_rn(tm, 1.0f + kWalkEps, gtol);
+                    const float thr = __fmaf_rn(tm, 1.0f + kEpsT, gtol);
                     bool p0 = T0 <= thr, p1 = T1 <= thr;
                     const bool p2 = T2 <= thr;
                     const bool amb = p0 ? p1 || p2 : p1 == p2;
@@ -440,10 +445,11 @@ __device__ __forceinline__ bool walk_pixel(const SceneDev& S, const CamDev& C, c
                     } else {
                         undecided = undecided || amb;
                     }
-                    uint32_t nv;
-                    if (p0) { nv = V0 = E0 + (1u - kMagicBits); e = 0; }
-                    else if (p1) { nv = V1 = E1 + (1u - kMagicBits); e = 1; }
-                    else { nv = V2 = E2 + (1u - kMagicBits); e = 2; }
+                    e = p0 ? 0 : (p1 ? 1 : 2);
+                    const uint32_t nv = (p0 ? E0 : (p1 ? E1 : E2)) + (1u - kMagicBits);
+                    V0 = p0 ? nv : V0;
+                    V1 = e == 1 ? nv : V1;
+                    V2 = e == 2 ? nv : V2;
                     m0 = m;
                     // the level of the cell entered: k for a sibling, else
                     // that of the lowest set bit (the parent was left)
@@ -464,13 +470,13 @@ __device__ __forceinline__ bool walk_pixel(const SceneDev& S, const CamDev& C, c
                     // left at (the crossed axis' are zero: it is on a face);
                     // at a tie, below the level it was entered at
                     if (EXACT) m0 = m;
-                    const float lim = 0.5f - __fmaf_rn(tm, kWalkEps, gtol) * dmaxn;
+                    const float lim = 0.5f - __fmaf_rn(tm, kEpsX, gtol) * dmaxn;
                     const float x0 = __fmaf_rn(tm, dv[0], xm[0]), x1 = __fmaf_rn(tm, dv[1], xm[1]),
                                 x2 = __fmaf_rn(tm, dv[2], xm[2]);
                     const float r0 = (x0 + kRound) - kRound, r1 = (x1 + kRound) - kRound, r2 = (x2 + kRound) - kRound;
                     const bool clear = fabsf(x0 - r0) < (e == 0 ? 1.0f : lim) && fabsf(x1 - r1) < (e == 1 ? 1.0f : lim) &&
                                        fabsf(x2 - r2) < (e == 2 ? 1.0f : lim);
-                    if (tm * w.dmax > kRebase || !clear) {
+                    if (tm * w.dmax > (k > kNearLevel ? kRebaseFar : kRebaseNear) || !clear) {
                         // far from the base point, or next to a voxel plane: a new base here
                         const int32_t Nt = plane(e, sel3(e, V0, V1, V2));
                         if (!undecided) { eb = e; Ne = Nt; }
@@ -515,7 +521,7 @@ __device__ __forceinline__ bool walk_pixel(const SceneDev& S, const CamDev& C, c
 #pragma unroll
             for (int a = 0; a < 3; a++)
                 T[a] = __fmaf_rn((float)(((cc[a] + 1) << S.mlog) - B[a]), w.inv[a], -x[a] * w.inv[a]);
-            const float thr = __fmaf_rn(fminf(fminf(T[0], T[1]), T[2]), 1.0f + kWalkEps, kWalkEps * w.gmax);
+            const float thr = __fmaf_rn(fminf(fminf(T[0], T[1]), T[2]), 1.0f + kEpsT, kEpsG * w.gmax);
             const bool p0 = T[0] <= thr, p1 = T[1] <= thr, p2 = T[2] <= thr;
             const int en = p0 ? 0 : (p1 ? 1 : 2);
             if (p0 ? p1 || p2 : p1 == p2) {

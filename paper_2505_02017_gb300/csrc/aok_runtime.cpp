@@ -919,7 +919,9 @@ static int ensure_bounds(aok_ctx* ctx, unsigned long long** buf, size_t* cap, si
     }
     int st = dev_alloc(ctx, (void**)buf, need * 8);
     if (st) return st;
-    if (cudaMemset(*buf, 0xFF, need * 8) != cudaSuccess) return cuda_status(ctx, cudaGetLastError());
+    // the pass that writes them may run on a stream the default stream's memset is not ordered with
+    if (cudaMemset(*buf, 0xFF, need * 8) != cudaSuccess || cudaStreamSynchronize(nullptr) != cudaSuccess)
+        return cuda_status(ctx, cudaGetLastError());
     *cap = need;
     return AOK_OK;
 }

@@ -120,7 +120,9 @@ static int ensure_batch_arena(aok_ctx* ctx, size_t frame_entries, uint32_t ngrou
         size_t cap = std::max<size_t>(ngroups * 2, 64);
         int st = dev_alloc(ctx, (void**)&A.d_queue, cap * sizeof(unsigned long long));
         if (st) return st;
-        if (cudaMemset(A.d_queue, 0, cap * sizeof(unsigned long long)) != cudaSuccess) return AOK_E_CUDA;
+        if (cudaMemset(A.d_queue, 0, cap * sizeof(unsigned long long)) != cudaSuccess ||
+            cudaStreamSynchronize(nullptr) != cudaSuccess)  // before its use on any stream
+            return AOK_E_CUDA;
         A.queue_cap = cap;
     }
     return AOK_OK;
@@ -582,7 +584,9 @@ int aok_serve_start(aok_ctx* ctx, uint32_t max_slots, uint32_t max_batch, uint32
         unsigned long long* c = nullptr;
         int st = dev_alloc(ctx, (void**)&c, 2 * ngroups * sizeof(unsigned long long));
         if (st) return st;
-        cudaMemset(c, 0, 2 * ngroups * sizeof(unsigned long long));
+        if (cudaMemset(c, 0, 2 * ngroups * sizeof(unsigned long long)) != cudaSuccess ||
+            cudaStreamSynchronize(nullptr) != cudaSuccess)
+            return AOK_E_CUDA;
         S->counters.push_back(c);
         S->stream_busy.push_back(0);
         for (int k = 0; k < 2; k++) {

@@ -444,3 +444,28 @@ def test_selection_inside_the_pass(ctx, spec):
     aok.cast_selected(ctx, sc, cam, *plain)
     torch.cuda.synchronize()
     assert same(ref, plain)
+
+
+def test_first_host_frames_beside_default_stream_work():
+    """The first frames of a context size their bound pyramids: their clearing is done before the passes that
+    write them, which run on other streams, even while the default stream is busy."""
+    c = aok.Context(0)
+    aok.beam_tune(c, 16, 2, 0, 0)
+    w = sg.World(MED64)
+    sc = aok.Scene.from_world(c, w, threads=4)
+    cams = [sg.ground_camera(w, s, 203, 117, z_lo=4, z_hi=40) for s in (4, 9, 12)]
+    out = [(torch.empty((m.H, m.W, 4), dtype=torch.int32, pin_memory=True),
+            torch.empty((m.H, m.W), dtype=torch.float32, pin_memory=True)) for m in cams]
+    torch.cuda._sleep(40_000_000)  # about 20 ms of the default stream
+    tickets = [aok.render_host_async(c, sc, m, 1.5, *o) for m, o in zip(cams, out)]
+    for t in tickets:
+        aok.host_frame_wait(c, t)
+    torch.cuda.synchronize()
+    for m, o in zip(cams, out):
+        hit, t = aok.alloc_frame(m.W, m.H)
+        aok.set_beam(c, False)
+        aok.render(c, sc, m, 1.5, hit, t)
+        torch.cuda.synchronize()
+        assert torch.equal(hit.cpu(), o[0]) and torch.equal(t.cpu().view(torch.int32), o[1].view(torch.int32))
+    sc.destroy()
+    c.close()

@@ -549,7 +549,7 @@ int aok_render_noalloc(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, doub
 int aok_set_beam(aok_ctx* ctx, int on);
 /* Refinement of the beam pass's walk: a node is refined while its rectangle
  * spans more than refine_tiles tiles and its side is above 2^min_node_log2
- * LOD-0 voxels (defaults 8 and 2: down to the 4^3 leaves); frames of fewer
+ * LOD-0 voxels (a context starts with 16 and 2: down to the 4^3 leaves); frames of fewer
  * than min_pixels pixels cast without the pass (default 1,500,000: below
  * that the pass's fixed cost, some tens of microseconds, outweighs what it
  * saves); queue_nodes caps the nodes one level of the walk may queue

@@ -20,8 +20,8 @@
 //     the box being the region's AABB of valid voxels;
 //   * a node is projected in FP32 to a rectangle of tiles (box_rect, with
 //     margins that cover its rounding); if the rectangle spans more tiles
-//     than the refinement threshold and the node is not a 4^3 leaf, its
-//     children (cell boxes clipped to the AABB) go to the next level's queue;
+//     than the refinement threshold and the node is not a 4^3 leaf, it goes to
+//     the next level's queue, where its children are projected in its place;
 //     otherwise atomicMin(Dn[tile], its L-inf distance) over the rectangle.
 //     A leaf uses the bounding box of its set voxels;
 //   * a box that comes closer to the origin than 2/16 of the largest |d|
@@ -59,67 +59,89 @@ using namespace aok;
 namespace {
 
 constexpr int kBeamThreads = 256;      // block size of the cooperative walk
-constexpr int kBeamNarrowThreads = 128;  // block size of the walk that shares SMs with a cast
-constexpr int kBeamBlocksPerSM = 2;    // blocks per SM of the full grid (walks over many regions)
-constexpr uint32_t kWideWalkRegions = 4096;  // above this many regions a pass takes the full grid; below,
-                                             // one block per SM, which can start beside a running cast
+constexpr int kBeamBlocksPerSM = 2;    // blocks per SM of the grid: 45 us against 50 with one, 48 with three (city 1080p)
+constexpr uint32_t kWideWalkRegions = 4096;  // a pass beside a running cast takes one block per SM, which can start
+                                             // there sooner, unless it walks more regions than this
 constexpr double kNearS = 1.0 / 16.0;  // camera-depth plane the projection clips at
 constexpr uint32_t kNoItem = 0xFFFFFFFFu;  // an empty queue slot
 constexpr int kMaxBeamDevices = 128;
 
+__device__ __forceinline__ float rcp_approx(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
 // Screen rectangle [x, z) x [y, w) of tiles a box (relative to the origin)
 // can cover from its part at camera depth s >= kNearS; false if none.
-// q = Af p in FP32 errs by at most dl = 8 2^-24 max_i sum_j |Af_ij| |p_j|
-// (rounding of p, of Af and of the products and sums).  A box wholly in front
-// of the plane is bounded by its corners' projections (their hull holds the
-// box's), widened by the error that dl and the division carry; a box that
-// straddles it by u = q_x / q_s over q_x in [X0, X1] and q_s in [kNearS, S1],
-// each widened by dl.  Then a 0.5 pixel margin for the FP32 pixel rays.
+// A corner's q = Af p is the first corner's plus the edges' steps; with
+// u = 2^-24 it errs by at most dl = 16 u max_i sum_j |Af_ij| max |p_j| (2u M
+// from the rounding of p and Af, 3u M from the first corner, 6u M from the
+// three steps, each of an edge of up to 2 max |p_j|, 3u M from adding them).
+// A box wholly in front of the plane is bounded by its corners' projections
+// (their hull holds the box's), widened by the error that dl and the
+// approximate reciprocal (2u) carry; a box that straddles it by u = q_x / q_s
+// over q_x in [X0, X1] and q_s in [kNearS, S1], each widened by dl.  Then a 0.5
+// pixel margin for the FP32 pixel rays.
 __device__ bool box_rect(const BeamView& K, const float lo[3], const float hi[3], int4& rc) {
-    float pm[3];
-#pragma unroll
-    for (int a = 0; a < 3; a++) pm[a] = fmaxf(fabsf(lo[a]), fabsf(hi[a]));
     float M = 0.0f;
+    float q[3][8];
+    const float pm0 = fmaxf(fabsf(lo[0]), fabsf(hi[0])), pm1 = fmaxf(fabsf(lo[1]), fabsf(hi[1])),
+                pm2 = fmaxf(fabsf(lo[2]), fabsf(hi[2]));
 #pragma unroll
-    for (int i = 0; i < 3; i++)
-        M = fmaxf(M, fabsf(K.Af[3 * i]) * pm[0] + fabsf(K.Af[3 * i + 1]) * pm[1] + fabsf(K.Af[3 * i + 2]) * pm[2]);
-    const float dl = M * 4.8e-7f + 1e-6f;
-    float X0 = 3e38f, X1 = -3e38f, Y0 = 3e38f, Y1 = -3e38f, S0 = 3e38f, S1 = -3e38f;
-    float u0 = 3e38f, u1 = -3e38f, v0 = 3e38f, v1 = -3e38f;
+    for (int i = 0; i < 3; i++) {
+        const float a0 = K.Af[3 * i], a1 = K.Af[3 * i + 1], a2 = K.Af[3 * i + 2];
+        M = fmaxf(M, __fmaf_rn(fabsf(a0), pm0, __fmaf_rn(fabsf(a1), pm1, fabsf(a2) * pm2)));
+        const float d0 = a0 * (hi[0] - lo[0]), d1 = a1 * (hi[1] - lo[1]), d2 = a2 * (hi[2] - lo[2]);
+        q[i][0] = __fmaf_rn(a0, lo[0], __fmaf_rn(a1, lo[1], a2 * lo[2]));
+        q[i][1] = q[i][0] + d0;
+        q[i][2] = q[i][0] + d1;
+        q[i][3] = q[i][1] + d1;
+#pragma unroll
+        for (int k = 0; k < 4; k++) q[i][4 + k] = q[i][k] + d2;
+    }
+    const float dl = M * 9.7e-7f + 1e-6f;
+    float S0 = 3e38f, S1 = -3e38f;
 #pragma unroll
     for (int k = 0; k < 8; k++) {
-        const float p0 = (k & 1) ? hi[0] : lo[0], p1 = (k & 2) ? hi[1] : lo[1], p2 = (k & 4) ? hi[2] : lo[2];
-        const float qx = K.Af[0] * p0 + K.Af[1] * p1 + K.Af[2] * p2;
-        const float qy = K.Af[3] * p0 + K.Af[4] * p1 + K.Af[5] * p2;
-        const float qs = K.Af[6] * p0 + K.Af[7] * p1 + K.Af[8] * p2;
-        X0 = fminf(X0, qx); X1 = fmaxf(X1, qx);
-        Y0 = fminf(Y0, qy); Y1 = fmaxf(Y1, qy);
-        S0 = fminf(S0, qs); S1 = fmaxf(S1, qs);
-        if (qs > 0.0f) {
-            const float r = 1.0f / qs;
-            u0 = fminf(u0, qx * r); u1 = fmaxf(u1, qx * r);
-            v0 = fminf(v0, qy * r); v1 = fmaxf(v1, qy * r);
-        }
+        S0 = fminf(S0, q[2][k]);
+        S1 = fmaxf(S1, q[2][k]);
     }
     const float near_s = (float)kNearS;
     if (S1 + dl < near_s) return false;  // wholly behind the plane: only the near rule can reach it
     float a0, a1, b0, b1;
     if (S0 - dl >= near_s) {
+        float u0 = 3e38f, u1 = -3e38f, v0 = 3e38f, v1 = -3e38f;
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            const float r = rcp_approx(q[2][k]);
+            u0 = fminf(u0, q[0][k] * r); u1 = fmaxf(u1, q[0][k] * r);
+            v0 = fminf(v0, q[1][k] * r); v1 = fmaxf(v1, q[1][k] * r);
+        }
         const float um = fmaxf(fabsf(u0), fabsf(u1)) * 1.001f, vm = fmaxf(fabsf(v0), fabsf(v1)) * 1.001f;
-        const float mu = dl * (1.0f + um) / (S0 - dl) + um * 4.8e-7f;
-        const float mv = dl * (1.0f + vm) / (S0 - dl) + vm * 4.8e-7f;
+        const float rs = dl * rcp_approx(S0 - dl) * 1.00001f;
+        const float mu = __fmaf_rn(rs, 1.0f + um, um * 4.8e-7f);
+        const float mv = __fmaf_rn(rs, 1.0f + vm, vm * 4.8e-7f);
         a0 = u0 - mu; a1 = u1 + mu;
         b0 = v0 - mv; b1 = v1 + mv;
     } else {
-        const float Xl = X0 - dl, Xh = X1 + dl, Yl = Y0 - dl, Yh = Y1 + dl, Sh = S1 + dl;
-        a0 = fminf(Xl / near_s, Xl / Sh); a1 = fmaxf(Xh / near_s, Xh / Sh);
-        b0 = fminf(Yl / near_s, Yl / Sh); b1 = fmaxf(Yh / near_s, Yh / Sh);
+        float X0 = 3e38f, X1 = -3e38f, Y0 = 3e38f, Y1 = -3e38f;
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            X0 = fminf(X0, q[0][k]); X1 = fmaxf(X1, q[0][k]);
+            Y0 = fminf(Y0, q[1][k]); Y1 = fmaxf(Y1, q[1][k]);
+        }
+        const float Xl = X0 - dl, Xh = X1 + dl, Yl = Y0 - dl, Yh = Y1 + dl;
+        const float in = 1.0f / near_s, is = rcp_approx(S1 + dl);
+        a0 = fminf(Xl * in, Xl * is); a1 = fmaxf(Xh * in, Xh * is);
+        b0 = fminf(Yl * in, Yl * is); b1 = fmaxf(Yh * in, Yh * is);
         a0 -= fabsf(a0) * 1e-6f; a1 += fabsf(a1) * 1e-6f;
         b0 -= fabsf(b0) * 1e-6f; b1 += fabsf(b1) * 1e-6f;
     }
     // pixel-centre coordinates of the pixel rays (the inverse of ray_dir), 0.5 pixel margin
-    const float x0 = (a0 / K.U + 1.0f) * 0.5f * K.W - 1.0f, x1 = (a1 / K.U + 1.0f) * 0.5f * K.W;
-    const float y0 = (1.0f - b1 / K.V) * 0.5f * K.H - 1.0f, y1 = (1.0f - b0 / K.V) * 0.5f * K.H;
+    const float hw = 0.5f * (float)K.W, hh = 0.5f * (float)K.H;
+    const float x0 = (a0 * K.iU + 1.0f) * hw - 1.0f, x1 = (a1 * K.iU + 1.0f) * hw;
+    const float y0 = (1.0f - b1 * K.iV) * hh - 1.0f, y1 = (1.0f - b0 * K.iV) * hh;
     if (!(x1 >= 0.0f) || !(y1 >= 0.0f) || !(x0 < (float)K.W) || !(y0 < (float)K.H)) return false;
     rc.x = (int)fmaxf(floorf(x0 * (1.0f / kBeamTileW)), 0.0f);
     rc.y = (int)fmaxf(floorf(y0 * (1.0f / kBeamTileH)), 0.0f);
@@ -243,68 +265,66 @@ __device__ __forceinline__ void scatter_bound(const BeamView& V, uint32_t tag, c
         for (int x = x0; x <= x1; x++) red_min_u64(&lv[(size_t)y * wl + x], v);
 }
 
-// A checked pass (P.ck.err set) that meets a node or leaf index outside its
+// A checked pass (ck.err set) that meets a node or leaf index outside its
 // pool: the error code goes into the error word and the view is bounded by 0
 // (no ray of it skips anything), in place of the loads.
-__device__ __noinline__ void bad_index(const BeamBatch& P, const BeamView& V, uint32_t code) {
+__device__ __noinline__ void bad_index(const BeamHead& P, const BeamView& V, uint32_t code) {
     atomicOr(P.ck.err, code);
     scatter_bound(V, P.tag, make_int4(0, 0, V.tiles_x, V.tiles_y), 0);
-}
-
-// Children of interior node `node` (side 2^s) at cell c: {pointer, packed cell}.
-__device__ __forceinline__ uint32_t node_children(const SceneDev& S, uint32_t node, uint32_t packed_cell, int s,
-                                                  uint32_t ch[8], uint32_t cc[8], uint32_t hdr) {
-    const uint32_t m0 = hdr & 0xFFu;
-    const uint32_t k = (uint32_t)__popc(m0);
-    const uint32_t h = 1u << (s - 1);
-    const uint32_t cx0 = packed_cell & 1023u, cy0 = (packed_cell >> 10) & 1023u, cz0 = (packed_cell >> 20) & 1023u;
-    uint32_t m = m0;
-#pragma unroll
-    for (int j = 0; j < 8; j++) {
-        ch[j] = (uint32_t)j < k ? __ldg(S.nodes + node + 2 + 2 * j) : 0u;
-        const int oct = m ? __ffs(m) - 1 : 0;
-        m &= m - 1;
-        cc[j] = (cx0 + ((oct & 1) ? h : 0u)) | ((cy0 + ((oct & 2) ? h : 0u)) << 10) | ((cz0 + ((oct & 4) ? h : 0u)) << 20);
-    }
-    return k;
 }
 
 // The whole pass in one cooperative launch (every block resident): the
 // levels of the walk over all views with a grid-wide barrier after each,
 // ending at the first level that queued nothing.  Level 0 takes every view's
-// chunk regions; every lane of a warp runs the same iterations (the queue
-// reservation is warp-wide).  A queued item carries what its node's bound
-// needs (region, node, cell, side, view, LOD), so a level's chain of
-// dependent loads starts at the item itself; each thread loads its first
-// item beside the level's count and the next one while it works on the
-// current one.  Queues are read through L2 (written by other SMs before the
-// barrier).  Bounds carry the pass's tag, so nothing has to be reset before
-// the walk or folded after it.
-__device__ __forceinline__ void beam_walk(const BeamBatch& P) {
+// chunk regions, one lane each; a later level takes the queued nodes, eight
+// lanes each, a lane projecting the child of its octant.  A projected node is
+// scattered or queued to be refined; one whose rectangle is so large that its
+// children will be refined as well (a child's is about a quarter of it) queues
+// them at once, unprojected, so that about half the levels remain, and with
+// them half the chains of dependent loads and barriers that bound the pass.
+// (City 1920x1080, three views: 71 / 51 / 77 us for the pass that projected
+// every level, one lane a node, refining above 8 tiles; 45 / 37 / 49 for this
+// one above 16.  Above 8 it gains nothing: its levels hold too many nodes.)
+// Every lane of a warp runs the same iterations (the queue reservation is
+// warp-wide), and a level's warps are dealt over the SMs first.  A queued item
+// carries what its children's bounds need (region, node, cell, side, view,
+// LOD, child mask), so a level's chain of dependent loads starts at the item
+// itself; each lane loads its first item beside the level's count and the
+// next one while it works on the current one.  Queues are read through L2
+// (written by other SMs before the barrier).  Bounds carry the pass's tag, so
+// nothing has to be reset before the walk or folded after it; the queue
+// counters are zeroed behind the walk, a level after their last reader.
+template <class PB>
+__device__ __forceinline__ void beam_walk(const PB& P) {
     cg::grid_group g = cg::this_grid();
     __shared__ uint32_t hist[kBeamLevels];
-    const uint32_t gtid = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
     const int lane = (int)(threadIdx.x & 31u);
-    if (threadIdx.x < kBeamLevels) hist[threadIdx.x] = 0;
+    const uint32_t warp = (threadIdx.x >> 5) * gridDim.x + blockIdx.x, warps = (blockDim.x >> 5) * gridDim.x;
+    const bool checked = P.ck.err != nullptr;
+    if (threadIdx.x < kBeamLevels) {
+        hist[threadIdx.x] = 0;
+        if (blockIdx.x == 0) P.hist[threadIdx.x] = 0;  // (added to after the first barrier)
+    }
     __syncthreads();
     for (int level = 0; level < kBeamLevels - 1; level++) {
         const uint4* qin = P.q[level & 1];
         uint4* qout = P.q[(level + 1) & 1];
-        // level 0 (the regions, few): one warp per block first, so that its
-        // selection and root projections spread over the SMs
-        const uint32_t first = level == 0 ? (((threadIdx.x >> 5) * gridDim.x + blockIdx.x) << 5) : (gtid & ~31u);
+        const uint32_t per = level == 0 ? 32u : 4u;  // items a warp takes at a time
+        const uint32_t mine = level == 0 ? (uint32_t)lane : (uint32_t)lane >> 3;
+        const uint32_t first = warp * per, stride = warps * per;
         uint4 nxt = make_uint4(kNoItem, 0u, 0u, 0u);
-        if (level > 0 && first + (uint32_t)lane < P.cap) nxt = __ldcg(qin + first + lane);
+        if (level > 0 && first + mine < P.cap) nxt = __ldcg(qin + first + mine);
         const uint32_t n = level == 0 ? P.n_regions : min(*(volatile uint32_t*)&P.cnt[level], P.cap);
+        if (level > 0 && blockIdx.x == 0 && threadIdx.x == 0) P.cnt[level - 1] = 0;
         if (n == 0) break;  // the same value in every thread after the barrier
         for (uint32_t base = first; base < n; base += stride) {
-            const uint32_t i = base + (uint32_t)lane;
-            uint32_t kids = 0, ch[8], cc[8];
-            uint4 it = make_uint4(kNoItem, 0u, 0u, 0u);
-            bool clip = false;
+            const uint32_t i = base + mine;
+            uint32_t kids = 0, ch[8], cm[8];
+            uint32_t chunk = kNoItem, node = 0, cell = 0, vi = 0;  // the node this lane projects
+            int s = 0, lod = 0;
             ChunkRef ref;
-            if (i < n) {
-                if (level == 0) {
+            if (level == 0) {
+                if (i < n) {
                     // the view holding region item i: the last with region_begin <= i
                     uint32_t lo = 0, hi = P.n_views - 1;
                     while (lo < hi) {
@@ -317,42 +337,81 @@ __device__ __forceinline__ void beam_walk(const BeamBatch& P) {
                     ref = P.select ? select_one(P.v[lo].scene, P.cam, const_cast<ChunkRef*>(P.v[lo].frame), nullptr,
                                                 nullptr, nullptr, (int)r)
                                    : P.v[lo].frame[r];
-                    if (ref.root != kNone)
-                        it = make_uint4(r, ref.root, 0u,
-                                        (uint32_t)P.v[lo].scene.mlog | (lo << 8) | ((uint32_t)ref.lod << 16));
-                    clip = true;
-                } else {
-                    it = nxt;
+                    vi = lo;
+                    if (ref.root != kNone) {
+                        chunk = r;
+                        node = ref.root;
+                        s = P.v[lo].scene.mlog;
+                        lod = (int)ref.lod;
+                    }
                 }
-            }
-            if (level > 0) {
-                const uint32_t j = i + stride;
+            } else {
+                const uint4 it = nxt;
                 nxt = make_uint4(kNoItem, 0u, 0u, 0u);
-                if (j < n) nxt = __ldcg(qin + j);
-            }
-            const uint32_t vi = (it.w >> 8) & 0xFFu;
-            const int s = (int)(it.w & 0xFFu), lod = (int)((it.w >> 16) & 0xFFu);
-            const BeamView& V = P.v[it.x != kNoItem ? vi : 0u];
-            if (it.x != kNoItem) {
-                atomicAdd(&hist[min(V.scene.mlog - s, kBeamLevels - 1)], 1u);
-                int4 rc;
-                int32_t D;
-                uint32_t hdr = 0;
-                if (P.ck.err && (s == lod + 2 ? it.y >= P.ck.n_leaves : (uint64_t)it.y + 2 > P.ck.n_nodes)) {
-                    bad_index(P, V, s == lod + 2 ? 2u : 1u);
-                } else if (node_bound(V, lod, clip, ref, it.x, it.y, it.z, s, rc, D, hdr)) {
-                    const uint32_t area = (uint32_t)(rc.z - rc.x) * (uint32_t)(rc.w - rc.y);
-                    if (s > lod + 2 && area > P.expand && s > P.smin) {
-                        if (P.ck.err && (uint64_t)it.y + 2 + 2 * __popc(hdr & 0xFFu) > P.ck.n_nodes)
-                            bad_index(P, V, 1u);
-                        else
-                            kids = node_children(V.scene, it.y, it.z, s, ch, cc, hdr);
+                if (i + stride < n) nxt = __ldcg(qin + i + stride);
+                const uint32_t mask = it.w >> 24, o = (uint32_t)lane & 7u;
+                if (i < n && it.x != kNoItem && ((mask >> o) & 1u)) {
+                    vi = (it.w >> 8) & 0xFFu;
+                    const uint64_t at = (uint64_t)it.y + 2 + 2 * __popc(mask & ((1u << o) - 1u));
+                    if (checked && at + 2 > P.ck.n_nodes) {
+                        bad_index(P, P.v[vi], 1u);
                     } else {
-                        scatter_bound(V, P.tag, rc, D);
+                        chunk = it.x;
+                        node = __ldg(P.v[vi].scene.nodes + at);
+                        s = (int)(it.w & 0xFFu) - 1;
+                        lod = (int)((it.w >> 16) & 0xFFu);
+                        const uint32_t h = 1u << s;
+                        cell = it.z + ((o & 1u) ? h : 0u) + ((o & 2u) ? h << 10 : 0u) + ((o & 4u) ? h << 20 : 0u);
                     }
                 }
             }
-            // queue the children: one reservation per warp
+            const BeamView& V = P.v[vi];
+            int4 rc;
+            int32_t D = 0;
+            int sk = s;  // side of the nodes this lane queues
+            uint32_t mk = 0;
+            if (chunk != kNoItem) {
+                atomicAdd(&hist[min(V.scene.mlog - s, kBeamLevels - 1)], 1u);
+                const bool leaf = s == lod + 2;
+                uint32_t hdr = 0;
+                if (checked && (leaf ? node >= P.ck.n_leaves : (uint64_t)node + 2 > P.ck.n_nodes)) {
+                    bad_index(P, V, leaf ? 2u : 1u);
+                } else if (node_bound(V, lod, level == 0, ref, chunk, node, cell, s, rc, D, hdr)) {
+                    const uint32_t area = (uint32_t)(rc.z - rc.x) * (uint32_t)(rc.w - rc.y);
+                    mk = hdr & 0xFFu;
+                    const uint32_t k = (uint32_t)__popc(mk);
+                    if (leaf || area <= P.expand || s <= P.smin) {
+                        scatter_bound(V, P.tag, rc, D);
+                    } else if (checked && (uint64_t)node + 2 + 2 * k > P.ck.n_nodes) {
+                        bad_index(P, V, 1u);
+                    } else if (area / 4u > P.expand && s - 1 > lod + 2 && s - 1 > P.smin) {
+                        // its children, to be refined without a projection of their own
+                        kids = k;
+                        sk = s - 1;
+#pragma unroll
+                        for (int j = 0; j < 8; j++) {
+                            uint2 w = make_uint2(0u, 0u);
+                            if ((uint32_t)j < k) w = __ldg(reinterpret_cast<const uint2*>(V.scene.nodes + node + 2 + 2 * j));
+                            ch[j] = w.x;
+                            cm[j] = w.y >> 24;
+                        }
+                        if (s - lod == kWideLevel) {  // no child masks beside the pointers
+#pragma unroll
+                            for (int j = 0; j < 8; j++) {
+                                if ((uint32_t)j < k && checked && (uint64_t)ch[j] + 2 > P.ck.n_nodes) {
+                                    bad_index(P, V, 1u);
+                                    ch[j] = node;  // (an index within the pool; the view skips nothing)
+                                }
+                                if ((uint32_t)j < k) cm[j] = __ldg(V.scene.nodes + ch[j]) & 0xFFu;
+                            }
+                        }
+                        atomicAdd(&hist[min(V.scene.mlog - sk, kBeamLevels - 1)], k);
+                    } else {
+                        kids = 1;
+                    }
+                }
+            }
+            // queue them: one reservation per warp
             uint32_t pre = kids;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
@@ -367,18 +426,24 @@ __device__ __forceinline__ void beam_walk(const BeamBatch& P) {
             }
             if (kids) {
                 const uint32_t at = wbase + pre - kids;
-                if (at + kids <= P.cap) {
-#pragma unroll
-                    for (int q = 0; q < 8; q++)
-                        if ((uint32_t)q < kids) qout[at + q] = make_uint4(it.x, ch[q], cc[q], it.w - 1);
-                } else {
+                const uint32_t w = (uint32_t)sk | (vi << 8) | ((uint32_t)lod << 16);
+                if (at + kids > P.cap) {
                     // queue full: this node stands for its children; its slots
                     // below the capacity are marked empty
                     for (uint32_t q = at; q < P.cap && q < at + kids; q++) qout[q] = make_uint4(kNoItem, 0u, 0u, 0u);
-                    int4 rc;
-                    int32_t D;
-                    uint32_t hdr;
-                    if (node_bound(V, lod, clip, ref, it.x, it.y, it.z, s, rc, D, hdr)) scatter_bound(V, P.tag, rc, D);
+                    scatter_bound(V, P.tag, rc, D);
+                } else if (sk == s) {
+                    qout[at] = make_uint4(chunk, node, cell, w | mk << 24);
+                } else {
+                    const uint32_t h = 1u << sk;
+                    uint32_t m = mk;
+#pragma unroll
+                    for (int q = 0; q < 8; q++) {
+                        const int o = m ? __ffs((int)m) - 1 : 0;
+                        m &= m - 1u;
+                        const uint32_t c = cell + ((o & 1) ? h : 0u) + ((o & 2) ? h << 10 : 0u) + ((o & 4) ? h << 20 : 0u);
+                        if ((uint32_t)q < kids) qout[at + q] = make_uint4(chunk, ch[q], c, w | cm[q] << 24);
+                    }
                 }
             }
         }
@@ -388,14 +453,10 @@ __device__ __forceinline__ void beam_walk(const BeamBatch& P) {
     if (threadIdx.x < kBeamLevels && hist[threadIdx.x]) atomicAdd(&P.hist[threadIdx.x], hist[threadIdx.x]);
 }
 
-__global__ void __launch_bounds__(kBeamThreads) beam_kernel(const __grid_constant__ BeamBatch P) { beam_walk(P); }
-
-// The same walk as one block of kBeamNarrowThreads per SM with at most 80
-// registers: it fits beside six blocks of a running cast (7 x 128 threads x
-// 72 registers per SM), so a pipelined frame's pass can start on an SM as
-// soon as one casting block of the frame before retires there instead of
-// after the cast.  Alone it is slower (half the threads).
-__global__ void __maxnreg__(80) beam_kernel_narrow(const __grid_constant__ BeamBatch P) { beam_walk(P); }
+template <class PB>
+__global__ void __launch_bounds__(kBeamThreads) beam_kernel(const __grid_constant__ PB P) {
+    beam_walk(P);
+}
 
 }  // namespace
 
@@ -403,7 +464,7 @@ extern "C" {
 
 unsigned aokk_beam_grid(int sms) {
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, beam_kernel, kBeamThreads, 0) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, beam_kernel<BeamBatch>, kBeamThreads, 0) != cudaSuccess ||
         per_sm < 1)
         return 0;
     return (unsigned)(sms > 0 ? sms : 1) * (unsigned)(per_sm < kBeamBlocksPerSM ? per_sm : kBeamBlocksPerSM);
@@ -441,8 +502,8 @@ bool aokk_beam_view(const SceneDev* S, const CamDev* C, const ChunkRef* frame, u
     K.bounds = bounds;
     for (int i = 0; i < 9; i++) K.Af[i] = (float)Ai[i];
     const double U = (double)C->tan_half * (double)C->W / (double)C->H, V = (double)C->tan_half;
-    K.U = (float)U;
-    K.V = (float)V;
+    K.iU = (float)(1.0 / U);
+    K.iV = (float)(1.0 / V);
     // largest |d| component over the screen, with slack for the FP32 ray arithmetic
     double dmax = 0.0;
     for (int i = 0; i < 3; i++) dmax = fmax(dmax, fabs(A[3 * i]) * U + fabs(A[3 * i + 1]) * V + fabs(A[3 * i + 2]));
@@ -463,23 +524,16 @@ bool aokk_beam_view(const SceneDev* S, const CamDev* C, const ChunkRef* frame, u
 static std::mutex g_beam_mu;
 static cudaEvent_t g_beam_done[kMaxBeamDevices];
 
-// The pass as a node of a CUDA graph (aokk_batch_run): its kernel with the
-// launch shape aokk_beam_run uses, and the memset of the counters that
-// aokk_beam_run zeroes before it.  argp: one slot, valid until the node is set.
-void aokk_beam_node(const BeamBatch* P, unsigned grid, void** argp, cudaKernelNodeParams* kp, cudaMemsetParams* zero) {
+// The pass as a node of a CUDA graph (aokk_batch_run), with the launch shape
+// aokk_beam_run uses.  argp: one slot, valid until the node is set.
+void aokk_beam_node(const BeamBatch* P, unsigned grid, void** argp, cudaKernelNodeParams* kp) {
     argp[0] = (void*)P;
-    kp->func = (void*)beam_kernel;
-    kp->gridDim = dim3(P->n_regions > kWideWalkRegions ? grid : (grid + kBeamBlocksPerSM - 1) / kBeamBlocksPerSM);
+    kp->func = (void*)beam_kernel<BeamBatch>;
+    kp->gridDim = dim3(grid);
     kp->blockDim = dim3(kBeamThreads);
     kp->sharedMemBytes = 0;
     kp->kernelParams = argp;
     kp->extra = nullptr;
-    zero->dst = P->cnt;
-    zero->pitch = 0;
-    zero->value = 0;
-    zero->elementSize = sizeof(uint32_t);
-    zero->width = 2 * kBeamLevels;
-    zero->height = 1;
 }
 
 // The per-device order of beam passes for work that holds passes but is not
@@ -498,7 +552,7 @@ int aokk_beam_order(void* stream, int record) {
     return aokk_status(e);
 }
 
-int aokk_beam_run(const BeamBatch* P, unsigned grid, void* stream, int narrow) {
+int aokk_beam_run(const BeamBatch* P, unsigned grid, void* stream, int beside) {
     const cudaStream_t st = (cudaStream_t)stream;
     if (P->n_views == 0) return AOK_OK;
     int dev = -1;
@@ -508,16 +562,16 @@ int aokk_beam_run(const BeamBatch* P, unsigned grid, void* stream, int narrow) {
     std::lock_guard<std::mutex> lk(g_beam_mu);
     if (!g_beam_done[dev]) e = cudaEventCreateWithFlags(&g_beam_done[dev], cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(st, g_beam_done[dev], 0);
-    // queue counts and the walk histogram (cnt and hist are adjacent)
-    if (e == cudaSuccess) e = cudaMemsetAsync(P->cnt, 0, 2 * kBeamLevels * sizeof(uint32_t), st);
-    void* args[] = {(void*)P};
-    const bool wide = P->n_regions > kWideWalkRegions;
-    const unsigned g = wide ? grid : (grid + kBeamBlocksPerSM - 1) / kBeamBlocksPerSM;
-    if (e == cudaSuccess) {
-        if (narrow && !wide)  // one narrow block per SM
-            e = cudaLaunchCooperativeKernel((const void*)beam_kernel_narrow, g, kBeamNarrowThreads, args, 0, st);
-        else
-            e = cudaLaunchCooperativeKernel((const void*)beam_kernel, g, kBeamThreads, args, 0, st);
+    const unsigned g = beside && P->n_regions <= kWideWalkRegions ? (grid + kBeamBlocksPerSM - 1) / kBeamBlocksPerSM : grid;
+    if (e == cudaSuccess && P->n_views == 1) {
+        BeamParams<1> one;
+        static_cast<BeamHead&>(one) = *P;
+        one.v[0] = P->v[0];
+        void* args[] = {&one};
+        e = cudaLaunchCooperativeKernel((const void*)beam_kernel<BeamParams<1>>, g, kBeamThreads, args, 0, st);
+    } else if (e == cudaSuccess) {
+        void* args[] = {(void*)P};
+        e = cudaLaunchCooperativeKernel((const void*)beam_kernel<BeamBatch>, g, kBeamThreads, args, 0, st);
     }
     if (e == cudaSuccess) e = cudaEventRecord(g_beam_done[dev], st);
     return aokk_status(e);

@@ -116,7 +116,7 @@ struct BeamView {
     const ChunkRef* frame;
     unsigned long long* bounds;  // the view's pyramid (beam_entries(W, H) entries)
     float Af[9];                 // row-major inverse of A = [R col 0, R col 1, -R col 2] (d = A (u, v, 1)), FP32
-    float U, V;                  // u and v at the screen edges: tan_half * W / H, tan_half
+    float iU, iV;                // 1 / u and 1 / v at the screen edges: 1 / (tan_half * W / H), 1 / tan_half
     float near_dn;               // numerator units: boxes closer than this cover every tile
     float view_num;              // > 0: boxes farther than this (Euclidean, numerator units) are dropped
     int32_t W, H, tiles_x, tiles_y;
@@ -124,21 +124,27 @@ struct BeamView {
     uint32_t region_begin;       // first item of this view among the pass's regions
 };
 
-// The parameter block of one beam pass over up to kBeamViews views.
-struct BeamBatch {
+// The parameter block of one beam pass over up to N views (a single view's
+// pass copies and launches 0.6 KB of parameters instead of 27).
+struct BeamHead {
     uint32_t n_views, n_regions;  // views; chunk regions of all views
     uint32_t expand;              // refine nodes whose rectangle spans more tiles than this ...
     int32_t smin;                 // ... and whose side is above 2^smin LOD-0 voxels
     uint32_t tag;                 // the pass's tag: decreases from pass to pass
     uint32_t cap;                 // queue capacity in items
-    uint4* q[2];                  // node queues of alternate levels: {chunk, node, cell x | y << 10 | z << 20, log2 size | view << 8 | LOD << 16}
-    uint32_t* cnt;                // [kBeamLevels] items queued per level
+    uint4* q[2];                  // queues of nodes to refine, of alternate levels: {chunk, node, cell x | y << 10 | z << 20,
+                                  // log2 size | view << 8 | LOD << 16 | child mask << 24}
+    uint32_t* cnt;                // [kBeamLevels] items queued per level; zero between passes
     uint32_t* hist;               // [kBeamLevels] nodes walked per depth below the region roots
     uint32_t select;              // 1: one view whose frame table the pass selects first (cam)
     CamDev cam;                   // that view's camera (select == 1)
     CheckDev ck;                  // ck.err != nullptr: node and leaf indices tested before their loads
-    BeamView v[kBeamViews];
 };
+template <int N>
+struct BeamParams : BeamHead {
+    BeamView v[N];
+};
+using BeamBatch = BeamParams<kBeamViews>;
 static_assert(sizeof(BeamBatch) < 32000, "a beam pass's parameters must fit the kernel parameter space");
 
 // What a casting kernel reads of a view's beam pass (bounds == nullptr: none).
@@ -213,7 +219,7 @@ static_assert(sizeof(BatchParams) < 32000, "batched launch parameters must fit t
 struct GraphCache {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
-    std::vector<cudaGraphNode_t> nodes;  // per group: select, [counter memset, beam pass], cast
+    std::vector<cudaGraphNode_t> nodes;  // per group: select, [beam pass], cast
     std::vector<uint64_t> key;
 };
 
@@ -233,17 +239,16 @@ int aokk_cast(const aok::SceneDev* s, const aok::CamDev* c, const aok::ChunkRef*
               uint32_t* counts, void* stream, const aok::CheckDev* ck, const aok::BeamRead* beam = nullptr);
 // Beam pass (aok_beam.cu).  aokk_beam_view fills a view's projection (false:
 // the camera matrix has no usable inverse; leave the view out, it casts
-// without bounds); aokk_beam_run zeroes P's counters and launches the pass
-// (narrow: as one 128-thread block per SM that fits beside a running cast,
-// for walks over at most 4096 regions; the pipelined host frames use it).
+// without bounds); aokk_beam_run launches the pass
+// (beside: with one block per SM, for a pass that starts beside the cast of
+// the frame before, as in the pipelined host frames).
 bool aokk_beam_view(const aok::SceneDev* S, const aok::CamDev* C, const aok::ChunkRef* frame,
                     unsigned long long* bounds, aok::BeamView* out);
-int aokk_beam_run(const aok::BeamBatch* P, unsigned grid, void* stream, int narrow = 0);
-// The pass as a graph node (kernel + counter memset) and the per-device pass
+int aokk_beam_run(const aok::BeamBatch* P, unsigned grid, void* stream, int beside = 0);
+// The pass as a graph's kernel node and the per-device pass
 // order around a graph launch (record = 0: wait for the previous pass before;
 // 1: mark the end of the launch as the point the next pass waits for).
-void aokk_beam_node(const aok::BeamBatch* P, unsigned grid, void** argp, cudaKernelNodeParams* kp,
-                    cudaMemsetParams* zero);
+void aokk_beam_node(const aok::BeamBatch* P, unsigned grid, void** argp, cudaKernelNodeParams* kp);
 int aokk_beam_order(void* stream, int record);
 // Blocks of the beam pass's cooperative launch on `sms` SMs (0 on error).
 unsigned aokk_beam_grid(int sms);

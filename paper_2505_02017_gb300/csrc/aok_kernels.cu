@@ -260,7 +260,7 @@ int aokk_cast_batch(const BatchParams* p, uint32_t ctas, uint32_t threads, void*
 // group's beam pass (beams[g], one cooperative launch) runs between its
 // selection and its cast.  With a cache and no hand-off stream, the whole
 // sequence is one CUDA graph built per shape (group sizes, launch dims, which
-// groups hold a beam pass) -- select, counter memset and cooperative beam
+// groups hold a beam pass) -- select, cooperative beam
 // kernel, cast per group, chained -- whose nodes are updated with the new
 // parameters on every call; a graph holding beam passes keeps the per-device
 // order of passes around its launch.
@@ -329,11 +329,7 @@ int aokk_batch_run(const BatchParams* groups, uint32_t n_groups, uint32_t ctas, 
             if (e != cudaSuccess) break;
             add(node);
             if (has_beam(g)) {
-                cudaMemsetParams zp;
-                aokk_beam_node(&beams[g], beam_grid, argp, &kp, &zp);
-                e = cudaGraphAddMemsetNode(&node, gc->graph, &prev, 1, &zp);
-                if (e != cudaSuccess) break;
-                add(node);
+                aokk_beam_node(&beams[g], beam_grid, argp, &kp);
                 e = cudaGraphAddKernelNode(&node, gc->graph, &prev, 1, &kp);
                 if (e != cudaSuccess) break;
                 cudaLaunchAttributeValue coop;
@@ -362,10 +358,8 @@ int aokk_batch_run(const BatchParams* groups, uint32_t n_groups, uint32_t ctas, 
             params(g, true, argp, kp);
             e = cudaGraphExecKernelNodeSetParams(gc->exec, gc->nodes[i++], &kp);
             if (e == cudaSuccess && has_beam(g)) {
-                cudaMemsetParams zp;
-                aokk_beam_node(&beams[g], beam_grid, argp, &kp, &zp);
-                e = cudaGraphExecMemsetNodeSetParams(gc->exec, gc->nodes[i++], &zp);
-                if (e == cudaSuccess) e = cudaGraphExecKernelNodeSetParams(gc->exec, gc->nodes[i++], &kp);
+                aokk_beam_node(&beams[g], beam_grid, argp, &kp);
+                e = cudaGraphExecKernelNodeSetParams(gc->exec, gc->nodes[i++], &kp);
             }
             if (e == cudaSuccess) {
                 params(g, false, argp, kp);

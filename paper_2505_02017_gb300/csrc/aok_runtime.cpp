@@ -899,6 +899,11 @@ static int ensure_beam_queues(aok_ctx* ctx) {
     b.q[1] = (uint4*)((char*)block + sq);
     b.cnt = (uint32_t*)((char*)block + 2 * sq);
     b.hist = b.cnt + kBeamLevels;
+    // (each pass leaves the queue counters at zero)
+    if (cudaMemset(b.cnt, 0, sc) != cudaSuccess || cudaStreamSynchronize(nullptr) != cudaSuccess) {
+        dev_free(ctx, block, 2 * sq + sc);
+        return cuda_status(ctx, cudaGetLastError());
+    }
     b.qblock = block;
     b.qbytes = 2 * sq + sc;
     b.grid = aokk_beam_grid(ctx->sm_count);

@@ -160,7 +160,7 @@ struct aok_ctx {
     aok::TileState tiles;
     aok::BeamState beam;
     int beam_on = 1;  // single-view renders run the beam pass before casting
-    uint32_t beam_refine = 8;  // refine nodes spanning more tiles than this ...
+    uint32_t beam_refine = 16;  // refine nodes spanning more tiles than this ...
     int beam_min_log2 = 2;     // ... whose side is above 2^this LOD-0 voxels
     uint64_t beam_min_pixels = 1500000;  // smaller frames cast without the pass
     uint32_t beam_queue = 0;             // nodes a queue level may hold (0: the allocated 2^20)

@@ -250,9 +250,9 @@ def bench_batched(aok, ctx, scene, world, flush, reps=5):
     equal = equal and all(torch.equal(a[0], b[0]) and torch.equal(a[1].view(torch.int32), b[1].view(torch.int32))
                           for a, b in zip(plain, eager))
     ctas, threads, packet = aok.get_launch(ctx)
-    # the beam pass runs for views of at least 1.5 M pixels: one launch per
+    # the beam pass runs for views of at least 0.8 M pixels: one launch per
     # such plain render, one for the batch (grid launch)
-    big = sum(1 for c in cams if c.W * c.H >= 1_500_000) if BEAM_DEFAULT else 0
+    big = sum(1 for c in cams if c.W * c.H >= 800_000) if BEAM_DEFAULT else 0
     return {"workload": "city4096, 64 views (seed 104), resolutions uniform over "
                         "{320x180, 640x360, 1280x720, 1920x1080, 2560x1440}, tau = 1 px",
             "rays": rays, "plain_rays_per_s": rays / (p_med / 1e3), "batched_rays_per_s": rays / (b_med / 1e3),

@@ -527,7 +527,7 @@ int aok_render_noalloc(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, doub
  * Sec. 2; here exact): with on = 1, aok_render, aok_render_counted,
  * aok_render_host(_async), aok_cast_selected, aok_render_batch (grid
  * launch) and the render server of this context first compute, for every 8 x 4 pixel tile of each
- * frame of at least 1.5 M pixels (aok_beam_tune), a lower bound on the
+ * frame of at least 0.8 M pixels (aok_beam_tune), a lower bound on the
  * L-infinity distance from the camera origin of every solid voxel of the
  * frame's LOD-cut scene that the tile's rays can meet: a level-by-level walk
  * of the selected DAGs (all views of a batch in one launch), refining a node
@@ -550,7 +550,7 @@ int aok_set_beam(aok_ctx* ctx, int on);
 /* Refinement of the beam pass's walk: a node is refined while its rectangle
  * spans more than refine_tiles tiles and its side is above 2^min_node_log2
  * LOD-0 voxels (a context starts with 16 and 2: down to the 4^3 leaves); frames of fewer
- * than min_pixels pixels cast without the pass (default 1,500,000: below
+ * than min_pixels pixels cast without the pass (a context starts with 800,000: below
  * that the pass's fixed cost, some tens of microseconds, outweighs what it
  * saves); queue_nodes caps the nodes one level of the walk may queue
  * (0: the allocated 2^20; past the cap a node stands for its children).

@@ -20,6 +20,8 @@ using namespace aok;
 
 namespace {
 
+constexpr int kMaxDevices = 128;
+
 __global__ void select_kernel(SceneDev S, CamDev C, ChunkRef* __restrict__ frame, int8_t* __restrict__ lod_out,
                               uint8_t* __restrict__ vis_out, uint32_t* __restrict__ n_visible) {
     const int nch = S.grid[0] * S.grid[1] * S.grid[2];
@@ -64,24 +66,56 @@ __device__ __forceinline__ int32_t beam_bound_warp(const BeamLookup& b, int px, 
 // 8 blocks per SM (72 and 7 blocks: overview 3840x2160 511 us a frame instead
 // of 491, city 1080p 360 instead of 354; 56 and 9 blocks: 482 and 352, but
 // 320x180 views, where occupancy does not matter, 3% slower).
+//
+// Without bounds a warp may take a smaller tile, wl and hl its sides' logs (3
+// and 2: 8 x 4), in its first lanes: see cast_tile.
 template <bool COUNT, bool BEAM = false>
 __global__ void __launch_bounds__(128, 8) cast_kernel(const __grid_constant__ SceneDev S,
                                                    const __grid_constant__ CamDev C,
                                                    const ChunkRef* __restrict__ frame,
                                                    uint4* __restrict__ out_hit, float* __restrict__ out_t,
                                                    uint32_t* __restrict__ counts,
-                                                   const __grid_constant__ BeamLookup beam) {
+                                                   const __grid_constant__ BeamLookup beam, int wl, int hl) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int px = blockIdx.x * 16 + (warp & 1) * 8 + (lane & 7);
-    const int py = blockIdx.y * 8 + (warp >> 1) * 4 + (lane >> 3);
-    const uint32_t lanes = __ballot_sync(0xFFFFFFFFu, px < C.W && py < C.H);
-    const int wx = px - (lane & 7), wy = py - (lane >> 3);  // the warp's tile
-    if (wx >= C.W || wy >= C.H) return;
+    if (BEAM) { wl = 3; hl = 2; }
+    const int wx = (blockIdx.x * 2 + (warp & 1)) << wl, wy = (blockIdx.y * 2 + (warp >> 1)) << hl;  // the warp's tile
+    const int px = wx + (lane & ((1 << wl) - 1)), py = wy + (lane >> wl);
+    const bool in = px < C.W && py < C.H && lane < 1 << (wl + hl);
+    const uint32_t lanes = __ballot_sync(0xFFFFFFFFu, in);
+    if (!lanes) return;
     const int32_t Dn = BEAM ? beam_bound_warp(beam, wx, wy, lane) : 0;
-    if (px >= C.W || py >= C.H) return;
+    if (!in) return;
     const size_t pix = (size_t)py * C.W + px;
     if (COUNT) trace_pixel<true, false, BEAM>(S, C, frame, px, py, out_hit, out_t, counts, pix, nullptr, Dn);
     else cast_pixel<BEAM>(S, C, frame, px, py, out_hit, out_t, pix, Dn, lanes);
+}
+
+// Warp tile of a frame cast without bounds.  A frame of fewer pixels than the
+// GPU holds threads ends when its slowest warp does, and a warp takes as long
+// as the paths of all its rays together, step by step: with fewer rays a warp
+// there are as many chains, each shorter, on schedulers that idle otherwise.
+// So the smallest tile whose warps still fit one resident wave (8 blocks of 4
+// warps per SM; 4,864 warps on 152 SMs): 16 rays up to 77,824 pixels, 8 up to
+// 38,912, and so on to one.  Four city views each, 8 x 4 tiles -> this rule:
+// 320x180 66 / 78 / 96 / 68 -> 62 / 72 / 85 / 62 us, 160x90 74 / 70 / 154 / 60
+// -> 51 / 45 / 102 / 45, 96x54 76 / 84 / 135 / 66 -> 39 / 39 / 68 / 41; past
+// one wave it turns (480x270, 16 rays: 90 / 77 / 123 / 117 -> 99 / 82 / 115 / 104).
+static void cast_tile(const CamDev& c, int& wl, int& hl) {
+    static std::atomic<int> sms[kMaxDevices];
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) dev = 0;
+    n = sms[dev].load(std::memory_order_relaxed);
+    if (!n) {
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) n = 1;
+        sms[dev].store(n, std::memory_order_relaxed);
+    }
+    wl = 3;
+    hl = 2;
+    const int64_t px = (int64_t)c.W * c.H, warps = (int64_t)n * 32;
+    while (wl + hl > 0 && px <= warps << (wl + hl - 1)) {
+        if (wl > hl) wl--;
+        else hl--;
+    }
 }
 
 // The same casting with every pool index checked (CheckDev); BEAM: with the
@@ -222,23 +256,32 @@ int aokk_select(const SceneDev* s, const CamDev* c, ChunkRef* frame, int8_t* lod
     return status_of(cudaGetLastError());
 }
 
+static void cast_plain(const SceneDev* s, const CamDev* c, const ChunkRef* frame, uint4* hit, float* t,
+                       cudaStream_t st) {
+    int wl, hl;
+    cast_tile(*c, wl, hl);
+    dim3 grid((c->W + (2 << wl) - 1) >> (wl + 1), (c->H + (2 << hl) - 1) >> (hl + 1));
+    cast_kernel<false><<<grid, 128, 0, st>>>(*s, *c, frame, hit, t, nullptr, beam_lookup(nullptr, 0, 0), wl, hl);
+}
+
 int aokk_cast(const SceneDev* s, const CamDev* c, const ChunkRef* frame, uint4* hit, float* t, uint32_t* counts,
               void* stream, const CheckDev* ck, const BeamRead* beam) {
     dim3 grid((c->W + 15) / 16, (c->H + 7) / 8);
     const cudaStream_t st = (cudaStream_t)stream;
+    int wl = 3, hl = 2;
     const BeamLookup bl = beam_lookup(beam, c->W, c->H);
     if (ck && !counts && beam)
         cast_kernel_checked<true><<<grid, 128, 0, st>>>(*s, *c, frame, hit, t, *ck, bl);
     else if (ck && !counts)
         cast_kernel_checked<false><<<grid, 128, 0, st>>>(*s, *c, frame, hit, t, *ck, bl);
     else if (counts && beam)
-        cast_kernel<true, true><<<grid, 128, 0, st>>>(*s, *c, frame, hit, t, counts, bl);
+        cast_kernel<true, true><<<grid, 128, 0, st>>>(*s, *c, frame, hit, t, counts, bl, wl, hl);
     else if (counts)
-        cast_kernel<true><<<grid, 128, 0, st>>>(*s, *c, frame, hit, t, counts, bl);
+        cast_kernel<true><<<grid, 128, 0, st>>>(*s, *c, frame, hit, t, counts, bl, wl, hl);
     else if (beam)
-        cast_kernel<false, true><<<grid, 128, 0, st>>>(*s, *c, frame, hit, t, nullptr, bl);
+        cast_kernel<false, true><<<grid, 128, 0, st>>>(*s, *c, frame, hit, t, nullptr, bl, wl, hl);
     else
-        cast_kernel<false><<<grid, 128, 0, st>>>(*s, *c, frame, hit, t, nullptr, bl);
+        cast_plain(s, c, frame, hit, t, st);
     return status_of(cudaGetLastError());
 }
 
@@ -446,8 +489,7 @@ int aokk_read_bw(const void* buf, size_t n16, int passes, uint32_t* sink, int sm
 // ---------------------------------------------------------------------------
 static __device__ __align__(256) ChunkRef g_noalloc_frame[AOK_NOALLOC_MAX_CHUNKS];
 
-static constexpr int kMaxNoallocDevices = 128;
-static std::atomic<ChunkRef*> g_noalloc_ptr[kMaxNoallocDevices];
+static std::atomic<ChunkRef*> g_noalloc_ptr[kMaxDevices];
 static std::mutex g_noalloc_mu;
 
 int aokk_render_noalloc(const SceneDev* s, const CamDev* c, uint4* hit, float* t, void* stream, const CheckDev* ck) {
@@ -455,7 +497,7 @@ int aokk_render_noalloc(const SceneDev* s, const CamDev* c, uint4* hit, float* t
     if (nch > AOK_NOALLOC_MAX_CHUNKS) return AOK_E_INVALID;
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess) return AOK_E_CUDA;
-    if (dev < 0 || dev >= kMaxNoallocDevices) return AOK_E_INVALID;
+    if (dev < 0 || dev >= kMaxDevices) return AOK_E_INVALID;
     ChunkRef* frame = g_noalloc_ptr[dev].load(std::memory_order_acquire);
     if (!frame) {
         std::lock_guard<std::mutex> g(g_noalloc_mu);
@@ -474,7 +516,7 @@ int aokk_render_noalloc(const SceneDev* s, const CamDev* c, uint4* hit, float* t
     if (ck)
         cast_kernel_checked<false><<<grid, 128, 0, st>>>(*s, *c, frame, hit, t, *ck, beam_lookup(nullptr, 0, 0));
     else
-        cast_kernel<false><<<grid, 128, 0, st>>>(*s, *c, frame, hit, t, nullptr, beam_lookup(nullptr, 0, 0));
+        cast_plain(s, c, frame, hit, t, st);
     return status_of(cudaGetLastError());
 }
 

@@ -95,3 +95,15 @@ def test_walk_of_scaled_directions(ctx, scale):
     assert torch.equal(want, got)
     _equal_to_march(ctx, sc, cam, 1.5 / scale)
     sc.destroy()
+
+
+@pytest.mark.parametrize("size", [(1, 1), (3, 2), (61, 79), (64, 76), (139, 70), (139, 71), (278, 140), (278, 141), (399, 390)])
+def test_small_frames_at_the_edges_of_the_warp_tiles(ctx, size):
+    # frames around the sizes where a warp takes 1, 2, 4, 8, 16 or 32 rays (152 SMs), with ragged edges
+    w = sg.World(MED64)
+    sc = aok.Scene.from_world(ctx, w, threads=4)
+    aok.beam_tune(ctx, 16, 2, 1 << 40, 0)
+    for seed in (4, 9):
+        _equal_to_march(ctx, sc, sg.ground_camera(w, seed, *size, z_lo=4, z_hi=40), 1.5)
+    aok.beam_tune(ctx)
+    sc.destroy()

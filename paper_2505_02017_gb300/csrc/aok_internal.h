@@ -72,8 +72,7 @@ struct CamDev {
 // Device buffers of the tile-chunk pipeline (Sec. 3.5) for one resolution.
 constexpr int kTileStats = 8;
 struct TileDev {
-    unsigned long long* vis;   // [W*H][2] visibility records: key (distance | march order | chunk), ~0 = none;
-                               // payload (hit voxel, LOD, entry axis, material)
+    unsigned long long* vis;   // [W*H] visibility records (march order | chunk | hit), ~0 = none
     float* hiz_prev;           // [tiles] previous frame's per-tile max hit distance (no culling: huge)
     float* hiz;                // [tiles] per-tile max distance after pass 1 of this frame
     float* hiz_next;           // [tiles] this frame's final per-tile max distance
@@ -82,10 +81,13 @@ struct TileDev {
     int32_t* dfar;             // [chunks] largest L-inf distance (2^-12 units) from the camera origin to a
                                // point of the AABB
     uint32_t* area;            // [chunks] tiles in the rectangle (0: no pairs)
-    uint32_t* list;            // [chunks] chunks with pairs, ascending
+    uint32_t* list;            // [chunks] chunks with pairs, roughly front to back
     unsigned long long* offs;  // [chunks + 1] exclusive prefix of their areas; offs[n_list] = pairs
     unsigned long long* stats; // [kTileStats] n_list, items traced / culled per pass, pixel traces ...
     int32_t tiles_x, tiles_y;
+    // a record's chunk: its grid coordinates along axes ax[0] and ax[1] in ba
+    // and bb bits; the one along ax[2] (the longest) follows from the order
+    int32_t ax[3], ba, bb;
 };
 
 // The beam pass (ESVO's beam optimisation, Sec. 2; aok_beam.cu): per 8 x 4

@@ -1184,7 +1184,7 @@ static int ensure_tiles(aok_ctx* ctx, uint32_t scene, int32_t W, int32_t H, int6
     const int32_t tx = (W + 7) / 8, ty = (H + 7) / 8;
     const size_t tiles = (size_t)tx * ty, px = (size_t)W * H, n = (size_t)nch;
     auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
-    const size_t sz[] = {px * 16, tiles * 4, tiles * 4, tiles * 4, n * 16, n * 4, n * 4, n * 4, (n + 1) * 8,
+    const size_t sz[] = {px * 8, tiles * 4, tiles * 4, tiles * 4, n * 16, n * 4, n * 4, n * 4, (n + 1) * 8,
                          kTileStats * 8, n * 4};
     constexpr int kParts = (int)(sizeof(sz) / sizeof(sz[0]));
     size_t total = 0;
@@ -1209,7 +1209,7 @@ static int ensure_tiles(aok_ctx* ctx, uint32_t scene, int32_t W, int32_t H, int6
     d.dfar = (int32_t*)q[10];
     d.tiles_x = tx;
     d.tiles_y = ty;
-    cudaError_t e = cudaMemsetAsync(d.vis, 0xFF, px * 16, s);
+    cudaError_t e = cudaMemsetAsync(d.vis, 0xFF, px * 8, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(d.hiz_prev, 0x7F, tiles * 4, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(d.stats, 0, kTileStats * 8, s);
     if (e != cudaSuccess) {
@@ -1227,6 +1227,23 @@ static int ensure_tiles(aok_ctx* ctx, uint32_t scene, int32_t W, int32_t H, int6
     return AOK_OK;
 }
 
+// How a visibility record holds its region for this grid (the longest axis last).
+static void tile_axes(const SceneDev& sd, TileDev& d) {
+    int last = 0;
+    for (int a = 1; a < 3; a++)
+        if (sd.grid[a] > sd.grid[last]) last = a;
+    d.ax[0] = last == 0 ? 1 : 0;
+    d.ax[1] = last == 2 ? 1 : 2;
+    d.ax[2] = last;
+    auto bits = [](int32_t v) {
+        int n = 0;
+        while (v >> n) n++;
+        return n;
+    };
+    d.ba = bits(sd.grid[d.ax[0]] - 1);
+    d.bb = bits(sd.grid[d.ax[1]] - 1);
+}
+
 int aok_render_tiles(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, double tau, const aok_frame* frame,
                      void* stream) {
     if (!ctx || !frame || !frame->hit || !frame->t) return AOK_E_INVALID;
@@ -1241,14 +1258,17 @@ int aok_render_tiles(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, double
     st = ensure_tiles(ctx, scene, cd.W, cd.H, sc->n_chunks, (cudaStream_t)stream);
     if (st) return st;
     SceneDev sd = scene_dev(sc);
+    tile_axes(sd, ctx->tiles.dev);
     sc->select_gen++;
-    st = aokk_select(&sd, &cd, sc->d_frame, nullptr, nullptr, nullptr, stream);
     // the beam pass's bounds cull the pairs in front of every voxel a tile's
-    // rays can meet and restart the rays of the others (as in the march)
+    // rays can meet and restart the rays of the others (as in the march); the
+    // pass selects the frame table as its first step
     const BeamRead* beam = nullptr;
-    if (!st && beam_wanted(ctx, cd.W, cd.H)) {
-        st = run_beam(ctx, scene, sc, sd, cd, stream);
+    if (beam_wanted(ctx, cd.W, cd.H)) {
+        st = run_beam(ctx, scene, sc, sd, cd, stream, true);
         beam = &ctx->beam.read;
+    } else {
+        st = aokk_select(&sd, &cd, sc->d_frame, nullptr, nullptr, nullptr, stream);
     }
     if (!st) st = aokk_tiles_frame(&sd, &cd, sc->d_frame, &ctx->tiles.dev, (uint4*)frame->hit, frame->t,
                                    ctx->sm_count, stream, beam);

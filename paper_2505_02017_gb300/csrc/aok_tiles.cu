@@ -25,56 +25,45 @@
 // nearer one.  With the beam pass (aok_beam.cu) a half tile (8 x 4 pixels,
 // one beam tile) also skips the pairs whose chunk AABB lies wholly nearer
 // than its bound -- no voxel there can be met -- and its rays start each
-// remaining pair at the bound's restart plane, as in the march.  Differences from the paper: the pair list is implicit (a
-// prefix sum over the chunks' rectangle areas, searched by the marching warps)
+// remaining pair at the bound's restart plane, as in the march.  Differences
+// from the paper: the pair list is implicit (a prefix sum over the chunks'
+// rectangle areas, front to back, stepped through by the marching warps)
 // instead of an appended TileInfo buffer with indirect dispatch; the key is
-// widened; each marching warp takes half a tile (32 pixels).
+// the march order; each marching warp takes half a tile (32 pixels).
 //
-// Visibility record: 16 bytes per pixel, a key and a payload installed
-// together by a 128-bit compare-and-swap (the paper's 64-bit InterlockedMax
-// record of depth | normal | 13-bit chunk ID | 24-bit position cannot address
-// 512^3 chunks).  Payload: the hit voxel's world LOD-0 corner x, y, z (17 bits
-// each), its LOD (3 bits), the entry axis (2 bits; 3: origin inside) and the
-// material (8 bits) -- with the ray, everything the output record needs.
-// Key:
-//   bits 63..32  top 32 bits of the FP64 ray parameter t of the hit (t >= 0,
-//                so the IEEE bits order as integers; truncation keeps order)
-//   bits 31..16  place of the chunk region in the march order along the ray:
-//                the sum of its mirrored grid coordinates, which grows by one
-//                from each region of a ray's march to the next
-//   bits 15..0   chunk region index (scenes of at most 65536 regions)
-// The minimum key is the hit of the first region along the ray that has one,
-// the march's answer: a later region's hit never has a smaller t, and equal
-// truncated t falls back to the march order.
+// Visibility record: 64 bits per pixel, installed by an atomic minimum.  From
+// the top:
+//   the place of the chunk region in the march order along the ray: the sum
+//       of its mirrored grid coordinates, which grows by one from each region
+//       of a ray's march to the next;
+//   the region's grid coordinates along its two shorter axes (the third
+//       follows from the order): at most 19 bits with the order for the 65,536
+//       regions a scene may have;
+//   40 bits of the hit: the voxel's index in the region's DAG (9 bits per
+//       axis), its LOD (3), the entry axis (2; 3: origin inside), the material
+//       (8) -- with the ray, everything the output record needs.
+// The minimum is the hit of the first region along the ray that has one, the
+// march's answer.  (The paper's record has the depth on top, which orders the
+// hits of different chunks as the march does, but needs a division a hit, and
+// here an FP64 one so that keys cannot misorder.)  City 1920x1080, changing
+// views: 1236 us a frame with 32-bit depth keys and a 128-bit compare-and-swap
+// of key and payload, exact 64-bit comparisons and regions in index order; 645
+// with this record, the FP32 walk (aok_walk.cuh) and regions front to back.
 #include <cuda_runtime.h>
 
 #include <cstdint>
 
 #include "aok_internal.h"
 #include "aok_trace.cuh"
+#include "aok_walk.cuh"
 
 using namespace aok;
 
 namespace {
 
 constexpr unsigned long long kNoKey = ~0ull;
-constexpr int kCasLimit = 4096;  // attempts: each failure means another chunk's smaller key went in
-
-// 128-bit compare-and-swap on a 16-byte aligned record (sm_90+): returns the
-// previous record.
-__device__ __forceinline__ ulonglong2 cas128(unsigned long long* p, ulonglong2 cmp, ulonglong2 val) {
-    ulonglong2 old;
-    asm volatile("{\n\t.reg .b128 d, c, n;\n\t"
-                 "mov.b128 c, {%2, %3};\n\t"
-                 "mov.b128 n, {%4, %5};\n\t"
-                 "atom.global.cas.b128 d, [%6], c, n;\n\t"
-                 "mov.b128 {%0, %1}, d;\n\t}"
-                 : "=l"(old.x), "=l"(old.y)
-                 : "l"(cmp.x), "l"(cmp.y), "l"(val.x), "l"(val.y), "l"(p)
-                 : "memory");
-    return old;
-}
-enum { kStList = 0, kStTraced1, kStCulled1, kStTraced2, kStCulled2, kStPixelTraces, kStPixelSkips, kStCasExhausted };
+constexpr int kHitBits = 40;  // a record's bits below the region's
+enum { kStList = 0, kStTraced1, kStCulled1, kStTraced2, kStCulled2, kStPixelTraces, kStPixelSkips };
 
 __device__ __forceinline__ void region_coords(const SceneDev& S, uint32_t chunk, int32_t u[3]) {
     u[0] = (int32_t)(chunk % (uint32_t)S.grid[0]);
@@ -82,10 +71,72 @@ __device__ __forceinline__ void region_coords(const SceneDev& S, uint32_t chunk,
     u[2] = (int32_t)(chunk / ((uint32_t)S.grid[0] * (uint32_t)S.grid[1]));
 }
 
-// top 32 bits of t = N / (2^12 |d_e|) in FP64 (N >= 0; exact operands, one rounding)
-__device__ __forceinline__ uint32_t t_key(int32_t N, float de) {
-    const double t = __ddiv_rn((double)N, __dmul_rn(4096.0, fabs((double)de)));
-    return (uint32_t)((unsigned long long)__double_as_longlong(t) >> 32);
+// The record of a hit in region u (order: its place in the march order).
+__device__ __forceinline__ unsigned long long pack_hit(const SceneDev& S, const TileDev& T, const int32_t u[3],
+                                                       uint32_t order, uint32_t mir, int n, const HitRec& hit,
+                                                       uint32_t mat) {
+    const int32_t side = (1 << (S.mlog - n)) - 1;
+    unsigned long long r = 0;
+#pragma unroll
+    for (int a = 0; a < 3; a++)
+        r |= (unsigned long long)(uint32_t)(((mir >> a) & 1u) ? side - hit.c[a] : hit.c[a]) << (9 * a);
+    r |= (unsigned long long)n << 27 | (unsigned long long)hit.e << 30 | (unsigned long long)mat << 32;
+    const unsigned long long reg = ((unsigned long long)order << (T.ba + T.bb)) |
+                                   ((unsigned long long)(uint32_t)sel3(T.ax[0], u[0], u[1], u[2]) << T.bb) |
+                                   (uint32_t)sel3(T.ax[1], u[0], u[1], u[2]);
+    return reg << kHitBits | r;
+}
+
+// Atomic minimum without a return value (a reduction the SM does not wait for).
+__device__ __forceinline__ void red_min_u64(unsigned long long* p, unsigned long long v) {
+    asm volatile("red.global.min.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
+// A record decoded for its ray (direction d): voxel corner, LOD, entry axis,
+// material and the hit distance, as emit_hit computes it.
+struct VisHit {
+    uint32_t c[3], mat;
+    int n, e;
+    uint32_t normal;
+    float dist;
+};
+__device__ __forceinline__ VisHit unpack_hit(const SceneDev& S, const CamDev& C, const TileDev& T,
+                                             unsigned long long key, const float d[3]) {
+    const uint32_t mir = (d[0] < 0.0f ? 1u : 0u) | (d[1] < 0.0f ? 2u : 0u) | (d[2] < 0.0f ? 4u : 0u);
+    const uint32_t reg = (uint32_t)(key >> kHitBits);
+    const int32_t ua = (int32_t)((reg >> T.bb) & ((1u << T.ba) - 1u)), ub = (int32_t)(reg & ((1u << T.bb) - 1u));
+    const int a0 = T.ax[0], a1 = T.ax[1], a2 = T.ax[2];
+    auto mirrored = [&](int a, int32_t v) {
+        return ((mir >> a) & 1u) ? sel3(a, S.grid[0], S.grid[1], S.grid[2]) - 1 - v : v;
+    };
+    const int32_t uc = mirrored(a2, (int32_t)(reg >> (T.ba + T.bb)) - mirrored(a0, ua) - mirrored(a1, ub));
+    VisHit h;
+    h.n = (int)((key >> 27) & 7u);
+    h.e = (int)((key >> 30) & 3u);
+    h.mat = (uint32_t)(key >> 32) & 0xFFu;
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        const int32_t u = a == a0 ? ua : (a == a1 ? ub : uc);
+        h.c[a] = (uint32_t)((u << S.mlog) + (int32_t)(((uint32_t)(key >> (9 * a)) & 511u) << h.n));
+    }
+    h.dist = 0.0f;
+    h.normal = 7u;
+    if (h.e < 3) {
+        // entry plane: the voxel's face the mirrored ray meets first, as a numerator
+        const bool m = (mir >> h.e) & 1u;
+        const int32_t we = (int32_t)sel3(h.e, h.c[0], h.c[1], h.c[2]), G = sel3(h.e, S.grid[0], S.grid[1], S.grid[2]),
+                      O = sel3(h.e, C.O[0], C.O[1], C.O[2]);
+        const int32_t face = m ? (G << S.mlog) - we - (1 << h.n) : we;
+        const int32_t Ow = m ? (G << (S.mlog + kFix)) - O : O;
+        const int32_t Ne = (int32_t)((uint32_t)face << kFix) - Ow;
+        RayState r;
+        r.d[0] = d[0];
+        r.d[1] = d[1];
+        r.d[2] = d[2];
+        h.dist = __fdiv_rn((float)Ne * (1.0f / 4096.0f), fabsf(sel3(h.e, d[0], d[1], d[2]))) * ray_norm(r);
+        h.normal = (uint32_t)(2 * h.e) + ((mir >> h.e) & 1u);
+    }
+    return h;
 }
 
 // How the march enters chunk region u: entry axis e (3: the origin lies in
@@ -172,22 +223,21 @@ __device__ __forceinline__ bool aabb_pass(const SceneDev& S, const CamDev& C, co
     return tn <= tf;
 }
 
-// One pixel of a pair: 0 = region not entered, 1 = traced, 2 = skipped (the
-// pixel already holds a hit nearer than the region's entry, or the beam
-// bound Dn puts every voxel the ray can meet past the region).  Dn > 0: the
+// One pixel of a pair with exact comparisons throughout: 0 = region not
+// entered, 1 = traced, 2 = skipped (the pixel already holds a hit of an earlier
+// region, or the beam bound Dn puts every voxel the ray can meet past the
+// region).  Dn > 0: the
 // ray starts at the bound's restart plane when that lies later than the
 // region's entry (trace_pixel_t's beam restart, within one region).
 template <bool FAST, bool BEAM>
 __device__ __forceinline__ int pair_pixel(const SceneDev& S, const CamDev& C, const ChunkRef& ref, uint32_t chunk,
-                                          const RayState& r, size_t pix, unsigned long long* __restrict__ vis,
-                                          int32_t Dn) {
+                                          const RayState& r, size_t pix, const TileDev& T, int32_t Dn) {
     int32_t u[3];
     region_coords(S, chunk, u);
     Entry en;
     if (!enter_region<FAST>(S, C, r, u, en) || !aabb_pass(S, C, r, ref, u)) return 0;
-    unsigned long long* rec = vis + 2 * pix;
-    const unsigned long long cur = __ldcg(rec);
-    if (cur != kNoKey && en.e < 3 && t_key(en.Ne, r.d[en.e]) > (uint32_t)(cur >> 32)) return 2;
+    const unsigned long long cur = __ldcg(T.vis + pix);
+    if (cur != kNoKey && (uint32_t)(cur >> kHitBits) >> (T.ba + T.bb) < en.order) return 2;
     int e = en.e;
     int32_t Ne = en.Ne;
     if (BEAM && Dn > 0) {
@@ -215,30 +265,133 @@ __device__ __forceinline__ int pair_pixel(const SceneDev& S, const CamDev& C, co
     Counters cnt = {0, 0, 0};
     if (trace_chunk<FAST, false, false, BEAM>(S, ref, r, en.Oloc, e, Ne, hit, cnt) &&
         (lowest_entry_face<FAST>(r, en.Oloc, (int)ref.lod, hit), within_view(S, r, hit))) {
-        const uint32_t tk = hit.e < 3 ? t_key(hit.Ne, r.d[hit.e]) : 0u;
-        const int n = (int)ref.lod;
-        const int32_t side = (1 << (S.mlog - n)) - 1;
-        unsigned long long pay = 0;
-#pragma unroll
-        for (int a = 0; a < 3; a++) {
-            const int32_t uv = ((r.mir >> a) & 1u) ? side - hit.c[a] : hit.c[a];
-            pay |= (unsigned long long)(uint32_t)((u[a] << S.mlog) + (uv << n)) << (17 * a);
-        }
-        const uint32_t mat = hit_material(S, ref, hit.idx);
-        pay |= (unsigned long long)n << 51 | (unsigned long long)hit.e << 54 | (unsigned long long)mat << 56;
-        const ulonglong2 mine = make_ulonglong2(
-            ((unsigned long long)tk << 32) | ((unsigned long long)(en.order & 0xFFFFu) << 16) | chunk, pay);
-        // install the record if its key is the smallest so far
-        ulonglong2 seen = make_ulonglong2(cur, __ldcg(rec + 1));
-        int tries = 0;
-        while (seen.x > mine.x) {
-            if (++tries > kCasLimit) return 3;
-            const ulonglong2 old = cas128(rec, seen, mine);
-            if (old.x == seen.x && old.y == seen.y) break;
-            seen = old;
-        }
+        red_min_u64(T.vis + pix, pack_hit(S, T, u, en.order, r.mir, (int)ref.lod, hit, hit_material(S, ref, hit.idx)));
     }
     return 1;
+}
+
+// The exact version as the fallback of pair_walk (out of line: rare).
+template <bool BEAM>
+__device__ __noinline__ int pair_exact(const SceneDev& S, const CamDev& C, const ChunkRef* __restrict__ frame,
+                                       uint32_t chunk, int px, int py, const TileDev& T, int32_t Dn) {
+    const ChunkRef ref = frame[chunk];
+    RayState r;
+    const size_t pix = (size_t)py * C.W + px;
+    return make_ray(C, px, py, r) ? pair_pixel<true, BEAM>(S, C, ref, chunk, r, pix, T, Dn)
+                                  : pair_pixel<false, BEAM>(S, C, ref, chunk, r, pix, T, Dn);
+}
+
+// One pixel of a pair (results of pair_pixel): entry, skip tests and walk in
+// FP32 as in walk_pixel, the exact version where a decision is left open.
+// Called by all lanes of a warp for the same pair; `in`: the lane has a pixel.
+template <bool BEAM>
+__device__ __forceinline__ int pair_walk(const SceneDev& S, const CamDev& C, const ChunkRef* __restrict__ frame,
+                                         uint32_t chunk, bool in, int px, int py, const TileDev& T, int32_t Dn) {
+    const uint4* fr = reinterpret_cast<const uint4*>(frame + chunk);
+    const uint4 ra = __ldg(fr), rb = __ldg(fr + 1);
+    const size_t pix = (size_t)py * C.W + px;
+    float d[3];
+    ray_dir(C, px, py, d);
+    const uint32_t mir = (d[0] < 0.0f ? 1u : 0u) | (d[1] < 0.0f ? 2u : 0u) | (d[2] < 0.0f ? 4u : 0u);
+    WalkRay w;
+    w.dmax = fmaxf(fmaxf(fabsf(d[0]), fabsf(d[1])), fabsf(d[2]));
+    bool undecided = !(w.dmax > 0x1p-40f && w.dmax < 0x1p40f);
+    w.gmax = 0.0f;
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        w.ad[a] = fabsf(d[a]);
+        w.inv[a] = w.ad[a] > 0.0f ? rcp_approx(w.ad[a]) : kZeroInv;
+        if (w.ad[a] > 0.0f) w.gmax = fmaxf(w.gmax, w.inv[a]);
+    }
+    int32_t u[3], Ow[3], cc[3], Hi[3];
+    region_coords(S, chunk, u);
+    const int cs = S.mlog + kFix;
+    const int32_t M = 1 << S.mlog;
+    const int32_t alo[3] = {(int32_t)(rb.x & 0xFFFFu), (int32_t)(rb.x >> 16), (int32_t)(rb.y & 0xFFFFu)};
+    const int32_t ahi[3] = {(int32_t)(rb.y >> 16), (int32_t)(rb.z & 0xFFFFu), (int32_t)(rb.z >> 16)};
+    uint32_t order = 0;
+    int e = 3;
+    int32_t Ne = 0;
+    bool enter = in;
+    float tin = -1.0f, tin2 = -1.0f, tout = 3.0e38f, tn = 0.0f, tf = 3.0e38f;
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        const bool m = (mir >> a) & 1u;
+        Ow[a] = m ? (S.grid[a] << cs) - C.O[a] : C.O[a];
+        cc[a] = m ? S.grid[a] - 1 - u[a] : u[a];
+        order += (uint32_t)cc[a];
+        const int32_t Lo = (cc[a] << cs) - Ow[a];
+        Hi[a] = Lo + (1 << cs);
+        if (Hi[a] <= 0 || (w.ad[a] == 0.0f && Lo > 0)) enter = false;
+        const float ti = Lo > 0 ? (float)Lo * w.inv[a] : -1.0f;
+        tout = fminf(tout, (float)Hi[a] * w.inv[a]);
+        if (ti > tin) { tin2 = tin; tin = ti; e = a; Ne = Lo; }
+        else tin2 = fmaxf(tin2, ti);
+        // the solid voxels' box grown by 1/16 voxel
+        tn = fmaxf(tn, (float)(Lo + ((m ? M - ahi[a] : alo[a]) << kFix) - 256) * w.inv[a]);
+        tf = fminf(tf, (float)(Lo + ((m ? M - alo[a] : ahi[a]) << kFix) + 256) * w.inv[a]);
+    }
+    if (!undecided && tin > tout * (1.0f + kWalkEps)) enter = false;
+    else if (!(tin < tout * (1.0f - kWalkEps) && (e == 3 || tin2 < tin * (1.0f - kWalkEps)))) undecided = true;
+    if (!undecided && tn > tf) enter = false;
+    undecided = undecided && enter;
+    int res = 0;
+    bool traced = enter && !undecided;
+    if (traced) {
+        res = 1;
+        const unsigned long long cur = __ldcg(T.vis + pix);
+        if (cur != kNoKey && (uint32_t)(cur >> kHitBits) >> (T.ba + T.bb) < order) res = 2;
+        if (BEAM && Dn > 0) {
+            // the last integer plane of the dominant axis crossed before the ray's
+            // L-inf distance reaches Dn; at or past the region's exit: no hit here
+            int as = 0;
+            if (w.ad[1] > w.ad[0]) as = 1;
+            if (w.ad[2] > fmaxf(w.ad[0], w.ad[1])) as = 2;
+            const int32_t O = sel3(as, Ow[0], Ow[1], Ow[2]);
+            const long long Nl = ((((long long)Dn - 1 + O) >> kFix) << kFix) - O;
+            if (Nl >= (long long)sel3(as, Hi[0], Hi[1], Hi[2])) {
+                res = 2;
+            } else if (Nl > 0) {
+                const float ts = (float)(int32_t)Nl * sel3(as, w.inv[0], w.inv[1], w.inv[2]);
+                if (ts > tout * (1.0f + kWalkEps)) {
+                    res = 2;  // left the region before the restart point
+                } else if (ts < tout * (1.0f - kWalkEps) && (e == 3 || ts > tin * (1.0f + kWalkEps))) {
+                    e = as;
+                    Ne = (int32_t)Nl;
+                }
+            }
+        }
+        traced = res == 1;
+    }
+    int32_t B[3];
+    float x[3];
+    int eb = 0;
+    HitRec hit;
+    if (traced && !walk_base<false>(w, Ow, e, Ne, B, x)) {
+        undecided = true;
+        traced = false;
+    }
+    bool found = false;
+    if (__any_sync(0xFFFFFFFFu, traced))
+        found = walk_chunk<false>(S, w, mir, Ow, cc, traced, true, ra.x, (int)ra.y, e, Ne, eb, B, x, undecided, hit);
+    if (found) {
+        const int n = (int)ra.y;
+        RayState r;
+        hit.Ne = 0;
+        if (e < 3)
+            hit.Ne = (((sel3(e, cc[0], cc[1], cc[2]) << S.mlog) + (sel3(e, hit.c[0], hit.c[1], hit.c[2]) << n)) << kFix) -
+                     sel3(e, Ow[0], Ow[1], Ow[2]);
+#pragma unroll
+        for (int a = 0; a < 3; a++) r.d[a] = d[a];
+        if (within_view(S, r, hit)) {
+            ChunkRef ref;
+            ref.mat_base = (uint64_t)ra.z | (uint64_t)ra.w << 32;
+            ref.nblocks = rb.w;
+            red_min_u64(T.vis + pix, pack_hit(S, T, u, order, mir, n, hit, hit_material(S, ref, hit.idx)));
+        }
+    }
+    if (undecided) res = pair_exact<BEAM>(S, C, frame, chunk, px, py, T, Dn);
+    return res;
 }
 
 // ---------------------------------------------------------------------------
@@ -325,46 +478,62 @@ __global__ void __launch_bounds__(128) tc_rect_kernel(SceneDev S, CamDev C, cons
     }
 }
 
-// Compacts the regions with pairs (ascending) and their exclusive area prefix
-// (one block); zeroes the frame's statistics.
+// Lists the regions with pairs front to back -- by the leading bits of their
+// depth, so that most of a pixel's farther pairs meet a record that ends them
+// -- and their exclusive area prefix (one block); zeroes the frame's
+// statistics.
+constexpr int kDepthBuckets = 4096;  // exponent and 4 bits of the depth's mantissa
+__device__ __forceinline__ uint32_t depth_bucket(float dm) {
+    return min(__float_as_uint(fmaxf(dm, 0.0f)) >> 19, (uint32_t)kDepthBuckets - 1u);
+}
 __global__ void __launch_bounds__(1024) tc_scan_kernel(int nch, TileDev T) {
+    __shared__ uint32_t s_hist[kDepthBuckets];
     __shared__ unsigned long long s_sum[1024];
-    __shared__ uint32_t s_cnt[1024];
     const int tid = threadIdx.x;
-    const int per = (nch + 1023) / 1024;
-    const int b = min(tid * per, nch), e = min(b + per, nch);
-    unsigned long long sum = 0;
-    uint32_t cnt = 0;
-    for (int i = b; i < e; i++) {
-        const uint32_t a = T.area[i];
-        sum += a;
-        cnt += a ? 1u : 0u;
-    }
-    s_sum[tid] = sum;
-    s_cnt[tid] = cnt;
-    __syncthreads();
-    for (int off = 1; off < 1024; off <<= 1) {
-        const unsigned long long vs = tid >= off ? s_sum[tid - off] : 0ull;
-        const uint32_t vc = tid >= off ? s_cnt[tid - off] : 0u;
+    // exclusive prefix over the block of one value per thread; the last entry is the total
+    auto scan = [&](unsigned long long v) -> unsigned long long {
+        s_sum[tid] = v;
         __syncthreads();
-        s_sum[tid] += vs;
-        s_cnt[tid] += vc;
-        __syncthreads();
-    }
-    unsigned long long base = s_sum[tid] - sum;
-    uint32_t pos = s_cnt[tid] - cnt;
-    for (int i = b; i < e; i++) {
-        const uint32_t a = T.area[i];
-        if (a) {
-            T.list[pos] = (uint32_t)i;
-            T.offs[pos] = base;
-            pos++;
-            base += a;
+        for (int off = 1; off < 1024; off <<= 1) {
+            const unsigned long long p = tid >= off ? s_sum[tid - off] : 0ull;
+            __syncthreads();
+            s_sum[tid] += p;
+            __syncthreads();
         }
+        return s_sum[tid] - v;
+    };
+    for (int i = tid; i < kDepthBuckets; i += 1024) s_hist[i] = 0;
+    __syncthreads();
+    for (int i = tid; i < nch; i += 1024)
+        if (T.area[i]) atomicAdd(&s_hist[depth_bucket(T.dmin[i])], 1u);
+    __syncthreads();
+    uint32_t h[kDepthBuckets / 1024];
+    uint32_t cnt = 0;
+#pragma unroll
+    for (int k = 0; k < kDepthBuckets / 1024; k++) {
+        h[k] = cnt;
+        cnt += s_hist[tid * (kDepthBuckets / 1024) + k];
+    }
+    const uint32_t at = (uint32_t)scan(cnt);
+    const uint32_t n_list = (uint32_t)s_sum[1023];
+#pragma unroll
+    for (int k = 0; k < kDepthBuckets / 1024; k++) s_hist[tid * (kDepthBuckets / 1024) + k] = at + h[k];
+    __syncthreads();
+    for (int i = tid; i < nch; i += 1024)
+        if (T.area[i]) T.list[atomicAdd(&s_hist[depth_bucket(T.dmin[i])], 1u)] = (uint32_t)i;
+    __syncthreads();
+    const uint32_t per = (n_list + 1023) / 1024;
+    const uint32_t b = min((uint32_t)tid * per, n_list), e = min(b + per, n_list);
+    unsigned long long sum = 0;
+    for (uint32_t i = b; i < e; i++) sum += T.area[T.list[i]];
+    unsigned long long base = scan(sum);
+    for (uint32_t i = b; i < e; i++) {
+        T.offs[i] = base;
+        base += T.area[T.list[i]];
     }
     if (tid == 1023) {
-        T.offs[s_cnt[1023]] = s_sum[1023];
-        T.stats[kStList] = s_cnt[1023];
+        T.offs[n_list] = s_sum[1023];
+        T.stats[kStList] = n_list;
     }
     if (tid > 0 && tid < kTileStats) T.stats[tid] = 0ull;
 }
@@ -376,23 +545,20 @@ __global__ void __launch_bounds__(1024) tc_scan_kernel(int nch, TileDev T) {
 // frame's keeps.
 // ---------------------------------------------------------------------------
 template <int PASS, bool BEAM>
-__global__ void __launch_bounds__(128, 7) tc_cast_kernel(SceneDev S, CamDev C, const ChunkRef* __restrict__ frame,
-                                                      TileDev T, const BeamLookup beam) {
+__global__ void __launch_bounds__(128, 7) tc_cast_kernel(const __grid_constant__ SceneDev S,
+                                                      const __grid_constant__ CamDev C,
+                                                      const ChunkRef* __restrict__ frame,
+                                                      const __grid_constant__ TileDev T, const BeamLookup beam) {
     const uint32_t n_list = (uint32_t)T.stats[kStList];
     if (n_list == 0) return;
     const unsigned long long n_items = 2ull * T.offs[n_list];
     const int lane = threadIdx.x & 31;
     const unsigned long long nw = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
-    uint32_t traced = 0, culled = 0, pix_traced = 0, pix_skipped = 0;
+    uint32_t traced = 0, culled = 0, pix_traced = 0, pix_skipped = 0, lo = 0;
     for (unsigned long long item = ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; item < n_items;
          item += nw) {
         const unsigned long long pair = item >> 1;
-        uint32_t lo = 0, hi = n_list - 1;  // last listed region with offs <= pair
-        while (lo < hi) {
-            const uint32_t mid = (lo + hi + 1) >> 1;
-            if (T.offs[mid] <= pair) lo = mid;
-            else hi = mid - 1;
-        }
+        while (lo + 1 < n_list && T.offs[lo + 1] <= pair) lo++;  // last listed region with offs <= pair
         const uint32_t chunk = T.list[lo];
         const uint32_t local = (uint32_t)(pair - T.offs[lo]);
         const int4 rc = T.rect[chunk];
@@ -415,16 +581,9 @@ __global__ void __launch_bounds__(128, 7) tc_cast_kernel(SceneDev S, CamDev C, c
         }
         traced++;
         const int px = tx * 8 + (lane & 7), py = by * 4 + (lane >> 3);
-        if (px < C.W && py < C.H) {
-            const ChunkRef ref = frame[chunk];
-            RayState r;
-            const size_t pix = (size_t)py * C.W + px;
-            const int res = make_ray(C, px, py, r) ? pair_pixel<true, BEAM>(S, C, ref, chunk, r, pix, T.vis, Dn)
-                                                   : pair_pixel<false, BEAM>(S, C, ref, chunk, r, pix, T.vis, Dn);
-            pix_traced += res == 1;
-            pix_skipped += res == 2;
-            if (res == 3) atomicAdd(&T.stats[kStCasExhausted], 1ull);
-        }
+        const int res = pair_walk<BEAM>(S, C, frame, chunk, px < C.W && py < C.H, px, py, T, Dn);
+        pix_traced += res == 1;
+        pix_skipped += res == 2;
     }
     pix_traced = __reduce_add_sync(0xFFFFFFFFu, pix_traced);
     pix_skipped = __reduce_add_sync(0xFFFFFFFFu, pix_skipped);
@@ -441,7 +600,7 @@ __global__ void __launch_bounds__(128, 7) tc_cast_kernel(SceneDev S, CamDev C, c
 // an upper bound of the distance of the pixel's hit so far (+inf: none yet).
 // One warp per tile.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) tc_hiz_kernel(CamDev C, TileDev T) {
+__global__ void __launch_bounds__(256) tc_hiz_kernel(SceneDev S, CamDev C, TileDev T) {
     const int lane = threadIdx.x & 31;
     const int tile = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (tile >= T.tiles_x * T.tiles_y) return;
@@ -451,16 +610,12 @@ __global__ void __launch_bounds__(256) tc_hiz_kernel(CamDev C, TileDev T) {
     for (int k = 0; k < 2; k++) {
         const int px = tx * 8 + (lane & 7), py = ty * 8 + k * 4 + (lane >> 3);
         if (px < C.W && py < C.H) {
-            const unsigned long long key = __ldcg(T.vis + 2 * ((size_t)py * C.W + px));
+            const unsigned long long key = __ldcg(T.vis + ((size_t)py * C.W + px));
             float dist = __int_as_float(0x7F800000);
             if (key != kNoKey) {
                 float d[3];
                 ray_dir(C, px, py, d);
-                // upper bounds in FP32 with upward rounding: |d| and t (the key's next value)
-                const float dn = __fsqrt_ru(__fadd_ru(__fadd_ru(__fmul_ru(d[0], d[0]), __fmul_ru(d[1], d[1])),
-                                                      __fmul_ru(d[2], d[2])));
-                const float t_up = __double2float_ru(__longlong_as_double((long long)(((key >> 32) + 1ull) << 32)));
-                dist = __fmul_ru(t_up, dn);
+                dist = __fmul_ru(unpack_hit(S, C, T, key, d).dist, 1.000001f);
             }
             m = fmaxf(m, dist);
         }
@@ -483,35 +638,19 @@ __global__ void __launch_bounds__(128) tc_resolve_kernel(SceneDev S, CamDev C, c
     float dist_up = 0.0f;
     if (px < C.W && py < C.H) {
         const size_t pix = (size_t)py * C.W + px;
-        const ulonglong2 rec = __ldcg(reinterpret_cast<const ulonglong2*>(T.vis) + pix);
-        if (rec.x == kNoKey) {
+        const unsigned long long key = __ldcg(T.vis + pix);
+        if (key == kNoKey) {
             emit_miss(out_hit, out_t, pix);
             dist_up = __int_as_float(0x7F800000);
         } else {
-            // the output record of emit_hit, rebuilt from the payload and the ray
-            RayState r;
-            ray_dir(C, px, py, r.d);
-            r.mir = (r.d[0] < 0.0f ? 1u : 0u) | (r.d[1] < 0.0f ? 2u : 0u) | (r.d[2] < 0.0f ? 4u : 0u);
-            const unsigned long long pay = rec.y;
-            const uint32_t x = (uint32_t)(pay & 0x1FFFFu), y = (uint32_t)((pay >> 17) & 0x1FFFFu),
-                           z = (uint32_t)((pay >> 34) & 0x1FFFFu);
-            const int n = (int)((pay >> 51) & 7u), e = (int)((pay >> 54) & 3u);
-            const uint32_t mat = (uint32_t)(pay >> 56);
-            float dist = 0.0f;
-            if (e < 3) {
-                // entry plane: the voxel's face the mirrored ray meets first, as a numerator
-                const uint32_t w[3] = {x, y, z};
-                const bool m = (r.mir >> e) & 1u;
-                const int32_t wext = S.grid[e] << S.mlog;
-                const int32_t face = m ? wext - (int32_t)w[e] - (1 << n) : (int32_t)w[e];
-                const int32_t Ow = m ? (S.grid[e] << (S.mlog + kFix)) - C.O[e] : C.O[e];
-                const int32_t Ne = (face << kFix) - Ow;
-                dist = __fdiv_rn((float)Ne * (1.0f / 4096.0f), fabsf(r.d[e])) * ray_norm(r);
-            }
-            const uint32_t normal = e == 3 ? 7u : (uint32_t)(2 * e) + ((r.mir >> e) & 1u);
-            out_hit[pix] = make_uint4(x, y, z, (uint32_t)n | (mat << 8) | (normal << 16) | (1u << 19));
-            out_t[pix] = dist;
-            dist_up = __fmul_ru(dist, 1.000001f);
+            // the output record of emit_hit, rebuilt from the record and the ray
+            float d[3];
+            ray_dir(C, px, py, d);
+            const VisHit h = unpack_hit(S, C, T, key, d);
+            out_hit[pix] = make_uint4(h.c[0], h.c[1], h.c[2],
+                                      (uint32_t)h.n | (h.mat << 8) | (h.normal << 16) | (1u << 19));
+            out_t[pix] = h.dist;
+            dist_up = __fmul_ru(h.dist, 1.000001f);
         }
     }
 #pragma unroll
@@ -546,11 +685,11 @@ int aokk_tiles_frame(const SceneDev* S, const CamDev* C, const ChunkRef* frame, 
     tc_scan_kernel<<<1, 1024, 0, s>>>(nch, *T);
     if (bl.bounds) tc_cast_kernel<1, true><<<sms * per_sm[0], 128, 0, s>>>(*S, *C, frame, *T, bl);
     else tc_cast_kernel<1, false><<<sms * per_sm[0], 128, 0, s>>>(*S, *C, frame, *T, bl);
-    tc_hiz_kernel<<<(tiles + 7) / 8, 256, 0, s>>>(*C, *T);
+    tc_hiz_kernel<<<(tiles + 7) / 8, 256, 0, s>>>(*S, *C, *T);
     if (bl.bounds) tc_cast_kernel<2, true><<<sms * per_sm[1], 128, 0, s>>>(*S, *C, frame, *T, bl);
     else tc_cast_kernel<2, false><<<sms * per_sm[1], 128, 0, s>>>(*S, *C, frame, *T, bl);
     tc_resolve_kernel<<<dim3((C->W + 15) / 16, (C->H + 7) / 8), 128, 0, s>>>(*S, *C, frame, *T, hit, t);
-    e = cudaMemsetAsync(T->vis, 0xFF, (size_t)C->W * C->H * 16, s);  // re-armed for the next frame
+    e = cudaMemsetAsync(T->vis, 0xFF, (size_t)C->W * C->H * 8, s);  // re-armed for the next frame
     if (e != cudaSuccess) return AOK_E_CUDA;
     return tiles_status(cudaGetLastError());
 }

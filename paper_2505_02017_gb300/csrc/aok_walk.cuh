@@ -133,6 +133,240 @@ __device__ __forceinline__ bool walk_base(const WalkRay& w, const int32_t Ow[3],
     return clear;
 }
 
+// One chunk's part of a walk, called by all of a warp's lanes together, those
+// with `traced` taking part: the traversal of the sparse voxel DAG `root` (LOD
+// lod) of chunk cell cc from the ray's base point (based) or its crossing of
+// plane (e, Ne).  True: a hit (c, e and idx of `hit`; e its entry axis).
+// Otherwise, unless undecided, e is the axis the chunk is left through.
+// (eb, Ne) follows the base point.
+template <bool EXACT>
+__device__ __forceinline__ bool walk_chunk(const SceneDev& S, const WalkRay& w, uint32_t mir, const int32_t (&Ow)[3],
+                                           const int32_t (&cc)[3], bool traced, bool based, uint32_t root, int lod,
+                                           int& e, int32_t& Ne, int& eb, int32_t (&B)[3], float (&x)[3],
+                                           bool& undecided, HitRec& hit) {
+    const uint32_t* __restrict__ nodes = S.nodes;
+    // Voxel coordinates of the current cell at every level, in voxels
+    // of the LOD, axis a shifted left by a: the octant of level k is
+    // then bits k, k + 1, k + 2 of the three merged words.
+    bool go = traced, occ = false;
+    int n = 0, R = 3, k = 2;
+    float gtol = 0.0f, dmaxn = 0.0f;
+    uint32_t V0 = 0, V1 = 0, V2 = 0;
+    float Kp[3], gs[3], hp[3], xm[3], dv[3];
+    // {node, child mask | its place among its parent's children << 8}
+    // of the path's interior levels R .. 3; an
+    // EXACT walk keeps to the octree inside leaf blocks too (at a tie
+    // the cells visited depend on it) and holds level 2 as well
+    constexpr int kLow = EXACT ? 2 : 3;
+    uint2 st[kMaxLevels - kLow];
+    uint32_t pidx = 0, pm8 = 0, o = 0;
+    uint64_t lmu = 0;
+    // numerator of the plane at scaled coordinate P of axis a
+    auto plane = [&](int a, uint32_t P) -> int32_t {
+        return (((sel3(a, cc[0], cc[1], cc[2]) << S.mlog) + (int32_t)((P >> a) << n)) << kFix) -
+               sel3(a, Ow[0], Ow[1], Ow[2]);
+    };
+    // crossing parameters and coordinates from the base point, the
+    // latter kept within the cell of coordinates V with bits `low` free
+    auto rebase = [&](uint32_t low) {
+        const float up = pow2(n), down = pow2(-n);
+        uint32_t J[3] = {V0, V1 >> 1, V2 >> 2};
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            const int32_t l = B[a] - (cc[a] << S.mlog);
+            // (a decided base point lies in the cell: only EXACT can meet its upper face, at a tie)
+            J[a] = EXACT ? (uint32_t)max((int32_t)(J[a] & ~low), min(l >> n, (int32_t)(J[a] | low)))
+                         : (J[a] & ~low) | ((uint32_t)(l >> n) & low);
+            const int32_t below = EXACT ? l - (int32_t)(J[a] << n) : l & ((1 << n) - 1);
+            const float xn = ((float)below + x[a]) * down;
+            const float g = w.inv[a] * up;
+            gs[a] = g * (1.0f / (float)(1 << a));
+            hp[a] = __fmaf_rn(-xn, g, gs[a]);
+            xm[a] = xn - 0.5f;
+            dv[a] = w.ad[a] * down;
+            Kp[a] = __uint_as_float(kMagicBits | (J[a] << a));
+        }
+        V0 = J[0];
+        V1 = J[1] << 1;
+        V2 = J[2] << 2;
+    };
+    // octant of the level-k cell in its parent, stored order: bits k,
+    // k + 1, k + 2 of the three words merged (m = ~0 << k)
+    uint32_t m = ~0u;
+    auto octant = [&]() -> uint32_t {
+        const uint32_t hi = (V2 & (m << 2)) | (V1 & ~(m << 2));
+        return ((((hi & (m << 1)) | (V0 & ~(m << 1))) >> k) & 7u) ^ mir;
+    };
+    if (traced) {
+        n = lod;
+        R = S.mlog - n;
+        gtol = kEpsG * w.gmax * pow2(n);
+        dmaxn = w.dmax * pow2(-n);
+        pidx = root;
+        pm8 = nodes[pidx] & 0xFFu;
+        if (!based) undecided = !walk_base<EXACT>(w, Ow, e, Ne, B, x) && !EXACT;
+        eb = e;
+        rebase((1u << R) - 1u);
+        st[R - kLow] = make_uint2(pidx, pm8);
+        k = R - 1;
+        m = ~0u << k;
+        o = octant();
+        occ = (pm8 >> o) & 1u;
+    }
+    while (go) {
+        while (occ && k > (EXACT ? 0 : 2)) {
+            // into the occupied cell: its node and child mask
+            if (EXACT && k == 1) {
+                // the voxel bits of a leaf block's 2x2x2 group
+                const uint64_t v = lmu >> ((o & 1u) * 2 + (o & 2u) * 4 + (o & 4u) * 8);
+                pm8 = (uint32_t)((v & 3) | ((v >> 2) & 0xC) | ((v >> 12) & 0x30) | ((v >> 14) & 0xC0));
+            } else {
+                const uint32_t rank = __popc(pm8 & ~(~0u << o));
+                const uint2 ch = __ldg(reinterpret_cast<const uint2*>(nodes + pidx + 2 + 2 * rank));
+                pidx = ch.x;
+                pm8 = ch.y >> 24;
+                if (k == kWideLevel - 1) pm8 = nodes[pidx] & 0xFFu;
+                if (EXACT && k == 2) {
+                    lmu = __ldg(S.leaves + pidx);
+                    uint64_t q = lmu | (lmu >> 1);
+                    q |= q >> 4;
+                    q |= q >> 16;  // the occupied groups
+                    pm8 = (uint32_t)((q & 1) | ((q >> 1) & 2) | ((q >> 6) & 4) | ((q >> 7) & 8) |
+                                     ((q >> 28) & 16) | ((q >> 29) & 32) | ((q >> 34) & 64) | ((q >> 35) & 128));
+                }
+                st[k - kLow] = make_uint2(pidx, pm8 | rank << 8);
+            }
+            k--;
+            m = ~0u << k;
+            o = octant();
+            occ = (pm8 >> o) & 1u;
+        }
+        float tm = 0.0f;
+        if (EXACT) {
+            go = !occ;  // occupied at level 0: the hit
+        } else if (occ) {
+            // a 4^3 leaf block: voxel by voxel, to a set bit or out of
+            // it; i: bit of the voxel in the mirrored frame
+            lmu = __ldg(S.leaves + __ldg(nodes + pidx + 2 + 2 * __popc(pm8 & ~(~0u << o))));
+            float T0 = __fmaf_rn(__uint_as_float(V0 | kMagicBits) - Kp[0], gs[0], hp[0]);
+            float T1 = __fmaf_rn(__uint_as_float(V1 | 1u | kMagicBits) - Kp[1], gs[1], hp[1]);
+            float T2 = __fmaf_rn(__uint_as_float(V2 | 3u | kMagicBits) - Kp[2], gs[2], hp[2]);
+            uint32_t i = (V0 & 3u) | ((V1 & 6u) << 1) | ((V2 & 12u) << 2), inc = 0;
+            const uint32_t mi = ((mir & 1u) | ((mir & 2u) << 1) | ((mir & 4u) << 2)) * 3u;
+            for (;;) {
+                const uint32_t j = i ^ mi;
+                occ = (((j & 32u) ? (uint32_t)(lmu >> 32) : (uint32_t)lmu) >> (j & 31u)) & 1u;
+                if (occ) break;
+                tm = fminf(fminf(T0, T1), T2);
+                const float thr = __fmaf_rn(tm, 1.0f + kEpsLeaf, gtol);
+                const bool p0 = T0 <= thr, p1 = T1 <= thr, p2 = T2 <= thr;
+                undecided = undecided || (p0 ? p1 || p2 : p1 == p2);
+                if (p0) { T0 = T0 + gs[0]; inc = 1u; }
+                else if (p1) { T1 = __fmaf_rn(gs[1], 2.0f, T1); inc = 4u; }
+                else { T2 = __fmaf_rn(gs[2], 4.0f, T2); inc = 16u; }
+                i += inc;
+                if (!(i & (3u * inc))) break;  // left the block
+            }
+            if (occ) {
+                if (inc) e = inc == 1u ? 0 : (inc == 4u ? 1 : 2);
+                V0 = (V0 & ~3u) | (i & 3u);
+                V1 = (V1 & ~6u) | ((i >> 1) & 6u);
+                V2 = (V2 & ~12u) | ((i >> 2) & 12u);
+                go = false;  // the hit
+            }
+        }
+        // leave empty cells through their nearest exit face until an
+        // occupied one or the chunk's end
+        uint32_t m0 = m;
+        while (!occ) {
+            const uint32_t E0 = V0 | ~m | kMagicBits, E1 = V1 | ~(m << 1) | kMagicBits,
+                           E2 = V2 | ~(m << 2) | kMagicBits;
+            const float T0 = __fmaf_rn(__uint_as_float(E0) - Kp[0], gs[0], hp[0]);
+            const float T1 = __fmaf_rn(__uint_as_float(E1) - Kp[1], gs[1], hp[1]);
+            const float T2 = __fmaf_rn(__uint_as_float(E2) - Kp[2], gs[2], hp[2]);
+            tm = fminf(fminf(T0, T1), T2);
+            const float thr = __fmaf_rn(tm, 1.0f + kEpsT, gtol);
+            bool p0 = T0 <= thr, p1 = T1 <= thr;
+            const bool p2 = T2 <= thr;
+            const bool amb = p0 ? p1 || p2 : p1 == p2;
+            if (EXACT) {
+                if (amb) {
+                    const int a = exact_nearest(plane(0, E0 + (1u - kMagicBits)), plane(1, E1 + (1u - kMagicBits)),
+                                                plane(2, E2 + (1u - kMagicBits)), w.ad[0], w.ad[1], w.ad[2]);
+                    p0 = a == 0;
+                    p1 = a == 1;
+                    tm = sel3(a, T0, T1, T2);
+                }
+            } else {
+                undecided = undecided || amb;
+            }
+            e = p0 ? 0 : (p1 ? 1 : 2);
+            const uint32_t nv = (p0 ? E0 : (p1 ? E1 : E2)) + (1u - kMagicBits);
+            V0 = p0 ? nv : V0;
+            V1 = e == 1 ? nv : V1;
+            V2 = e == 2 ? nv : V2;
+            m0 = m;
+            // the level of the cell entered: k for a sibling, else
+            // that of the lowest set bit (the parent was left)
+            const int K = __ffs((int)nv) - 1 - e;
+            if (K >= R) { go = false; break; }  // left the chunk
+            if (K != k) {
+                const uint2 par = st[K + 1 - kLow];
+                pidx = par.x;
+                pm8 = par.y;
+            }
+            k = K;
+            m = ~0u << k;
+            o = octant();
+            occ = (pm8 >> o) & 1u;
+        }
+        if (go) {
+            // the entered cell's coordinates below the level it was
+            // left at (the crossed axis' are zero: it is on a face);
+            // at a tie, below the level it was entered at
+            if (EXACT) m0 = m;
+            const float lim = 0.5f - __fmaf_rn(tm, kEpsX, gtol) * dmaxn;
+            const float x0 = __fmaf_rn(tm, dv[0], xm[0]), x1 = __fmaf_rn(tm, dv[1], xm[1]),
+                        x2 = __fmaf_rn(tm, dv[2], xm[2]);
+            const float r0 = (x0 + kRound) - kRound, r1 = (x1 + kRound) - kRound, r2 = (x2 + kRound) - kRound;
+            const bool clear = fabsf(x0 - r0) < (e == 0 ? 1.0f : lim) && fabsf(x1 - r1) < (e == 1 ? 1.0f : lim) &&
+                               fabsf(x2 - r2) < (e == 2 ? 1.0f : lim);
+            if (tm * w.dmax > (k > kNearLevel ? kRebaseFar : kRebaseNear) || !clear) {
+                // far from the base point, or next to a voxel plane: a new base here
+                const int32_t Nt = plane(e, sel3(e, V0, V1, V2));
+                if (!undecided) { eb = e; Ne = Nt; }
+                undecided = (!walk_base<EXACT>(w, Ow, e, Nt, B, x) && !EXACT) || undecided;
+                rebase(~m0);
+            } else {
+                const uint32_t k0 = e == 0 ? ~0u : m0, k1 = e == 1 ? ~0u : m0 << 1, k2 = e == 2 ? ~0u : m0 << 2;
+                V0 = (V0 & k0) | (__float_as_uint(r0 + Kp[0]) & ~k0);
+                V1 = (V1 & k1) | (__float_as_uint(__fmaf_rn(r1, 2.0f, Kp[1])) & ~k1);
+                V2 = (V2 & k2) | (__float_as_uint(__fmaf_rn(r2, 4.0f, Kp[2])) & ~k2);
+            }
+        }
+    }
+    if ((!EXACT && undecided) || !traced || !occ) return false;
+    hit.c[0] = (int32_t)V0;
+    hit.c[1] = (int32_t)(V1 >> 1);
+    hit.c[2] = (int32_t)(V2 >> 2);
+    hit.e = e;
+    // depth-first index (Sec. 3.3): the prefix beside each child
+    // pointer of the path, then the leaf block's earlier voxels
+    uint32_t idx;
+    if (EXACT) {
+        idx = nodes[st[1].x + 3 + 2 * (st[0].y >> 8)];
+    } else {
+        idx = nodes[pidx + 3 + 2 * __popc(pm8 & ~(~0u << o))];
+    }
+    idx &= kPrefixBits;
+    for (int j = R; j > 3; j--)
+        idx += nodes[st[j - kLow].x + 3 + 2 * (st[j - 1 - kLow].y >> 8)] & (j == kWideLevel ? ~0u : kPrefixBits);
+    const uint32_t bit = ((V0 & 3u) | ((V1 & 6u) << 1) | ((V2 & 12u) << 2)) ^
+                         (((mir & 1u) | ((mir & 2u) << 1) | ((mir & 4u) << 2)) * 3u);
+    hit.idx = idx + (uint32_t)__popcll(lmu & ((1ull << bit) - 1ull));
+    return true;
+}
+
 // Cast the pixel's ray and write its record.  BEAM: restart past the beam
 // pass's bound Dn (0: none).  lanes: the warp's lanes that call it.  False
 // (never with EXACT; nothing written): undecided at `at`, where an EXACT walk
@@ -255,7 +489,6 @@ __device__ __forceinline__ bool walk_pixel(const SceneDev& S, const CamDev& C, c
         return reinterpret_cast<const uint4*>(
             frame + ((uint32_t)u[0] + (uint32_t)S.grid[0] * ((uint32_t)u[1] + (uint32_t)S.grid[1] * (uint32_t)u[2])));
     };
-    const uint32_t* __restrict__ nodes = S.nodes;
     bool based = true;  // the base point lies on the entry of the current chunk
     while (EXACT ? alive : __any_sync(lanes, alive)) {
         bool traced = false;
@@ -290,230 +523,9 @@ __device__ __forceinline__ bool walk_pixel(const SceneDev& S, const CamDev& C, c
             }
         }
         if (EXACT ? traced : __any_sync(lanes, traced)) {
-            // Voxel coordinates of the current cell at every level, in voxels
-            // of the LOD, axis a shifted left by a: the octant of level k is
-            // then bits k, k + 1, k + 2 of the three merged words.
-            bool go = traced, occ = false;
-            int n = 0, R = 3, k = 2;
-            float gtol = 0.0f, dmaxn = 0.0f;
-            uint32_t V0 = 0, V1 = 0, V2 = 0;
-            float Kp[3], gs[3], hp[3], xm[3], dv[3];
-            // {node, child mask | its place among its parent's children << 8}
-            // of the path's interior levels R .. 3; an
-            // EXACT walk keeps to the octree inside leaf blocks too (at a tie
-            // the cells visited depend on it) and holds level 2 as well
-            constexpr int kLow = EXACT ? 2 : 3;
-            uint2 st[kMaxLevels - kLow];
-            uint32_t pidx = 0, pm8 = 0, o = 0;
-            uint64_t lmu = 0;
-            // numerator of the plane at scaled coordinate P of axis a
-            auto plane = [&](int a, uint32_t P) -> int32_t {
-                return (((sel3(a, cc[0], cc[1], cc[2]) << S.mlog) + (int32_t)((P >> a) << n)) << kFix) -
-                       sel3(a, Ow[0], Ow[1], Ow[2]);
-            };
-            // crossing parameters and coordinates from the base point, the
-            // latter kept within the cell of coordinates V with bits `low` free
-            auto rebase = [&](uint32_t low) {
-                const float up = pow2(n), down = pow2(-n);
-                uint32_t J[3] = {V0, V1 >> 1, V2 >> 2};
-#pragma unroll
-                for (int a = 0; a < 3; a++) {
-                    const int32_t l = B[a] - (cc[a] << S.mlog);
-                    // (a decided base point lies in the cell: only EXACT can meet its upper face, at a tie)
-                    J[a] = EXACT ? (uint32_t)max((int32_t)(J[a] & ~low), min(l >> n, (int32_t)(J[a] | low)))
-                                 : (J[a] & ~low) | ((uint32_t)(l >> n) & low);
-                    const int32_t below = EXACT ? l - (int32_t)(J[a] << n) : l & ((1 << n) - 1);
-                    const float xn = ((float)below + x[a]) * down;
-                    const float g = w.inv[a] * up;
-                    gs[a] = g * (1.0f / (float)(1 << a));
-                    hp[a] = __fmaf_rn(-xn, g, gs[a]);
-                    xm[a] = xn - 0.5f;
-                    dv[a] = w.ad[a] * down;
-                    Kp[a] = __uint_as_float(kMagicBits | (J[a] << a));
-                }
-                V0 = J[0];
-                V1 = J[1] << 1;
-                V2 = J[2] << 2;
-            };
-            // octant of the level-k cell in its parent, stored order: bits k,
-            // k + 1, k + 2 of the three words merged (m = ~0 << k)
-            uint32_t m = ~0u;
-            auto octant = [&]() -> uint32_t {
-                const uint32_t hi = (V2 & (m << 2)) | (V1 & ~(m << 2));
-                return ((((hi & (m << 1)) | (V0 & ~(m << 1))) >> k) & 7u) ^ mir;
-            };
-            if (traced) {
-                n = (int)lod;
-                R = S.mlog - n;
-                gtol = kEpsG * w.gmax * pow2(n);
-                dmaxn = w.dmax * pow2(-n);
-                pidx = root;
-                pm8 = nodes[pidx] & 0xFFu;
-                if (!based) undecided = !walk_base<EXACT>(w, Ow, e, Ne, B, x) && !EXACT;
-                eb = e;
-                rebase((1u << R) - 1u);
-                st[R - kLow] = make_uint2(pidx, pm8);
-                k = R - 1;
-                m = ~0u << k;
-                o = octant();
-                occ = (pm8 >> o) & 1u;
-            }
-            while (go) {
-                while (occ && k > (EXACT ? 0 : 2)) {
-                    // into the occupied cell: its node and child mask
-                    if (EXACT && k == 1) {
-                        // the voxel bits of a leaf block's 2x2x2 group
-                        const uint64_t v = lmu >> ((o & 1u) * 2 + (o & 2u) * 4 + (o & 4u) * 8);
-                        pm8 = (uint32_t)((v & 3) | ((v >> 2) & 0xC) | ((v >> 12) & 0x30) | ((v >> 14) & 0xC0));
-                    } else {
-                        const uint32_t rank = __popc(pm8 & ~(~0u << o));
-                        const uint2 ch = __ldg(reinterpret_cast<const uint2*>(nodes + pidx + 2 + 2 * rank));
-                        pidx = ch.x;
-                        pm8 = ch.y >> 24;
-                        if (k == kWideLevel - 1) pm8 = nodes[pidx] & 0xFFu;
-                        if (EXACT && k == 2) {
-                            lmu = __ldg(S.leaves + pidx);
-                            uint64_t q = lmu | (lmu >> 1);
-                            q |= q >> 4;
-                            q |= q >> 16;  // the occupied groups
-                            pm8 = (uint32_t)((q & 1) | ((q >> 1) & 2) | ((q >> 6) & 4) | ((q >> 7) & 8) |
-                                             ((q >> 28) & 16) | ((q >> 29) & 32) | ((q >> 34) & 64) | ((q >> 35) & 128));
-                        }
-                        st[k - kLow] = make_uint2(pidx, pm8 | rank << 8);
-                    }
-                    k--;
-                    m = ~0u << k;
-                    o = octant();
-                    occ = (pm8 >> o) & 1u;
-                }
-                float tm = 0.0f;
-                if (EXACT) {
-                    go = !occ;  // occupied at level 0: the hit
-                } else if (occ) {
-                    // a 4^3 leaf block: voxel by voxel, to a set bit or out of
-                    // it; i: bit of the voxel in the mirrored frame
-                    lmu = __ldg(S.leaves + __ldg(nodes + pidx + 2 + 2 * __popc(pm8 & ~(~0u << o))));
-                    float T0 = __fmaf_rn(__uint_as_float(V0 | kMagicBits) - Kp[0], gs[0], hp[0]);
-                    float T1 = __fmaf_rn(__uint_as_float(V1 | 1u | kMagicBits) - Kp[1], gs[1], hp[1]);
-                    float T2 = __fmaf_rn(__uint_as_float(V2 | 3u | kMagicBits) - Kp[2], gs[2], hp[2]);
-                    uint32_t i = (V0 & 3u) | ((V1 & 6u) << 1) | ((V2 & 12u) << 2), inc = 0;
-                    const uint32_t mi = ((mir & 1u) | ((mir & 2u) << 1) | ((mir & 4u) << 2)) * 3u;
-                    for (;;) {
-                        const uint32_t j = i ^ mi;
-                        occ = (((j & 32u) ? (uint32_t)(lmu >> 32) : (uint32_t)lmu) >> (j & 31u)) & 1u;
-                        if (occ) break;
-                        tm = fminf(fminf(T0, T1), T2);
-                        const float thr = __fmaf_rn(tm, 1.0f + kEpsLeaf, gtol);
-                        const bool p0 = T0 <= thr, p1 = T1 <= thr, p2 = T2 <= thr;
-                        undecided = undecided || (p0 ? p1 || p2 : p1 == p2);
-                        if (p0) { T0 = T0 + gs[0]; inc = 1u; }
-                        else if (p1) { T1 = __fmaf_rn(gs[1], 2.0f, T1); inc = 4u; }
-                        else { T2 = __fmaf_rn(gs[2], 4.0f, T2); inc = 16u; }
-                        i += inc;
-                        if (!(i & (3u * inc))) break;  // left the block
-                    }
-                    if (occ) {
-                        if (inc) e = inc == 1u ? 0 : (inc == 4u ? 1 : 2);
-                        V0 = (V0 & ~3u) | (i & 3u);
-                        V1 = (V1 & ~6u) | ((i >> 1) & 6u);
-                        V2 = (V2 & ~12u) | ((i >> 2) & 12u);
-                        go = false;  // the hit
-                    }
-                }
-                // leave empty cells through their nearest exit face until an
-                // occupied one or the chunk's end
-                uint32_t m0 = m;
-                while (!occ) {
-                    const uint32_t E0 = V0 | ~m | kMagicBits, E1 = V1 | ~(m << 1) | kMagicBits,
-                                   E2 = V2 | ~(m << 2) | kMagicBits;
-                    const float T0 = __fmaf_rn(__uint_as_float(E0) - Kp[0], gs[0], hp[0]);
-                    const float T1 = __fmaf_rn(__uint_as_float(E1) - Kp[1], gs[1], hp[1]);
-                    const float T2 = __fmaf_rn(__uint_as_float(E2) - Kp[2], gs[2], hp[2]);
-                    tm = fminf(fminf(T0, T1), T2);
-                    const float thr = __fmaf_rn(tm, 1.0f + kEpsT, gtol);
-                    bool p0 = T0 <= thr, p1 = T1 <= thr;
-                    const bool p2 = T2 <= thr;
-                    const bool amb = p0 ? p1 || p2 : p1 == p2;
-                    if (EXACT) {
-                        if (amb) {
-                            const int a = exact_nearest(plane(0, E0 + (1u - kMagicBits)), plane(1, E1 + (1u - kMagicBits)),
-                                                        plane(2, E2 + (1u - kMagicBits)), w.ad[0], w.ad[1], w.ad[2]);
-                            p0 = a == 0;
-                            p1 = a == 1;
-                            tm = sel3(a, T0, T1, T2);
-                        }
-                    } else {
-                        undecided = undecided || amb;
-                    }
-                    e = p0 ? 0 : (p1 ? 1 : 2);
-                    const uint32_t nv = (p0 ? E0 : (p1 ? E1 : E2)) + (1u - kMagicBits);
-                    V0 = p0 ? nv : V0;
-                    V1 = e == 1 ? nv : V1;
-                    V2 = e == 2 ? nv : V2;
-                    m0 = m;
-                    // the level of the cell entered: k for a sibling, else
-                    // that of the lowest set bit (the parent was left)
-                    const int K = __ffs((int)nv) - 1 - e;
-                    if (K >= R) { go = false; break; }  // left the chunk
-                    if (K != k) {
-                        const uint2 par = st[K + 1 - kLow];
-                        pidx = par.x;
-                        pm8 = par.y;
-                    }
-                    k = K;
-                    m = ~0u << k;
-                    o = octant();
-                    occ = (pm8 >> o) & 1u;
-                }
-                if (go) {
-                    // the entered cell's coordinates below the level it was
-                    // left at (the crossed axis' are zero: it is on a face);
-                    // at a tie, below the level it was entered at
-                    if (EXACT) m0 = m;
-                    const float lim = 0.5f - __fmaf_rn(tm, kEpsX, gtol) * dmaxn;
-                    const float x0 = __fmaf_rn(tm, dv[0], xm[0]), x1 = __fmaf_rn(tm, dv[1], xm[1]),
-                                x2 = __fmaf_rn(tm, dv[2], xm[2]);
-                    const float r0 = (x0 + kRound) - kRound, r1 = (x1 + kRound) - kRound, r2 = (x2 + kRound) - kRound;
-                    const bool clear = fabsf(x0 - r0) < (e == 0 ? 1.0f : lim) && fabsf(x1 - r1) < (e == 1 ? 1.0f : lim) &&
-                                       fabsf(x2 - r2) < (e == 2 ? 1.0f : lim);
-                    if (tm * w.dmax > (k > kNearLevel ? kRebaseFar : kRebaseNear) || !clear) {
-                        // far from the base point, or next to a voxel plane: a new base here
-                        const int32_t Nt = plane(e, sel3(e, V0, V1, V2));
-                        if (!undecided) { eb = e; Ne = Nt; }
-                        undecided = (!walk_base<EXACT>(w, Ow, e, Nt, B, x) && !EXACT) || undecided;
-                        rebase(~m0);
-                    } else {
-                        const uint32_t k0 = e == 0 ? ~0u : m0, k1 = e == 1 ? ~0u : m0 << 1, k2 = e == 2 ? ~0u : m0 << 2;
-                        V0 = (V0 & k0) | (__float_as_uint(r0 + Kp[0]) & ~k0);
-                        V1 = (V1 & k1) | (__float_as_uint(__fmaf_rn(r1, 2.0f, Kp[1])) & ~k1);
-                        V2 = (V2 & k2) | (__float_as_uint(__fmaf_rn(r2, 4.0f, Kp[2])) & ~k2);
-                    }
-                }
-            }
-            if (!EXACT && undecided) {
-                alive = false;
-            } else if (traced && occ) {
-                hit.c[0] = (int32_t)V0;
-                hit.c[1] = (int32_t)(V1 >> 1);
-                hit.c[2] = (int32_t)(V2 >> 2);
-                hit.e = e;
-                // depth-first index (Sec. 3.3): the prefix beside each child
-                // pointer of the path, then the leaf block's earlier voxels
-                uint32_t idx;
-                if (EXACT) {
-                    idx = nodes[st[1].x + 3 + 2 * (st[0].y >> 8)];
-                } else {
-                    idx = nodes[pidx + 3 + 2 * __popc(pm8 & ~(~0u << o))];
-                }
-                idx &= kPrefixBits;
-                for (int j = R; j > 3; j--)
-                    idx += nodes[st[j - kLow].x + 3 + 2 * (st[j - 1 - kLow].y >> 8)] & (j == kWideLevel ? ~0u : kPrefixBits);
-                const uint32_t bit = ((V0 & 3u) | ((V1 & 6u) << 1) | ((V2 & 12u) << 2)) ^
-                                     (((mir & 1u) | ((mir & 2u) << 1) | ((mir & 4u) << 2)) * 3u);
-                hit.idx = idx + (uint32_t)__popcll(lmu & ((1ull << bit) - 1ull));
-                found = true;
-                alive = false;
-            }
+            found = walk_chunk<EXACT>(S, w, mir, Ow, cc, traced, based, root, (int)lod, e, Ne, eb, B, x, undecided, hit) ||
+                    found;
+            if (found || (!EXACT && undecided)) alive = false;
         }
         if (alive && !traced) {
             // over this chunk cell: its nearest exit face

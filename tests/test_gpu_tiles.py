@@ -241,3 +241,28 @@ def test_limits_and_errors():
     assert L.aok_render_tiles(c.h, 12345, ctypes.byref(cam), 1.0, ctypes.byref(f), None) == aok.AOK_E_NOT_RESIDENT
     L.aok_scene_destroy(c.h, sid.value)
     c.close()
+
+
+@pytest.mark.parametrize("grid", [(16, 2, 2), (2, 16, 3), (2, 3, 16), (1, 1, 8), (33, 3, 1), (1, 1, 1)])
+def test_records_of_any_grid_shape(ctx, grid):
+    """A visibility record holds its region by the march order and the grid coordinates along the two shorter axes:
+    views from every side (all mirrorings) of grids whose longest axis is x, y or z."""
+    from dataclasses import replace
+    spec = replace(sg.CITY_4096, name="grid%dx%dx%d" % grid, seed=9, wx=8 * grid[0], wy=8 * grid[1], wz=8 * grid[2], chunk=8,
+                   n_lods=1, period0=16, h_min=2, h_max=max(4, 5 * grid[2]), crust=2, n_boxes=10, box_min=1, box_max=6)
+    w = sg.World(spec)
+    sc = aok.Scene.from_world(ctx, w, threads=4)
+    c = (spec.wx / 2, spec.wy / 2, spec.wz / 2)
+    r = 0.75 * max(spec.wx, spec.wy, spec.wz) + 8.0
+    for sx in (-1, 1):
+        for sy in (-1, 1):
+            for sz in (-1, 1):
+                o = (c[0] + sx * r * 0.8, c[1] + sy * r * 0.55, c[2] + sz * r * 0.35)
+                cam = sg.make_camera(o, tuple(c[a] - o[a] for a in range(3)), 141, 99)
+                a, b = aok.alloc_frame(cam.W, cam.H), aok.alloc_frame(cam.W, cam.H)
+                aok.render(ctx, sc, cam, 1.0, *a)
+                aok.render_tiles(ctx, sc, cam, 1.0, *b)
+                torch.cuda.synchronize()
+                assert torch.equal(a[0], b[0]) and torch.equal(a[1].view(torch.int32), b[1].view(torch.int32))
+                assert bool(((a[0][..., 3] >> 19) & 1).any())
+    sc.destroy()

@@ -19,7 +19,7 @@ constexpr int kFix = 12;            // camera origin fixed point: multiples of 2
 constexpr int kMaxLevels = 10;      // log2(512) + 1
 // A device node's prefix words hold 24 bits of prefix and the child's mask
 // above them, except in a node of this side (2^kWideLevel voxels of its LOD).
-constexpr int kWideLevel = 9, kWideSide = 1 << kWideLevel;
+constexpr int kWideLevel = 9;
 constexpr uint32_t kPrefixBits = 0xFFFFFFu;
 constexpr int kMaxImageHeight = 65535 * 8;  // 8-row casting blocks, at most 65535 in grid y
 

@@ -126,6 +126,19 @@ struct BeamState {
     int32_t W = 0, H = 0;
 };
 
+// The reachable nodes of a chunk blob by depth, found while it is validated
+// and used to lay it out.  The vectors keep their storage from one blob to the
+// next (a blob's would be fresh pages of several MB each time).
+struct BlobPlan {
+    std::vector<uint32_t> ord;    // [blob words] place of the node at this word in `node`, or kNoOrd
+    std::vector<uint32_t> node;   // word index of every reachable node, by depth
+    std::vector<uint32_t> level;  // [levels + 1] first place of each depth
+    std::vector<uint32_t> off;    // device word offset of every reachable node
+    std::vector<uint16_t> box;    // solid-voxel box of every reachable node: lo x, y, z, hi x, y, z
+    uint64_t words = 0;           // device words of the nodes
+    static constexpr uint32_t kNoOrd = 0xFFFFFFFFu;
+};
+
 struct aok_ctx_impl;
 
 }  // namespace aok
@@ -142,6 +155,7 @@ struct aok_ctx {
     uint32_t next_scene = 0;
     void* staging = nullptr;
     size_t staging_cap = 0;
+    aok::BlobPlan upload_plan;  // (with the staging buffer, under upload_mu)
     uint32_t* pinned_word = nullptr;
     uint32_t* d_counter = nullptr;
     // persistent casting launch shape (0 = defaults) and single-view kernel choice
@@ -198,6 +212,7 @@ struct Staging {
     size_t cap = 0;
     cudaStream_t stream = nullptr;
     size_t min_cap = (size_t)64 << 20;  // smallest buffer allocated when it grows
+    BlobPlan plan;
 };
 int stage_chunk(aok_ctx* ctx, Scene* sc, int64_t di, uint32_t lod, const aok_chunk_blob* blob, bool evict_old_first,
                 Staging* stg, std::mutex* pool_mu, ChunkAlloc* out_a, ChunkRef* out_ref);

@@ -1,5 +1,6 @@
 """The casting kernels' FP32 decisions (view distance, voxel walk) at the
 places where they hand over to exact arithmetic."""
+import ctypes
 from dataclasses import replace
 
 import numpy as np
@@ -107,3 +108,49 @@ def test_small_frames_at_the_edges_of_the_warp_tiles(ctx, size):
         _equal_to_march(ctx, sc, sg.ground_camera(w, seed, *size, z_lo=4, z_hi=40), 1.5)
     aok.beam_tune(ctx)
     sc.destroy()
+
+
+def test_blob_nodes_in_any_order(ctx):
+    # a blob's nodes may lie in any order, with unused words between them: the same scene
+    w = sg.World(MED64)
+    built = aok.BuiltWorld(w)
+    spec = MED64
+    a = aok.Scene.from_world(ctx, w, built=built)
+    b = aok.Scene(ctx, spec, 2 * built.node_words, built.leaves, built.mat_bytes)
+    rng = np.random.default_rng(7)
+    gx, gy, _ = b.grid
+    keep = []
+    for i in range(len(built)):
+        for lod in range(spec.n_lods):
+            c, blob = built.blob(i, lod)
+            if blob.n_node_words:
+                src = np.ctypeslib.as_array(ctypes.cast(blob.nodes, ctypes.POINTER(ctypes.c_uint32)), (blob.n_node_words,))
+                depth, todo = {int(blob.root): 0}, [int(blob.root)]
+                last = int(np.log2(spec.chunk >> lod)) - 3  # depth of the nodes above the leaf blocks
+                while todo:
+                    n = todo.pop()
+                    if depth[n] < last:
+                        for ch in src[n + 2:n + 2 + int(src[n]).bit_count()]:
+                            if int(ch) not in depth:
+                                depth[int(ch)] = depth[n] + 1
+                                todo.append(int(ch))
+                order = rng.permutation(sorted(depth))
+                at, pos = {}, 0
+                for n in order:
+                    at[int(n)] = pos
+                    pos += 2 + int(src[n]).bit_count() + int(rng.integers(0, 2))
+                dst = np.full(pos + 1, 0xDEADBEEF, np.uint32)
+                for n in order:
+                    n, k = int(n), int(src[n]).bit_count()
+                    dst[at[n]:at[n] + 2] = src[n:n + 2]
+                    ch = src[n + 2:n + 2 + k]
+                    dst[at[n] + 2:at[n] + 2 + k] = ch if depth[n] == last else [at[int(x)] for x in ch]
+                keep.append(dst)
+                blob.nodes, blob.n_node_words, blob.root = dst.ctypes.data, len(dst), at[int(blob.root)]
+            b.upload(c % gx, (c // gx) % gy, c // (gx * gy), lod, blob)
+    for seed in (4, 9):
+        cam = sg.ground_camera(w, seed, 203, 117, z_lo=4, z_hi=40)
+        x, y = _render(ctx, a, cam, 1.5), _render(ctx, b, cam, 1.5)
+        assert torch.equal(x[0], y[0]) and torch.equal(x[1].view(torch.int32), y[1].view(torch.int32))
+    a.destroy()
+    b.destroy()

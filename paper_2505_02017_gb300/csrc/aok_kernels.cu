@@ -22,10 +22,16 @@ namespace {
 
 constexpr int kMaxDevices = 128;
 
+// Programmatic dependent launch: the selection lets the cast after it on its
+// stream be launched at once; the cast waits for it before anything else.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_prerequisites() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __global__ void select_kernel(SceneDev S, CamDev C, ChunkRef* __restrict__ frame, int8_t* __restrict__ lod_out,
                               uint8_t* __restrict__ vis_out, uint32_t* __restrict__ n_visible) {
     const int nch = S.grid[0] * S.grid[1] * S.grid[2];
     const int chunk = blockIdx.x * blockDim.x + threadIdx.x;
+    launch_dependents();
     if (chunk < nch) select_one(S, C, frame, lod_out, vis_out, n_visible, chunk);
 }
 
@@ -83,6 +89,7 @@ __global__ void __launch_bounds__(128, 8) cast_kernel(const __grid_constant__ Sc
     const bool in = px < C.W && py < C.H && lane < 1 << (wl + hl);
     const uint32_t lanes = __ballot_sync(0xFFFFFFFFu, in);
     if (!lanes) return;
+    if (!BEAM) wait_prerequisites();
     const int32_t Dn = BEAM ? beam_bound_warp(beam, wx, wy, lane) : 0;
     if (!in) return;
     const size_t pix = (size_t)py * C.W + px;
@@ -256,12 +263,24 @@ int aokk_select(const SceneDev* s, const CamDev* c, ChunkRef* frame, int8_t* lod
     return status_of(cudaGetLastError());
 }
 
-static void cast_plain(const SceneDev* s, const CamDev* c, const ChunkRef* frame, uint4* hit, float* t,
-                       cudaStream_t st) {
+static cudaError_t cast_plain(const SceneDev* s, const CamDev* c, const ChunkRef* frame, uint4* hit, float* t,
+                              cudaStream_t st) {
     int wl, hl;
     cast_tile(*c, wl, hl);
     dim3 grid((c->W + (2 << wl) - 1) >> (wl + 1), (c->H + (2 << hl) - 1) >> (hl + 1));
-    cast_kernel<false><<<grid, 128, 0, st>>>(*s, *c, frame, hit, t, nullptr, beam_lookup(nullptr, 0, 0), wl, hl);
+    // launched while the selection before it runs: 38 / 46 / 57 -> 36 / 44 / 55 us for 256x256 views, 63 / 71 / 86
+    // -> 61 / 70 / 83 for 320x180 (behind a beam pass, whose SMs its blocks would crowd, frames got 1% longer)
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(128);
+    cfg.stream = st;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, cast_kernel<false>, *s, *c, frame, hit, t, (uint32_t*)nullptr,
+                              beam_lookup(nullptr, 0, 0), wl, hl);
 }
 
 int aokk_cast(const SceneDev* s, const CamDev* c, const ChunkRef* frame, uint4* hit, float* t, uint32_t* counts,
@@ -281,7 +300,7 @@ int aokk_cast(const SceneDev* s, const CamDev* c, const ChunkRef* frame, uint4* 
     else if (beam)
         cast_kernel<false, true><<<grid, 128, 0, st>>>(*s, *c, frame, hit, t, nullptr, bl, wl, hl);
     else
-        cast_plain(s, c, frame, hit, t, st);
+        return status_of(cast_plain(s, c, frame, hit, t, st));
     return status_of(cudaGetLastError());
 }
 
@@ -516,7 +535,7 @@ int aokk_render_noalloc(const SceneDev* s, const CamDev* c, uint4* hit, float* t
     if (ck)
         cast_kernel_checked<false><<<grid, 128, 0, st>>>(*s, *c, frame, hit, t, *ck, beam_lookup(nullptr, 0, 0));
     else
-        cast_plain(s, c, frame, hit, t, st);
+        return status_of(cast_plain(s, c, frame, hit, t, st));
     return status_of(cudaGetLastError());
 }
 

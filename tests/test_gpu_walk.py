@@ -154,3 +154,24 @@ def test_blob_nodes_in_any_order(ctx):
         assert torch.equal(x[0], y[0]) and torch.equal(x[1].view(torch.int32), y[1].view(torch.int32))
     a.destroy()
     b.destroy()
+
+
+def test_small_frame_in_a_cuda_graph(ctx):
+    # the selection and the cast that is launched beside it, captured and replayed
+    w = sg.World(MED64)
+    sc = aok.Scene.from_world(ctx, w, threads=4)
+    cam = sg.ground_camera(w, 4, 160, 90, z_lo=4, z_hi=40)
+    want = _render(ctx, sc, cam, 1.5)
+    hit, t = aok.alloc_frame(cam.W, cam.H)
+    s = torch.cuda.Stream()
+    g = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g, stream=s):
+        aok.render(ctx, sc, cam, 1.5, hit, t, stream=s)
+    for _ in range(3):
+        hit.zero_()
+        t.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(want[0], hit) and torch.equal(want[1].view(torch.int32), t.view(torch.int32))
+    sc.destroy()

@@ -525,7 +525,8 @@ int aok_render_noalloc(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, doub
  * Sec. 2; here exact): with on = 1, aok_render, aok_render_counted,
  * aok_render_host(_async), aok_cast_selected, aok_render_batch (grid
  * launch) and the render server of this context first compute, for every 8 x 4 pixel tile of each
- * frame of at least 0.8 M pixels (aok_beam_tune), a lower bound on the
+ * frame of at least 1.5 M pixels (aok_beam_tune), and of smaller ones from
+ * 0.8 M pixels where the pass can run, a lower bound on the
  * L-infinity distance from the camera origin of every solid voxel of the
  * frame's LOD-cut scene that the tile's rays can meet: a level-by-level walk
  * of the selected DAGs (all views of a batch in one launch), refining a node
@@ -536,21 +537,30 @@ int aok_render_noalloc(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, doub
  * distance.  Output records are identical with the pass on or off.  Buffers
  * (about 11 B per 8 x 4 pixel tile, grown to the largest frame or batch seen,
  * and two 16 MiB node queues) are charged to the budget when first needed.
- * The render server runs it for its batches too (per-request pyramids).
- * Not used by the persistent single-view and batch kernels,
- * aok_render_noalloc or the tile pipeline; with checked casting it runs with
+ * The render server runs it for its batches too (per-request pyramids, or
+ * one arena per stream for the frames below 1.5 M pixels).
+ * aok_render_tiles uses the same bounds.  Not used by the persistent
+ * single-view and batch kernels or
+ * aok_render_noalloc; with checked casting it runs with
  * its node and leaf indices checked.  Default on.  The pass's
- * buffers belong to the context: with it on, renders of one context on
+ * buffers belong to the context: with it on, renders of 1.5 M pixels and more
+ * of one context on
  * different streams must be ordered (an event or a synchronisation between
- * them).  The passes of all contexts of a process run one after another on a
+ * them).  Frames from 0.8 to 1.5 M pixels cast without the pass on a stream
+ * that is being captured and where its buffers don't fit the budget; when an
+ * allocation of this context finds no room, buffers that only such frames
+ * have used are given back, and the context casts them without the pass until
+ * aok_set_beam or aok_beam_tune is called.
+ * The passes of all contexts of a process run one after another on a
  * device (each waits for the previous one's launch to finish). */
 int aok_set_beam(aok_ctx* ctx, int on);
 /* Refinement of the beam pass's walk: a node is refined while its rectangle
  * spans more than refine_tiles tiles and its side is above 2^min_node_log2
  * LOD-0 voxels (a context starts with 16 and 2: down to the 4^3 leaves); frames of fewer
- * than min_pixels pixels cast without the pass (a context starts with 800,000: below
- * that the pass's fixed cost, some tens of microseconds, outweighs what it
- * saves); queue_nodes caps the nodes one level of the walk may queue
+ * than min_pixels pixels cast without the pass, and all others take it (a
+ * context starts with 1,500,000, and with the optional pass from 800,000 on:
+ * below that the pass's fixed cost, some tens of microseconds, outweighs what
+ * it saves); queue_nodes caps the nodes one level of the walk may queue
  * (0: the allocated 2^20; past the cap a node stands for its children).
  * Any setting gives the same output records.  AOK_E_INVALID for
  * min_node_log2 outside [2, 16]. */

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstring>
 #include <map>
@@ -41,7 +42,7 @@ void uncharge(aok_ctx* ctx, size_t bytes) {
     ctx->used -= std::min(ctx->used, bytes);
 }
 
-int dev_alloc(aok_ctx* ctx, void** p, size_t bytes) {
+static int dev_alloc_once(aok_ctx* ctx, void** p, size_t bytes) {
     *p = nullptr;
     if (bytes == 0) return AOK_OK;
     int st = charge(ctx, bytes);
@@ -54,6 +55,12 @@ int dev_alloc(aok_ctx* ctx, void** p, size_t bytes) {
         return e == cudaErrorMemoryAllocation ? AOK_E_OOM : cuda_status(ctx, e);
     }
     return AOK_OK;
+}
+
+int dev_alloc(aok_ctx* ctx, void** p, size_t bytes) {
+    int st = dev_alloc_once(ctx, p, bytes);
+    if (st == AOK_E_OOM && beam_reclaim(ctx)) st = dev_alloc_once(ctx, p, bytes);
+    return st;
 }
 
 void dev_free(aok_ctx* ctx, void* p, size_t bytes) {
@@ -429,7 +436,9 @@ void aok_destroy(aok_ctx* ctx) {
     dev_free(ctx, ctx->d_single_queue, 2 * sizeof(unsigned long long));
     dev_free(ctx, ctx->tiles.block, ctx->tiles.bytes);
     dev_free(ctx, ctx->beam.qblock, ctx->beam.qbytes);
-    dev_free(ctx, ctx->beam.bounds, ctx->beam.bounds_cap * 8);
+    dev_free(ctx, ctx->beam.bounds.p, ctx->beam.bounds.cap * 8);
+    dev_free(ctx, ctx->beam.opt.p, ctx->beam.opt.cap * 8);
+    if (ctx->beam.opt_read) cudaEventDestroy(ctx->beam.opt_read);
     pipe_release(ctx);
     if (ctx->pipe.prep) cudaStreamDestroy(ctx->pipe.prep);
     if (ctx->pipe.render) cudaStreamDestroy(ctx->pipe.render);
@@ -442,8 +451,9 @@ void aok_destroy(aok_ctx* ctx) {
 
 int aok_memory(aok_ctx* ctx, size_t* used, size_t* budget) {
     if (!ctx) return AOK_E_INVALID;
+    const size_t spare = beam_spare_bytes(ctx);  // given back to whatever needs them
     std::lock_guard<std::mutex> g(ctx->mem_mu);
-    if (used) *used = ctx->used;
+    if (used) *used = ctx->used - std::min(ctx->used, spare);
     if (budget) *budget = ctx->budget;
     return AOK_OK;
 }
@@ -909,22 +919,31 @@ static const CheckDev* check_dev(aok_ctx* ctx, const Scene* sc, CheckDev* ck) {
 // ---------------------------------------------------------------------------
 static constexpr uint32_t kBeamCap = 1u << 20;  // queued nodes per level
 
+// Fill new pass buffers; the pass may run on any stream, so the fill is done
+// before it is enqueued.
+static bool fill_now(aok_ctx* ctx, void* p, int byte, size_t bytes) {
+    return cudaMemsetAsync(p, byte, bytes, ctx->copy_stream) == cudaSuccess &&
+           cudaStreamSynchronize(ctx->copy_stream) == cudaSuccess;
+}
+
 // The walk's queues, counters and launch grid (shared by single-view and
-// batch passes, which run in stream order).
-static int ensure_beam_queues(aok_ctx* ctx) {
+// batch passes, which run in stream order).  required: a frame that has to
+// take the pass uses them.
+static int ensure_beam_queues(aok_ctx* ctx, bool required) {
     BeamState& b = ctx->beam;
     std::lock_guard<std::mutex> lk(b.mu);
+    b.q_hard |= required;
     if (b.qblock) return AOK_OK;
     const size_t sq = (size_t)kBeamCap * 16, sc = 2 * kBeamLevels * 4;
     void* block = nullptr;
-    int st = dev_alloc(ctx, &block, 2 * sq + sc);
+    int st = required ? dev_alloc(ctx, &block, 2 * sq + sc) : dev_alloc_once(ctx, &block, 2 * sq + sc);
     if (st) return st;
     b.q[0] = (uint4*)block;
     b.q[1] = (uint4*)((char*)block + sq);
     b.cnt = (uint32_t*)((char*)block + 2 * sq);
     b.hist = b.cnt + kBeamLevels;
     // (each pass leaves the queue counters at zero)
-    if (cudaMemset(b.cnt, 0, sc) != cudaSuccess || cudaStreamSynchronize(nullptr) != cudaSuccess) {
+    if (!fill_now(ctx, b.cnt, 0, sc)) {
         dev_free(ctx, block, 2 * sq + sc);
         return cuda_status(ctx, cudaGetLastError());
     }
@@ -936,23 +955,78 @@ static int ensure_beam_queues(aok_ctx* ctx) {
     return AOK_OK;
 }
 
-// A grow-only array of bound entries, all without a pass tag when allocated
-// (entries carry their pass's tag, so a change of layout needs no clearing).
-static int ensure_bounds(aok_ctx* ctx, unsigned long long** buf, size_t* cap, size_t need) {
-    if (need <= *cap) return AOK_OK;
-    if (*buf) {
-        cudaDeviceSynchronize();
-        dev_free(ctx, *buf, *cap * 8);
-        *buf = nullptr;
-        *cap = 0;
-    }
-    int st = dev_alloc(ctx, (void**)buf, need * 8);
+static int alloc_bounds(aok_ctx* ctx, BoundBuf& b, size_t need, bool required) {
+    void* p = nullptr;
+    int st = required ? dev_alloc(ctx, &p, need * 8) : dev_alloc_once(ctx, &p, need * 8);
     if (st) return st;
-    // the pass that writes them may run on a stream the default stream's memset is not ordered with
-    if (cudaMemset(*buf, 0xFF, need * 8) != cudaSuccess || cudaStreamSynchronize(nullptr) != cudaSuccess)
+    if (!fill_now(ctx, p, 0xFF, need * 8)) {
+        dev_free(ctx, p, need * 8);
         return cuda_status(ctx, cudaGetLastError());
-    *cap = need;
+    }
+    b.p = (unsigned long long*)p;
+    b.cap = need;
     return AOK_OK;
+}
+
+// Room for `need` entries, `required` of them for passes that have to run;
+// all are without a pass tag when allocated (entries carry their pass's tag,
+// so a change of layout needs no clearing).  Where only the required ones
+// fit, b.cap stays below `need`.
+static int ensure_bounds(aok_ctx* ctx, BoundBuf& b, size_t need, size_t required) {
+    b.hard = std::max(b.hard, required);
+    if (need <= b.cap) return AOK_OK;
+    if (need > required && ctx->beam.no_room) {
+        if (required <= b.cap) return required ? AOK_OK : AOK_E_OOM;
+        need = required;
+    }
+    if (b.p) {
+        cudaDeviceSynchronize();
+        dev_free(ctx, b.p, b.cap * 8);
+        b.p = nullptr;
+        b.cap = 0;
+    }
+    if (need <= required) return alloc_bounds(ctx, b, need, true);
+    int st = alloc_bounds(ctx, b, need, false);
+    if (st != AOK_E_OOM) return st;
+    ctx->beam.no_room = true;
+    if (b.hard) st = alloc_bounds(ctx, b, b.hard, true);
+    return required || st != AOK_OK ? st : AOK_E_OOM;
+}
+
+static std::array<BoundBuf*, 3 + kHostSlots> bound_bufs(aok_ctx* ctx) {
+    std::array<BoundBuf*, 3 + kHostSlots> r{&ctx->beam.bounds, &ctx->beam.opt, &ctx->batch.beam_bounds};
+    for (int i = 0; i < kHostSlots; i++) r[3 + i] = &ctx->pipe.slot[i].bounds;
+    return r;
+}
+
+extern "C++" size_t aok::beam_spare_bytes(aok_ctx* ctx) {
+    const BeamState& b = ctx->beam;
+    std::lock_guard<std::recursive_mutex> lk(ctx->beam.use);
+    size_t n = serve_beam_bytes(ctx) + (b.qblock && !b.q_hard ? b.qbytes : 0);
+    for (const BoundBuf* s : bound_bufs(ctx)) n += s->cap > s->hard ? (s->cap - s->hard) * 8 : 0;
+    return n;
+}
+
+extern "C++" bool aok::beam_reclaim(aok_ctx* ctx) {
+    BeamState& b = ctx->beam;
+    std::lock_guard<std::recursive_mutex> lk(b.use);
+    if (!beam_spare_bytes(ctx) || cudaDeviceSynchronize() != cudaSuccess) return false;
+    b.no_room = true;
+    const bool queues = b.qblock && !b.q_hard;
+    if (queues || b.opt.cap || b.bounds.cap > b.bounds.hard) b.valid = false;
+    if (queues) {
+        dev_free(ctx, b.qblock, b.qbytes);
+        b.qblock = nullptr;
+    }
+    for (BoundBuf* s : bound_bufs(ctx))
+        if (s->cap > s->hard) {
+            dev_free(ctx, s->p, s->cap * 8);
+            s->p = nullptr;
+            s->cap = 0;
+            if (s->hard) alloc_bounds(ctx, *s, s->hard, false);  // (else at the next pass that needs it)
+        }
+    serve_beam_release(ctx);
+    return true;
 }
 
 // The next pass's tag (tags count down); before they wrap every bound array
@@ -962,9 +1036,10 @@ static int next_beam_tag(aok_ctx* ctx, void* stream, uint32_t* tag) {
     std::lock_guard<std::mutex> lk(b.mu);
     if (++b.passes >= 0xFFFFFFF0u) {
         const cudaStream_t s = (cudaStream_t)stream;
-        if ((b.bounds && cudaMemsetAsync(b.bounds, 0xFF, b.bounds_cap * 8, s) != cudaSuccess) ||
-            (ctx->batch.beam_bounds &&
-             cudaMemsetAsync(ctx->batch.beam_bounds, 0xFF, ctx->batch.beam_cap * 8, s) != cudaSuccess))
+        const BoundBuf& bb = ctx->batch.beam_bounds;
+        if ((b.bounds.p && cudaMemsetAsync(b.bounds.p, 0xFF, b.bounds.cap * 8, s) != cudaSuccess) ||
+            (b.opt.p && cudaMemsetAsync(b.opt.p, 0xFF, b.opt.cap * 8, s) != cudaSuccess) ||
+            (bb.p && cudaMemsetAsync(bb.p, 0xFF, bb.cap * 8, s) != cudaSuccess))
             return AOK_E_CUDA;
         b.passes = 1;
         b.valid = false;
@@ -987,20 +1062,34 @@ static void beam_header(aok_ctx* ctx, BeamBatch* P, uint32_t tag) {
     std::memset(&P->ck, 0, sizeof(P->ck));  // unchecked
 }
 
-// The beam pass over the scene's current frame table, remembered with what
-// it was computed for.  select: the frame table is not selected yet; the
+// A view's pass buffers.
+static int beam_buffers(aok_ctx* ctx, BoundBuf& b, const CamDev& cd, bool optional) {
+    const size_t need = beam_entries((uint32_t)cd.W, (uint32_t)cd.H);
+    RelaxedCapture rc(optional);
+    int st = ensure_beam_queues(ctx, !optional);
+    if (!st) st = ensure_bounds(ctx, b, need, optional ? 0 : need);
+    if (st == AOK_E_OOM && optional) ctx->beam.no_room = true;
+    return st;
+}
+
+// The beam pass over the scene's current frame table; *rd: what the cast
+// reads.  select: the frame table is not selected yet; the
 // pass selects it as its first step (one launch fewer), or, for a view
 // without a usable projection, the selection kernel does.  ck: checked
 // casting's pool sizes and error word (the pass tests its node and leaf
-// indices too), or null.
+// indices too), or null.  optional: AOK_E_OOM leaves the frame as it was, to be
+// cast without the pass; the cast is followed by beam_was_read.  keep: the
+// pass is remembered with what it was computed for.  Called with the pass's
+// buffers held (b.use).
 static int run_beam(aok_ctx* ctx, uint32_t scene, Scene* sc, const SceneDev& sd, const CamDev& cd, void* stream,
-                    bool select = false, const CheckDev* ck = nullptr) {
-    int st = ensure_beam_queues(ctx);
-    if (st) return st;
+                    BeamRead* rd, bool select, const CheckDev* ck, bool optional, bool keep) {
     BeamState& b = ctx->beam;
-    st = ensure_bounds(ctx, &b.bounds, &b.bounds_cap, beam_entries((uint32_t)cd.W, (uint32_t)cd.H));
+    BoundBuf& buf = optional ? b.opt : b.bounds;
+    int st = beam_buffers(ctx, buf, cd, optional);
     if (st) return st;
-    b.valid = false;
+    if (optional && b.opt_read && cudaStreamWaitEvent((cudaStream_t)stream, b.opt_read, 0) != cudaSuccess)
+        return AOK_E_CUDA;
+    if (keep || b.read.bounds == buf.p) b.valid = false;
     uint32_t tag;
     st = next_beam_tag(ctx, stream, &tag);
     if (st) return st;
@@ -1009,13 +1098,12 @@ static int run_beam(aok_ctx* ctx, uint32_t scene, Scene* sc, const SceneDev& sd,
     if (ck) P->ck = *ck;
     P->n_views = 0;
     P->n_regions = 0;
-    b.read.bounds = nullptr;  // no usable projection: no bounds, nothing is skipped
-    b.read.tag = tag;
-    if (aokk_beam_view(&sd, &cd, sc->d_frame, b.bounds, &P->v[0])) {
+    *rd = BeamRead{nullptr, tag};  // no usable projection: no bounds, nothing is skipped
+    if (aokk_beam_view(&sd, &cd, sc->d_frame, buf.p, &P->v[0])) {
         P->v[0].region_begin = 0;
         P->n_views = 1;
         P->n_regions = (uint32_t)sc->n_chunks;
-        b.read.bounds = b.bounds;
+        rd->bounds = buf.p;
         if (select) {
             P->select = 1;
             P->cam = cd;
@@ -1025,7 +1113,8 @@ static int run_beam(aok_ctx* ctx, uint32_t scene, Scene* sc, const SceneDev& sd,
         if (st) return st;
     }
     st = aokk_beam_run(P, b.grid, stream);
-    if (st) return st;
+    if (st || !keep) return st;
+    b.read = *rd;
     b.valid = true;
     b.scene = scene;
     b.gen = sc->select_gen;
@@ -1036,8 +1125,26 @@ static int run_beam(aok_ctx* ctx, uint32_t scene, Scene* sc, const SceneDev& sd,
     return AOK_OK;
 }
 
-extern "C++" bool aok::beam_wanted(const aok_ctx* ctx, int32_t W, int32_t H) {
-    return ctx->beam_on && (uint64_t)W * (uint64_t)H >= ctx->beam_min_pixels;
+// After a cast that read an optional pass's pyramid: the next optional pass,
+// on whatever stream, waits for it.
+static int beam_was_read(aok_ctx* ctx, void* stream) {
+    cudaEvent_t& ev = ctx->beam.opt_read;
+    cudaError_t e = ev ? cudaSuccess : cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventRecord(ev, (cudaStream_t)stream);
+    return cuda_status(ctx, e);
+}
+
+extern "C++" BeamUse aok::beam_use(const aok_ctx* ctx, int32_t W, int32_t H, void* stream) {
+    const uint64_t px = (uint64_t)W * (uint64_t)H;
+    if (!ctx->beam_on) return kBeamNone;
+    if (px >= ctx->beam_min_pixels) return kBeamRequired;
+    if (px < ctx->beam_min_optional || ctx->beam.no_room) return kBeamNone;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing((cudaStream_t)stream, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return kBeamNone;
+    }
+    return cap == cudaStreamCaptureStatusNone ? kBeamOptional : kBeamNone;
 }
 
 extern "C++" int aok::beam_for_batch(aok_ctx* ctx, BatchParams* groups, uint32_t ngroups,
@@ -1045,23 +1152,31 @@ extern "C++" int aok::beam_for_batch(aok_ctx* ctx, BatchParams* groups, uint32_t
                                      unsigned long long* const* view_bounds) {
     out.clear();
     if (!ctx->beam_on) return AOK_OK;
-    size_t need = 0, n_big = 0;
+    // entries of the views with a required pass, and with an optional one
+    size_t need[3] = {0, 0, 0}, flat = 0;
     for (uint32_t g = 0; g < ngroups; g++)
-        for (uint32_t i = 0; i < groups[g].n_views; i++) {
+        for (uint32_t i = 0; i < groups[g].n_views; i++, flat++) {
             const CamDev& c = groups[g].v[i].cam;
-            if (beam_wanted(ctx, c.W, c.H)) {
-                need += beam_entries((uint32_t)c.W, (uint32_t)c.H);
-                n_big++;
-            }
+            if (view_bounds && !view_bounds[flat]) continue;
+            need[beam_use(ctx, c.W, c.H, stream)] += beam_entries((uint32_t)c.W, (uint32_t)c.H);
         }
-    if (!n_big) return AOK_OK;
-    int st = ensure_beam_queues(ctx);
-    if (!st && !view_bounds) st = ensure_bounds(ctx, &ctx->batch.beam_bounds, &ctx->batch.beam_cap, need);
+    const size_t req = need[kBeamRequired], opt = need[kBeamOptional];
+    if (!req && !opt) return AOK_OK;
+    RelaxedCapture rc(!req);
+    BoundBuf& bb = ctx->batch.beam_bounds;
+    int st = ensure_beam_queues(ctx, req > 0);
+    if (!st && !view_bounds) st = ensure_bounds(ctx, bb, req + opt, req);
+    if (st == AOK_E_OOM && !req) {
+        ctx->beam.no_room = true;
+        return AOK_OK;
+    }
     uint32_t tag = 0;
     if (!st) st = next_beam_tag(ctx, stream, &tag);
     if (st) return st;
+    const bool all = view_bounds || bb.cap >= req + opt;  // else the optional passes don't fit
     out.resize(ngroups);
-    size_t off = 0, flat = 0;
+    size_t off = 0;
+    flat = 0;
     for (uint32_t g = 0; g < ngroups; g++) {
         BeamBatch& B = out[g];
         beam_header(ctx, &B, tag);
@@ -1071,8 +1186,9 @@ extern "C++" int aok::beam_for_batch(aok_ctx* ctx, BatchParams* groups, uint32_t
         for (uint32_t i = 0; i < groups[g].n_views; i++, flat++) {
             ViewDev& d = groups[g].v[i];
             d.beam = nullptr;
-            if (!beam_wanted(ctx, d.cam.W, d.cam.H)) continue;
-            unsigned long long* bnd = view_bounds ? view_bounds[flat] : ctx->batch.beam_bounds + off;
+            const BeamUse use = beam_use(ctx, d.cam.W, d.cam.H, stream);
+            if (use == kBeamNone || (use == kBeamOptional && !all)) continue;
+            unsigned long long* bnd = view_bounds ? view_bounds[flat] : bb.p + off;
             off += beam_entries((uint32_t)d.cam.W, (uint32_t)d.cam.H);
             if (!bnd) continue;
             if (!aokk_beam_view(&d.scene, &d.cam, d.frame, bnd, &B.v[B.n_views])) continue;  // casts without
@@ -1103,19 +1219,27 @@ static int cast_single(aok_ctx* ctx, uint32_t scene, Scene* sc, const SceneDev& 
                        const aok_frame* frame, uint32_t* counts, void* stream, bool selected = true) {
     CheckDev ck;
     const CheckDev* ckp = check_dev(ctx, sc, &ck);
+    BeamRead rd{nullptr, 0};
     const BeamRead* beam = nullptr;
     int st = AOK_OK;
-    if (ctx->beam_on && (uint64_t)cd.W * (uint64_t)cd.H >= ctx->beam_min_pixels) {
-        if (!selected || !beam_fresh(ctx, scene, sc, cd)) {
-            st = run_beam(ctx, scene, sc, sd, cd, stream, !selected, ckp);
-            if (st) return st;
+    std::lock_guard<std::recursive_mutex> lk(ctx->beam.use);
+    const BeamUse use = beam_use(ctx, cd.W, cd.H, stream);
+    if (use != kBeamNone) {
+        const bool optional = use == kBeamOptional;
+        if (selected && beam_fresh(ctx, scene, sc, cd)) rd = ctx->beam.read;
+        else st = run_beam(ctx, scene, sc, sd, cd, stream, &rd, !selected, ckp, optional, !optional);
+        if (st == AOK_OK) {
             selected = true;
+            beam = &rd;
+        } else if (st != AOK_E_OOM || use == kBeamRequired) {
+            return st;
         }
-        beam = &ctx->beam.read;
+        st = AOK_OK;
     }
     if (!selected) st = aokk_select(&sd, &cd, sc->d_frame, nullptr, nullptr, nullptr, stream);
     if (st) return st;
-    return aokk_cast(&sd, &cd, sc->d_frame, (uint4*)frame->hit, frame->t, counts, stream, ckp, beam);
+    st = aokk_cast(&sd, &cd, sc->d_frame, (uint4*)frame->hit, frame->t, counts, stream, ckp, beam);
+    return st || !beam || use != kBeamOptional ? st : beam_was_read(ctx, stream);
 }
 
 static int render_impl(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, double tau, const aok_frame* frame,
@@ -1287,15 +1411,19 @@ int aok_render_tiles(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, double
     // the beam pass's bounds cull the pairs in front of every voxel a tile's
     // rays can meet and restart the rays of the others (as in the march); the
     // pass selects the frame table as its first step
+    BeamRead rd{nullptr, 0};
     const BeamRead* beam = nullptr;
-    if (beam_wanted(ctx, cd.W, cd.H)) {
-        st = run_beam(ctx, scene, sc, sd, cd, stream, true);
-        beam = &ctx->beam.read;
-    } else {
-        st = aokk_select(&sd, &cd, sc->d_frame, nullptr, nullptr, nullptr, stream);
+    std::lock_guard<std::recursive_mutex> lk(ctx->beam.use);
+    const BeamUse use = beam_use(ctx, cd.W, cd.H, stream);
+    if (use != kBeamNone) {
+        st = run_beam(ctx, scene, sc, sd, cd, stream, &rd, true, nullptr, use == kBeamOptional, use == kBeamRequired);
+        if (!st) beam = &rd;
     }
+    if (use == kBeamNone || (use == kBeamOptional && st == AOK_E_OOM))
+        st = aokk_select(&sd, &cd, sc->d_frame, nullptr, nullptr, nullptr, stream);
     if (!st) st = aokk_tiles_frame(&sd, &cd, sc->d_frame, &ctx->tiles.dev, (uint4*)frame->hit, frame->t,
                                    ctx->sm_count, stream, beam);
+    if (!st && beam && use == kBeamOptional) st = beam_was_read(ctx, stream);
     if (st) return st == AOK_E_CUDA ? launch_failure(ctx) : st;
     std::swap(ctx->tiles.dev.hiz_prev, ctx->tiles.dev.hiz_next);  // this frame's depth culls the next one
     return AOK_OK;
@@ -1319,6 +1447,7 @@ int aok_tiles_forget(aok_ctx* ctx) {
 int aok_set_beam(aok_ctx* ctx, int on) {
     if (!ctx) return AOK_E_INVALID;
     ctx->beam_on = on ? 1 : 0;
+    ctx->beam.no_room = false;
     return AOK_OK;
 }
 
@@ -1327,8 +1456,9 @@ int aok_beam_tune(aok_ctx* ctx, uint32_t refine_tiles, int32_t min_node_log2, ui
     if (!ctx || min_node_log2 < 2 || min_node_log2 > 16) return AOK_E_INVALID;
     ctx->beam_refine = refine_tiles;
     ctx->beam_min_log2 = min_node_log2;
-    ctx->beam_min_pixels = min_pixels;
+    ctx->beam_min_pixels = ctx->beam_min_optional = min_pixels;
     ctx->beam_queue = queue_nodes;
+    ctx->beam.no_room = false;
     return AOK_OK;
 }
 
@@ -1341,7 +1471,9 @@ int aok_beam_selected(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, void*
     if (st) return st;
     cudaSetDevice(ctx->device);
     SceneDev sd = scene_dev(sc);
-    st = run_beam(ctx, scene, sc, sd, cd, stream);
+    std::lock_guard<std::recursive_mutex> lk(ctx->beam.use);
+    BeamRead rd;
+    st = run_beam(ctx, scene, sc, sd, cd, stream, &rd, false, nullptr, false, true);
     if (st == AOK_E_CUDA) return launch_failure(ctx);
     return st;
 }
@@ -1357,9 +1489,12 @@ int aok_select_beam(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, double 
     SceneDev sd = scene_dev(sc);
     sc->select_gen++;
     CheckDev ck;
-    if (ctx->beam_on && (uint64_t)cd.W * (uint64_t)cd.H >= ctx->beam_min_pixels)
-        st = run_beam(ctx, scene, sc, sd, cd, stream, true, check_dev(ctx, sc, &ck));
-    else
+    std::lock_guard<std::recursive_mutex> lk(ctx->beam.use);
+    const BeamUse use = beam_use(ctx, cd.W, cd.H, stream);
+    BeamRead rd;
+    if (use != kBeamNone)
+        st = run_beam(ctx, scene, sc, sd, cd, stream, &rd, true, check_dev(ctx, sc, &ck), use == kBeamOptional, true);
+    if (use == kBeamNone || (use == kBeamOptional && st == AOK_E_OOM))
         st = aokk_select(&sd, &cd, sc->d_frame, nullptr, nullptr, nullptr, stream);
     if (st == AOK_E_CUDA) return launch_failure(ctx);
     return st;
@@ -1466,7 +1601,7 @@ static void pipe_release(aok_ctx* ctx) {
         dev_free(ctx, sl.hit, p.px * 16);
         dev_free(ctx, sl.t, p.px * 4);
         dev_free(ctx, sl.frame, sl.frame_cap * sizeof(ChunkRef));
-        dev_free(ctx, sl.bounds, sl.bounds_cap * 8);
+        dev_free(ctx, sl.bounds.p, sl.bounds.cap * 8);
         if (sl.prepped) cudaEventDestroy(sl.prepped);
         if (sl.rendered) cudaEventDestroy(sl.rendered);
         if (sl.copied) cudaEventDestroy(sl.copied);
@@ -1522,11 +1657,13 @@ static int pipe_render(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, doub
         if (st) return st;
         sl.frame_cap = (size_t)sc->n_chunks;
     }
-    const bool beam = beam_wanted(ctx, cd.W, cd.H);
+    std::lock_guard<std::recursive_mutex> lk(ctx->beam.use);
+    const BeamUse use = beam_use(ctx, cd.W, cd.H, p.prep);
+    bool beam = use != kBeamNone;
     if (beam) {
-        st = ensure_beam_queues(ctx);
-        if (!st) st = ensure_bounds(ctx, &sl.bounds, &sl.bounds_cap, beam_entries((uint32_t)cd.W, (uint32_t)cd.H));
-        if (st) return st;
+        st = beam_buffers(ctx, sl.bounds, cd, use == kBeamOptional);
+        if (st == AOK_E_OOM && use == kBeamOptional) beam = false;
+        else if (st) return st;
     }
     const SceneDev sd = scene_dev(sc);
     // the selection kernel, then the pass (measured faster here than the pass
@@ -1542,11 +1679,11 @@ static int pipe_render(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, doub
         beam_header(ctx, P, tag);
         P->n_views = 0;
         P->n_regions = 0;
-        if (aokk_beam_view(&sd, &cd, sl.frame, sl.bounds, &P->v[0])) {
+        if (aokk_beam_view(&sd, &cd, sl.frame, sl.bounds.p, &P->v[0])) {
             P->v[0].region_begin = 0;
             P->n_views = 1;
             P->n_regions = (uint32_t)sc->n_chunks;
-            rd.bounds = sl.bounds;
+            rd.bounds = sl.bounds.p;
             rd.tag = tag;
         }
         st = aokk_beam_run(P, ctx->beam.grid, p.prep, 1);  // beside the previous frame's cast

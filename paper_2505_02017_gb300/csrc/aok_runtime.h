@@ -53,13 +53,19 @@ struct Scene {
 // its loads and quarantined space; the object stays for aok_stream_destroy.
 void stream_detach(aok_stream* s);
 
+// A grow-only array of beam pyramid entries.
+struct BoundBuf {
+    unsigned long long* p = nullptr;
+    size_t cap = 0;   // entries
+    size_t hard = 0;  // entries that frames with a required pass have needed
+};
+
 // Device arena of aok_render_batch: per-view frame tables, work counters and
 // the CUDA graph of the last list shape.
 struct BatchArena {
     ChunkRef* d_frames = nullptr;
     size_t frames_cap = 0;
-    unsigned long long* beam_bounds = nullptr;  // the views' bound pyramids (grow-only)
-    size_t beam_cap = 0;                        // entries
+    BoundBuf beam_bounds;                   // the views' bound pyramids
     unsigned long long* d_queue = nullptr;  // 2 per group, zero between launches
     size_t queue_cap = 0;
     GraphCache graph;
@@ -77,8 +83,7 @@ struct HostSlot {
     float* t = nullptr;
     ChunkRef* frame = nullptr;  // the slot's chunk table
     size_t frame_cap = 0;       // entries
-    unsigned long long* bounds = nullptr;  // the slot's bound pyramid
-    size_t bounds_cap = 0;                 // entries
+    BoundBuf bounds;            // the slot's bound pyramid
     cudaEvent_t prepped = nullptr, rendered = nullptr, copied = nullptr;
     uint64_t ticket = 0;  // frame in this slot (0: none yet)
 };
@@ -106,16 +111,24 @@ struct TileState {
 // the context), the single-view bound pyramid and what its last pass was
 // computed for.
 struct BeamState {
+    // held from a pass's buffers being looked up to its launches being enqueued: another thread that runs short of
+    // memory may give the buffers back (beam_reclaim)
+    std::recursive_mutex use;
     std::mutex mu;  // the queues' allocation and the pass counter (the serving thread shares them)
     void* qblock = nullptr;
     size_t qbytes = 0;
+    bool q_hard = false;   // a frame that has to take the pass has used the queues
+    std::atomic<bool> no_room{false};  // memory ran short: frames that need not take the pass no longer do
     uint4* q[2] = {nullptr, nullptr};
     uint32_t* cnt = nullptr;   // [kBeamLevels] queue counts, then [kBeamLevels] walk histogram
     uint32_t* hist = nullptr;
     unsigned grid = 0;         // blocks of the cooperative launch
     std::unique_ptr<BeamBatch> P;  // host parameter block (~26 KB)
-    unsigned long long* bounds = nullptr;  // single-view pyramid (grow-only)
-    size_t bounds_cap = 0;                 // entries
+    BoundBuf bounds;                       // single-view pyramid
+    // the pyramid of frames that need not take the pass, and the last cast
+    // that read it: they may come on streams that nothing orders
+    BoundBuf opt;
+    cudaEvent_t opt_read = nullptr;
     uint32_t passes = 0;                   // passes run (their tags count down)
     // the last single-view pass: a scene, its selection, a camera
     bool valid = false;
@@ -176,9 +189,11 @@ struct aok_ctx {
     int beam_on = 1;  // single-view renders run the beam pass before casting
     uint32_t beam_refine = 16;  // refine nodes spanning more tiles than this ...
     int beam_min_log2 = 2;     // ... whose side is above 2^this LOD-0 voxels
-    // smaller frames cast without the pass (city views of 1120 x 630 break even at 160-240 us, 1280 x 720 ones
-    // gain 12% on average with it, -29% to +12%, and 960 x 540 ones nothing)
-    uint64_t beam_min_pixels = 800000;
+    // Frames of beam_min_pixels take the pass.  Those of beam_min_optional take it where it can run: not on a stream
+    // that is being captured (the passes of a device wait for one another by events a capture can't hold) and not
+    // where its 33 MB of queues don't fit the budget.  Smaller ones cast without it (city views of 1120 x 630 break
+    // even at 160-240 us, 1280 x 720 ones gain 12% on average with it, -29% to +12%, and 960 x 540 ones nothing).
+    uint64_t beam_min_pixels = 1500000, beam_min_optional = 800000;
     uint32_t beam_queue = 0;             // nodes a queue level may hold (0: the allocated 2^20)
     aok::HostPipe pipe;
     int checked = 0;  // single-view casts check every pool index (error word: d_counter[8])
@@ -204,8 +219,32 @@ void free_alloc(Scene* sc, ChunkAlloc& a);
 // Leaves `out` empty if no view takes the pass.
 int beam_for_batch(aok_ctx* ctx, BatchParams* groups, uint32_t ngroups, std::vector<BeamBatch>& out, void* stream,
                    unsigned long long* const* view_bounds = nullptr);
-// Whether a frame of W x H pixels takes the beam pass in this context.
-bool beam_wanted(const aok_ctx* ctx, int32_t W, int32_t H);
+// Whether a frame of W x H pixels on `stream` takes the beam pass in this
+// context, and whether it may also be cast without.
+inline bool beam_required(const aok_ctx* ctx, int32_t W, int32_t H) {
+    return ctx->beam_on && (uint64_t)W * (uint64_t)H >= ctx->beam_min_pixels;
+}
+enum BeamUse { kBeamNone, kBeamOptional, kBeamRequired };
+BeamUse beam_use(const aok_ctx* ctx, int32_t W, int32_t H, void* stream);
+// Frees the pass's buffers that only optional passes have needed (true: there
+// were some); the context runs no optional pass any more.
+bool beam_reclaim(aok_ctx* ctx);
+size_t beam_spare_bytes(aok_ctx* ctx);  // what it would free
+// ... the serving loop's share of them.
+size_t serve_beam_bytes(aok_ctx* ctx);
+void serve_beam_release(aok_ctx* ctx);
+// Lets this thread allocate while another one captures a stream in the global
+// capture mode (whose capture an allocation here would end).
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    const bool on;
+    explicit RelaxedCapture(bool use) : on(use) {
+        if (on) cudaThreadExchangeStreamCaptureMode(&mode);
+    }
+    ~RelaxedCapture() {
+        if (on) cudaThreadExchangeStreamCaptureMode(&mode);
+    }
+};
 // Pinned staging memory and the stream its copies go on.
 struct Staging {
     void* buf = nullptr;

@@ -133,7 +133,7 @@ void batch_release(aok_ctx* ctx) {
     aokk_graph_destroy(&A.graph);
     dev_free(ctx, A.d_frames, A.frames_cap * sizeof(ChunkRef));
     dev_free(ctx, A.d_queue, A.queue_cap * sizeof(unsigned long long));
-    dev_free(ctx, A.beam_bounds, A.beam_cap * 8);
+    dev_free(ctx, A.beam_bounds.p, A.beam_bounds.cap * 8);
     A = BatchArena();
 }
 
@@ -150,7 +150,9 @@ static int render_batch_impl(aok_ctx* ctx, const aok_view* views, uint32_t n, vo
     if (st) return st;
     // the beam pass for the views large enough (grid launch only)
     std::vector<BeamBatch> beams;
+    std::unique_lock<std::recursive_mutex> lk(ctx->beam.use, std::defer_lock);
     if (L.ctas == 0) {
+        lk.lock();
         st = beam_for_batch(ctx, prep.groups.data(), (uint32_t)prep.groups.size(), beams, stream);
         if (st) return st;
     }
@@ -237,6 +239,7 @@ struct ServeState {
     std::vector<cudaEvent_t> beam_ev;    // per stream: selection done, beam pass done
     std::vector<unsigned long long*> counters;  // 2 * kBatchViews-group pairs per stream
     std::vector<uint32_t> stream_busy;
+    std::vector<BoundBuf> arena;  // per stream: pyramids of requests that need not take the pass
     std::mutex mu;
     std::condition_variable cv, done_cv;
     std::deque<uint64_t> pending;
@@ -270,13 +273,65 @@ static void CUDART_CB on_batch_done(void* p) {
 }
 
 // A request's device memory: frame record, distances, chunk table and, for a
-// frame that takes the beam pass, its bound pyramid.
+// frame that has to take the beam pass, its bound pyramid.
 static size_t request_bytes(const aok_ctx* ctx, const Scene* sc, const aok_camera& cam) {
     const size_t px = (size_t)cam.width * cam.height;
     size_t b = ((px * 16 + 255) & ~(size_t)255) + ((px * 4 + 255) & ~(size_t)255) +
                (((size_t)sc->n_chunks * sizeof(ChunkRef) + 255) & ~(size_t)255);
-    if (beam_wanted(ctx, cam.width, cam.height)) b += (size_t)beam_entries((uint32_t)cam.width, (uint32_t)cam.height) * 8;
+    if (beam_required(ctx, cam.width, cam.height))
+        b += (size_t)beam_entries((uint32_t)cam.width, (uint32_t)cam.height) * 8;
     return b;
+}
+
+// Room in a stream's arena for the pyramids of the requests that need not take
+// the pass (nullptr: none, they are cast without).  The stream's batches use
+// it one after another; it is replaced in stream order.
+static unsigned long long* serve_bounds(aok_ctx* ctx, ServeState& S, uint32_t slot, size_t need) {
+    BoundBuf& a = S.arena[slot];
+    if (need <= a.cap) return a.p;
+    const cudaStream_t st = S.streams[slot];
+    if (a.p) {
+        cudaFreeAsync(a.p, st);
+        uncharge(ctx, a.cap * 8);
+        a = BoundBuf();
+    }
+    const size_t cap = need + need / 2;
+    void* p = nullptr;
+    if (charge(ctx, cap * 8) != AOK_OK) {
+        ctx->beam.no_room = true;
+        return nullptr;
+    }
+    if (cudaMallocFromPoolAsync(&p, cap * 8, S.pool, st) != cudaSuccess) {
+        cudaGetLastError();
+        uncharge(ctx, cap * 8);
+        ctx->beam.no_room = true;
+        return nullptr;
+    }
+    cudaMemsetAsync(p, 0xFF, cap * 8, st);  // no entry has a pass's tag
+    a.p = (unsigned long long*)p;
+    a.cap = cap;
+    return a.p;
+}
+
+size_t serve_beam_bytes(aok_ctx* ctx) {
+    size_t n = 0;
+    if (ctx->serve)
+        for (const BoundBuf& a : ctx->serve->arena) n += a.cap * 8;
+    return n;
+}
+
+// (the device is idle)
+void serve_beam_release(aok_ctx* ctx) {
+    if (!ctx->serve) return;
+    ServeState& S = *ctx->serve;
+    for (size_t i = 0; i < S.arena.size(); i++)
+        if (S.arena[i].p) {
+            cudaFreeAsync(S.arena[i].p, S.streams[i]);
+            cudaStreamSynchronize(S.streams[i]);
+            uncharge(ctx, S.arena[i].cap * 8);
+            S.arena[i] = BoundBuf();
+        }
+    cudaMemPoolTrimTo(S.pool, 0);
 }
 
 static void free_ticket_memory(aok_ctx* ctx, Ticket& t, cudaStream_t s) {
@@ -348,18 +403,20 @@ static void serve_loop(aok_ctx* ctx) {
                     continue;
                 }
                 const size_t bytes = request_bytes(ctx, sc, t.req.cam);
-                if (charge(ctx, bytes) != AOK_OK) break;  // wait for memory to free up
                 void* mem = nullptr;
-                if (cudaMallocFromPoolAsync(&mem, bytes, S.pool, S.streams[slot]) != cudaSuccess) {
+                auto take = [&] {
+                    if (charge(ctx, bytes) != AOK_OK) return false;
+                    if (cudaMallocFromPoolAsync(&mem, bytes, S.pool, S.streams[slot]) == cudaSuccess) return true;
                     cudaGetLastError();
                     uncharge(ctx, bytes);
-                    break;
-                }
+                    return false;
+                };
+                if (!take() && !(beam_reclaim(ctx) && take())) break;  // wait for memory to free up
                 const size_t px = (size_t)t.req.cam.width * t.req.cam.height;
                 t.hit = mem;
                 t.t = (float*)((char*)mem + ((px * 16 + 255) & ~(size_t)255));
                 t.frame = (ChunkRef*)((char*)t.t + ((px * 4 + 255) & ~(size_t)255));
-                t.bounds = beam_wanted(ctx, t.req.cam.width, t.req.cam.height)
+                t.bounds = beam_required(ctx, t.req.cam.width, t.req.cam.height)
                                ? (unsigned long long*)((char*)t.frame +
                                                        (((size_t)sc->n_chunks * sizeof(ChunkRef) + 255) & ~(size_t)255))
                                : nullptr;
@@ -410,10 +467,12 @@ static void serve_loop(aok_ctx* ctx) {
                 P.total_tiles = tiles;
             }
         }
-        // the beam pass for the large requests (grid launch): their pyramids
-        // are fresh pool memory, so every entry is first set to "no tag"
+        // the beam pass for the large requests (grid launch): pyramids in a
+        // request's fresh pool memory are first set to "no tag" everywhere
         std::vector<BeamBatch> beams;
+        std::unique_lock<std::recursive_mutex> use(ctx->beam.use, std::defer_lock);
         if (rc == AOK_OK && L.ctas == 0) {
+            use.lock();
             std::vector<unsigned long long*> vb(batch.size(), nullptr);
             {
                 std::lock_guard<std::mutex> g(S.mu);
@@ -426,6 +485,21 @@ static void serve_loop(aok_ctx* ctx) {
                     cudaSuccess)
                     rc = AOK_E_CUDA;
             }
+            size_t need = 0, off = 0;
+            auto entries = [&](size_t i) {
+                const ViewDev& d = S.params[i / kBatchViews].v[i % kBatchViews];
+                return vb[i] || beam_use(ctx, d.cam.W, d.cam.H, st) != kBeamOptional
+                           ? (size_t)0
+                           : (size_t)beam_entries((uint32_t)d.cam.W, (uint32_t)d.cam.H);
+            };
+            for (size_t i = 0; i < batch.size(); i++) need += entries(i);
+            unsigned long long* arena = need ? serve_bounds(ctx, S, slot, need) : nullptr;
+            for (size_t i = 0; i < batch.size() && arena; i++)
+                if (const size_t n = entries(i)) {
+                    vb[i] = arena + off;
+                    off += n;
+                }
+            RelaxedCapture relaxed(true);
             if (rc == AOK_OK) rc = beam_for_batch(ctx, S.params.data(), ngroups, beams, st, vb.data());
         }
         if (rc == AOK_OK) {
@@ -435,6 +509,7 @@ static void serve_loop(aok_ctx* ctx) {
             rc = aokk_batch_run(S.params.data(), ngroups, L.ctas, L.threads, st, beams.empty() ? nullptr : beams.data(),
                                 ctx->beam.grid, &ho, nullptr);
         }
+        if (use.owns_lock()) use.unlock();
         std::lock_guard<std::mutex> g(S.mu);
         if (rc != AOK_OK) {
             for (uint64_t id : batch) {
@@ -589,6 +664,7 @@ int aok_serve_start(aok_ctx* ctx, uint32_t max_slots, uint32_t max_batch, uint32
             return AOK_E_CUDA;
         S->counters.push_back(c);
         S->stream_busy.push_back(0);
+        S->arena.emplace_back();
         for (int k = 0; k < 2; k++) {
             cudaEvent_t e;
             if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) return AOK_E_CUDA;
@@ -634,6 +710,11 @@ int aok_serve_stop(aok_ctx* ctx) {
     cudaSetDevice(ctx->device);
     for (auto& kv : S->tickets) free_ticket_memory(ctx, kv.second, S->streams[0]);
     for (cudaStream_t s : S->streams) cudaStreamSynchronize(s);
+    {
+        std::lock_guard<std::recursive_mutex> lk(ctx->beam.use);
+        serve_beam_release(ctx);
+        ctx->serve = nullptr;
+    }
     if (S->beam_stream) {
         cudaStreamSynchronize(S->beam_stream);
         cudaStreamDestroy(S->beam_stream);

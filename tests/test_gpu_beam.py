@@ -5,6 +5,7 @@ non-ambiguous pixel; every tile's bound is at most the L-infinity distance
 from the camera of every voxel hit in it; a camera matrix the pass cannot
 invert turns it off (all bounds 0); on the benchmark's 4096^3 frame the pass
 removes node visits."""
+import ctypes
 from dataclasses import replace
 
 import numpy as np
@@ -467,5 +468,130 @@ def test_first_host_frames_beside_default_stream_work():
         aok.render(c, sc, m, 1.5, hit, t)
         torch.cuda.synchronize()
         assert torch.equal(hit.cpu(), o[0]) and torch.equal(t.cpu().view(torch.int32), o[1].view(torch.int32))
+    sc.destroy()
+    c.close()
+
+
+def _optional_setup(budget=0):
+    """A context with its initial settings, a scene, three 1280x720 cameras (a size that takes the pass only where it
+    can run) and their frames without the pass."""
+    c = aok.Context(0, budget_bytes=budget)
+    w = sg.World(MED64)
+    sc = aok.Scene.from_world(c, w, threads=4)
+    cams = [sg.ground_camera(w, s, 1280, 720, z_lo=4, z_hi=40) for s in (4, 9, 12)]
+    aok.set_beam(c, False)
+    refs = [aok.alloc_frame(m.W, m.H) for m in cams]
+    for m, r in zip(cams, refs):
+        aok.render(c, sc, m, 1.5, *r)
+    torch.cuda.synchronize()
+    aok.set_beam(c, True)
+    return c, sc, cams, refs
+
+
+def _equal(x, y):
+    return torch.equal(x[0], y[0]) and torch.equal(x[1].view(torch.int32), y[1].view(torch.int32))
+
+
+def test_optional_pass_under_capture():
+    c, sc, cams, refs = _optional_setup()
+    out = aok.alloc_frame(1280, 720)
+    for warm in range(2):
+        for what in range(2):
+            s, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+            torch.cuda.synchronize()
+            with torch.cuda.graph(g, stream=s):
+                if what == 0:
+                    aok.render(c, sc, cams[0], 1.5, *out, stream=s)
+                else:
+                    aok.select_beam(c, sc, cams[0], 1.5, stream=s)
+                    aok.cast_selected(c, sc, cams[0], *out, stream=s)
+            for _ in range(2):
+                out[0].zero_()
+                out[1].zero_()
+                g.replay()
+                torch.cuda.synchronize()
+                assert _equal(out, refs[0]), (warm, what)
+        aok.render(c, sc, cams[1], 1.5, *out)  # with the pass
+        torch.cuda.synchronize()
+        assert _equal(out, refs[1])
+    sc.destroy()
+    c.close()
+
+
+@pytest.mark.parametrize("room_mb", [24, 60])
+def test_optional_pass_within_the_budget(room_mb):
+    """24 MB: the pass's queues don't fit and the frames are cast without it.  60 MB: they do, and are given back
+    when a scene needs their room.  The memory a context reports holds neither."""
+    c, sc, cams, refs = _optional_setup()
+    used = c.memory()[0]
+    sc.destroy()
+    c.close()
+    c, sc, cams, refs = _optional_setup(used + (room_mb << 20))
+    assert c.memory()[0] == used
+    outs = [aok.alloc_frame(1280, 720) for _ in cams]
+
+    def frames():
+        for m, o, r in zip(cams, outs, refs):
+            aok.render(c, sc, m, 1.5, *o)
+            torch.cuda.synchronize()
+            assert _equal(o, r)
+        aok.render_batch(c, [aok.make_view(sc, m, 1.5, *o) for m, o in zip(cams, outs)])
+        torch.cuda.synchronize()
+        assert all(_equal(o, r) for o, r in zip(outs, refs))
+
+    aok.render(c, sc, cams[0], 1.5, *outs[0])
+    torch.cuda.synchronize()
+    assert _equal(outs[0], refs[0]) and c.memory()[0] == used
+    frames()
+    d, sid = aok.SceneDesc(), ctypes.c_uint32()
+    d.grid[0] = d.grid[1] = d.grid[2] = 1
+    d.chunk_res, d.n_lods = 64, 1
+    d.node_words, d.leaf_count, d.mat_bytes = 5 << 20, 1, 1  # 40 MB in the device layout
+    st = aok.lib().aok_scene_create(c.h, ctypes.byref(d), ctypes.byref(sid))
+    assert st == (aok.AOK_E_OOM if room_mb == 24 else aok.AOK_OK)
+    frames()
+    sc.destroy()
+    c.close()
+
+
+def test_optional_passes_on_unordered_streams():
+    c, sc, cams, refs = _optional_setup()
+    w2 = sg.World(MED64)
+    sc2 = aok.Scene.from_world(c, w2, threads=4)  # (its own chunk table)
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    a = [aok.alloc_frame(1280, 720) for _ in range(12)]
+    b = [aok.alloc_frame(1280, 720) for _ in range(12)]
+    torch.cuda.synchronize()
+    for i in range(12):
+        aok.render(c, sc, cams[i % 3], 1.5, *a[i], stream=s1)
+        aok.render(c, sc2, cams[(i + 1) % 3], 1.5, *b[i], stream=s2)
+    torch.cuda.synchronize()
+    for i in range(12):
+        assert _equal(a[i], refs[i % 3]) and _equal(b[i], refs[(i + 1) % 3]), i
+    sc.destroy()
+    sc2.destroy()
+    c.close()
+
+
+@pytest.mark.parametrize("room_mb", [0, 24, 60])
+def test_optional_pass_in_the_server(room_mb):
+    """room_mb 0: no limit.  24: one request's frame at a time and no queues.  60: the queues, given back when
+    a second request's frame needs their room."""
+    c, sc, cams, refs = _optional_setup()
+    used = c.memory()[0]
+    if room_mb:
+        sc.destroy()
+        c.close()
+        c, sc, cams, refs = _optional_setup(used + (room_mb << 20))
+    srv = aok.Server(c, max_slots=8, max_batch=4, n_streams=2)
+    for rep in range(2):
+        held = [srv.submit(sc, m, 1.5) for m in (cams if room_mb != 24 else cams[:1])]
+        for tk, r in zip(held, refs):
+            st, f = srv.wait(tk, 20000)
+            assert st == aok.AOK_OK and _equal(srv.result(tk, f), r)
+        torch.cuda.synchronize()
+        for tk in held:
+            assert srv.release(tk) == aok.AOK_OK
+    srv.stop()
     sc.destroy()
     c.close()

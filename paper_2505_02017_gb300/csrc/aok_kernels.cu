@@ -66,6 +66,23 @@ __device__ __forceinline__ int32_t beam_bound_warp(const BeamLookup& b, int px, 
     return (int32_t)__reduce_min_sync(0xFFFFFFFFu, (uint32_t)(v >> 32) == b.tag ? (uint32_t)v : (uint32_t)INT_MAX);
 }
 
+// The same for a view of a batch, whose pyramid's level offsets are not at hand.
+__device__ __forceinline__ int32_t beam_bound_warp(const unsigned long long* __restrict__ b, uint32_t tag, int W, int H,
+                                                   int px, int py, int lane) {
+    if (!b) return 0;
+    const uint32_t tx = (uint32_t)(W + kBeamTileW - 1) / kBeamTileW, ty = (uint32_t)(H + kBeamTileH - 1) / kBeamTileH;
+    const int L = min(lane, kBeamPyr - 1);
+    uint32_t off = 0;
+#pragma unroll
+    for (int l = 0; l < kBeamPyr - 1; l++) {
+        const uint32_t n = ((tx + (1u << l) - 1) >> l) * ((ty + (1u << l) - 1) >> l);
+        if (l < L) off += n;
+    }
+    const uint32_t x = ((uint32_t)px / kBeamTileW) >> L, y = ((uint32_t)py / kBeamTileH) >> L;
+    const unsigned long long v = __ldcg(b + off + y * ((tx + (1u << L) - 1) >> L) + x);
+    return (int32_t)__reduce_min_sync(0xFFFFFFFFu, (uint32_t)(v >> 32) == tag ? (uint32_t)v : (uint32_t)INT_MAX);
+}
+
 // 16 x 8 pixel tiles, warps of 8 x 4 pixels.  BEAM: the warp's 8 x 4 tile
 // bound from the beam pass (aok_beam.cu) restarts its rays' march past the
 // space in front of the nearest voxel they can meet.  At most 64 registers:
@@ -208,12 +225,14 @@ __global__ void __launch_bounds__(128, 8) cast_grid(const __grid_constant__ Batc
     const int twl = P.tile_w_log, tw = 1 << twl, th = 32 >> twl;
     const int bw = (v.cam.W + 2 * tw - 1) / (2 * tw);
     const int32_t local = (int32_t)(blk - v.tile_begin);
-    const int px = (local % bw) * 2 * tw + (warp & 1) * tw + (lane & (tw - 1));
-    const int py = (local / bw) * 2 * th + (warp >> 1) * th + (lane >> twl);
+    const int wx = ((local % bw) * 2 + (warp & 1)) * tw, wy = ((local / bw) * 2 + (warp >> 1)) * th;
+    const int px = wx + (lane & (tw - 1)), py = wy + (lane >> twl);
     const uint32_t lanes = __ballot_sync(0xFFFFFFFFu, px < v.cam.W && py < v.cam.H);
+    if (!lanes) return;
+    // with a bound of 0 (no beam pass for this view) the march is the plain one
+    const int32_t Dn = twl == 3 ? beam_bound_warp(v.beam, P.beam_tag, v.cam.W, v.cam.H, wx, wy, lane)
+                                : beam_bound(v.beam, P.beam_tag, v.cam.W, v.cam.H, min(px, v.cam.W - 1), min(py, v.cam.H - 1));
     if (px < v.cam.W && py < v.cam.H) {
-        // with a bound of 0 (no beam pass for this view) the march is the plain one
-        const int32_t Dn = beam_bound(v.beam, P.beam_tag, v.cam.W, v.cam.H, px, py);
         cast_pixel<true>(v.scene, v.cam, v.frame, px, py, v.hit, v.t, (size_t)py * v.cam.W + px, Dn, lanes);
     }
 }

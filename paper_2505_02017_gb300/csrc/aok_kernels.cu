@@ -110,6 +110,10 @@ __global__ void __launch_bounds__(128, 8) cast_kernel(const __grid_constant__ Sc
     const int32_t Dn = BEAM ? beam_bound_warp(beam, wx, wy, lane) : 0;
     if (!in) return;
     const size_t pix = (size_t)py * C.W + px;
+    if (BEAM && !COUNT && Dn == INT_MAX) {  // nothing solid in the tile's view
+        emit_miss(out_hit, out_t, pix);
+        return;
+    }
     if (COUNT) trace_pixel<true, false, BEAM>(S, C, frame, px, py, out_hit, out_t, counts, pix, nullptr, Dn);
     else cast_pixel<BEAM>(S, C, frame, px, py, out_hit, out_t, pix, Dn, lanes);
 }
@@ -212,7 +216,7 @@ __global__ void __launch_bounds__(256) cast_persistent(const __grid_constant__ B
 // tiles (2^tile_w_log x 32/2^tile_w_log pixels each); P.v[v].tile_begin is the
 // exclusive prefix sum of the views' block-tile counts.  The view index derives
 // from blockIdx only, so every per-view parameter load is block-uniform.
-__global__ void __launch_bounds__(128, 8) cast_grid(const __grid_constant__ BatchParams P) {
+__global__ void __launch_bounds__(128, 9) cast_grid(const __grid_constant__ BatchParams P) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint64_t blk = blockIdx.x;
     uint32_t lo = 0, hi = P.n_views - 1;  // last view with tile_begin <= blk
@@ -232,9 +236,10 @@ __global__ void __launch_bounds__(128, 8) cast_grid(const __grid_constant__ Batc
     // with a bound of 0 (no beam pass for this view) the march is the plain one
     const int32_t Dn = twl == 3 ? beam_bound_warp(v.beam, P.beam_tag, v.cam.W, v.cam.H, wx, wy, lane)
                                 : beam_bound(v.beam, P.beam_tag, v.cam.W, v.cam.H, min(px, v.cam.W - 1), min(py, v.cam.H - 1));
-    if (px < v.cam.W && py < v.cam.H) {
-        cast_pixel<true>(v.scene, v.cam, v.frame, px, py, v.hit, v.t, (size_t)py * v.cam.W + px, Dn, lanes);
-    }
+    if (px >= v.cam.W || py >= v.cam.H) return;
+    const size_t pix = (size_t)py * v.cam.W + px;
+    if (twl == 3 && Dn == INT_MAX) emit_miss(v.hit, v.t, pix);  // nothing solid in the tile's view
+    else cast_pixel<true>(v.scene, v.cam, v.frame, px, py, v.hit, v.t, pix, Dn, lanes);
 }
 
 // Descriptor patches in the order the host queued them (one thread: a later

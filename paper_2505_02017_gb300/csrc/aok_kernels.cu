@@ -110,7 +110,10 @@ __global__ void __launch_bounds__(128, 8) cast_kernel(const __grid_constant__ Sc
     const int32_t Dn = BEAM ? beam_bound_warp(beam, wx, wy, lane) : 0;
     if (!in) return;
     const size_t pix = (size_t)py * C.W + px;
-    if (BEAM && !COUNT && Dn == INT_MAX) {  // nothing solid in the tile's view
+    // Nothing solid in the tile's view: the miss is written without setting the
+    // ray up (overview 3840x2160 470 / 487 / 467 -> 418 / 439 / 418 us, walk
+    // views 1920x1080 318 / 239 / 290 -> 316 / 236 / 290).
+    if (BEAM && !COUNT && Dn == INT_MAX) {
         emit_miss(out_hit, out_t, pix);
         return;
     }
@@ -215,7 +218,9 @@ __global__ void __launch_bounds__(256) cast_persistent(const __grid_constant__ B
 // covers block tile b of the concatenated views, a block tile being 2x2 warp
 // tiles (2^tile_w_log x 32/2^tile_w_log pixels each); P.v[v].tile_begin is the
 // exclusive prefix sum of the views' block-tile counts.  The view index derives
-// from blockIdx only, so every per-view parameter load is block-uniform.
+// from blockIdx only, so every per-view parameter load is block-uniform.  9
+// blocks per SM (56 registers): 24 views 3546 / 3067 / 3674 us, 8 blocks 3595 /
+// 3105 / 3725, 10 blocks 3572 / 3103 / 3707 (one view's kernel gains nothing).
 __global__ void __launch_bounds__(128, 9) cast_grid(const __grid_constant__ BatchParams P) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint64_t blk = blockIdx.x;

@@ -8,13 +8,19 @@
 // Why: the exact march spends two 32 x 32 -> 64-bit products (half-rate
 // multiplies) and a 64-bit compare on every comparison of plane crossings, and
 // compares again at every level it descends.  Here a crossing is one FMA, the
-// nearest of three and its distance from the second one are a minimum and
-// three compares, and a cell's coordinates at all levels are found at once
+// nearest of three and its distance from the second one are the minimum and
+// the median of three, and a cell's coordinates at all levels are found at once
 // when an occupied cell is entered, so that descending costs no comparison.
-// Bound: instruction issue (about 70% of it) and the divergence of neighbour
-// rays (19 of 32 lanes).  Frames, exact march -> this walk: city 1920x1080
+// Bound: instruction issue (about 70% of it, the ALU pipe 67%) and the
+// divergence of neighbour rays (17.5 of 32 lanes; 7 at the entry of a leaf
+// block, 9 in its steps).  Frames, exact march -> this walk when it was new:
+// city 1920x1080
 // 484 -> 334 us, overview 3840x2160 743 -> 530, open world 2560x1440
 // 801 -> 557, 24 views 6404 -> 4278, 320x180 147 -> 83, 256x256 74 -> 54 us.
+// Three shapes that are slower here, frames of city 1920x1080 (315 / 232 / 290
+// us at the time): the rays that reach a leaf block wait for the others before
+// any enters (412 / 277 / 344), one way out of the leaf block's loop (330 / 241
+// / 303), its three-way branch by selects (346 / 249 / 312).
 //
 // Numbers.  The ray is taken in the frame mirrored so that d >= 0.  Its
 // parameter t counts from a base point on the ray, known to 2^-24 of a voxel:
@@ -255,12 +261,16 @@ __device__ __forceinline__ bool walk_chunk(const SceneDev& S, const WalkRay& w, 
             const uint32_t mi = ((mir & 1u) | ((mir & 2u) << 1) | ((mir & 4u) << 2)) * 3u;
             for (;;) {
                 const uint32_t j = i ^ mi;
-                occ = (((j & 32u) ? (uint32_t)(lmu >> 32) : (uint32_t)lmu) >> (j & 31u)) & 1u;
+                occ = (lmu >> j) & 1u;
                 if (occ) break;
-                tm = fminf(fminf(T0, T1), T2);
+                // (decided when the second smallest, the median, lies past
+                // thr; against three compares with thr and their logic, here
+                // and below, 315 / 232 / 290 -> 307 / 229 / 282 us)
+                const float lo01 = fminf(T0, T1), hi01 = fmaxf(T0, T1);
+                tm = fminf(lo01, T2);
                 const float thr = __fmaf_rn(tm, 1.0f + kEpsLeaf, gtol);
-                const bool p0 = T0 <= thr, p1 = T1 <= thr, p2 = T2 <= thr;
-                undecided = undecided || (p0 ? p1 || p2 : p1 == p2);
+                undecided = undecided || !(fminf(hi01, fmaxf(lo01, T2)) > thr);
+                const bool p2 = T2 < lo01, p0 = !p2 && T0 < T1, p1 = !p2 && !p0;
                 if (p0) { T0 = T0 + gs[0]; inc = 1u; }
                 else if (p1) { T1 = __fmaf_rn(gs[1], 2.0f, T1); inc = 4u; }
                 else { T2 = __fmaf_rn(gs[2], 4.0f, T2); inc = 16u; }
@@ -284,11 +294,12 @@ __device__ __forceinline__ bool walk_chunk(const SceneDev& S, const WalkRay& w, 
             const float T0 = __fmaf_rn(__uint_as_float(E0) - Kp[0], gs[0], hp[0]);
             const float T1 = __fmaf_rn(__uint_as_float(E1) - Kp[1], gs[1], hp[1]);
             const float T2 = __fmaf_rn(__uint_as_float(E2) - Kp[2], gs[2], hp[2]);
-            tm = fminf(fminf(T0, T1), T2);
+            const float lo01 = fminf(T0, T1), hi01 = fmaxf(T0, T1);
+            tm = fminf(lo01, T2);
             const float thr = __fmaf_rn(tm, 1.0f + kEpsT, gtol);
-            bool p0 = T0 <= thr, p1 = T1 <= thr;
-            const bool p2 = T2 <= thr;
-            const bool amb = p0 ? p1 || p2 : p1 == p2;
+            const bool p2 = T2 < lo01;
+            bool p0 = !p2 && T0 < T1, p1 = !p2 && !p0;
+            const bool amb = !(fminf(hi01, fmaxf(lo01, T2)) > thr);
             if (EXACT) {
                 if (amb) {
                     const int a = exact_nearest(plane(0, E0 + (1u - kMagicBits)), plane(1, E1 + (1u - kMagicBits)),
@@ -303,8 +314,8 @@ __device__ __forceinline__ bool walk_chunk(const SceneDev& S, const WalkRay& w, 
             e = p0 ? 0 : (p1 ? 1 : 2);
             const uint32_t nv = (p0 ? E0 : (p1 ? E1 : E2)) + (1u - kMagicBits);
             V0 = p0 ? nv : V0;
-            V1 = e == 1 ? nv : V1;
-            V2 = e == 2 ? nv : V2;
+            V1 = p1 ? nv : V1;
+            V2 = p0 || p1 ? V2 : nv;
             m0 = m;
             // the level of the cell entered: k for a sibling, else
             // that of the lowest set bit (the parent was left)
@@ -329,8 +340,8 @@ __device__ __forceinline__ bool walk_chunk(const SceneDev& S, const WalkRay& w, 
             const float x0 = __fmaf_rn(tm, dv[0], xm[0]), x1 = __fmaf_rn(tm, dv[1], xm[1]),
                         x2 = __fmaf_rn(tm, dv[2], xm[2]);
             const float r0 = (x0 + kRound) - kRound, r1 = (x1 + kRound) - kRound, r2 = (x2 + kRound) - kRound;
-            const bool clear = fabsf(x0 - r0) < (e == 0 ? 1.0f : lim) && fabsf(x1 - r1) < (e == 1 ? 1.0f : lim) &&
-                               fabsf(x2 - r2) < (e == 2 ? 1.0f : lim);
+            const float f0 = e == 0 ? 0.0f : x0 - r0, f1 = e == 1 ? 0.0f : x1 - r1, f2 = e == 2 ? 0.0f : x2 - r2;
+            const bool clear = fmaxf(fmaxf(fabsf(f0), fabsf(f1)), fabsf(f2)) < lim;
             if (tm * w.dmax > (k > kNearLevel ? kRebaseFar : kRebaseNear) || !clear) {
                 // far from the base point, or next to a voxel plane: a new base here
                 const int32_t Nt = plane(e, sel3(e, V0, V1, V2));

@@ -363,8 +363,8 @@ int aok_render(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, double lod_t
  * Buffers (visibility records 8 B per pixel, per-tile and per-region arrays)
  * are allocated on first use and when the resolution or grid changes,
  * charged to the budget.  Not for concurrent calls on one context.
- * AOK_E_INVALID for scenes of more than AOK_TILES_MAX_CHUNKS regions (the key
- * holds a 16-bit region index) or a misaligned frame. */
+ * AOK_E_INVALID for scenes of more than AOK_TILES_MAX_CHUNKS regions or a
+ * misaligned frame. */
 #define AOK_TILES_MAX_CHUNKS 65536
 int aok_render_tiles(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, double lod_threshold_px,
                      const aok_frame* frame, void* stream);

@@ -86,9 +86,14 @@ __device__ __forceinline__ int32_t beam_bound_warp(const unsigned long long* __r
 // 16 x 8 pixel tiles, warps of 8 x 4 pixels.  BEAM: the warp's 8 x 4 tile
 // bound from the beam pass (aok_beam.cu) restarts its rays' march past the
 // space in front of the nearest voxel they can meet.  At most 64 registers:
-// 8 blocks per SM (72 and 7 blocks: overview 3840x2160 511 us a frame instead
-// of 491, city 1080p 360 instead of 354; 56 and 9 blocks: 482 and 352, but
-// 320x180 views, where occupancy does not matter, 3% slower).
+// 8 blocks per SM (three views each, city 1920x1080 318 / 241 / 291 us, overview
+// 3840x2160 468 / 486 / 467, open world 2560x1440 414 / 468 / 589; 7 blocks 323 /
+// 239 / 292, 481 / 498 / 479, 416 / 473 / 601; 9 blocks 320 / 243 / 293, 463 /
+// 482 / 464, 422 / 470 / 589; 10 blocks 319 / 247 / 294, 459 / 478 / 458, 437 /
+// 475 / 592).  A warp takes 12 to 20 us on average and up to 140, so a frame
+// ends with few warps left; other orders of the rows and smaller or larger
+// blocks shorten some views and lengthen others (rows from below: city 303 /
+// 228 / 278 -> 325 / 184 / 320 us; blocks of one warp 313 / 247 / 285).
 //
 // Without bounds a warp may take a smaller tile, wl and hl its sides' logs (3
 // and 2: 8 x 4), in its first lanes: see cast_tile.

@@ -1085,11 +1085,11 @@ static int run_beam(aok_ctx* ctx, uint32_t scene, Scene* sc, const SceneDev& sd,
                     BeamRead* rd, bool select, const CheckDev* ck, bool optional, bool keep) {
     BeamState& b = ctx->beam;
     BoundBuf& buf = optional ? b.opt : b.bounds;
+    if (keep || b.read.bounds == buf.p) b.valid = false;  // (the buffer may move)
     int st = beam_buffers(ctx, buf, cd, optional);
     if (st) return st;
     if (optional && b.opt_read && cudaStreamWaitEvent((cudaStream_t)stream, b.opt_read, 0) != cudaSuccess)
         return AOK_E_CUDA;
-    if (keep || b.read.bounds == buf.p) b.valid = false;
     uint32_t tag;
     st = next_beam_tag(ctx, stream, &tag);
     if (st) return st;

@@ -595,3 +595,19 @@ def test_optional_pass_in_the_server(room_mb):
     srv.stop()
     sc.destroy()
     c.close()
+
+
+def test_optional_pass_kept_while_its_buffer_grows():
+    """A selection's bounds are not used after a larger frame's pass has replaced their buffer."""
+    c, sc, cams, refs = _optional_setup()
+    sc2 = aok.Scene.from_world(c, sg.World(MED64), threads=4)
+    big = aok.alloc_frame(1400, 1000)
+    out = aok.alloc_frame(1280, 720)
+    aok.select_beam(c, sc, cams[0], 1.5)
+    aok.render(c, sc2, replace(cams[1], W=1400, H=1000), 1.5, *big)
+    aok.cast_selected(c, sc, cams[0], *out)
+    torch.cuda.synchronize()
+    assert _equal(out, refs[0])
+    sc.destroy()
+    sc2.destroy()
+    c.close()

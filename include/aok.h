@@ -526,7 +526,7 @@ int aok_render_noalloc(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, doub
  * aok_render_host(_async), aok_cast_selected, aok_render_batch (grid
  * launch) and the render server of this context first compute, for every 8 x 4 pixel tile of each
  * frame of at least 1.5 M pixels (aok_beam_tune), and of smaller ones from
- * 0.8 M pixels where the pass can run, a lower bound on the
+ * 0.8 M pixels where the pass can run (not aok_render_counted's), a lower bound on the
  * L-infinity distance from the camera origin of every solid voxel of the
  * frame's LOD-cut scene that the tile's rays can meet: a level-by-level walk
  * of the selected DAGs (all views of a batch in one launch), refining a node

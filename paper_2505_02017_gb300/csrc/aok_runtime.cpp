@@ -1223,7 +1223,8 @@ static int cast_single(aok_ctx* ctx, uint32_t scene, Scene* sc, const SceneDev& 
     const BeamRead* beam = nullptr;
     int st = AOK_OK;
     std::lock_guard<std::recursive_mutex> lk(ctx->beam.use);
-    const BeamUse use = beam_use(ctx, cd.W, cd.H, stream);
+    BeamUse use = beam_use(ctx, cd.W, cd.H, stream);
+    if (counts && use == kBeamOptional) use = kBeamNone;  // its visits would depend on whether the pass could run
     if (use != kBeamNone) {
         const bool optional = use == kBeamOptional;
         if (selected && beam_fresh(ctx, scene, sc, cd)) rd = ctx->beam.read;

@@ -611,3 +611,17 @@ def test_optional_pass_kept_while_its_buffer_grows():
     sc.destroy()
     sc2.destroy()
     c.close()
+
+
+def test_counts_do_not_depend_on_the_optional_pass():
+    c, sc, cams, refs = _optional_setup()
+    counts = [torch.zeros((720, 1280, 3), dtype=torch.int32, device="cuda") for _ in range(2)]
+    out = aok.alloc_frame(1280, 720)
+    for k in range(2):
+        aok.set_beam(c, k == 1)
+        aok.render_counted(c, sc, cams[0], 1.5, *out, counts[k])
+        torch.cuda.synchronize()
+        assert _equal(out, refs[0])
+    assert torch.equal(*counts)
+    sc.destroy()
+    c.close()

@@ -591,6 +591,14 @@ int aok_select_beam(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, double 
  * that parents stand in for their children) and tiles_xy (nullable, 2).
  * AOK_E_INVALID before the first beam pass or if n_bounds is too small. */
 int aok_beam_info(aok_ctx* ctx, int32_t* bounds, uint64_t n_bounds, uint32_t* level_counts, int32_t* tiles_xy);
+/* Beam passes this context has run: one for a single view's frame, one for
+ * all views of a batch or of a server's batch. */
+int aok_beam_passes(aok_ctx* ctx, uint64_t* passes);
+/* Diagnostics.  A pass marks its bounds with a 32-bit tag that counts down;
+ * after 2^32 - 17 passes the tags start over and each bound array is cleared
+ * before its next use.  This moves the counter on, as if all but `left` of
+ * them had been used.  AOK_E_INVALID if fewer are left already. */
+int aok_beam_tags_left(aok_ctx* ctx, uint32_t left);
 
 /* ------------------------------------------------------------------ */
 /* Diagnostics                                                        */

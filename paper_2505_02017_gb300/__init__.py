@@ -125,6 +125,8 @@ def lib() -> ctypes.CDLL:
             "aok_set_beam": [vp, ctypes.c_int],
             "aok_beam_tune": [vp, u32, ctypes.c_int32, u64, u32],
             "aok_beam_info": [vp, P(ctypes.c_int32), u64, P(u32), P(ctypes.c_int32)],
+            "aok_beam_passes": [vp, P(u64)],
+            "aok_beam_tags_left": [vp, u32],
             "aok_beam_selected": [vp, u32, P(Camera), vp],
             "aok_select_beam": [vp, u32, P(Camera), dbl, vp],
             "aok_checked_errors": [vp, P(u32)],
@@ -467,6 +469,18 @@ def beam_info(ctx: Context):
     check(lib().aok_beam_info(ctx.h, b.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)), b.size, None, None),
           "aok_beam_info")
     return b, [int(v) for v in lv]
+
+
+def beam_passes(ctx: Context) -> int:
+    """Beam passes the context has run (aok_beam_passes)."""
+    n = ctypes.c_uint64()
+    check(lib().aok_beam_passes(ctx.h, ctypes.byref(n)), "aok_beam_passes")
+    return n.value
+
+
+def beam_tags_left(ctx: Context, left: int):
+    """Leave `left` pass tags before they start over (aok_beam_tags_left)."""
+    return check(lib().aok_beam_tags_left(ctx.h, left), "aok_beam_tags_left")
 
 
 def checked_errors(ctx: Context) -> int:

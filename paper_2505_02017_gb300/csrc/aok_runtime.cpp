@@ -965,6 +965,7 @@ static int alloc_bounds(aok_ctx* ctx, BoundBuf& b, size_t need, bool required) {
     }
     b.p = (unsigned long long*)p;
     b.cap = need;
+    b.epoch = ctx->beam.epoch;
     return AOK_OK;
 }
 
@@ -1029,22 +1030,30 @@ extern "C++" bool aok::beam_reclaim(aok_ctx* ctx) {
     return true;
 }
 
-// The next pass's tag (tags count down); before they wrap every bound array
-// is cleared.
-static int next_beam_tag(aok_ctx* ctx, void* stream, uint32_t* tag) {
+static constexpr uint32_t kBeamTags = 0xFFFFFFEFu;  // tags of an epoch
+
+// The next pass's tag (tags count down; after the last one a new epoch begins)
+// and its epoch.
+static uint32_t next_beam_tag(aok_ctx* ctx, uint32_t* epoch) {
     BeamState& b = ctx->beam;
     std::lock_guard<std::mutex> lk(b.mu);
-    if (++b.passes >= 0xFFFFFFF0u) {
-        const cudaStream_t s = (cudaStream_t)stream;
-        const BoundBuf& bb = ctx->batch.beam_bounds;
-        if ((b.bounds.p && cudaMemsetAsync(b.bounds.p, 0xFF, b.bounds.cap * 8, s) != cudaSuccess) ||
-            (b.opt.p && cudaMemsetAsync(b.opt.p, 0xFF, b.opt.cap * 8, s) != cudaSuccess) ||
-            (bb.p && cudaMemsetAsync(bb.p, 0xFF, bb.cap * 8, s) != cudaSuccess))
-            return AOK_E_CUDA;
+    b.total++;
+    if (++b.passes > kBeamTags) {
         b.passes = 1;
-        b.valid = false;
+        b.epoch++;
     }
-    *tag = 0xFFFFFFFFu - b.passes;
+    *epoch = b.epoch;
+    return 0xFFFFFFFFu - b.passes;
+}
+
+// Before a pass of `epoch` writes into `b` on `stream`: a buffer last written
+// in an earlier epoch is cleared, in the order of its users (each buffer has
+// one at a time), since the entries of that epoch's last passes would win
+// against the new ones and read as "nothing solid".
+static int beam_renew(BoundBuf& b, uint32_t epoch, void* stream) {
+    if (!b.p || b.epoch == epoch) return AOK_OK;
+    if (cudaMemsetAsync(b.p, 0xFF, b.cap * 8, (cudaStream_t)stream) != cudaSuccess) return AOK_E_CUDA;
+    b.epoch = epoch;
     return AOK_OK;
 }
 
@@ -1090,8 +1099,9 @@ static int run_beam(aok_ctx* ctx, uint32_t scene, Scene* sc, const SceneDev& sd,
     if (st) return st;
     if (optional && b.opt_read && cudaStreamWaitEvent((cudaStream_t)stream, b.opt_read, 0) != cudaSuccess)
         return AOK_E_CUDA;
-    uint32_t tag;
-    st = next_beam_tag(ctx, stream, &tag);
+    uint32_t epoch;
+    const uint32_t tag = next_beam_tag(ctx, &epoch);
+    st = beam_renew(buf, epoch, stream);
     if (st) return st;
     BeamBatch* P = b.P.get();
     beam_header(ctx, P, tag);
@@ -1149,7 +1159,7 @@ extern "C++" BeamUse aok::beam_use(const aok_ctx* ctx, int32_t W, int32_t H, voi
 
 extern "C++" int aok::beam_for_batch(aok_ctx* ctx, BatchParams* groups, uint32_t ngroups,
                                      std::vector<BeamBatch>& out, void* stream,
-                                     unsigned long long* const* view_bounds) {
+                                     unsigned long long* const* view_bounds, BoundBuf* arena) {
     out.clear();
     if (!ctx->beam_on) return AOK_OK;
     // entries of the views with a required pass, and with an optional one
@@ -1170,8 +1180,11 @@ extern "C++" int aok::beam_for_batch(aok_ctx* ctx, BatchParams* groups, uint32_t
         ctx->beam.no_room = true;
         return AOK_OK;
     }
-    uint32_t tag = 0;
-    if (!st) st = next_beam_tag(ctx, stream, &tag);
+    if (st) return st;
+    uint32_t epoch;
+    const uint32_t tag = next_beam_tag(ctx, &epoch);
+    if (!view_bounds) arena = &bb;
+    if (arena) st = beam_renew(*arena, epoch, stream);
     if (st) return st;
     const bool all = view_bounds || bb.cap >= req + opt;  // else the optional passes don't fit
     out.resize(ngroups);
@@ -1539,6 +1552,21 @@ int aok_beam_info(aok_ctx* ctx, int32_t* bounds, uint64_t n_bounds, uint32_t* le
     return AOK_OK;
 }
 
+int aok_beam_passes(aok_ctx* ctx, uint64_t* passes) {
+    if (!ctx || !passes) return AOK_E_INVALID;
+    std::lock_guard<std::mutex> lk(ctx->beam.mu);
+    *passes = ctx->beam.total;
+    return AOK_OK;
+}
+
+int aok_beam_tags_left(aok_ctx* ctx, uint32_t left) {
+    if (!ctx) return AOK_E_INVALID;
+    std::lock_guard<std::mutex> lk(ctx->beam.mu);
+    if (left > kBeamTags - ctx->beam.passes) return AOK_E_INVALID;
+    ctx->beam.passes = kBeamTags - left;
+    return AOK_OK;
+}
+
 int aok_set_checked(aok_ctx* ctx, int on) {
     if (!ctx || on < 0 || on > 1) return AOK_E_INVALID;
     ctx->checked = on;
@@ -1673,8 +1701,9 @@ static int pipe_render(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, doub
     if (st) return launch_failure(ctx);
     BeamRead rd{nullptr, 0};
     if (beam) {
-        uint32_t tag;
-        st = next_beam_tag(ctx, p.prep, &tag);
+        uint32_t epoch;
+        const uint32_t tag = next_beam_tag(ctx, &epoch);
+        st = beam_renew(sl.bounds, epoch, p.prep);
         if (st) return st;
         BeamBatch* P = p.P.get();
         beam_header(ctx, P, tag);

@@ -58,6 +58,7 @@ struct BoundBuf {
     unsigned long long* p = nullptr;
     size_t cap = 0;   // entries
     size_t hard = 0;  // entries that frames with a required pass have needed
+    uint32_t epoch = 0;  // of the tags in it (beam_renew)
 };
 
 // Device arena of aok_render_batch: per-view frame tables, work counters and
@@ -129,7 +130,9 @@ struct BeamState {
     // that read it: they may come on streams that nothing orders
     BoundBuf opt;
     cudaEvent_t opt_read = nullptr;
-    uint32_t passes = 0;                   // passes run (their tags count down)
+    uint32_t passes = 0;                   // passes run in this epoch (their tags count down)
+    std::atomic<uint32_t> epoch{0};        // times the tags have started over
+    uint64_t total = 0;                    // passes run
     // the last single-view pass: a scene, its selection, a camera
     bool valid = false;
     uint32_t scene = 0xFFFFFFFFu;
@@ -217,8 +220,10 @@ void free_alloc(Scene* sc, ChunkAlloc& a);
 // context's beam frame size; sets the views' bounds, in the batch arena or,
 // with view_bounds, in view_bounds[view] (nullptr: that view casts without).
 // Leaves `out` empty if no view takes the pass.
+// (arena: the buffer that some of view_bounds lie in; the others are cleared
+// for every pass.)
 int beam_for_batch(aok_ctx* ctx, BatchParams* groups, uint32_t ngroups, std::vector<BeamBatch>& out, void* stream,
-                   unsigned long long* const* view_bounds = nullptr);
+                   unsigned long long* const* view_bounds = nullptr, BoundBuf* arena = nullptr);
 // Whether a frame of W x H pixels on `stream` takes the beam pass in this
 // context, and whether it may also be cast without.
 inline bool beam_required(const aok_ctx* ctx, int32_t W, int32_t H) {

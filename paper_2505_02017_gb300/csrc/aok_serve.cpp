@@ -310,6 +310,7 @@ static unsigned long long* serve_bounds(aok_ctx* ctx, ServeState& S, uint32_t sl
     cudaMemsetAsync(p, 0xFF, cap * 8, st);  // no entry has a pass's tag
     a.p = (unsigned long long*)p;
     a.cap = cap;
+    a.epoch = ctx->beam.epoch;
     return a.p;
 }
 
@@ -500,7 +501,8 @@ static void serve_loop(aok_ctx* ctx) {
                     off += n;
                 }
             RelaxedCapture relaxed(true);
-            if (rc == AOK_OK) rc = beam_for_batch(ctx, S.params.data(), ngroups, beams, st, vb.data());
+            if (rc == AOK_OK) rc = beam_for_batch(ctx, S.params.data(), ngroups, beams, st, vb.data(),
+                                              arena ? &S.arena[slot] : nullptr);
         }
         if (rc == AOK_OK) {
             // the server's passes share one stream: a pass waits only for its

@@ -1,0 +1,91 @@
+"""State that beam passes share within a context: tags, buffers, the record of
+the last pass.  Frames of 1280 x 720 take the pass where it can run, frames of
+1600 x 1000 always; each equals the frame without the pass bit for bit."""
+from dataclasses import replace
+
+import pytest
+
+import scenegen as sg
+from worlds import MED64
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA device", allow_module_level=True)
+
+import paper_2505_02017_gb300 as aok  # noqa: E402
+
+OPTIONAL, REQUIRED = (1280, 720), (1600, 1000)
+
+
+class Setup:
+    """A context with its initial settings, a scene of it, and frames without the pass to compare with."""
+
+    def __init__(self, budget=0):
+        self.c = aok.Context(0, budget_bytes=budget)
+        self.world = sg.World(MED64)
+        self.sc = aok.Scene.from_world(self.c, self.world, threads=4)
+
+    def cam(self, k, size=OPTIONAL):
+        return sg.ground_camera(self.world, (4, 9, 12)[k % 3], *size, z_lo=4, z_hi=40)
+
+    def ref(self, cam, tau=1.5):
+        aok.set_beam(self.c, False)
+        out = aok.alloc_frame(cam.W, cam.H)
+        aok.render(self.c, self.sc, cam, tau, *out)
+        torch.cuda.synchronize()
+        aok.set_beam(self.c, True)
+        return out
+
+    def close(self):
+        self.sc.destroy()
+        self.c.close()
+
+
+def equal(x, y):
+    return torch.equal(x[0].cpu(), y[0].cpu()) and torch.equal(x[1].cpu().view(torch.int32), y[1].cpu().view(torch.int32))
+
+
+def draw(s, kind, cam, srv=None):
+    """The frame of `cam` through one of the calls that run the pass."""
+    if kind == "host":
+        out = (torch.empty((cam.H, cam.W, 4), dtype=torch.int32, pin_memory=True),
+               torch.empty((cam.H, cam.W), dtype=torch.float32, pin_memory=True))
+        aok.host_frame_wait(s.c, aok.render_host_async(s.c, s.sc, cam, 1.5, *out))
+        return out
+    if kind == "serve":
+        tk = srv.submit(s.sc, cam, 1.5)
+        st, f = srv.wait(tk, 20000)
+        assert st == aok.AOK_OK
+        out = tuple(x.clone() for x in srv.result(tk, f))
+        torch.cuda.synchronize()
+        assert srv.release(tk) == aok.AOK_OK
+        return out
+    out = aok.alloc_frame(cam.W, cam.H)
+    if kind == "batch":
+        aok.render_batch(s.c, [aok.make_view(s.sc, cam, 1.5, *out)])
+    elif kind == "tiles":
+        aok.render_tiles(s.c, s.sc, cam, 1.5, *out)
+    else:
+        aok.render(s.c, s.sc, cam, 1.5, *out)
+    torch.cuda.synchronize()
+    return out
+
+
+@pytest.mark.parametrize("size", [OPTIONAL, REQUIRED], ids=["optional", "required"])
+@pytest.mark.parametrize("kind", ["single", "tiles", "host", "batch", "serve"])
+def test_tags_start_over(kind, size):
+    """Bounds left by the last passes before the tags start over are not read as the new passes'."""
+    s = Setup()
+    cams = [s.cam(k, size) for k in range(3)]
+    refs = [s.ref(m) for m in cams]
+    srv = aok.Server(s.c, max_slots=4, max_batch=2, n_streams=1) if kind == "serve" else None
+    before = aok.beam_passes(s.c)
+    aok.beam_tags_left(s.c, 4)
+    for i in range(12):  # (host frames: each of the three slots on both sides)
+        assert equal(draw(s, kind, cams[i % 3], srv), refs[i % 3]), i
+    assert aok.beam_passes(s.c) == before + 12
+    if srv:
+        srv.stop()
+    s.close()

@@ -582,14 +582,17 @@ int aok_beam_selected(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, void*
  * scene and camera casts the selection with these bounds.  Arguments and
  * stream rules as for aok_select_chunks and aok_cast_selected. */
 int aok_select_beam(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, double lod_threshold_px, void* stream);
-/* The last beam pass of this context (synchronises the device): bounds
+/* The last beam pass of this context for a single view (aok_render, _counted,
+ * _tiles, _host, aok_cast_selected, aok_select_beam, aok_beam_selected; not
+ * those of batches, pipelined host frames and the server), as long as its
+ * buffers hold it (synchronises the device): bounds
  * (nullable, n_bounds >= tiles_x * tiles_y entries, row-major, numerator
  * units of 2^-12 LOD-0 voxels, INT32_MAX = no solid voxel reachable; 0
  * everywhere if the camera matrix has no usable inverse), level_counts
  * (nullable, 16 entries: nodes walked at each depth below the region roots,
  * depth 0 the selected regions; a queue holds 2^20 nodes per level, past
  * that parents stand in for their children) and tiles_xy (nullable, 2).
- * AOK_E_INVALID before the first beam pass or if n_bounds is too small. */
+ * AOK_E_INVALID before the first such pass or if n_bounds is too small. */
 int aok_beam_info(aok_ctx* ctx, int32_t* bounds, uint64_t n_bounds, uint32_t* level_counts, int32_t* tiles_xy);
 /* Beam passes this context has run: one for a single view's frame, one for
  * all views of a batch or of a server's batch. */

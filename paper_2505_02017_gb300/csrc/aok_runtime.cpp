@@ -934,7 +934,7 @@ static int ensure_beam_queues(aok_ctx* ctx, bool required) {
     std::lock_guard<std::mutex> lk(b.mu);
     b.q_hard |= required;
     if (b.qblock) return AOK_OK;
-    const size_t sq = (size_t)kBeamCap * 16, sc = 2 * kBeamLevels * 4;
+    const size_t sq = (size_t)kBeamCap * 16, sc = 3 * kBeamLevels * 4;
     void* block = nullptr;
     int st = required ? dev_alloc(ctx, &block, 2 * sq + sc) : dev_alloc_once(ctx, &block, 2 * sq + sc);
     if (st) return st;
@@ -942,6 +942,7 @@ static int ensure_beam_queues(aok_ctx* ctx, bool required) {
     b.q[1] = (uint4*)((char*)block + sq);
     b.cnt = (uint32_t*)((char*)block + 2 * sq);
     b.hist = b.cnt + kBeamLevels;
+    b.view_hist = b.hist + kBeamLevels;
     // (each pass leaves the queue counters at zero)
     if (!fill_now(ctx, b.cnt, 0, sc)) {
         dev_free(ctx, block, 2 * sq + sc);
@@ -1014,7 +1015,7 @@ extern "C++" bool aok::beam_reclaim(aok_ctx* ctx) {
     if (!beam_spare_bytes(ctx) || cudaDeviceSynchronize() != cudaSuccess) return false;
     b.no_room = true;
     const bool queues = b.qblock && !b.q_hard;
-    if (queues || b.opt.cap || b.bounds.cap > b.bounds.hard) b.valid = false;
+    if (queues || b.opt.cap || b.bounds.cap > b.bounds.hard) b.valid = b.ran = false;
     if (queues) {
         dev_free(ctx, b.qblock, b.qbytes);
         b.qblock = nullptr;
@@ -1095,6 +1096,7 @@ static int run_beam(aok_ctx* ctx, uint32_t scene, Scene* sc, const SceneDev& sd,
     BeamState& b = ctx->beam;
     BoundBuf& buf = optional ? b.opt : b.bounds;
     if (keep || b.read.bounds == buf.p) b.valid = false;  // (the buffer may move)
+    if (b.last.bounds == buf.p) b.ran = false;
     int st = beam_buffers(ctx, buf, cd, optional);
     if (st) return st;
     if (optional && b.opt_read && cudaStreamWaitEvent((cudaStream_t)stream, b.opt_read, 0) != cudaSuccess)
@@ -1105,6 +1107,7 @@ static int run_beam(aok_ctx* ctx, uint32_t scene, Scene* sc, const SceneDev& sd,
     if (st) return st;
     BeamBatch* P = b.P.get();
     beam_header(ctx, P, tag);
+    P->hist = b.view_hist;
     if (ck) P->ck = *ck;
     P->n_views = 0;
     P->n_regions = 0;
@@ -1123,15 +1126,18 @@ static int run_beam(aok_ctx* ctx, uint32_t scene, Scene* sc, const SceneDev& sd,
         if (st) return st;
     }
     st = aokk_beam_run(P, b.grid, stream);
-    if (st || !keep) return st;
+    if (st) return st;
+    b.last = *rd;
+    b.ran = true;
+    b.W = cd.W;
+    b.H = cd.H;
+    if (!keep) return AOK_OK;
     b.read = *rd;
     b.valid = true;
     b.scene = scene;
     b.gen = sc->select_gen;
     b.cam = cd;
     b.cam.sf = 0.0;  // the LOD threshold does not enter the bounds
-    b.W = cd.W;
-    b.H = cd.H;
     return AOK_OK;
 }
 
@@ -1517,7 +1523,8 @@ int aok_select_beam(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, double 
 int aok_beam_info(aok_ctx* ctx, int32_t* bounds, uint64_t n_bounds, uint32_t* level_counts, int32_t* tiles_xy) {
     if (!ctx) return AOK_E_INVALID;
     const BeamState& b = ctx->beam;
-    if (!b.valid) return AOK_E_INVALID;
+    std::lock_guard<std::recursive_mutex> lk(ctx->beam.use);
+    if (!b.ran) return AOK_E_INVALID;
     const uint32_t tx = (uint32_t)(b.W + kBeamTileW - 1) / kBeamTileW, ty = (uint32_t)(b.H + kBeamTileH - 1) / kBeamTileH;
     const uint64_t n = (uint64_t)tx * ty;
     if (bounds && n_bounds < n) return AOK_E_INVALID;
@@ -1528,10 +1535,10 @@ int aok_beam_info(aok_ctx* ctx, int32_t* bounds, uint64_t n_bounds, uint32_t* le
         // cells of the pyramid among entries of the last pass's tag, or 0
         // everywhere if that pass could not project
         std::vector<unsigned long long> e(beam_entries((uint32_t)b.W, (uint32_t)b.H));
-        if (b.read.bounds &&
-            cudaMemcpy(e.data(), b.read.bounds, e.size() * 8, cudaMemcpyDeviceToHost) != cudaSuccess)
+        if (b.last.bounds &&
+            cudaMemcpy(e.data(), b.last.bounds, e.size() * 8, cudaMemcpyDeviceToHost) != cudaSuccess)
             return cuda_status(ctx, cudaGetLastError());
-        const unsigned long long tag = (unsigned long long)b.read.tag << 32;
+        const unsigned long long tag = (unsigned long long)b.last.tag << 32;
         for (uint32_t y = 0; y < ty; y++)
             for (uint32_t x = 0; x < tx; x++) {
                 unsigned long long v = ~0ull;
@@ -1540,10 +1547,10 @@ int aok_beam_info(aok_ctx* ctx, int32_t* bounds, uint64_t n_bounds, uint32_t* le
                     v = std::min(v, e[beam_level_offset(tx, ty, L) + (size_t)(y >> L) * wl + (x >> L)]);
                 }
                 bounds[(size_t)y * tx + x] =
-                    !b.read.bounds ? 0 : ((v & 0xFFFFFFFF00000000ull) == tag ? (int32_t)(uint32_t)v : INT32_MAX);
+                    !b.last.bounds ? 0 : ((v & 0xFFFFFFFF00000000ull) == tag ? (int32_t)(uint32_t)v : INT32_MAX);
             }
     }
-    if (level_counts && cudaMemcpy(level_counts, b.hist, kBeamLevels * 4, cudaMemcpyDeviceToHost) != cudaSuccess)
+    if (level_counts && cudaMemcpy(level_counts, b.view_hist, kBeamLevels * 4, cudaMemcpyDeviceToHost) != cudaSuccess)
         return cuda_status(ctx, cudaGetLastError());
     if (tiles_xy) {
         tiles_xy[0] = (int32_t)tx;

@@ -121,8 +121,9 @@ struct BeamState {
     bool q_hard = false;   // a frame that has to take the pass has used the queues
     std::atomic<bool> no_room{false};  // memory ran short: frames that need not take the pass no longer do
     uint4* q[2] = {nullptr, nullptr};
-    uint32_t* cnt = nullptr;   // [kBeamLevels] queue counts, then [kBeamLevels] walk histogram
-    uint32_t* hist = nullptr;
+    uint32_t* cnt = nullptr;   // [kBeamLevels] queue counts, then two walk histograms [kBeamLevels]:
+    uint32_t* hist = nullptr;  // of the last batch or host frame, and
+    uint32_t* view_hist = nullptr;  // of the last single view's pass
     unsigned grid = 0;         // blocks of the cooperative launch
     std::unique_ptr<BeamBatch> P;  // host parameter block (~26 KB)
     BoundBuf bounds;                       // single-view pyramid
@@ -133,13 +134,16 @@ struct BeamState {
     uint32_t passes = 0;                   // passes run in this epoch (their tags count down)
     std::atomic<uint32_t> epoch{0};        // times the tags have started over
     uint64_t total = 0;                    // passes run
-    // the last single-view pass: a scene, its selection, a camera
+    // the last single-view pass, for aok_beam_info
+    bool ran = false;
+    BeamRead last{nullptr, 0};
+    int32_t W = 0, H = 0;
+    // the last one kept for the cast of its selection: a scene, its selection, a camera
     bool valid = false;
     uint32_t scene = 0xFFFFFFFFu;
     uint64_t gen = 0;
     CamDev cam{};
     BeamRead read{nullptr, 0};
-    int32_t W = 0, H = 0;
 };
 
 // The reachable nodes of a chunk blob by depth, found while it is validated

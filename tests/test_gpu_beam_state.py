@@ -89,3 +89,29 @@ def test_tags_start_over(kind, size):
     if srv:
         srv.stop()
     s.close()
+
+
+def test_info_is_of_the_last_view():
+    """aok_beam_info reports the last single view's pass, its bounds and its level counts together, also for
+    frames that need not take the pass; a batch in between changes neither."""
+    s = Setup()
+    with pytest.raises(aok.AokError):
+        aok.beam_info(s.c)
+    seen = {}
+    for size in (OPTIONAL, REQUIRED, OPTIONAL):
+        cam = s.cam(0, size)
+        draw(s, "single", cam)
+        b, levels = aok.beam_info(s.c)
+        assert b.shape == ((cam.H + 3) // 4, (cam.W + 7) // 8) and levels[0] > 0
+        draw(s, "batch", s.cam(1, REQUIRED))
+        assert (aok.beam_info(s.c)[0] == b).all() and aok.beam_info(s.c)[1] == levels
+        # the same pass by itself (kept, in the buffer of the large frames)
+        aok.beam_selected(s.c, s.sc, cam)
+        b2, levels2 = aok.beam_info(s.c)
+        assert (b2 == b).all() and levels2 == levels
+        assert seen.setdefault(size, levels) == levels
+    assert seen[OPTIONAL] != seen[REQUIRED]
+    aok.beam_selected(s.c, s.sc, s.cam(0, REQUIRED))
+    draw(s, "single", s.cam(2))
+    assert aok.beam_info(s.c)[0].shape == (180, 160)
+    s.close()

@@ -1144,10 +1144,25 @@ static int run_beam(aok_ctx* ctx, uint32_t scene, Scene* sc, const SceneDev& sd,
 // After a cast that read an optional pass's pyramid: the next optional pass,
 // on whatever stream, waits for it.
 static int beam_was_read(aok_ctx* ctx, void* stream) {
-    cudaEvent_t& ev = ctx->beam.opt_read;
-    cudaError_t e = ev ? cudaSuccess : cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventRecord(ev, (cudaStream_t)stream);
+    BeamState& b = ctx->beam;
+    cudaError_t e = b.opt_read ? cudaSuccess : cudaEventCreateWithFlags(&b.opt_read, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaStreamGetId((cudaStream_t)stream, &b.opt_stream);
+    if (e == cudaSuccess) e = cudaEventRecord(b.opt_read, (cudaStream_t)stream);
     return cuda_status(ctx, e);
+}
+
+// Whether that record, made anew after a cast on `stream`, still stands for
+// every cast that reads the pyramid: the last one is over, or comes before on
+// the same stream.
+static bool beam_read_alone(aok_ctx* ctx, void* stream) {
+    const BeamState& b = ctx->beam;
+    if (!b.opt_read) return true;
+    unsigned long long id = 0;
+    if (cudaStreamGetId((cudaStream_t)stream, &id) == cudaSuccess && id == b.opt_stream) return true;
+    RelaxedCapture rc(true);  // (a query would end another stream's capture)
+    if (cudaEventQuery(b.opt_read) == cudaSuccess) return true;
+    cudaGetLastError();  // "not ready" is no error of the next launch
+    return false;
 }
 
 extern "C++" BeamUse aok::beam_use(const aok_ctx* ctx, int32_t W, int32_t H, void* stream) {
@@ -1246,8 +1261,11 @@ static int cast_single(aok_ctx* ctx, uint32_t scene, Scene* sc, const SceneDev& 
     if (counts && use == kBeamOptional) use = kBeamNone;  // its visits would depend on whether the pass could run
     if (use != kBeamNone) {
         const bool optional = use == kBeamOptional;
-        if (selected && beam_fresh(ctx, scene, sc, cd)) rd = ctx->beam.read;
-        else st = run_beam(ctx, scene, sc, sd, cd, stream, &rd, !selected, ckp, optional, !optional);
+        if (selected && beam_fresh(ctx, scene, sc, cd)) {
+            rd = ctx->beam.read;
+            // a second cast of one selection, beside the first: without the bounds
+            if (optional && rd.bounds == ctx->beam.opt.p && !beam_read_alone(ctx, stream)) st = AOK_E_OOM;
+        } else st = run_beam(ctx, scene, sc, sd, cd, stream, &rd, !selected, ckp, optional, !optional);
         if (st == AOK_OK) {
             selected = true;
             beam = &rd;

@@ -131,6 +131,7 @@ struct BeamState {
     // that read it: they may come on streams that nothing orders
     BoundBuf opt;
     cudaEvent_t opt_read = nullptr;
+    unsigned long long opt_stream = 0;  // that cast's stream
     uint32_t passes = 0;                   // passes run in this epoch (their tags count down)
     std::atomic<uint32_t> epoch{0};        // times the tags have started over
     uint64_t total = 0;                    // passes run

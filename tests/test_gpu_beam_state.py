@@ -115,3 +115,26 @@ def test_info_is_of_the_last_view():
     draw(s, "single", s.cam(2))
     assert aok.beam_info(s.c)[0].shape == (180, 160)
     s.close()
+
+
+def test_two_casts_of_one_selection():
+    """Two casts of one selection on two streams, the first held back, and then another frame's pass: it must
+    not replace the bounds before both have read them."""
+    s = Setup()
+    cams = [s.cam(k) for k in range(3)]
+    refs = [s.ref(m) for m in cams]
+    outs = [aok.alloc_frame(m.W, m.H) for m in cams]
+    s1, s2, s3 = (torch.cuda.Stream() for _ in range(3))
+    sc3 = aok.Scene.from_world(s.c, s.world, threads=4)  # (its own chunk table)
+    aok.select_beam(s.c, s.sc, cams[0], 1.5)
+    assert aok.beam_info(s.c)[1][0] > 0
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s1):
+        torch.cuda._sleep(40_000_000)  # about 20 ms
+    aok.cast_selected(s.c, s.sc, cams[0], *outs[0], stream=s1)
+    aok.cast_selected(s.c, s.sc, cams[0], *outs[1], stream=s2)
+    aok.render(s.c, sc3, cams[2], 1.5, *outs[2], stream=s3)
+    torch.cuda.synchronize()
+    assert equal(outs[0], refs[0]) and equal(outs[1], refs[0]) and equal(outs[2], refs[2])
+    sc3.destroy()
+    s.close()

@@ -537,8 +537,9 @@ int aok_render_noalloc(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, doub
  * distance.  Output records are identical with the pass on or off.  Buffers
  * (about 11 B per 8 x 4 pixel tile, grown to the largest frame or batch seen,
  * and two 16 MiB node queues) are charged to the budget when first needed.
- * The render server runs it for its batches too (per-request pyramids, or
- * one arena per stream for the frames below 1.5 M pixels).
+ * The render server runs it for its batches too (per-request pyramids, or,
+ * for the frames below 1.5 M pixels, an arena per stream of 2 to 16 MB beside
+ * the budget; frames beyond its room are cast without).
  * aok_render_tiles uses the same bounds.  Not used by the persistent
  * single-view and batch kernels or
  * aok_render_noalloc; with checked casting it runs with

@@ -1004,7 +1004,7 @@ static std::array<BoundBuf*, 3 + kHostSlots> bound_bufs(aok_ctx* ctx) {
 extern "C++" size_t aok::beam_spare_bytes(aok_ctx* ctx) {
     const BeamState& b = ctx->beam;
     std::lock_guard<std::recursive_mutex> lk(ctx->beam.use);
-    size_t n = serve_beam_bytes(ctx) + (b.qblock && !b.q_hard ? b.qbytes : 0);
+    size_t n = b.qblock && !b.q_hard ? b.qbytes : 0;
     for (const BoundBuf* s : bound_bufs(ctx)) n += s->cap > s->hard ? (s->cap - s->hard) * 8 : 0;
     return n;
 }
@@ -1027,7 +1027,6 @@ extern "C++" bool aok::beam_reclaim(aok_ctx* ctx) {
             s->cap = 0;
             if (s->hard) alloc_bounds(ctx, *s, s->hard, false);  // (else at the next pass that needs it)
         }
-    serve_beam_release(ctx);
     return true;
 }
 

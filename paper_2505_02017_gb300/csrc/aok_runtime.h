@@ -240,9 +240,6 @@ BeamUse beam_use(const aok_ctx* ctx, int32_t W, int32_t H, void* stream);
 // were some); the context runs no optional pass any more.
 bool beam_reclaim(aok_ctx* ctx);
 size_t beam_spare_bytes(aok_ctx* ctx);  // what it would free
-// ... the serving loop's share of them.
-size_t serve_beam_bytes(aok_ctx* ctx);
-void serve_beam_release(aok_ctx* ctx);
 // Lets this thread allocate while another one captures a stream in the global
 // capture mode (whose capture an allocation here would end).
 struct RelaxedCapture {

@@ -283,56 +283,35 @@ static size_t request_bytes(const aok_ctx* ctx, const Scene* sc, const aok_camer
     return b;
 }
 
-// Room in a stream's arena for the pyramids of the requests that need not take
-// the pass (nullptr: none, they are cast without).  The stream's batches use
-// it one after another; it is replaced in stream order.
-static unsigned long long* serve_bounds(aok_ctx* ctx, ServeState& S, uint32_t slot, size_t need) {
+// A stream's arena: pyramids of the requests that need not take the pass, for
+// its batches one after another.  It comes from the request pool and, like the
+// memory the pool keeps, is not charged to the budget: requests and scenes
+// find the room that they would find without the pass.
+constexpr size_t kArenaFirst = (size_t)1 << 18, kArenaMost = (size_t)1 << 21;  // entries (8 bytes)
+
+// The stream's arena with room for `need` entries or, beyond kArenaMost or
+// where memory is short, for fewer.  It is replaced in stream order.
+static BoundBuf& serve_arena(aok_ctx* ctx, ServeState& S, uint32_t slot, size_t need) {
     BoundBuf& a = S.arena[slot];
-    if (need <= a.cap) return a.p;
+    need = std::min(need, kArenaMost);
+    if (need <= a.cap) return a;
     const cudaStream_t st = S.streams[slot];
-    if (a.p) {
-        cudaFreeAsync(a.p, st);
-        uncharge(ctx, a.cap * 8);
-        a = BoundBuf();
-    }
-    const size_t cap = need + need / 2;
+    const size_t cap = std::min(std::max(need + need / 2, kArenaFirst), kArenaMost);
     void* p = nullptr;
-    if (charge(ctx, cap * 8) != AOK_OK) {
-        ctx->beam.no_room = true;
-        return nullptr;
-    }
     if (cudaMallocFromPoolAsync(&p, cap * 8, S.pool, st) != cudaSuccess) {
         cudaGetLastError();
-        uncharge(ctx, cap * 8);
-        ctx->beam.no_room = true;
-        return nullptr;
+        return a;
     }
-    cudaMemsetAsync(p, 0xFF, cap * 8, st);  // no entry has a pass's tag
+    if (cudaMemsetAsync(p, 0xFF, cap * 8, st) != cudaSuccess) {  // no entry has a pass's tag
+        cudaGetLastError();
+        cudaFreeAsync(p, st);
+        return a;
+    }
+    if (a.p) cudaFreeAsync(a.p, st);
     a.p = (unsigned long long*)p;
     a.cap = cap;
     a.epoch = ctx->beam.epoch;
-    return a.p;
-}
-
-size_t serve_beam_bytes(aok_ctx* ctx) {
-    size_t n = 0;
-    if (ctx->serve)
-        for (const BoundBuf& a : ctx->serve->arena) n += a.cap * 8;
-    return n;
-}
-
-// (the device is idle)
-void serve_beam_release(aok_ctx* ctx) {
-    if (!ctx->serve) return;
-    ServeState& S = *ctx->serve;
-    for (size_t i = 0; i < S.arena.size(); i++)
-        if (S.arena[i].p) {
-            cudaFreeAsync(S.arena[i].p, S.streams[i]);
-            cudaStreamSynchronize(S.streams[i]);
-            uncharge(ctx, S.arena[i].cap * 8);
-            S.arena[i] = BoundBuf();
-        }
-    cudaMemPoolTrimTo(S.pool, 0);
+    return a;
 }
 
 static void free_ticket_memory(aok_ctx* ctx, Ticket& t, cudaStream_t s) {
@@ -494,15 +473,14 @@ static void serve_loop(aok_ctx* ctx) {
                            : (size_t)beam_entries((uint32_t)d.cam.W, (uint32_t)d.cam.H);
             };
             for (size_t i = 0; i < batch.size(); i++) need += entries(i);
-            unsigned long long* arena = need ? serve_bounds(ctx, S, slot, need) : nullptr;
+            BoundBuf* arena = need ? &serve_arena(ctx, S, slot, need) : nullptr;
             for (size_t i = 0; i < batch.size() && arena; i++)
-                if (const size_t n = entries(i)) {
-                    vb[i] = arena + off;
+                if (const size_t n = entries(i); n && off + n <= arena->cap) {  // (the others are cast without)
+                    vb[i] = arena->p + off;
                     off += n;
                 }
             RelaxedCapture relaxed(true);
-            if (rc == AOK_OK) rc = beam_for_batch(ctx, S.params.data(), ngroups, beams, st, vb.data(),
-                                              arena ? &S.arena[slot] : nullptr);
+            if (rc == AOK_OK) rc = beam_for_batch(ctx, S.params.data(), ngroups, beams, st, vb.data(), arena);
         }
         if (rc == AOK_OK) {
             // the server's passes share one stream: a pass waits only for its
@@ -685,6 +663,7 @@ int aok_serve_start(aok_ctx* ctx, uint32_t max_slots, uint32_t max_batch, uint32
     }
     uint64_t keep = (uint64_t)ctx->budget;
     cudaMemPoolSetAttribute(S->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    for (uint32_t i = 0; i < n_streams; i++) serve_arena(ctx, *S, i, kArenaFirst);  // not in the first request's time
     cudaDeviceSynchronize();
     ctx->serve = S;
     S->loop = std::thread(serve_loop, ctx);
@@ -712,11 +691,8 @@ int aok_serve_stop(aok_ctx* ctx) {
     cudaSetDevice(ctx->device);
     for (auto& kv : S->tickets) free_ticket_memory(ctx, kv.second, S->streams[0]);
     for (cudaStream_t s : S->streams) cudaStreamSynchronize(s);
-    {
-        std::lock_guard<std::recursive_mutex> lk(ctx->beam.use);
-        serve_beam_release(ctx);
-        ctx->serve = nullptr;
-    }
+    for (size_t i = 0; i < S->arena.size(); i++)
+        if (S->arena[i].p) cudaFreeAsync(S->arena[i].p, S->streams[i]);
     if (S->beam_stream) {
         cudaStreamSynchronize(S->beam_stream);
         cudaStreamDestroy(S->beam_stream);

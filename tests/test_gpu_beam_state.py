@@ -138,3 +138,27 @@ def test_two_casts_of_one_selection():
     assert equal(outs[0], refs[0]) and equal(outs[1], refs[0]) and equal(outs[2], refs[2])
     sc3.destroy()
     s.close()
+
+
+@pytest.mark.parametrize("room_kb", range(0, 1200, 200))
+def test_server_batch_of_both_kinds_in_a_tight_budget(room_kb):
+    """The queues of the large request's pass are the last to fit: what the small request's pass uses must stay."""
+    s = Setup()
+    used = s.c.memory()[0]
+    s.close()
+    need = sum(w * h * 20 + ((w * h) >> 2) for w, h in (OPTIONAL, REQUIRED)) + (33 << 20)
+    s = Setup(used + need + (room_kb << 10))
+    cams = [s.cam(0), s.cam(1, REQUIRED), s.cam(2)]
+    refs = [s.ref(m) for m in cams]
+    srv = aok.Server(s.c, max_slots=8, max_batch=4, n_streams=1)
+    for k in ((0, 1), (1, 2), (2, 1), (0, 1)):
+        held = [srv.submit(s.sc, cams[i], 1.5) for i in k]
+        for i, tk in zip(k, held):
+            st, f = srv.wait(tk, 20000)
+            assert st == aok.AOK_OK and equal(srv.result(tk, f), refs[i])
+        torch.cuda.synchronize()
+        for tk in held:
+            assert srv.release(tk) == aok.AOK_OK
+    assert aok.beam_passes(s.c) > 0
+    srv.stop()
+    s.close()

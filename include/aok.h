@@ -56,7 +56,8 @@ typedef struct aok_ctx aok_ctx;
 /* Create a context on CUDA device `device`.  All device memory the library
  * allocates (scene pools, per-frame tables, serving slots) is charged
  * against `hbm_budget_bytes` (0 = 90% of the device's free memory at
- * creation).  Returns AOK_E_INVALID for a bad device, AOK_E_CUDA on
+ * creation), but for a fixed block of 14 MB per context and 2 to 16 MB per
+ * serving stream (aok_set_beam).  Returns AOK_E_INVALID for a bad device, AOK_E_CUDA on
  * initialisation failure. */
 int aok_create(aok_ctx** out, int device, size_t hbm_budget_bytes);
 /* Wait for the context's work, free every allocation, stop serving. */
@@ -526,7 +527,8 @@ int aok_render_noalloc(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, doub
  * aok_render_host(_async), aok_cast_selected, aok_render_batch (grid
  * launch) and the render server of this context first compute, for every 8 x 4 pixel tile of each
  * frame of at least 1.5 M pixels (aok_beam_tune), and of smaller ones from
- * 0.8 M pixels where the pass can run (not aok_render_counted's), a lower bound on the
+ * 0.8 M pixels where the pass can run (an optional pass; not for
+ * aok_render_counted), a lower bound on the
  * L-infinity distance from the camera origin of every solid voxel of the
  * frame's LOD-cut scene that the tile's rays can meet: a level-by-level walk
  * of the selected DAGs (all views of a batch in one launch), refining a node
@@ -536,7 +538,8 @@ int aok_render_noalloc(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, doub
  * last integer plane of its dominant axis that the ray crosses before that
  * distance.  Output records are identical with the pass on or off.  Buffers
  * (about 11 B per 8 x 4 pixel tile, grown to the largest frame or batch seen,
- * and two 16 MiB node queues) are charged to the budget when first needed.
+ * and two 16 MiB node queues) are charged to the budget when first needed;
+ * an optional pass uses a block that the context holds from its creation.
  * The render server runs it for its batches too (per-request pyramids, or,
  * for the frames below 1.5 M pixels, an arena per stream of 2 to 16 MB beside
  * the budget; frames beyond its room are cast without).
@@ -548,10 +551,9 @@ int aok_render_noalloc(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, doub
  * of one context on
  * different streams must be ordered (an event or a synchronisation between
  * them).  Frames from 0.8 to 1.5 M pixels cast without the pass on a stream
- * that is being captured and where its buffers don't fit the budget; when an
- * allocation of this context finds no room, buffers that only such frames
- * have used are given back, and the context casts them without the pass until
- * aok_set_beam or aok_beam_tune is called.
+ * that is being captured and where the block has no room (a shape of very few
+ * rows or columns, more than about 16 such views in a batch); they can be
+ * rendered on any streams.
  * The passes of all contexts of a process run one after another on a
  * device (each waits for the previous one's launch to finish). */
 int aok_set_beam(aok_ctx* ctx, int on);

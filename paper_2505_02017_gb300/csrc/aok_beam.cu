@@ -552,7 +552,9 @@ int aokk_beam_order(void* stream, int record) {
     return aokk_status(e);
 }
 
-int aokk_beam_run(const BeamBatch* P, unsigned grid, void* stream, int beside) {
+extern "C++" {
+template <class PB>
+static int launch_pass(const PB* P, unsigned grid, void* stream) {
     const cudaStream_t st = (cudaStream_t)stream;
     if (P->n_views == 0) return AOK_OK;
     int dev = -1;
@@ -562,19 +564,24 @@ int aokk_beam_run(const BeamBatch* P, unsigned grid, void* stream, int beside) {
     std::lock_guard<std::mutex> lk(g_beam_mu);
     if (!g_beam_done[dev]) e = cudaEventCreateWithFlags(&g_beam_done[dev], cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(st, g_beam_done[dev], 0);
-    const unsigned g = beside && P->n_regions <= kWideWalkRegions ? (grid + kBeamBlocksPerSM - 1) / kBeamBlocksPerSM : grid;
-    if (e == cudaSuccess && P->n_views == 1) {
-        BeamParams<1> one;
-        static_cast<BeamHead&>(one) = *P;
-        one.v[0] = P->v[0];
-        void* args[] = {&one};
-        e = cudaLaunchCooperativeKernel((const void*)beam_kernel<BeamParams<1>>, g, kBeamThreads, args, 0, st);
-    } else if (e == cudaSuccess) {
-        void* args[] = {(void*)P};
-        e = cudaLaunchCooperativeKernel((const void*)beam_kernel<BeamBatch>, g, kBeamThreads, args, 0, st);
-    }
+    void* args[] = {(void*)P};
+    if (e == cudaSuccess) e = cudaLaunchCooperativeKernel((const void*)beam_kernel<PB>, grid, kBeamThreads, args, 0, st);
     if (e == cudaSuccess) e = cudaEventRecord(g_beam_done[dev], st);
     return aokk_status(e);
+}
+}  // extern "C++"
+
+int aokk_beam_run_view(const BeamParams<1>* P, unsigned grid, void* stream, int beside) {
+    return launch_pass(P, beside && P->n_regions <= kWideWalkRegions ? (grid + kBeamBlocksPerSM - 1) / kBeamBlocksPerSM : grid,
+                       stream);
+}
+
+int aokk_beam_run(const BeamBatch* P, unsigned grid, void* stream) {
+    if (P->n_views != 1) return launch_pass(P, grid, stream);
+    BeamParams<1> one;
+    static_cast<BeamHead&>(one) = *P;
+    one.v[0] = P->v[0];
+    return launch_pass(&one, grid, stream);
 }
 
 }  // extern "C"

@@ -241,12 +241,13 @@ int aokk_cast(const aok::SceneDev* s, const aok::CamDev* c, const aok::ChunkRef*
               uint32_t* counts, void* stream, const aok::CheckDev* ck, const aok::BeamRead* beam = nullptr);
 // Beam pass (aok_beam.cu).  aokk_beam_view fills a view's projection (false:
 // the camera matrix has no usable inverse; leave the view out, it casts
-// without bounds); aokk_beam_run launches the pass
-// (beside: with one block per SM, for a pass that starts beside the cast of
-// the frame before, as in the pipelined host frames).
+// without bounds); aokk_beam_run launches a pass, aokk_beam_run_view one of a
+// single view (beside: with one block per SM, for a pass that starts beside
+// the cast of the frame before, as in the pipelined host frames).
 bool aokk_beam_view(const aok::SceneDev* S, const aok::CamDev* C, const aok::ChunkRef* frame,
                     unsigned long long* bounds, aok::BeamView* out);
-int aokk_beam_run(const aok::BeamBatch* P, unsigned grid, void* stream, int beside = 0);
+int aokk_beam_run(const aok::BeamBatch* P, unsigned grid, void* stream);
+int aokk_beam_run_view(const aok::BeamParams<1>* P, unsigned grid, void* stream, int beside);
 // The pass as a graph's kernel node and the per-device pass
 // order around a graph launch (record = 0: wait for the previous pass before;
 // 1: mark the end of the launch as the point the next pass waits for).

@@ -42,7 +42,7 @@ void uncharge(aok_ctx* ctx, size_t bytes) {
     ctx->used -= std::min(ctx->used, bytes);
 }
 
-static int dev_alloc_once(aok_ctx* ctx, void** p, size_t bytes) {
+int dev_alloc(aok_ctx* ctx, void** p, size_t bytes) {
     *p = nullptr;
     if (bytes == 0) return AOK_OK;
     int st = charge(ctx, bytes);
@@ -55,12 +55,6 @@ static int dev_alloc_once(aok_ctx* ctx, void** p, size_t bytes) {
         return e == cudaErrorMemoryAllocation ? AOK_E_OOM : cuda_status(ctx, e);
     }
     return AOK_OK;
-}
-
-int dev_alloc(aok_ctx* ctx, void** p, size_t bytes) {
-    int st = dev_alloc_once(ctx, p, bytes);
-    if (st == AOK_E_OOM && beam_reclaim(ctx)) st = dev_alloc_once(ctx, p, bytes);
-    return st;
 }
 
 void dev_free(aok_ctx* ctx, void* p, size_t bytes) {
@@ -368,6 +362,7 @@ static void layout_blob(const aok_chunk_blob* b, int res, uint32_t node_base, ui
 }
 
 static void pipe_release(aok_ctx* ctx);
+static void beam_reserve(aok_ctx* ctx);
 
 // ---------------------------------------------------------------------------
 // C ABI
@@ -417,6 +412,8 @@ int aok_create(aok_ctx** out, int device, size_t budget) {
         return AOK_E_CUDA;
     }
     ctx->sm_count = aokk_sm_count(device);
+    ctx->beam.grid = aokk_beam_grid(ctx->sm_count);
+    beam_reserve(ctx);
     *out = ctx;
     return AOK_OK;
 }
@@ -437,7 +434,7 @@ void aok_destroy(aok_ctx* ctx) {
     dev_free(ctx, ctx->tiles.block, ctx->tiles.bytes);
     dev_free(ctx, ctx->beam.qblock, ctx->beam.qbytes);
     dev_free(ctx, ctx->beam.bounds.p, ctx->beam.bounds.cap * 8);
-    dev_free(ctx, ctx->beam.opt.p, ctx->beam.opt.cap * 8);
+    if (ctx->beam.opt_block) cudaFree(ctx->beam.opt_block);
     if (ctx->beam.opt_read) cudaEventDestroy(ctx->beam.opt_read);
     pipe_release(ctx);
     if (ctx->pipe.prep) cudaStreamDestroy(ctx->pipe.prep);
@@ -451,9 +448,8 @@ void aok_destroy(aok_ctx* ctx) {
 
 int aok_memory(aok_ctx* ctx, size_t* used, size_t* budget) {
     if (!ctx) return AOK_E_INVALID;
-    const size_t spare = beam_spare_bytes(ctx);  // given back to whatever needs them
     std::lock_guard<std::mutex> g(ctx->mem_mu);
-    if (used) *used = ctx->used - std::min(ctx->used, spare);
+    if (used) *used = ctx->used;
     if (budget) *budget = ctx->budget;
     return AOK_OK;
 }
@@ -926,39 +922,42 @@ static bool fill_now(aok_ctx* ctx, void* p, int byte, size_t bytes) {
            cudaStreamSynchronize(ctx->copy_stream) == cudaSuccess;
 }
 
-// The walk's queues, counters and launch grid (shared by single-view and
-// batch passes, which run in stream order).  required: a frame that has to
-// take the pass uses them.
-static int ensure_beam_queues(aok_ctx* ctx, bool required) {
+// The queues and counters of the passes that frames have to take (shared by
+// single-view and batch passes, which run in stream order).
+static int ensure_beam_queues(aok_ctx* ctx) {
     BeamState& b = ctx->beam;
     std::lock_guard<std::mutex> lk(b.mu);
-    b.q_hard |= required;
     if (b.qblock) return AOK_OK;
-    const size_t sq = (size_t)kBeamCap * 16, sc = 3 * kBeamLevels * 4;
+    if (!b.grid) return AOK_E_CUDA;
+    const size_t sq = (size_t)kBeamCap * 16, sc = 2 * kBeamLevels * 4;
     void* block = nullptr;
-    int st = required ? dev_alloc(ctx, &block, 2 * sq + sc) : dev_alloc_once(ctx, &block, 2 * sq + sc);
+    int st = dev_alloc(ctx, &block, 2 * sq + sc);
     if (st) return st;
-    b.q[0] = (uint4*)block;
-    b.q[1] = (uint4*)((char*)block + sq);
-    b.cnt = (uint32_t*)((char*)block + 2 * sq);
-    b.hist = b.cnt + kBeamLevels;
-    b.view_hist = b.hist + kBeamLevels;
+    uint32_t* cnt = (uint32_t*)((char*)block + 2 * sq);
     // (each pass leaves the queue counters at zero)
-    if (!fill_now(ctx, b.cnt, 0, sc)) {
+    if (!fill_now(ctx, cnt, 0, sc)) {
         dev_free(ctx, block, 2 * sq + sc);
         return cuda_status(ctx, cudaGetLastError());
     }
+    b.q = BeamQueues{{(uint4*)block, (uint4*)((char*)block + sq)}, cnt, cnt + kBeamLevels, kBeamCap};
+    if (!b.view_hist) b.view_hist = b.q.hist;
     b.qblock = block;
     b.qbytes = 2 * sq + sc;
-    b.grid = aokk_beam_grid(ctx->sm_count);
-    if (!b.grid) return AOK_E_CUDA;
-    if (!b.P) b.P.reset(new BeamBatch);
     return AOK_OK;
 }
 
-static int alloc_bounds(aok_ctx* ctx, BoundBuf& b, size_t need, bool required) {
+// Room for `need` entries, all without a pass tag when allocated (entries
+// carry their pass's tag, so a change of layout needs no clearing).
+static int ensure_bounds(aok_ctx* ctx, BoundBuf& b, size_t need) {
+    if (need <= b.cap) return AOK_OK;
+    if (b.p) {
+        cudaDeviceSynchronize();
+        dev_free(ctx, b.p, b.cap * 8);
+        b.p = nullptr;
+        b.cap = 0;
+    }
     void* p = nullptr;
-    int st = required ? dev_alloc(ctx, &p, need * 8) : dev_alloc_once(ctx, &p, need * 8);
+    int st = dev_alloc(ctx, &p, need * 8);
     if (st) return st;
     if (!fill_now(ctx, p, 0xFF, need * 8)) {
         dev_free(ctx, p, need * 8);
@@ -970,65 +969,44 @@ static int alloc_bounds(aok_ctx* ctx, BoundBuf& b, size_t need, bool required) {
     return AOK_OK;
 }
 
-// Room for `need` entries, `required` of them for passes that have to run;
-// all are without a pass tag when allocated (entries carry their pass's tag,
-// so a change of layout needs no clearing).  Where only the required ones
-// fit, b.cap stays below `need`.
-static int ensure_bounds(aok_ctx* ctx, BoundBuf& b, size_t need, size_t required) {
-    b.hard = std::max(b.hard, required);
-    if (need <= b.cap) return AOK_OK;
-    if (need > required && ctx->beam.no_room) {
-        if (required <= b.cap) return required ? AOK_OK : AOK_E_OOM;
-        need = required;
-    }
-    if (b.p) {
-        cudaDeviceSynchronize();
-        dev_free(ctx, b.p, b.cap * 8);
-        b.p = nullptr;
-        b.cap = 0;
-    }
-    if (need <= required) return alloc_bounds(ctx, b, need, true);
-    int st = alloc_bounds(ctx, b, need, false);
-    if (st != AOK_E_OOM) return st;
-    ctx->beam.no_room = true;
-    if (b.hard) st = alloc_bounds(ctx, b, b.hard, true);
-    return required || st != AOK_OK ? st : AOK_E_OOM;
-}
-
-static std::array<BoundBuf*, 3 + kHostSlots> bound_bufs(aok_ctx* ctx) {
-    std::array<BoundBuf*, 3 + kHostSlots> r{&ctx->beam.bounds, &ctx->beam.opt, &ctx->batch.beam_bounds};
-    for (int i = 0; i < kHostSlots; i++) r[3 + i] = &ctx->pipe.slot[i].bounds;
-    return r;
-}
-
-extern "C++" size_t aok::beam_spare_bytes(aok_ctx* ctx) {
-    const BeamState& b = ctx->beam;
-    std::lock_guard<std::recursive_mutex> lk(ctx->beam.use);
-    size_t n = b.qblock && !b.q_hard ? b.qbytes : 0;
-    for (const BoundBuf* s : bound_bufs(ctx)) n += s->cap > s->hard ? (s->cap - s->hard) * 8 : 0;
-    return n;
-}
-
-extern "C++" bool aok::beam_reclaim(aok_ctx* ctx) {
+// The block of the passes that frames need not take.  A level of a 1080p
+// frame's walk queues up to 6,608 nodes, so 2^17 serve the views of a batch as
+// well (a full queue costs tighter bounds, no more); a pyramid of 2^16 entries
+// serves a frame of 1.5 M pixels (62,600 at usual shapes), 2^20 sixteen of
+// them in a batch.
+static constexpr uint32_t kOptQueue = 1u << 17;
+static constexpr size_t kOptView = (size_t)1 << 16, kOptBatch = (size_t)1 << 20;
+extern "C++" {
+static void beam_reserve(aok_ctx* ctx) {
     BeamState& b = ctx->beam;
-    std::lock_guard<std::recursive_mutex> lk(b.use);
-    if (!beam_spare_bytes(ctx) || cudaDeviceSynchronize() != cudaSuccess) return false;
-    b.no_room = true;
-    const bool queues = b.qblock && !b.q_hard;
-    if (queues || b.opt.cap || b.bounds.cap > b.bounds.hard) b.valid = b.ran = false;
-    if (queues) {
-        dev_free(ctx, b.qblock, b.qbytes);
-        b.qblock = nullptr;
+    const size_t sq = (size_t)kOptQueue * 16, sb = ((1 + kHostSlots) * kOptView + kOptBatch) * 8, sc = 3 * kBeamLevels * 4;
+    void* block = nullptr;
+    if (!b.grid) return;
+    if (cudaMalloc(&block, 2 * sq + sb + sc) != cudaSuccess) {
+        cudaGetLastError();
+        return;
     }
-    for (BoundBuf* s : bound_bufs(ctx))
-        if (s->cap > s->hard) {
-            dev_free(ctx, s->p, s->cap * 8);
-            s->p = nullptr;
-            s->cap = 0;
-            if (s->hard) alloc_bounds(ctx, *s, s->hard, false);  // (else at the next pass that needs it)
-        }
-    return true;
+    auto* e = (unsigned long long*)((char*)block + 2 * sq);
+    auto* cnt = (uint32_t*)((char*)block + 2 * sq + sb);
+    if (!fill_now(ctx, e, 0xFF, sb) || !fill_now(ctx, cnt, 0, sc) ||
+        cudaEventCreateWithFlags(&b.opt_read, cudaEventDisableTiming) != cudaSuccess) {
+        cudaGetLastError();
+        cudaFree(block);
+        return;
+    }
+    auto take = [&](BoundBuf& v, size_t n) {
+        v.p = e;
+        v.cap = n;
+        e += n;
+    };
+    take(b.opt, kOptView);
+    for (BoundBuf& v : b.opt_host) take(v, kOptView);
+    take(b.opt_batch, kOptBatch);
+    b.opt_q = BeamQueues{{(uint4*)block, (uint4*)((char*)block + sq)}, cnt, cnt + kBeamLevels, kOptQueue};
+    b.view_hist = cnt + 2 * kBeamLevels;
+    b.opt_block = block;
 }
+}  // extern "C++"
 
 static constexpr uint32_t kBeamTags = 0xFFFFFFEFu;  // tags of an epoch
 
@@ -1058,27 +1036,31 @@ static int beam_renew(BoundBuf& b, uint32_t epoch, void* stream) {
 }
 
 // Fill the pass header of P (views and regions are filled by the caller).
-static void beam_header(aok_ctx* ctx, BeamBatch* P, uint32_t tag) {
+static void beam_header(aok_ctx* ctx, BeamHead* P, uint32_t tag, const BeamQueues& q) {
+    P->n_views = 0;
+    P->n_regions = 0;
     P->expand = ctx->beam_refine;
     P->smin = ctx->beam_min_log2;
     P->tag = tag;
-    P->cap = ctx->beam_queue && ctx->beam_queue < kBeamCap ? ctx->beam_queue : kBeamCap;
-    P->q[0] = ctx->beam.q[0];
-    P->q[1] = ctx->beam.q[1];
-    P->cnt = ctx->beam.cnt;
-    P->hist = ctx->beam.hist;
+    P->cap = ctx->beam_queue ? std::min(ctx->beam_queue, q.cap) : q.cap;
+    P->q[0] = q.q[0];
+    P->q[1] = q.q[1];
+    P->cnt = q.cnt;
+    P->hist = q.hist;
     P->select = 0;
     std::memset(&P->ck, 0, sizeof(P->ck));  // unchecked
 }
 
-// A view's pass buffers.
-static int beam_buffers(aok_ctx* ctx, BoundBuf& b, const CamDev& cd, bool optional) {
+// The pyramid and queues of a view's pass (AOK_E_BUSY: the pass is optional
+// and has no room for it).
+static int beam_buffers(aok_ctx* ctx, BoundBuf& required, BoundBuf& opt, const CamDev& cd, bool optional,
+                        BoundBuf** buf, const BeamQueues** q) {
     const size_t need = beam_entries((uint32_t)cd.W, (uint32_t)cd.H);
-    RelaxedCapture rc(optional);
-    int st = ensure_beam_queues(ctx, !optional);
-    if (!st) st = ensure_bounds(ctx, b, need, optional ? 0 : need);
-    if (st == AOK_E_OOM && optional) ctx->beam.no_room = true;
-    return st;
+    *buf = optional ? &opt : &required;
+    *q = optional ? &ctx->beam.opt_q : &ctx->beam.q;
+    if (optional) return need <= opt.cap ? AOK_OK : AOK_E_BUSY;
+    int st = ensure_beam_queues(ctx);
+    return st ? st : ensure_bounds(ctx, required, need);
 }
 
 // The beam pass over the scene's current frame table; *rd: what the cast
@@ -1086,45 +1068,44 @@ static int beam_buffers(aok_ctx* ctx, BoundBuf& b, const CamDev& cd, bool option
 // pass selects it as its first step (one launch fewer), or, for a view
 // without a usable projection, the selection kernel does.  ck: checked
 // casting's pool sizes and error word (the pass tests its node and leaf
-// indices too), or null.  optional: AOK_E_OOM leaves the frame as it was, to be
+// indices too), or null.  optional: AOK_E_BUSY leaves the frame as it was, to be
 // cast without the pass; the cast is followed by beam_was_read.  keep: the
 // pass is remembered with what it was computed for.  Called with the pass's
 // buffers held (b.use).
 static int run_beam(aok_ctx* ctx, uint32_t scene, Scene* sc, const SceneDev& sd, const CamDev& cd, void* stream,
                     BeamRead* rd, bool select, const CheckDev* ck, bool optional, bool keep) {
     BeamState& b = ctx->beam;
-    BoundBuf& buf = optional ? b.opt : b.bounds;
-    if (keep || b.read.bounds == buf.p) b.valid = false;  // (the buffer may move)
-    if (b.last.bounds == buf.p) b.ran = false;
-    int st = beam_buffers(ctx, buf, cd, optional);
+    if (keep || b.read.bounds == (optional ? b.opt.p : b.bounds.p)) b.valid = false;
+    if (!optional && b.last.bounds == b.bounds.p) b.ran = false;  // (the buffer may move)
+    BoundBuf* buf;
+    const BeamQueues* q;
+    int st = beam_buffers(ctx, b.bounds, b.opt, cd, optional, &buf, &q);
     if (st) return st;
-    if (optional && b.opt_read && cudaStreamWaitEvent((cudaStream_t)stream, b.opt_read, 0) != cudaSuccess)
+    if (optional && cudaStreamWaitEvent((cudaStream_t)stream, b.opt_read, 0) != cudaSuccess)
         return AOK_E_CUDA;
     uint32_t epoch;
     const uint32_t tag = next_beam_tag(ctx, &epoch);
-    st = beam_renew(buf, epoch, stream);
+    st = beam_renew(*buf, epoch, stream);
     if (st) return st;
-    BeamBatch* P = b.P.get();
-    beam_header(ctx, P, tag);
-    P->hist = b.view_hist;
-    if (ck) P->ck = *ck;
-    P->n_views = 0;
-    P->n_regions = 0;
+    BeamParams<1> P;
+    beam_header(ctx, &P, tag, *q);
+    P.hist = b.view_hist;
+    if (ck) P.ck = *ck;
     *rd = BeamRead{nullptr, tag};  // no usable projection: no bounds, nothing is skipped
-    if (aokk_beam_view(&sd, &cd, sc->d_frame, buf.p, &P->v[0])) {
-        P->v[0].region_begin = 0;
-        P->n_views = 1;
-        P->n_regions = (uint32_t)sc->n_chunks;
-        rd->bounds = buf.p;
+    if (aokk_beam_view(&sd, &cd, sc->d_frame, buf->p, &P.v[0])) {
+        P.v[0].region_begin = 0;
+        P.n_views = 1;
+        P.n_regions = (uint32_t)sc->n_chunks;
+        rd->bounds = buf->p;
         if (select) {
-            P->select = 1;
-            P->cam = cd;
+            P.select = 1;
+            P.cam = cd;
         }
     } else if (select) {
         st = aokk_select(&sd, &cd, sc->d_frame, nullptr, nullptr, nullptr, stream);
         if (st) return st;
     }
-    st = aokk_beam_run(P, b.grid, stream);
+    st = aokk_beam_run_view(&P, b.grid, stream, 0);
     if (st) return st;
     b.last = *rd;
     b.ran = true;
@@ -1144,8 +1125,7 @@ static int run_beam(aok_ctx* ctx, uint32_t scene, Scene* sc, const SceneDev& sd,
 // on whatever stream, waits for it.
 static int beam_was_read(aok_ctx* ctx, void* stream) {
     BeamState& b = ctx->beam;
-    cudaError_t e = b.opt_read ? cudaSuccess : cudaEventCreateWithFlags(&b.opt_read, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaStreamGetId((cudaStream_t)stream, &b.opt_stream);
+    cudaError_t e = cudaStreamGetId((cudaStream_t)stream, &b.opt_stream);
     if (e == cudaSuccess) e = cudaEventRecord(b.opt_read, (cudaStream_t)stream);
     return cuda_status(ctx, e);
 }
@@ -1155,10 +1135,9 @@ static int beam_was_read(aok_ctx* ctx, void* stream) {
 // the same stream.
 static bool beam_read_alone(aok_ctx* ctx, void* stream) {
     const BeamState& b = ctx->beam;
-    if (!b.opt_read) return true;
     unsigned long long id = 0;
     if (cudaStreamGetId((cudaStream_t)stream, &id) == cudaSuccess && id == b.opt_stream) return true;
-    RelaxedCapture rc(true);  // (a query would end another stream's capture)
+    RelaxedCapture rc;
     if (cudaEventQuery(b.opt_read) == cudaSuccess) return true;
     cudaGetLastError();  // "not ready" is no error of the next launch
     return false;
@@ -1168,7 +1147,7 @@ extern "C++" BeamUse aok::beam_use(const aok_ctx* ctx, int32_t W, int32_t H, voi
     const uint64_t px = (uint64_t)W * (uint64_t)H;
     if (!ctx->beam_on) return kBeamNone;
     if (px >= ctx->beam_min_pixels) return kBeamRequired;
-    if (px < ctx->beam_min_optional || ctx->beam.no_room) return kBeamNone;
+    if (px < ctx->beam_min_optional || !ctx->beam.opt_block) return kBeamNone;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing((cudaStream_t)stream, &cap) != cudaSuccess) {
         cudaGetLastError();
@@ -1192,37 +1171,37 @@ extern "C++" int aok::beam_for_batch(aok_ctx* ctx, BatchParams* groups, uint32_t
         }
     const size_t req = need[kBeamRequired], opt = need[kBeamOptional];
     if (!req && !opt) return AOK_OK;
-    RelaxedCapture rc(!req);
-    BoundBuf& bb = ctx->batch.beam_bounds;
-    int st = ensure_beam_queues(ctx, req > 0);
-    if (!st && !view_bounds) st = ensure_bounds(ctx, bb, req + opt, req);
-    if (st == AOK_E_OOM && !req) {
-        ctx->beam.no_room = true;
-        return AOK_OK;
-    }
+    BoundBuf &bb = ctx->batch.beam_bounds, &ob = ctx->beam.opt_batch;
+    int st = req ? ensure_beam_queues(ctx) : AOK_OK;
+    if (!st && !view_bounds) st = ensure_bounds(ctx, bb, req);
     if (st) return st;
     uint32_t epoch;
     const uint32_t tag = next_beam_tag(ctx, &epoch);
-    if (!view_bounds) arena = &bb;
     if (arena) st = beam_renew(*arena, epoch, stream);
+    if (!st && !view_bounds) st = beam_renew(bb, epoch, stream);
+    if (!st && !view_bounds && opt) st = beam_renew(ob, epoch, stream);
     if (st) return st;
-    const bool all = view_bounds || bb.cap >= req + opt;  // else the optional passes don't fit
     out.resize(ngroups);
-    size_t off = 0;
+    size_t off[3] = {0, 0, 0};
     flat = 0;
     for (uint32_t g = 0; g < ngroups; g++) {
         BeamBatch& B = out[g];
-        beam_header(ctx, &B, tag);
-        B.n_views = 0;
-        B.n_regions = 0;
+        beam_header(ctx, &B, tag, req ? ctx->beam.q : ctx->beam.opt_q);
         groups[g].beam_tag = tag;
         for (uint32_t i = 0; i < groups[g].n_views; i++, flat++) {
             ViewDev& d = groups[g].v[i];
             d.beam = nullptr;
             const BeamUse use = beam_use(ctx, d.cam.W, d.cam.H, stream);
-            if (use == kBeamNone || (use == kBeamOptional && !all)) continue;
-            unsigned long long* bnd = view_bounds ? view_bounds[flat] : bb.p + off;
-            off += beam_entries((uint32_t)d.cam.W, (uint32_t)d.cam.H);
+            if (use == kBeamNone) continue;
+            unsigned long long* bnd = nullptr;
+            if (view_bounds) {
+                bnd = view_bounds[flat];
+            } else {
+                const size_t n = beam_entries((uint32_t)d.cam.W, (uint32_t)d.cam.H);
+                const BoundBuf& v = use == kBeamRequired ? bb : ob;
+                if (off[use] + n <= v.cap) bnd = v.p + off[use];
+                if (bnd) off[use] += n;
+            }
             if (!bnd) continue;
             if (!aokk_beam_view(&d.scene, &d.cam, d.frame, bnd, &B.v[B.n_views])) continue;  // casts without
             B.v[B.n_views].region_begin = B.n_regions;
@@ -1263,12 +1242,12 @@ static int cast_single(aok_ctx* ctx, uint32_t scene, Scene* sc, const SceneDev& 
         if (selected && beam_fresh(ctx, scene, sc, cd)) {
             rd = ctx->beam.read;
             // a second cast of one selection, beside the first: without the bounds
-            if (optional && rd.bounds == ctx->beam.opt.p && !beam_read_alone(ctx, stream)) st = AOK_E_OOM;
+            if (optional && rd.bounds == ctx->beam.opt.p && !beam_read_alone(ctx, stream)) st = AOK_E_BUSY;
         } else st = run_beam(ctx, scene, sc, sd, cd, stream, &rd, !selected, ckp, optional, !optional);
         if (st == AOK_OK) {
             selected = true;
             beam = &rd;
-        } else if (st != AOK_E_OOM || use == kBeamRequired) {
+        } else if (st != AOK_E_BUSY) {
             return st;
         }
         st = AOK_OK;
@@ -1456,7 +1435,7 @@ int aok_render_tiles(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, double
         st = run_beam(ctx, scene, sc, sd, cd, stream, &rd, true, nullptr, use == kBeamOptional, use == kBeamRequired);
         if (!st) beam = &rd;
     }
-    if (use == kBeamNone || (use == kBeamOptional && st == AOK_E_OOM))
+    if (use == kBeamNone || st == AOK_E_BUSY)
         st = aokk_select(&sd, &cd, sc->d_frame, nullptr, nullptr, nullptr, stream);
     if (!st) st = aokk_tiles_frame(&sd, &cd, sc->d_frame, &ctx->tiles.dev, (uint4*)frame->hit, frame->t,
                                    ctx->sm_count, stream, beam);
@@ -1484,7 +1463,6 @@ int aok_tiles_forget(aok_ctx* ctx) {
 int aok_set_beam(aok_ctx* ctx, int on) {
     if (!ctx) return AOK_E_INVALID;
     ctx->beam_on = on ? 1 : 0;
-    ctx->beam.no_room = false;
     return AOK_OK;
 }
 
@@ -1495,7 +1473,6 @@ int aok_beam_tune(aok_ctx* ctx, uint32_t refine_tiles, int32_t min_node_log2, ui
     ctx->beam_min_log2 = min_node_log2;
     ctx->beam_min_pixels = ctx->beam_min_optional = min_pixels;
     ctx->beam_queue = queue_nodes;
-    ctx->beam.no_room = false;
     return AOK_OK;
 }
 
@@ -1531,7 +1508,7 @@ int aok_select_beam(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, double 
     BeamRead rd;
     if (use != kBeamNone)
         st = run_beam(ctx, scene, sc, sd, cd, stream, &rd, true, check_dev(ctx, sc, &ck), use == kBeamOptional, true);
-    if (use == kBeamNone || (use == kBeamOptional && st == AOK_E_OOM))
+    if (use == kBeamNone || st == AOK_E_BUSY)
         st = aokk_select(&sd, &cd, sc->d_frame, nullptr, nullptr, nullptr, stream);
     if (st == AOK_E_CUDA) return launch_failure(ctx);
     return st;
@@ -1672,7 +1649,6 @@ static int pipe_ensure(aok_ctx* ctx, size_t px) {
             cudaStreamCreateWithFlags(&p.render, cudaStreamNonBlocking) != cudaSuccess ||
             cudaStreamCreateWithFlags(&p.copy, cudaStreamNonBlocking) != cudaSuccess)
             return cuda_status(ctx, cudaGetLastError());
-        p.P.reset(new BeamBatch);
     }
     if (px <= p.px) return AOK_OK;
     pipe_release(ctx);
@@ -1712,12 +1688,12 @@ static int pipe_render(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, doub
     }
     std::lock_guard<std::recursive_mutex> lk(ctx->beam.use);
     const BeamUse use = beam_use(ctx, cd.W, cd.H, p.prep);
-    bool beam = use != kBeamNone;
-    if (beam) {
-        st = beam_buffers(ctx, sl.bounds, cd, use == kBeamOptional);
-        if (st == AOK_E_OOM && use == kBeamOptional) beam = false;
-        else if (st) return st;
-    }
+    BoundBuf* buf = nullptr;
+    const BeamQueues* q = nullptr;
+    st = use == kBeamNone ? AOK_E_BUSY
+                          : beam_buffers(ctx, sl.bounds, ctx->beam.opt_host[&sl - p.slot], cd, use == kBeamOptional, &buf, &q);
+    const bool beam = st == AOK_OK;
+    if (st && st != AOK_E_BUSY) return st;
     const SceneDev sd = scene_dev(sc);
     // the selection kernel, then the pass (measured faster here than the pass
     // that selects first: the pass runs beside the previous frame's cast)
@@ -1727,20 +1703,18 @@ static int pipe_render(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, doub
     if (beam) {
         uint32_t epoch;
         const uint32_t tag = next_beam_tag(ctx, &epoch);
-        st = beam_renew(sl.bounds, epoch, p.prep);
+        st = beam_renew(*buf, epoch, p.prep);
         if (st) return st;
-        BeamBatch* P = p.P.get();
-        beam_header(ctx, P, tag);
-        P->n_views = 0;
-        P->n_regions = 0;
-        if (aokk_beam_view(&sd, &cd, sl.frame, sl.bounds.p, &P->v[0])) {
-            P->v[0].region_begin = 0;
-            P->n_views = 1;
-            P->n_regions = (uint32_t)sc->n_chunks;
-            rd.bounds = sl.bounds.p;
+        BeamParams<1> P;
+        beam_header(ctx, &P, tag, *q);
+        if (aokk_beam_view(&sd, &cd, sl.frame, buf->p, &P.v[0])) {
+            P.v[0].region_begin = 0;
+            P.n_views = 1;
+            P.n_regions = (uint32_t)sc->n_chunks;
+            rd.bounds = buf->p;
             rd.tag = tag;
         }
-        st = aokk_beam_run(P, ctx->beam.grid, p.prep, 1);  // beside the previous frame's cast
+        st = aokk_beam_run_view(&P, ctx->beam.grid, p.prep, 1);  // beside the previous frame's cast
         if (st) return launch_failure(ctx);
     }
     cudaError_t e = cudaEventRecord(sl.prepped, p.prep);

@@ -56,8 +56,7 @@ void stream_detach(aok_stream* s);
 // A grow-only array of beam pyramid entries.
 struct BoundBuf {
     unsigned long long* p = nullptr;
-    size_t cap = 0;   // entries
-    size_t hard = 0;  // entries that frames with a required pass have needed
+    size_t cap = 0;      // entries
     uint32_t epoch = 0;  // of the tags in it (beam_renew)
 };
 
@@ -93,7 +92,6 @@ struct HostPipe {
     HostSlot slot[kHostSlots];
     size_t px = 0;        // pixels each slot holds
     uint64_t next = 0;    // last ticket issued
-    std::unique_ptr<BeamBatch> P;  // beam pass parameter block
 };
 
 // Buffers of the tile-chunk pipeline for one resolution and grid size (one
@@ -108,28 +106,36 @@ struct TileState {
     uint32_t scene = 0xFFFFFFFFu;
 };
 
+// A walk's queues of `cap` nodes a level, the counts per level and, of the
+// last pass (not a single view's), the walk histogram.
+struct BeamQueues {
+    uint4* q[2] = {nullptr, nullptr};
+    uint32_t *cnt = nullptr, *hist = nullptr;
+    uint32_t cap = 0;
+};
+
 // The beam pass: the walk's queues and launch grid (shared by all passes of
 // the context), the single-view bound pyramid and what its last pass was
 // computed for.
 struct BeamState {
-    // held from a pass's buffers being looked up to its launches being enqueued: another thread that runs short of
-    // memory may give the buffers back (beam_reclaim)
-    std::recursive_mutex use;
+    std::recursive_mutex use;  // the single-view passes' buffers and records, until their launches are enqueued
     std::mutex mu;  // the queues' allocation and the pass counter (the serving thread shares them)
     void* qblock = nullptr;
     size_t qbytes = 0;
-    bool q_hard = false;   // a frame that has to take the pass has used the queues
-    std::atomic<bool> no_room{false};  // memory ran short: frames that need not take the pass no longer do
-    uint4* q[2] = {nullptr, nullptr};
-    uint32_t* cnt = nullptr;   // [kBeamLevels] queue counts, then two walk histograms [kBeamLevels]:
-    uint32_t* hist = nullptr;  // of the last batch or host frame, and
-    uint32_t* view_hist = nullptr;  // of the last single view's pass
+    BeamQueues q;              // of the passes that frames have to take
     unsigned grid = 0;         // blocks of the cooperative launch
-    std::unique_ptr<BeamBatch> P;  // host parameter block (~26 KB)
-    BoundBuf bounds;                       // single-view pyramid
-    // the pyramid of frames that need not take the pass, and the last cast
-    // that read it: they may come on streams that nothing orders
-    BoundBuf opt;
+    BoundBuf bounds;           // single-view pyramid
+    // What the passes use that frames need not take: one block beside the
+    // budget, allocated with the context (14 MB), so that such a frame needs
+    // no memory of its own, in its first pass or later, and takes none from
+    // what the budget is for.  Without it (opt_block == nullptr: the device
+    // had no room) there are no such passes.
+    void* opt_block = nullptr;
+    BeamQueues opt_q;
+    uint32_t* view_hist = nullptr;  // walk histogram of the last single view's pass
+    BoundBuf opt, opt_host[kHostSlots], opt_batch;
+    // the last cast that read `opt`: the next one may come on a stream that
+    // nothing orders with it
     cudaEvent_t opt_read = nullptr;
     unsigned long long opt_stream = 0;  // that cast's stream
     uint32_t passes = 0;                   // passes run in this epoch (their tags count down)
@@ -199,7 +205,7 @@ struct aok_ctx {
     int beam_min_log2 = 2;     // ... whose side is above 2^this LOD-0 voxels
     // Frames of beam_min_pixels take the pass.  Those of beam_min_optional take it where it can run: not on a stream
     // that is being captured (the passes of a device wait for one another by events a capture can't hold) and not
-    // where its 33 MB of queues don't fit the budget.  Smaller ones cast without it (city views of 1120 x 630 break
+    // beyond the room of its buffers.  Smaller ones cast without it (city views of 1120 x 630 break
     // even at 160-240 us, 1280 x 720 ones gain 12% on average with it, -29% to +12%, and 960 x 540 ones nothing).
     uint64_t beam_min_pixels = 1500000, beam_min_optional = 800000;
     uint32_t beam_queue = 0;             // nodes a queue level may hold (0: the allocated 2^20)
@@ -236,21 +242,12 @@ inline bool beam_required(const aok_ctx* ctx, int32_t W, int32_t H) {
 }
 enum BeamUse { kBeamNone, kBeamOptional, kBeamRequired };
 BeamUse beam_use(const aok_ctx* ctx, int32_t W, int32_t H, void* stream);
-// Frees the pass's buffers that only optional passes have needed (true: there
-// were some); the context runs no optional pass any more.
-bool beam_reclaim(aok_ctx* ctx);
-size_t beam_spare_bytes(aok_ctx* ctx);  // what it would free
-// Lets this thread allocate while another one captures a stream in the global
-// capture mode (whose capture an allocation here would end).
+// Lets this thread query an event while another one captures a stream in the
+// global capture mode (whose capture the query would end).
 struct RelaxedCapture {
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    const bool on;
-    explicit RelaxedCapture(bool use) : on(use) {
-        if (on) cudaThreadExchangeStreamCaptureMode(&mode);
-    }
-    ~RelaxedCapture() {
-        if (on) cudaThreadExchangeStreamCaptureMode(&mode);
-    }
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
 };
 // Pinned staging memory and the stream its copies go on.
 struct Staging {

@@ -383,15 +383,13 @@ static void serve_loop(aok_ctx* ctx) {
                     continue;
                 }
                 const size_t bytes = request_bytes(ctx, sc, t.req.cam);
+                if (charge(ctx, bytes) != AOK_OK) break;  // wait for memory to free up
                 void* mem = nullptr;
-                auto take = [&] {
-                    if (charge(ctx, bytes) != AOK_OK) return false;
-                    if (cudaMallocFromPoolAsync(&mem, bytes, S.pool, S.streams[slot]) == cudaSuccess) return true;
+                if (cudaMallocFromPoolAsync(&mem, bytes, S.pool, S.streams[slot]) != cudaSuccess) {
                     cudaGetLastError();
                     uncharge(ctx, bytes);
-                    return false;
-                };
-                if (!take() && !(beam_reclaim(ctx) && take())) break;  // wait for memory to free up
+                    break;
+                }
                 const size_t px = (size_t)t.req.cam.width * t.req.cam.height;
                 t.hit = mem;
                 t.t = (float*)((char*)mem + ((px * 16 + 255) & ~(size_t)255));
@@ -479,7 +477,6 @@ static void serve_loop(aok_ctx* ctx) {
                     vb[i] = arena->p + off;
                     off += n;
                 }
-            RelaxedCapture relaxed(true);
             if (rc == AOK_OK) rc = beam_for_batch(ctx, S.params.data(), ngroups, beams, st, vb.data(), arena);
         }
         if (rc == AOK_OK) {

@@ -162,3 +162,58 @@ def test_server_batch_of_both_kinds_in_a_tight_budget(room_kb):
     assert aok.beam_passes(s.c) > 0
     srv.stop()
     s.close()
+
+
+@pytest.mark.parametrize("kind", ["single", "tiles", "host", "batch", "serve"])
+@pytest.mark.parametrize("room", [None, 1 << 20])
+def test_optional_pass_takes_nothing_from_the_budget(kind, room):
+    """The pass runs for frames of 1280 x 720 whatever the budget (room: what it leaves beside the scene and the
+    call's own buffers), also after an allocation that failed; the frames change neither the context's charged
+    memory nor, from the first one on, the device's free memory."""
+    if room is not None:
+        s = Setup()
+        for _ in range(3 if kind != "serve" else 0):
+            draw(s, kind, s.cam(0))
+        used = s.c.memory()[0]
+        s.close()
+    s = Setup(0 if room is None else used + (20 << 20 if kind == "serve" else 0) + room)
+    cams = [s.cam(k) for k in range(3)]
+    refs = [s.ref(m) for m in cams]
+    srv = aok.Server(s.c, max_slots=4, max_batch=2, n_streams=1) if kind == "serve" else None
+    aok.set_beam(s.c, False)
+    for _ in range(3):  # the call's own buffers (three slots of host frames)
+        draw(s, kind, cams[0], srv)
+    aok.set_beam(s.c, True)
+    mem, free = s.c.memory(), torch.cuda.mem_get_info()[0]
+    n = aok.beam_passes(s.c)
+    for i in range(2):
+        for m, r in zip(cams, refs):
+            assert equal(draw(s, kind, m, srv), r)
+            n += 1
+            assert aok.beam_passes(s.c) == n and s.c.memory() == mem
+        assert torch.cuda.mem_get_info()[0] == free
+        if room is not None:
+            with pytest.raises(aok.AokError):
+                aok.Scene(s.c, s.world.spec, node_words=64 << 20, leaves=1, mat_bytes=1)
+        free = torch.cuda.mem_get_info()[0]
+    if srv:
+        srv.stop()
+    s.close()
+
+
+def test_optional_passes_beyond_their_room():
+    """Views beyond the block's room are cast without bounds: the last of 30 in a batch, a frame of one row."""
+    s = Setup()
+    cams = [s.cam(k) for k in range(3)]
+    refs = [s.ref(m) for m in cams]
+    outs = [aok.alloc_frame(*OPTIONAL) for _ in range(30)]
+    n = aok.beam_passes(s.c)
+    aok.render_batch(s.c, [aok.make_view(s.sc, cams[i % 3], 1.5, *o) for i, o in enumerate(outs)])
+    torch.cuda.synchronize()
+    assert all(equal(o, refs[i % 3]) for i, o in enumerate(outs)) and aok.beam_passes(s.c) == n + 1
+    row = replace(cams[0], W=900000, H=1)
+    ref = s.ref(row)
+    for kind in ("single", "tiles", "host"):
+        assert equal(draw(s, kind, row), ref)
+    assert aok.beam_passes(s.c) == n + 1
+    s.close()

@@ -1071,7 +1071,7 @@ static int beam_buffers(aok_ctx* ctx, BoundBuf& required, BoundBuf& opt, const C
 // indices too), or null.  optional: AOK_E_BUSY leaves the frame as it was, to be
 // cast without the pass; the cast is followed by beam_was_read.  keep: the
 // pass is remembered with what it was computed for.  Called with the pass's
-// buffers held (b.use).
+// buffers held (b.view_mu).
 static int run_beam(aok_ctx* ctx, uint32_t scene, Scene* sc, const SceneDev& sd, const CamDev& cd, void* stream,
                     BeamRead* rd, bool select, const CheckDev* ck, bool optional, bool keep) {
     BeamState& b = ctx->beam;
@@ -1234,10 +1234,11 @@ static int cast_single(aok_ctx* ctx, uint32_t scene, Scene* sc, const SceneDev& 
     BeamRead rd{nullptr, 0};
     const BeamRead* beam = nullptr;
     int st = AOK_OK;
-    std::lock_guard<std::recursive_mutex> lk(ctx->beam.use);
     BeamUse use = beam_use(ctx, cd.W, cd.H, stream);
     if (counts && use == kBeamOptional) use = kBeamNone;  // its visits would depend on whether the pass could run
+    std::unique_lock<std::mutex> lk(ctx->beam.view_mu, std::defer_lock);
     if (use != kBeamNone) {
+        lk.lock();
         const bool optional = use == kBeamOptional;
         if (selected && beam_fresh(ctx, scene, sc, cd)) {
             rd = ctx->beam.read;
@@ -1429,9 +1430,10 @@ int aok_render_tiles(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, double
     // pass selects the frame table as its first step
     BeamRead rd{nullptr, 0};
     const BeamRead* beam = nullptr;
-    std::lock_guard<std::recursive_mutex> lk(ctx->beam.use);
+    std::unique_lock<std::mutex> lk(ctx->beam.view_mu, std::defer_lock);
     const BeamUse use = beam_use(ctx, cd.W, cd.H, stream);
     if (use != kBeamNone) {
+        lk.lock();
         st = run_beam(ctx, scene, sc, sd, cd, stream, &rd, true, nullptr, use == kBeamOptional, use == kBeamRequired);
         if (!st) beam = &rd;
     }
@@ -1485,7 +1487,7 @@ int aok_beam_selected(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, void*
     if (st) return st;
     cudaSetDevice(ctx->device);
     SceneDev sd = scene_dev(sc);
-    std::lock_guard<std::recursive_mutex> lk(ctx->beam.use);
+    std::lock_guard<std::mutex> lk(ctx->beam.view_mu);
     BeamRead rd;
     st = run_beam(ctx, scene, sc, sd, cd, stream, &rd, false, nullptr, false, true);
     if (st == AOK_E_CUDA) return launch_failure(ctx);
@@ -1503,11 +1505,12 @@ int aok_select_beam(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, double 
     SceneDev sd = scene_dev(sc);
     sc->select_gen++;
     CheckDev ck;
-    std::lock_guard<std::recursive_mutex> lk(ctx->beam.use);
     const BeamUse use = beam_use(ctx, cd.W, cd.H, stream);
     BeamRead rd;
-    if (use != kBeamNone)
+    if (use != kBeamNone) {
+        std::lock_guard<std::mutex> lk(ctx->beam.view_mu);
         st = run_beam(ctx, scene, sc, sd, cd, stream, &rd, true, check_dev(ctx, sc, &ck), use == kBeamOptional, true);
+    }
     if (use == kBeamNone || st == AOK_E_BUSY)
         st = aokk_select(&sd, &cd, sc->d_frame, nullptr, nullptr, nullptr, stream);
     if (st == AOK_E_CUDA) return launch_failure(ctx);
@@ -1517,7 +1520,7 @@ int aok_select_beam(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, double 
 int aok_beam_info(aok_ctx* ctx, int32_t* bounds, uint64_t n_bounds, uint32_t* level_counts, int32_t* tiles_xy) {
     if (!ctx) return AOK_E_INVALID;
     const BeamState& b = ctx->beam;
-    std::lock_guard<std::recursive_mutex> lk(ctx->beam.use);
+    std::lock_guard<std::mutex> lk(ctx->beam.view_mu);
     if (!b.ran) return AOK_E_INVALID;
     const uint32_t tx = (uint32_t)(b.W + kBeamTileW - 1) / kBeamTileW, ty = (uint32_t)(b.H + kBeamTileH - 1) / kBeamTileH;
     const uint64_t n = (uint64_t)tx * ty;
@@ -1686,7 +1689,6 @@ static int pipe_render(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, doub
         if (st) return st;
         sl.frame_cap = (size_t)sc->n_chunks;
     }
-    std::lock_guard<std::recursive_mutex> lk(ctx->beam.use);
     const BeamUse use = beam_use(ctx, cd.W, cd.H, p.prep);
     BoundBuf* buf = nullptr;
     const BeamQueues* q = nullptr;

@@ -118,7 +118,10 @@ struct BeamQueues {
 // the context), the single-view bound pyramid and what its last pass was
 // computed for.
 struct BeamState {
-    std::recursive_mutex use;  // the single-view passes' buffers and records, until their launches are enqueued
+    // The single-view passes' buffers and records, until a pass and the cast
+    // that reads it are enqueued.  Frames without the pass don't take it, nor
+    // do batches, host frames and the server, which have their own buffers.
+    std::mutex view_mu;
     std::mutex mu;  // the queues' allocation and the pass counter (the serving thread shares them)
     void* qblock = nullptr;
     size_t qbytes = 0;

@@ -150,9 +150,7 @@ static int render_batch_impl(aok_ctx* ctx, const aok_view* views, uint32_t n, vo
     if (st) return st;
     // the beam pass for the views large enough (grid launch only)
     std::vector<BeamBatch> beams;
-    std::unique_lock<std::recursive_mutex> lk(ctx->beam.use, std::defer_lock);
     if (L.ctas == 0) {
-        lk.lock();
         st = beam_for_batch(ctx, prep.groups.data(), (uint32_t)prep.groups.size(), beams, stream);
         if (st) return st;
     }
@@ -448,9 +446,7 @@ static void serve_loop(aok_ctx* ctx) {
         // the beam pass for the large requests (grid launch): pyramids in a
         // request's fresh pool memory are first set to "no tag" everywhere
         std::vector<BeamBatch> beams;
-        std::unique_lock<std::recursive_mutex> use(ctx->beam.use, std::defer_lock);
         if (rc == AOK_OK && L.ctas == 0) {
-            use.lock();
             std::vector<unsigned long long*> vb(batch.size(), nullptr);
             {
                 std::lock_guard<std::mutex> g(S.mu);
@@ -486,7 +482,6 @@ static void serve_loop(aok_ctx* ctx) {
             rc = aokk_batch_run(S.params.data(), ngroups, L.ctas, L.threads, st, beams.empty() ? nullptr : beams.data(),
                                 ctx->beam.grid, &ho, nullptr);
         }
-        if (use.owns_lock()) use.unlock();
         std::lock_guard<std::mutex> g(S.mu);
         if (rc != AOK_OK) {
             for (uint64_t id : batch) {

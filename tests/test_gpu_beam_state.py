@@ -1,6 +1,8 @@
 """State that beam passes share within a context: tags, buffers, the record of
 the last pass.  Frames of 1280 x 720 take the pass where it can run, frames of
 1600 x 1000 always; each equals the frame without the pass bit for bit."""
+import threading
+import time
 from dataclasses import replace
 
 import pytest
@@ -216,4 +218,64 @@ def test_optional_passes_beyond_their_room():
     for kind in ("single", "tiles", "host"):
         assert equal(draw(s, kind, row), ref)
     assert aok.beam_passes(s.c) == n + 1
+    s.close()
+
+
+def test_frames_without_the_pass_do_not_wait():
+    """A large frame's call waits for the device (its buffer grows behind 400 ms of other work); a small frame
+    of another scene is enqueued meanwhile by another thread."""
+    s = Setup()
+    sc2 = aok.Scene.from_world(s.c, s.world, threads=4)
+    small, big = s.cam(0, (320, 180)), s.cam(1, (2000, 1200))
+    refs = s.ref(small), s.ref(big)
+    outs = aok.alloc_frame(320, 180), aok.alloc_frame(2000, 1200)
+    draw(s, "single", s.cam(1, REQUIRED))
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    aok.render(s.c, sc2, small, 1.5, *outs[0], stream=s2)
+    torch.cuda.synchronize()
+    t0 = time.perf_counter()
+    with torch.cuda.stream(s1):
+        torch.cuda._sleep(800_000_000)
+    th = threading.Thread(target=lambda: aok.render(s.c, s.sc, big, 1.5, *outs[1], stream=s1))
+    th.start()
+    time.sleep(0.05)
+    t1 = time.perf_counter()
+    aok.render(s.c, sc2, small, 1.5, *outs[0], stream=s2)
+    t2 = time.perf_counter()
+    th.join()
+    torch.cuda.synchronize()
+    t3 = time.perf_counter()
+    assert t3 - t0 > 0.3 and t2 - t1 < 0.1, (t3 - t0, t2 - t1)
+    assert equal(outs[0], refs[0]) and equal(outs[1], refs[1])
+    sc2.destroy()
+    s.close()
+
+
+def test_threads_with_scenes_of_their_own():
+    """Four host threads, each with a scene and a stream, sizes without the pass and with the optional one."""
+    s = Setup()
+    scenes = [aok.Scene.from_world(s.c, s.world, threads=4) for _ in range(4)]
+    cams = [s.cam(k, size) for k in range(3) for size in (OPTIONAL, (320, 180))]
+    refs = [s.ref(m) for m in cams]
+    bad = []
+
+    def work(i):
+        stream = torch.cuda.Stream()
+        for k in range(60):
+            j = (k + i) % len(cams)
+            out = aok.alloc_frame(cams[j].W, cams[j].H)
+            aok.render(s.c, scenes[i], cams[j], 1.5, *out, stream=stream)
+            stream.synchronize()
+            if not equal(out, refs[j]):
+                bad.append((i, k))
+
+    torch.cuda.synchronize()
+    ths = [threading.Thread(target=work, args=(i,)) for i in range(4)]
+    for th in ths:
+        th.start()
+    for th in ths:
+        th.join()
+    assert not bad
+    for sc in scenes:
+        sc.destroy()
     s.close()

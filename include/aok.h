@@ -555,7 +555,9 @@ int aok_render_noalloc(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, doub
  * rows or columns, more than about 16 such views in a batch); they can be
  * rendered on any streams.
  * The passes of all contexts of a process run one after another on a
- * device (each waits for the previous one's launch to finish). */
+ * device (each waits for the previous one's launch to finish); a frame (or a
+ * batch) that only has an optional pass is cast without it rather than wait
+ * for another stream. */
 int aok_set_beam(aok_ctx* ctx, int on);
 /* Refinement of the beam pass's walk: a node is refined while its rectangle
  * spans more than refine_tiles tiles and its side is above 2^min_node_log2

@@ -523,6 +523,28 @@ bool aokk_beam_view(const SceneDev* S, const CamDev* C, const ChunkRef* frame, u
 // blocks.
 static std::mutex g_beam_mu;
 static cudaEvent_t g_beam_done[kMaxBeamDevices];
+static unsigned long long g_beam_stream[kMaxBeamDevices];  // that pass's stream
+
+extern "C++" {
+// Whether a pass on `st` would wait for another stream's work (g_beam_mu held).
+static bool pass_waits(int dev, cudaStream_t st) {
+    unsigned long long id = 0;
+    if (!g_beam_done[dev] || (cudaStreamGetId(st, &id) == cudaSuccess && id == g_beam_stream[dev])) return false;
+    // (in the relaxed mode: a query would end another stream's capture)
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    const cudaError_t e = cudaEventQuery(g_beam_done[dev]);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e == cudaSuccess) return false;
+    cudaGetLastError();  // "not ready" is no error of the next launch
+    return true;
+}
+
+static cudaError_t pass_done(int dev, cudaStream_t st) {
+    const cudaError_t e = cudaStreamGetId(st, &g_beam_stream[dev]);
+    return e == cudaSuccess ? cudaEventRecord(g_beam_done[dev], st) : e;
+}
+}  // extern "C++"
 
 // The pass as a node of a CUDA graph (aokk_batch_run), with the launch shape
 // aokk_beam_run uses.  argp: one slot, valid until the node is set.
@@ -548,13 +570,20 @@ int aokk_beam_order(void* stream, int record) {
     if (dev < 0 || dev >= kMaxBeamDevices) return aokk_status(cudaErrorInvalidDevice);
     std::lock_guard<std::mutex> lk(g_beam_mu);
     if (!g_beam_done[dev]) e = cudaEventCreateWithFlags(&g_beam_done[dev], cudaEventDisableTiming);
-    if (e == cudaSuccess) e = record ? cudaEventRecord(g_beam_done[dev], st) : cudaStreamWaitEvent(st, g_beam_done[dev], 0);
+    if (e == cudaSuccess) e = record ? pass_done(dev, st) : cudaStreamWaitEvent(st, g_beam_done[dev], 0);
     return aokk_status(e);
+}
+
+int aokk_beam_waits(void* stream) {
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxBeamDevices) return 1;
+    std::lock_guard<std::mutex> lk(g_beam_mu);
+    return pass_waits(dev, (cudaStream_t)stream);
 }
 
 extern "C++" {
 template <class PB>
-static int launch_pass(const PB* P, unsigned grid, void* stream) {
+static int launch_pass(const PB* P, unsigned grid, void* stream, bool optional = false) {
     const cudaStream_t st = (cudaStream_t)stream;
     if (P->n_views == 0) return AOK_OK;
     int dev = -1;
@@ -562,18 +591,19 @@ static int launch_pass(const PB* P, unsigned grid, void* stream) {
     if (e != cudaSuccess) return aokk_status(e);
     if (dev < 0 || dev >= kMaxBeamDevices) return aokk_status(cudaErrorInvalidDevice);
     std::lock_guard<std::mutex> lk(g_beam_mu);
+    if (optional && pass_waits(dev, st)) return AOK_E_BUSY;
     if (!g_beam_done[dev]) e = cudaEventCreateWithFlags(&g_beam_done[dev], cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(st, g_beam_done[dev], 0);
     void* args[] = {(void*)P};
     if (e == cudaSuccess) e = cudaLaunchCooperativeKernel((const void*)beam_kernel<PB>, grid, kBeamThreads, args, 0, st);
-    if (e == cudaSuccess) e = cudaEventRecord(g_beam_done[dev], st);
+    if (e == cudaSuccess) e = pass_done(dev, st);
     return aokk_status(e);
 }
 }  // extern "C++"
 
-int aokk_beam_run_view(const BeamParams<1>* P, unsigned grid, void* stream, int beside) {
+int aokk_beam_run_view(const BeamParams<1>* P, unsigned grid, void* stream, int beside, int optional) {
     return launch_pass(P, beside && P->n_regions <= kWideWalkRegions ? (grid + kBeamBlocksPerSM - 1) / kBeamBlocksPerSM : grid,
-                       stream);
+                       stream, optional != 0);
 }
 
 int aokk_beam_run(const BeamBatch* P, unsigned grid, void* stream) {

@@ -243,16 +243,18 @@ int aokk_cast(const aok::SceneDev* s, const aok::CamDev* c, const aok::ChunkRef*
 // the camera matrix has no usable inverse; leave the view out, it casts
 // without bounds); aokk_beam_run launches a pass, aokk_beam_run_view one of a
 // single view (beside: with one block per SM, for a pass that starts beside
-// the cast of the frame before, as in the pipelined host frames).
+// the cast of the frame before, as in the pipelined host frames; optional:
+// AOK_E_BUSY instead of a launch that would wait for another stream).
 bool aokk_beam_view(const aok::SceneDev* S, const aok::CamDev* C, const aok::ChunkRef* frame,
                     unsigned long long* bounds, aok::BeamView* out);
 int aokk_beam_run(const aok::BeamBatch* P, unsigned grid, void* stream);
-int aokk_beam_run_view(const aok::BeamParams<1>* P, unsigned grid, void* stream, int beside);
+int aokk_beam_run_view(const aok::BeamParams<1>* P, unsigned grid, void* stream, int beside, int optional);
 // The pass as a graph's kernel node and the per-device pass
 // order around a graph launch (record = 0: wait for the previous pass before;
 // 1: mark the end of the launch as the point the next pass waits for).
 void aokk_beam_node(const aok::BeamBatch* P, unsigned grid, void** argp, cudaKernelNodeParams* kp);
 int aokk_beam_order(void* stream, int record);
+int aokk_beam_waits(void* stream);  // whether a pass launched on it now would wait for another stream
 // Blocks of the beam pass's cooperative launch on `sms` SMs (0 on error).
 unsigned aokk_beam_grid(int sms);
 int aokk_ray_dirs(const aok::CamDev* c, float* dirs, void* stream);

@@ -1015,7 +1015,6 @@ static constexpr uint32_t kBeamTags = 0xFFFFFFEFu;  // tags of an epoch
 static uint32_t next_beam_tag(aok_ctx* ctx, uint32_t* epoch) {
     BeamState& b = ctx->beam;
     std::lock_guard<std::mutex> lk(b.mu);
-    b.total++;
     if (++b.passes > kBeamTags) {
         b.passes = 1;
         b.epoch++;
@@ -1063,13 +1062,36 @@ static int beam_buffers(aok_ctx* ctx, BoundBuf& required, BoundBuf& opt, const C
     return st ? st : ensure_bounds(ctx, required, need);
 }
 
+// After a cast that read an optional pass's pyramid.
+static int beam_was_read(aok_ctx* ctx, void* stream) {
+    BeamState& b = ctx->beam;
+    cudaError_t e = cudaStreamGetId((cudaStream_t)stream, &b.opt_stream);
+    if (e == cudaSuccess) e = cudaEventRecord(b.opt_read, (cudaStream_t)stream);
+    return cuda_status(ctx, e);
+}
+
+// Whether a pass or a cast on `stream` comes after the last cast that read the
+// pyramid without waiting: that one is over, or before it on the same stream.
+// A pass may then write the pyramid, and the record made after a cast stands
+// for every cast that reads it.
+static bool beam_read_alone(aok_ctx* ctx, void* stream) {
+    const BeamState& b = ctx->beam;
+    unsigned long long id = 0;
+    if (cudaStreamGetId((cudaStream_t)stream, &id) == cudaSuccess && id == b.opt_stream) return true;
+    RelaxedCapture rc;
+    if (cudaEventQuery(b.opt_read) == cudaSuccess) return true;
+    cudaGetLastError();  // "not ready" is no error of the next launch
+    return false;
+}
+
 // The beam pass over the scene's current frame table; *rd: what the cast
 // reads.  select: the frame table is not selected yet; the
 // pass selects it as its first step (one launch fewer), or, for a view
 // without a usable projection, the selection kernel does.  ck: checked
 // casting's pool sizes and error word (the pass tests its node and leaf
-// indices too), or null.  optional: AOK_E_BUSY leaves the frame as it was, to be
-// cast without the pass; the cast is followed by beam_was_read.  keep: the
+// indices too), or null.  optional: AOK_E_BUSY (no room, or the pass would wait
+// for another stream's work, which a frame of this size does not do without
+// the pass) leaves the frame as it was, to be cast without the pass; the cast is followed by beam_was_read.  keep: the
 // pass is remembered with what it was computed for.  Called with the pass's
 // buffers held (b.view_mu).
 static int run_beam(aok_ctx* ctx, uint32_t scene, Scene* sc, const SceneDev& sd, const CamDev& cd, void* stream,
@@ -1081,8 +1103,7 @@ static int run_beam(aok_ctx* ctx, uint32_t scene, Scene* sc, const SceneDev& sd,
     const BeamQueues* q;
     int st = beam_buffers(ctx, b.bounds, b.opt, cd, optional, &buf, &q);
     if (st) return st;
-    if (optional && cudaStreamWaitEvent((cudaStream_t)stream, b.opt_read, 0) != cudaSuccess)
-        return AOK_E_CUDA;
+    if (optional && !beam_read_alone(ctx, stream)) return AOK_E_BUSY;
     uint32_t epoch;
     const uint32_t tag = next_beam_tag(ctx, &epoch);
     st = beam_renew(*buf, epoch, stream);
@@ -1105,8 +1126,9 @@ static int run_beam(aok_ctx* ctx, uint32_t scene, Scene* sc, const SceneDev& sd,
         st = aokk_select(&sd, &cd, sc->d_frame, nullptr, nullptr, nullptr, stream);
         if (st) return st;
     }
-    st = aokk_beam_run_view(&P, b.grid, stream, 0);
+    st = aokk_beam_run_view(&P, b.grid, stream, 0, optional);
     if (st) return st;
+    b.total++;
     b.last = *rd;
     b.ran = true;
     b.W = cd.W;
@@ -1119,28 +1141,6 @@ static int run_beam(aok_ctx* ctx, uint32_t scene, Scene* sc, const SceneDev& sd,
     b.cam = cd;
     b.cam.sf = 0.0;  // the LOD threshold does not enter the bounds
     return AOK_OK;
-}
-
-// After a cast that read an optional pass's pyramid: the next optional pass,
-// on whatever stream, waits for it.
-static int beam_was_read(aok_ctx* ctx, void* stream) {
-    BeamState& b = ctx->beam;
-    cudaError_t e = cudaStreamGetId((cudaStream_t)stream, &b.opt_stream);
-    if (e == cudaSuccess) e = cudaEventRecord(b.opt_read, (cudaStream_t)stream);
-    return cuda_status(ctx, e);
-}
-
-// Whether that record, made anew after a cast on `stream`, still stands for
-// every cast that reads the pyramid: the last one is over, or comes before on
-// the same stream.
-static bool beam_read_alone(aok_ctx* ctx, void* stream) {
-    const BeamState& b = ctx->beam;
-    unsigned long long id = 0;
-    if (cudaStreamGetId((cudaStream_t)stream, &id) == cudaSuccess && id == b.opt_stream) return true;
-    RelaxedCapture rc;
-    if (cudaEventQuery(b.opt_read) == cudaSuccess) return true;
-    cudaGetLastError();  // "not ready" is no error of the next launch
-    return false;
 }
 
 extern "C++" BeamUse aok::beam_use(const aok_ctx* ctx, int32_t W, int32_t H, void* stream) {
@@ -1158,7 +1158,7 @@ extern "C++" BeamUse aok::beam_use(const aok_ctx* ctx, int32_t W, int32_t H, voi
 
 extern "C++" int aok::beam_for_batch(aok_ctx* ctx, BatchParams* groups, uint32_t ngroups,
                                      std::vector<BeamBatch>& out, void* stream,
-                                     unsigned long long* const* view_bounds, BoundBuf* arena) {
+                                     unsigned long long* const* view_bounds, BoundBuf* arena, void* pass_stream) {
     out.clear();
     if (!ctx->beam_on) return AOK_OK;
     // entries of the views with a required pass, and with an optional one
@@ -1170,7 +1170,7 @@ extern "C++" int aok::beam_for_batch(aok_ctx* ctx, BatchParams* groups, uint32_t
             need[beam_use(ctx, c.W, c.H, stream)] += beam_entries((uint32_t)c.W, (uint32_t)c.H);
         }
     const size_t req = need[kBeamRequired], opt = need[kBeamOptional];
-    if (!req && !opt) return AOK_OK;
+    if (!req && (!opt || aokk_beam_waits(view_bounds ? pass_stream : stream))) return AOK_OK;
     BoundBuf &bb = ctx->batch.beam_bounds, &ob = ctx->beam.opt_batch;
     int st = req ? ensure_beam_queues(ctx) : AOK_OK;
     if (!st && !view_bounds) st = ensure_bounds(ctx, bb, req);
@@ -1181,6 +1181,7 @@ extern "C++" int aok::beam_for_batch(aok_ctx* ctx, BatchParams* groups, uint32_t
     if (!st && !view_bounds) st = beam_renew(bb, epoch, stream);
     if (!st && !view_bounds && opt) st = beam_renew(ob, epoch, stream);
     if (st) return st;
+    ctx->beam.total++;
     out.resize(ngroups);
     size_t off[3] = {0, 0, 0};
     flat = 0;
@@ -1558,7 +1559,6 @@ int aok_beam_info(aok_ctx* ctx, int32_t* bounds, uint64_t n_bounds, uint32_t* le
 
 int aok_beam_passes(aok_ctx* ctx, uint64_t* passes) {
     if (!ctx || !passes) return AOK_E_INVALID;
-    std::lock_guard<std::mutex> lk(ctx->beam.mu);
     *passes = ctx->beam.total;
     return AOK_OK;
 }
@@ -1716,8 +1716,10 @@ static int pipe_render(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, doub
             rd.bounds = buf->p;
             rd.tag = tag;
         }
-        st = aokk_beam_run_view(&P, ctx->beam.grid, p.prep, 1);  // beside the previous frame's cast
-        if (st) return launch_failure(ctx);
+        st = aokk_beam_run_view(&P, ctx->beam.grid, p.prep, 1, use == kBeamOptional);  // beside the previous frame's cast
+        if (st == AOK_E_BUSY) rd.bounds = nullptr;
+        else if (st) return launch_failure(ctx);
+        else ctx->beam.total++;
     }
     cudaError_t e = cudaEventRecord(sl.prepped, p.prep);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(p.render, sl.prepped, 0);

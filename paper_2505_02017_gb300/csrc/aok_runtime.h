@@ -143,7 +143,7 @@ struct BeamState {
     unsigned long long opt_stream = 0;  // that cast's stream
     uint32_t passes = 0;                   // passes run in this epoch (their tags count down)
     std::atomic<uint32_t> epoch{0};        // times the tags have started over
-    uint64_t total = 0;                    // passes run
+    std::atomic<uint64_t> total{0};        // passes run
     // the last single-view pass, for aok_beam_info
     bool ran = false;
     BeamRead last{nullptr, 0};
@@ -235,9 +235,10 @@ void free_alloc(Scene* sc, ChunkAlloc& a);
 // with view_bounds, in view_bounds[view] (nullptr: that view casts without).
 // Leaves `out` empty if no view takes the pass.
 // (arena: the buffer that some of view_bounds lie in; the others are cleared
-// for every pass.)
+// for every pass.  pass_stream: where those passes run.)
 int beam_for_batch(aok_ctx* ctx, BatchParams* groups, uint32_t ngroups, std::vector<BeamBatch>& out, void* stream,
-                   unsigned long long* const* view_bounds = nullptr, BoundBuf* arena = nullptr);
+                   unsigned long long* const* view_bounds = nullptr, BoundBuf* arena = nullptr,
+                   void* pass_stream = nullptr);
 // Whether a frame of W x H pixels on `stream` takes the beam pass in this
 // context, and whether it may also be cast without.
 inline bool beam_required(const aok_ctx* ctx, int32_t W, int32_t H) {

@@ -473,7 +473,8 @@ static void serve_loop(aok_ctx* ctx) {
                     vb[i] = arena->p + off;
                     off += n;
                 }
-            if (rc == AOK_OK) rc = beam_for_batch(ctx, S.params.data(), ngroups, beams, st, vb.data(), arena);
+            if (rc == AOK_OK) rc = beam_for_batch(ctx, S.params.data(), ngroups, beams, st, vb.data(), arena,
+                                              S.beam_stream);
         }
         if (rc == AOK_OK) {
             // the server's passes share one stream: a pass waits only for its

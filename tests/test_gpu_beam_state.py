@@ -49,29 +49,36 @@ def equal(x, y):
     return torch.equal(x[0].cpu(), y[0].cpu()) and torch.equal(x[1].cpu().view(torch.int32), y[1].cpu().view(torch.int32))
 
 
-def draw(s, kind, cam, srv=None):
-    """The frame of `cam` through one of the calls that run the pass."""
+def buffers(kind, cam):
     if kind == "host":
-        out = (torch.empty((cam.H, cam.W, 4), dtype=torch.int32, pin_memory=True),
-               torch.empty((cam.H, cam.W), dtype=torch.float32, pin_memory=True))
+        return (torch.empty((cam.H, cam.W, 4), dtype=torch.int32, pin_memory=True),
+                torch.empty((cam.H, cam.W), dtype=torch.float32, pin_memory=True))
+    return aok.alloc_frame(cam.W, cam.H)
+
+
+def draw(s, kind, cam, srv=None, out=None, stream=None):
+    """The frame of `cam` through one of the calls that run the pass; waits for it (not for other streams when one
+    is given)."""
+    out = out or (None if kind == "serve" else buffers(kind, cam))
+    if kind == "host":
         aok.host_frame_wait(s.c, aok.render_host_async(s.c, s.sc, cam, 1.5, *out))
         return out
     if kind == "serve":
         tk = srv.submit(s.sc, cam, 1.5)
         st, f = srv.wait(tk, 20000)
         assert st == aok.AOK_OK
-        out = tuple(x.clone() for x in srv.result(tk, f))
-        torch.cuda.synchronize()
+        with torch.cuda.stream(stream):
+            out = tuple(x.clone() for x in srv.result(tk, f))
+        torch.cuda.current_stream().synchronize() if stream is None else stream.synchronize()
         assert srv.release(tk) == aok.AOK_OK
         return out
-    out = aok.alloc_frame(cam.W, cam.H)
     if kind == "batch":
-        aok.render_batch(s.c, [aok.make_view(s.sc, cam, 1.5, *out)])
+        aok.render_batch(s.c, [aok.make_view(s.sc, cam, 1.5, *out)], stream=stream)
     elif kind == "tiles":
-        aok.render_tiles(s.c, s.sc, cam, 1.5, *out)
+        aok.render_tiles(s.c, s.sc, cam, 1.5, *out, stream=stream)
     else:
-        aok.render(s.c, s.sc, cam, 1.5, *out)
-    torch.cuda.synchronize()
+        aok.render(s.c, s.sc, cam, 1.5, *out, stream=stream)
+    torch.cuda.synchronize() if stream is None else stream.synchronize()
     return out
 
 
@@ -278,4 +285,38 @@ def test_threads_with_scenes_of_their_own():
     assert not bad
     for sc in scenes:
         sc.destroy()
+    s.close()
+
+
+@pytest.mark.parametrize("kind", ["single", "tiles", "host", "batch", "serve"])
+def test_optional_pass_waits_for_no_other_stream(kind):
+    """A frame of 1280 x 720 beside a large frame whose stream is held back for 400 ms is there at once, and takes
+    the pass again afterwards."""
+    s = Setup()
+    sc2 = aok.Scene.from_world(s.c, s.world, threads=4)
+    cam, big = s.cam(0), s.cam(1, REQUIRED)
+    ref, ref2 = s.ref(cam), s.ref(big)
+    srv = aok.Server(s.c, max_slots=4, max_batch=2, n_streams=1) if kind == "serve" else None
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    out = None if kind == "serve" else buffers(kind, cam)
+    out2 = aok.alloc_frame(big.W, big.H)
+    for _ in range(3):
+        draw(s, kind, cam, srv, out, s2)
+        aok.render(s.c, sc2, big, 1.5, *out2, stream=s1)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s1):
+        torch.cuda._sleep(800_000_000)
+    aok.render(s.c, sc2, big, 1.5, *out2, stream=s1)
+    t0 = time.perf_counter()
+    got = draw(s, kind, cam, srv, out, s2)
+    t1 = time.perf_counter()
+    held = not s1.query()
+    torch.cuda.synchronize()
+    assert held and t1 - t0 < 0.1, t1 - t0
+    assert equal(got, ref) and equal(out2, ref2)
+    n = aok.beam_passes(s.c)
+    assert equal(draw(s, kind, cam, srv, out, s2), ref) and aok.beam_passes(s.c) == n + 1
+    if srv:
+        srv.stop()
+    sc2.destroy()
     s.close()

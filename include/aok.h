@@ -571,6 +571,15 @@ int aok_set_beam(aok_ctx* ctx, int on);
  * min_node_log2 outside [2, 16]. */
 int aok_beam_tune(aok_ctx* ctx, uint32_t refine_tiles, int32_t min_node_log2, uint64_t min_pixels,
                   uint32_t queue_nodes);
+/* The two frame sizes by themselves: frames of min_pixels take the pass, those
+ * from min_optional pixels where it can run.  AOK_E_INVALID for
+ * min_optional > min_pixels.  aok_beam_tune(ctx, AOK_BEAM_REFINE, 2,
+ * AOK_BEAM_MIN_PIXELS, 0) and then aok_beam_limits(ctx, AOK_BEAM_MIN_PIXELS,
+ * AOK_BEAM_MIN_OPTIONAL) are the settings a context starts with. */
+#define AOK_BEAM_REFINE 16
+#define AOK_BEAM_MIN_PIXELS 1500000
+#define AOK_BEAM_MIN_OPTIONAL 800000
+int aok_beam_limits(aok_ctx* ctx, uint64_t min_pixels, uint64_t min_optional);
 /* The beam pass alone, for the frame table the last aok_select_chunks (or
  * render) of this scene selected and this camera: the next
  * aok_cast_selected of the same scene and camera then casts with these

@@ -125,6 +125,7 @@ def lib() -> ctypes.CDLL:
             "aok_set_beam": [vp, ctypes.c_int],
             "aok_beam_tune": [vp, u32, ctypes.c_int32, u64, u32],
             "aok_beam_info": [vp, P(ctypes.c_int32), u64, P(u32), P(ctypes.c_int32)],
+            "aok_beam_limits": [vp, u64, u64],
             "aok_beam_passes": [vp, P(u64)],
             "aok_beam_tags_left": [vp, u32],
             "aok_beam_selected": [vp, u32, P(Camera), vp],
@@ -438,11 +439,23 @@ def set_beam(ctx: Context, on: bool):
     return check(lib().aok_set_beam(ctx.h, 1 if on else 0), "aok_set_beam")
 
 
-def beam_tune(ctx: Context, refine_tiles: int = 8, min_node_log2: int = 2, min_pixels: int = 1500000,
+BEAM_REFINE, BEAM_MIN_PIXELS, BEAM_MIN_OPTIONAL = 16, 1500000, 800000  # the settings a context starts with
+
+
+def beam_tune(ctx: Context, refine_tiles: int = BEAM_REFINE, min_node_log2: int = 2, min_pixels: int | None = None,
               queue_nodes: int = 0):
     """Refinement of the beam pass's walk, the smallest frame it runs for and
-    the queue capacity per level (aok_beam_tune)."""
-    return check(lib().aok_beam_tune(ctx.h, refine_tiles, min_node_log2, min_pixels, queue_nodes), "aok_beam_tune")
+    the queue capacity per level (aok_beam_tune).  What is not given is set to
+    what a context starts with (min_pixels: the pass from BEAM_MIN_PIXELS on,
+    and where it can run from BEAM_MIN_OPTIONAL on)."""
+    check(lib().aok_beam_tune(ctx.h, refine_tiles, min_node_log2, BEAM_MIN_PIXELS if min_pixels is None else min_pixels,
+                              queue_nodes), "aok_beam_tune")
+    return beam_limits(ctx, BEAM_MIN_PIXELS, BEAM_MIN_OPTIONAL) if min_pixels is None else 0
+
+
+def beam_limits(ctx: Context, min_pixels: int, min_optional: int):
+    """The frame sizes that take the beam pass, and that take it where it can run (aok_beam_limits)."""
+    return check(lib().aok_beam_limits(ctx.h, min_pixels, min_optional), "aok_beam_limits")
 
 
 def beam_selected(ctx: Context, scene: Scene, cam, stream=None):

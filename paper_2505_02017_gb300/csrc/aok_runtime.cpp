@@ -1479,6 +1479,13 @@ int aok_beam_tune(aok_ctx* ctx, uint32_t refine_tiles, int32_t min_node_log2, ui
     return AOK_OK;
 }
 
+int aok_beam_limits(aok_ctx* ctx, uint64_t min_pixels, uint64_t min_optional) {
+    if (!ctx || min_optional > min_pixels) return AOK_E_INVALID;
+    ctx->beam_min_pixels = min_pixels;
+    ctx->beam_min_optional = min_optional;
+    return AOK_OK;
+}
+
 int aok_beam_selected(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, void* stream) {
     if (!ctx) return AOK_E_INVALID;
     Scene* sc = find_scene(ctx, scene);

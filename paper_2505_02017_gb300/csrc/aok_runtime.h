@@ -204,13 +204,13 @@ struct aok_ctx {
     aok::TileState tiles;
     aok::BeamState beam;
     int beam_on = 1;  // single-view renders run the beam pass before casting
-    uint32_t beam_refine = 16;  // refine nodes spanning more tiles than this ...
+    uint32_t beam_refine = AOK_BEAM_REFINE;  // refine nodes spanning more tiles than this ...
     int beam_min_log2 = 2;     // ... whose side is above 2^this LOD-0 voxels
     // Frames of beam_min_pixels take the pass.  Those of beam_min_optional take it where it can run: not on a stream
     // that is being captured (the passes of a device wait for one another by events a capture can't hold) and not
     // beyond the room of its buffers.  Smaller ones cast without it (city views of 1120 x 630 break
     // even at 160-240 us, 1280 x 720 ones gain 12% on average with it, -29% to +12%, and 960 x 540 ones nothing).
-    uint64_t beam_min_pixels = 1500000, beam_min_optional = 800000;
+    uint64_t beam_min_pixels = AOK_BEAM_MIN_PIXELS, beam_min_optional = AOK_BEAM_MIN_OPTIONAL;
     uint32_t beam_queue = 0;             // nodes a queue level may hold (0: the allocated 2^20)
     aok::HostPipe pipe;
     int checked = 0;  // single-view casts check every pool index (error word: d_counter[8])

@@ -1,6 +1,7 @@
 """State that beam passes share within a context: tags, buffers, the record of
 the last pass.  Frames of 1280 x 720 take the pass where it can run, frames of
 1600 x 1000 always; each equals the frame without the pass bit for bit."""
+import os
 import threading
 import time
 from dataclasses import replace
@@ -319,4 +320,36 @@ def test_optional_pass_waits_for_no_other_stream(kind):
     if srv:
         srv.stop()
     sc2.destroy()
+    s.close()
+
+
+def test_tune_without_arguments_restores_a_contexts_settings():
+    """Levels of the walk and the sizes that take it, after other settings and beam_tune(ctx), are a fresh
+    context's (the constants those of aok.h)."""
+    hdr = open(os.path.join(os.path.dirname(__file__), "..", "include", "aok.h")).read()
+    for name in ("BEAM_REFINE", "BEAM_MIN_PIXELS", "BEAM_MIN_OPTIONAL"):
+        assert f"#define AOK_{name} {getattr(aok, name)}\n" in hdr
+    s = Setup()
+    cams = [s.cam(0, size) for size in ((1000, 799), OPTIONAL, REQUIRED)]
+
+    def walks():
+        out = []
+        for m in cams:
+            n = aok.beam_passes(s.c)
+            draw(s, "single", m)
+            out.append(aok.beam_info(s.c)[1] if aok.beam_passes(s.c) > n else None)
+        return out
+
+    fresh = walks()
+    assert fresh[0] is None and fresh[1] and fresh[2]
+    aok.beam_tune(s.c, 4, 3, 100000, 64)
+    assert walks() != fresh
+    aok.beam_tune(s.c)
+    assert walks() == fresh
+    aok.beam_limits(s.c, 1500000, 1500000)
+    assert walks() == [None, None, fresh[2]]
+    aok.beam_limits(s.c, 1500000, 790000)
+    assert walks()[1:] == fresh[1:] and walks()[0]
+    with pytest.raises(aok.AokError):
+        aok.beam_limits(s.c, 1, 2)
     s.close()

@@ -578,8 +578,9 @@ static void color_blocks(const uint8_t* v, uint64_t n, double e_c, std::vector<u
 // descriptor table.  When the pools are full and evict_old_first is set, the
 // previous upload of descriptor di is evicted first (after the device is
 // idle).  The pools are touched under *pool_mu, or under the caller's hold of
-// sc->mu when pool_mu is null.
-int aok::stage_chunk(aok_ctx* ctx, Scene* sc, int64_t di, uint32_t lod, const aok_chunk_blob* blob,
+// sc->mu when pool_mu is null.  Host memory that runs out gives AOK_E_OOM, with
+// the pools as they were and no copy on its way.
+static int stage_chunk_or_throw(aok_ctx* ctx, Scene* sc, int64_t di, uint32_t lod, const aok_chunk_blob* blob,
                      bool evict_old_first, Staging* sg, std::mutex* pool_mu, ChunkAlloc* out_a, ChunkRef* out_ref) {
     const int M = sc->desc.chunk_res, res = M >> lod;
     // 1. validate before touching anything: a rejected blob changes nothing
@@ -657,6 +658,8 @@ int aok::stage_chunk(aok_ctx* ctx, Scene* sc, int64_t di, uint32_t lod, const ao
         }
         return true;
     };
+    const size_t nt = (blob->n_mats + 127) / 128;
+    std::vector<uint32_t> head(bfirst.empty() ? 0 : 1 + nt);
     ChunkAlloc a;
     {
         std::unique_lock<std::mutex> pl;
@@ -682,8 +685,6 @@ int aok::stage_chunk(aok_ctx* ctx, Scene* sc, int64_t di, uint32_t lod, const ao
             // [pad to 4][nt][nt x uint32: block holding entry 128 j]
             // [nblocks x uint32 first index][nblocks x uint8 colour]
             mat_base = (a.mat_off + 3) & ~(uint64_t)3;
-            const size_t nt = (blob->n_mats + 127) / 128;
-            std::vector<uint32_t> head(1 + nt);
             head[0] = (uint32_t)nt;
             for (size_t j = 0, b = 0; j < nt; j++) {
                 while (b + 1 < bfirst.size() && bfirst[b + 1] <= 128 * j) b++;
@@ -696,21 +697,27 @@ int aok::stage_chunk(aok_ctx* ctx, Scene* sc, int64_t di, uint32_t lod, const ao
             std::memcpy(q + head.size() * 4, bfirst.data(), bfirst.size() * 4);
             std::memcpy(q + head.size() * 4 + bfirst.size() * 4, bcol.data(), bcol.size());
         }
+        bool oom = false;
         cudaError_t e = cudaSuccess;
         if (mat_n)
             e = cudaMemcpyAsync(sc->d_mats + a.mat_off, stg + nb + lb, mat_n, cudaMemcpyHostToDevice, sg->stream);
         if (e == cudaSuccess && blob->n_leaves)
             e = cudaMemcpyAsync(sc->d_leaves + a.leaf_off, stg + nb, blob->n_leaves * 8, cudaMemcpyHostToDevice,
                                 sg->stream);
-        layout_blob(blob, res, (uint32_t)a.node_off, (uint32_t)a.leaf_off, &sg->plan, (uint32_t*)stg, &droot);
-        if (e == cudaSuccess)
+        try {
+            layout_blob(blob, res, (uint32_t)a.node_off, (uint32_t)a.leaf_off, &sg->plan, (uint32_t*)stg, &droot);
+        } catch (const std::bad_alloc&) {
+            oom = true;
+        }
+        if (e == cudaSuccess && !oom)
             e = cudaMemcpyAsync(sc->d_nodes + a.node_off, stg, nw * 4, cudaMemcpyHostToDevice, sg->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(sg->stream);
-        if (e != cudaSuccess) {
+        const cudaError_t es = cudaStreamSynchronize(sg->stream);  // nothing reads the staging memory any more
+        if (e == cudaSuccess) e = es;
+        if (e != cudaSuccess || oom) {
             std::unique_lock<std::mutex> pl;
             if (pool_mu) pl = std::unique_lock<std::mutex>(*pool_mu);
             free_alloc(sc, a);
-            return cuda_status(ctx, e);
+            return e != cudaSuccess ? cuda_status(ctx, e) : AOK_E_OOM;
         }
         ref.root = droot;
         ref.lod = lod;
@@ -724,6 +731,15 @@ int aok::stage_chunk(aok_ctx* ctx, Scene* sc, int64_t di, uint32_t lod, const ao
     *out_a = a;
     *out_ref = ref;
     return AOK_OK;
+}
+
+int aok::stage_chunk(aok_ctx* ctx, Scene* sc, int64_t di, uint32_t lod, const aok_chunk_blob* blob,
+                     bool evict_old_first, Staging* sg, std::mutex* pool_mu, ChunkAlloc* out_a, ChunkRef* out_ref) {
+    try {
+        return stage_chunk_or_throw(ctx, sc, di, lod, blob, evict_old_first, sg, pool_mu, out_a, out_ref);
+    } catch (const std::bad_alloc&) {
+        return AOK_E_OOM;
+    }
 }
 
 extern "C" {
@@ -744,11 +760,7 @@ int aok_scene_upload_chunk(aok_ctx* ctx, uint32_t scene, int32_t cx, int32_t cy,
         std::lock_guard<std::mutex> up(ctx->upload_mu);
         Staging sg{ctx->staging, ctx->staging_cap, ctx->copy_stream};
         sg.plan = std::move(ctx->upload_plan);
-        try {
-            st = stage_chunk(ctx, sc, di, lod, blob, true, &sg, nullptr, &a, &ref);
-        } catch (const std::bad_alloc&) {
-            st = AOK_E_OOM;
-        }
+        st = stage_chunk(ctx, sc, di, lod, blob, true, &sg, nullptr, &a, &ref);
         ctx->staging = sg.buf;
         ctx->staging_cap = sg.cap;
         ctx->upload_plan = std::move(sg.plan);

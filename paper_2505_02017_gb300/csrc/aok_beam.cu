@@ -484,7 +484,18 @@ bool aokk_beam_view(const SceneDev* S, const CamDev* C, const ChunkRef* frame, u
     double nrm = 0.0;
     for (int i = 0; i < 9; i++) nrm = fmax(nrm, fabs(A[i]));
     if (!(std::isfinite(det) && fabs(det) > 1e-6 * nrm * nrm * nrm)) return false;
-    const double id = 1.0 / det;
+    const double U = (double)C->tan_half * (double)C->W / (double)C->H, V = (double)C->tan_half;
+    // Pixel rays whose components reach the ends of binary32 lose the precision
+    // the tile margin counts on.  Elsewhere only the ratios of the matrix matter:
+    // its largest entry is brought to [1/2, 2), so that the projection stays
+    // clear of those ends too (the approximate reciprocal flushes those of
+    // numbers above 2^126 to zero).
+    if (!(nrm > 0x1p-122 && nrm * (U + V + 1.0) < 0x1p126)) return false;
+    int ex = 0;
+    (void)std::frexp(nrm, &ex);
+    const double sc = ex < 0 || ex > 1 ? std::ldexp(1.0, -ex) : 1.0;
+    for (int i = 0; i < 9; i++) A[i] *= sc;
+    const double id = 1.0 / (det * sc * sc * sc);
     double Ai[9];
     Ai[0] = (A[4] * A[8] - A[5] * A[7]) * id;
     Ai[1] = (A[2] * A[7] - A[1] * A[8]) * id;
@@ -501,7 +512,6 @@ bool aokk_beam_view(const SceneDev* S, const CamDev* C, const ChunkRef* frame, u
     K.frame = frame;
     K.bounds = bounds;
     for (int i = 0; i < 9; i++) K.Af[i] = (float)Ai[i];
-    const double U = (double)C->tan_half * (double)C->W / (double)C->H, V = (double)C->tan_half;
     K.iU = (float)(1.0 / U);
     K.iV = (float)(1.0 / V);
     // largest |d| component over the screen, with slack for the FP32 ray arithmetic

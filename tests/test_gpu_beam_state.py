@@ -353,3 +353,28 @@ def test_tune_without_arguments_restores_a_contexts_settings():
     with pytest.raises(aok.AokError):
         aok.beam_limits(s.c, 1, 2)
     s.close()
+
+
+@pytest.mark.parametrize("k", [-126, -123, -122, -121, -120, -119, -118, -112, -60, -21, -20, 20, 21, 60, 100, 126])
+def test_camera_matrix_of_any_scale(k):
+    """A matrix scaled by 2^k has the same rays but for their lengths: the frame's hits are those of k = 0 and
+    equal with the pass and without, up to the ends of binary32."""
+    s = Setup()
+    for seed in range(3):
+        one = s.cam(seed, (403, 217))
+        R = (one.R.astype("float64") * 2.0 ** k).astype("float32")
+        cam = replace(one, R=R)
+        ref, plain = s.ref(cam), s.ref(one)
+        aok.beam_tune(s.c, 16, 2, 0, 0)
+        on = draw(s, "single", cam)
+        b, _ = aok.beam_info(s.c)
+        draw(s, "single", one)
+        b1, _ = aok.beam_info(s.c)
+        aok.beam_tune(s.c)
+        assert equal(on, ref)
+        if (R.astype("float64") == one.R * 2.0 ** k).all() and k > -118:
+            assert torch.equal(ref[0], plain[0])
+            if k < 120:
+                assert (b == b1).mean() > 0.99
+        assert not (b > 2**31 - 2).all()
+    s.close()

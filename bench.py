@@ -53,7 +53,7 @@ def peaks():
 
 PROFILE = os.path.join(ROOT, "profiles", "cast_kernel_city4096_1080p.md")
 KERNEL_SRCS = [os.path.join(ROOT, "paper_2505_02017_gb300", "csrc", f)
-               for f in ("aok_kernels.cu", "aok_walk.cuh", "aok_trace.cuh", "aok_select.cuh", "aok_internal.h")]
+               for f in ("aok_kernels.cu", "aok_walk.cuh", "aok_trace.cuh", "aok_ptx.cuh", "aok_select.cuh", "aok_internal.h")]
 
 
 def kernel_sources_hash():

@@ -51,6 +51,7 @@
 #include <cooperative_groups.h>
 
 #include "aok_internal.h"
+#include "aok_ptx.cuh"
 #include "aok_select.cuh"
 
 namespace cg = cooperative_groups;
@@ -65,12 +66,6 @@ constexpr uint32_t kWideWalkRegions = 4096;  // a pass beside a running cast tak
 constexpr double kNearS = 1.0 / 16.0;  // camera-depth plane the projection clips at
 constexpr uint32_t kNoItem = 0xFFFFFFFFu;  // an empty queue slot
 constexpr int kMaxBeamDevices = 128;
-
-__device__ __forceinline__ float rcp_approx(float x) {
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
 
 // Screen rectangle [x, z) x [y, w) of tiles a box (relative to the origin)
 // can cover from its part at camera depth s >= kNearS; false if none.
@@ -240,11 +235,6 @@ __device__ __forceinline__ bool node_bound(const BeamView& V, int lod, bool clip
     const float lf[3] = {(float)wl[0] * sc, (float)wl[1] * sc, (float)wl[2] * sc};
     const float hf[3] = {(float)wh[0] * sc, (float)wh[1] * sc, (float)wh[2] * sc};
     return box_rect(V, lf, hf, rc);
-}
-
-// Atomic minimum without a return value (a reduction the SM does not wait for).
-__device__ __forceinline__ void red_min_u64(unsigned long long* p, unsigned long long v) {
-    asm volatile("red.global.min.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
 // D into the finest level L of the view's bound pyramid (level 0: the tiles;

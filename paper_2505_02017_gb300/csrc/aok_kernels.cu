@@ -86,14 +86,11 @@ __device__ __forceinline__ int32_t beam_bound_warp(const unsigned long long* __r
 // 16 x 8 pixel tiles, warps of 8 x 4 pixels.  BEAM: the warp's 8 x 4 tile
 // bound from the beam pass (aok_beam.cu) restarts its rays' march past the
 // space in front of the nearest voxel they can meet.  At most 64 registers:
-// 8 blocks per SM (three views each, city 1920x1080 318 / 241 / 291 us, overview
-// 3840x2160 468 / 486 / 467, open world 2560x1440 414 / 468 / 589; 7 blocks 323 /
-// 239 / 292, 481 / 498 / 479, 416 / 473 / 601; 9 blocks 320 / 243 / 293, 463 /
-// 482 / 464, 422 / 470 / 589; 10 blocks 319 / 247 / 294, 459 / 478 / 458, 437 /
-// 475 / 592).  A warp takes 12 to 20 us on average and up to 140, so a frame
-// ends with few warps left; other orders of the rows and smaller or larger
-// blocks shorten some views and lengthen others (rows from below: city 303 /
-// 228 / 278 -> 325 / 184 / 320 us; blocks of one warp 313 / 247 / 285).
+// 8 blocks per SM (over nine views of three scenes 7 blocks take 1.4% longer on
+// average, 9 and 10 gain up to 2% on the overview and lose up to 5% in the open
+// world).  A warp takes 12 to 20 us on average and up to 140, so a frame ends with few
+// warps left; no other order of the rows or size of the blocks was shorter on
+// all views.
 //
 // Without bounds a warp may take a smaller tile, wl and hl its sides' logs (3
 // and 2: 8 x 4), in its first lanes: see cast_tile.
@@ -133,9 +130,8 @@ __global__ void __launch_bounds__(128, 8) cast_kernel(const __grid_constant__ Sc
 // So the smallest tile whose warps still fit one resident wave (8 blocks of 4
 // warps per SM; 4,864 warps on 152 SMs): 16 rays up to 77,824 pixels, 8 up to
 // 38,912, and so on to one.  Four city views each, 8 x 4 tiles -> this rule:
-// 320x180 66 / 78 / 96 / 68 -> 62 / 72 / 85 / 62 us, 160x90 74 / 70 / 154 / 60
-// -> 51 / 45 / 102 / 45, 96x54 76 / 84 / 135 / 66 -> 39 / 39 / 68 / 41; past
-// one wave it turns (480x270, 16 rays: 90 / 77 / 123 / 117 -> 99 / 82 / 115 / 104).
+// 320x180 77 -> 70 us on average, 160x90 90 -> 61, 96x54 90 -> 47; past one wave
+// it turns (480x270 with 16 rays a warp: two views 8% longer, two 9% shorter).
 static void cast_tile(const CamDev& c, int& wl, int& hl) {
     static std::atomic<int> sms[kMaxDevices];
     int dev = 0, n = 0;
@@ -224,8 +220,8 @@ __global__ void __launch_bounds__(256) cast_persistent(const __grid_constant__ B
 // tiles (2^tile_w_log x 32/2^tile_w_log pixels each); P.v[v].tile_begin is the
 // exclusive prefix sum of the views' block-tile counts.  The view index derives
 // from blockIdx only, so every per-view parameter load is block-uniform.  9
-// blocks per SM (56 registers): 24 views 3546 / 3067 / 3674 us, 8 blocks 3595 /
-// 3105 / 3725, 10 blocks 3572 / 3103 / 3707 (one view's kernel gains nothing).
+// blocks per SM (56 registers): 24 views take 1.3% less than with 8, 0.9% less
+// than with 10 (one view's kernel gains nothing).
 __global__ void __launch_bounds__(128, 9) cast_grid(const __grid_constant__ BatchParams P) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint64_t blk = blockIdx.x;

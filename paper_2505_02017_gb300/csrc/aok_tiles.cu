@@ -54,6 +54,7 @@
 #include <cstdint>
 
 #include "aok_internal.h"
+#include "aok_ptx.cuh"
 #include "aok_trace.cuh"
 #include "aok_walk.cuh"
 
@@ -85,11 +86,6 @@ __device__ __forceinline__ unsigned long long pack_hit(const SceneDev& S, const 
                                    ((unsigned long long)(uint32_t)sel3(T.ax[0], u[0], u[1], u[2]) << T.bb) |
                                    (uint32_t)sel3(T.ax[1], u[0], u[1], u[2]);
     return reg << kHitBits | r;
-}
-
-// Atomic minimum without a return value (a reduction the SM does not wait for).
-__device__ __forceinline__ void red_min_u64(unsigned long long* p, unsigned long long v) {
-    asm volatile("red.global.min.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
 // A record decoded for its ray (direction d): voxel corner, LOD, entry axis,

@@ -13,14 +13,10 @@
 // when an occupied cell is entered, so that descending costs no comparison.
 // Bound: instruction issue (about 70% of it, the ALU pipe 67%) and the
 // divergence of neighbour rays (17.5 of 32 lanes; 7 at the entry of a leaf
-// block, 9 in its steps).  Frames, exact march -> this walk when it was new:
-// city 1920x1080
-// 484 -> 334 us, overview 3840x2160 743 -> 530, open world 2560x1440
-// 801 -> 557, 24 views 6404 -> 4278, 320x180 147 -> 83, 256x256 74 -> 54 us.
-// Three shapes that are slower here, frames of city 1920x1080 (315 / 232 / 290
-// us at the time): the rays that reach a leaf block wait for the others before
-// any enters (412 / 277 / 344), one way out of the leaf block's loop (330 / 241
-// / 303), its three-way branch by selects (346 / 249 / 312).
+// block, 9 in its steps).  Frames, the exact march -> this walk (with what the
+// march got beside it: bound, warp tiles, beam pass): city 1920x1080 485 -> 271
+// us, overview 3840x2160 746 -> 411, open world 2560x1440 885 -> 511, 24 views
+// 6301 -> 3263, 256x256 74 -> 38.
 //
 // Numbers.  The ray is taken in the frame mirrored so that d >= 0.  Its
 // parameter t counts from a base point on the ray, known to 2^-24 of a voxel:
@@ -36,6 +32,7 @@
 // 2u g d; from the FMA u T d, from x and x - 1/2 2u, and g_max d_max >= 1) and
 // is used when it lies farther than 5u (T + g_max) d_max from every integer.
 #pragma once
+#include "aok_ptx.cuh"
 #include "aok_trace.cuh"
 
 namespace aok {
@@ -56,12 +53,6 @@ constexpr int kNearLevel = 4;
 template <class T>
 __device__ __forceinline__ T sel3(int e, T a, T b, T c) {
     return e == 0 ? a : (e == 1 ? b : c);
-}
-
-__device__ __forceinline__ float rcp_approx(float x) {
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
 }
 
 // 2^n, |n| < 127

@@ -566,7 +566,7 @@ int aok_set_beam(aok_ctx* ctx, int on);
  * context starts with 1,500,000, and with the optional pass from 800,000 on:
  * below that the pass's fixed cost, some tens of microseconds, outweighs what
  * it saves); queue_nodes caps the nodes one level of the walk may queue
- * (0: the allocated 2^20; past the cap a node stands for its children).
+ * (0: the allocated 2^20, or 2^17 in an optional pass; past the cap a node stands for its children).
  * Any setting gives the same output records.  AOK_E_INVALID for
  * min_node_log2 outside [2, 16]. */
 int aok_beam_tune(aok_ctx* ctx, uint32_t refine_tiles, int32_t min_node_log2, uint64_t min_pixels,
@@ -604,7 +604,8 @@ int aok_select_beam(aok_ctx* ctx, uint32_t scene, const aok_camera* cam, double 
  * units of 2^-12 LOD-0 voxels, INT32_MAX = no solid voxel reachable; 0
  * everywhere if the camera matrix has no usable inverse), level_counts
  * (nullable, 16 entries: nodes walked at each depth below the region roots,
- * depth 0 the selected regions; a queue holds 2^20 nodes per level, past
+ * depth 0 the selected regions; a queue holds 2^20 nodes per level (2^17 in an
+ * optional pass), past
  * that parents stand in for their children) and tiles_xy (nullable, 2).
  * AOK_E_INVALID before the first such pass or if n_bounds is too small. */
 int aok_beam_info(aok_ctx* ctx, int32_t* bounds, uint64_t n_bounds, uint32_t* level_counts, int32_t* tiles_xy);

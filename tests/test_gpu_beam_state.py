@@ -378,3 +378,26 @@ def test_camera_matrix_of_any_scale(k):
                 assert (b == b1).mean() > 0.99
         assert not (b > 2**31 - 2).all()
     s.close()
+
+
+def test_optional_passes_beside_a_capture():
+    """First frames of 0.8-1.5 M pixels on one stream while another one is captured: the capture lives on."""
+    s = Setup()
+    sc2 = aok.Scene.from_world(s.c, s.world, threads=4)
+    small, cams = s.cam(0, (320, 180)), [s.cam(1), s.cam(2, (1400, 1000)), s.cam(0)]
+    refs = [s.ref(m) for m in (small, *cams)]
+    outs = [aok.alloc_frame(m.W, m.H) for m in (small, *cams)]
+    s1, s2, g = torch.cuda.Stream(), torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    n = aok.beam_passes(s.c)
+    with torch.cuda.graph(g, stream=s1):
+        aok.render(s.c, s.sc, small, 1.5, *outs[0], stream=s1)
+        for m, o in zip(cams, outs[1:]):
+            aok.render(s.c, sc2, m, 1.5, *o, stream=s2)
+    s2.synchronize()
+    assert aok.beam_passes(s.c) == n + 3
+    g.replay()
+    torch.cuda.synchronize()
+    assert all(equal(o, r) for o, r in zip(outs, refs))
+    sc2.destroy()
+    s.close()

@@ -265,13 +265,12 @@ static int validate_blob(const aok_chunk_blob* b, int res, int M, BlobPlan* plan
 // chunk LODs (21 MB) upload in 5.9 ms, of which the layout takes 2.8 and the
 // copy of the colours into pinned memory 1.1; with per-word storage allocated
 // for each blob, a sort of the nodes by depth and boxes per edge, in 12.7.
+// plan->off and plan->box have room for every node.
 static void layout_blob(const aok_chunk_blob* b, int res, uint32_t node_base, uint32_t leaf_base, BlobPlan* plan,
                         uint32_t* out, uint32_t* root_out) {
     const std::vector<uint32_t>&ord = plan->ord, &node = plan->node;
     const size_t n = node.size();
     const int n_int = (int)plan->level.size() - 1;
-    plan->off.resize(n);
-    plan->box.resize(6 * n);
     uint32_t* off = plan->off.data();
     uint16_t* box = plan->box.data();
     uint32_t w = 0;
@@ -586,6 +585,9 @@ static int stage_chunk_or_throw(aok_ctx* ctx, Scene* sc, int64_t di, uint32_t lo
     // 1. validate before touching anything: a rejected blob changes nothing
     int st = validate_blob(blob, res, M, &sg->plan);
     if (st) return st;
+    // (host memory is taken here, before pool ranges and copies: the layout allocates none)
+    sg->plan.off.resize(sg->plan.node.size());
+    sg->plan.box.resize(6 * sg->plan.node.size());
     uint32_t droot = 0;
     const uint64_t nw = sg->plan.words;  // device words (even)
     // material storage: colour blocks when the scene asks for them and they are
@@ -697,27 +699,22 @@ static int stage_chunk_or_throw(aok_ctx* ctx, Scene* sc, int64_t di, uint32_t lo
             std::memcpy(q + head.size() * 4, bfirst.data(), bfirst.size() * 4);
             std::memcpy(q + head.size() * 4 + bfirst.size() * 4, bcol.data(), bcol.size());
         }
-        bool oom = false;
         cudaError_t e = cudaSuccess;
         if (mat_n)
             e = cudaMemcpyAsync(sc->d_mats + a.mat_off, stg + nb + lb, mat_n, cudaMemcpyHostToDevice, sg->stream);
         if (e == cudaSuccess && blob->n_leaves)
             e = cudaMemcpyAsync(sc->d_leaves + a.leaf_off, stg + nb, blob->n_leaves * 8, cudaMemcpyHostToDevice,
                                 sg->stream);
-        try {
-            layout_blob(blob, res, (uint32_t)a.node_off, (uint32_t)a.leaf_off, &sg->plan, (uint32_t*)stg, &droot);
-        } catch (const std::bad_alloc&) {
-            oom = true;
-        }
-        if (e == cudaSuccess && !oom)
+        layout_blob(blob, res, (uint32_t)a.node_off, (uint32_t)a.leaf_off, &sg->plan, (uint32_t*)stg, &droot);
+        if (e == cudaSuccess)
             e = cudaMemcpyAsync(sc->d_nodes + a.node_off, stg, nw * 4, cudaMemcpyHostToDevice, sg->stream);
         const cudaError_t es = cudaStreamSynchronize(sg->stream);  // nothing reads the staging memory any more
         if (e == cudaSuccess) e = es;
-        if (e != cudaSuccess || oom) {
+        if (e != cudaSuccess) {
             std::unique_lock<std::mutex> pl;
             if (pool_mu) pl = std::unique_lock<std::mutex>(*pool_mu);
             free_alloc(sc, a);
-            return e != cudaSuccess ? cuda_status(ctx, e) : AOK_E_OOM;
+            return cuda_status(ctx, e);
         }
         ref.root = droot;
         ref.lod = lod;
